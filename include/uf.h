@@ -60,7 +60,11 @@ typedef enum {
 enum { UF_F32 = 0,   /* FP32 fields, FP64 reductions and coarsest MG solve */
        UF_F64 = 1 }; /* FP64 throughout                                     */
 
-enum { UF_PRECOND_MG = 0,      /* geometric multigrid V-cycle (default)       */
+enum { UF_PRECOND_MG = 0,      /* geometric multigrid V-cycle (default); FP32
+                                  grids with the default smoother and transfers
+                                  use the exact inverse by separation of
+                                  variables in its place (uf_tuning.coarse_start
+                                  below): same solution, fewer CG iterations    */
        UF_PRECOND_AI1 = 1,     /* approximate inverse, 1st order (Sec. 3)     */
        UF_PRECOND_JACOBI = 2,
        UF_PRECOND_NONE = 3,
@@ -419,18 +423,26 @@ typedef struct {
                                  BCs and the pressure right-hand side as
                                  three kernels.  Both forms give the same
                                  values bit for bit.  0 = all fused (default) */
-  int coarse_start;           /* first multigrid level of the V-cycle run as one
+  int coarse_start;           /* 0 = automatic: FP32 grids with the default
+                                 smoother (CHEBY) and transfers (LINEAR), nx <=
+                                 1024, ny <= 1392 and nz <= 400 run the exact
+                                 inverse of the operator (separation of
+                                 variables: cosine transforms along y and z,
+                                 tridiagonal solves along x) in place of the
+                                 V-cycle, and the other knobs of the solve
+                                 have no effect; all others run the V-cycle
+                                 with per-level launches.  -1 = the V-cycle
+                                 with per-level launches.  > 0: first
+                                 multigrid level of the V-cycle run as one
                                  thread-block-cluster launch (down legs, the
                                  tail, up legs); the levels above it use one
-                                 launch per level and leg.  0 = automatic
-                                 (per-level launches: on the coarse grids
-                                 measured so far the cluster, which holds
-                                 16 SMs at most, is no faster), -1 =
-                                 per-level launches only.  Both give the same
-                                 values bit for bit */
+                                 launch per level and leg.  -1 and > 0 give
+                                 the same values bit for bit, 0 the same
+                                 solution to the solver's tolerance */
 } uf_tuning;
 
-/* The knobs in use, resolved (no zeros).  levels: number of MG levels. */
+/* The knobs in use, resolved (no zeros, but for coarse_start = 0 where the
+ * separable inverse is in use).  levels: number of MG levels. */
 uf_status uf_get_tuning(uf_grid* g, uf_tuning* out, int* levels);
 
 /* Sets the knobs (NULL: back to automatic) and drops the captured graphs,
@@ -438,8 +450,8 @@ uf_status uf_get_tuning(uf_grid* g, uf_tuning* out, int* levels);
 uf_status uf_set_tuning(uf_grid* g, const uf_tuning* t);
 
 /* Autotuner: times `reps` pressure solves of a fixed synthetic right-hand
- * side from a zero guess for each candidate (tail level x uniform tile
- * depth), keeps the fastest and returns it in *chosen (may be NULL) with its
+ * side from a zero guess for each candidate (the automatic choice, and tail
+ * level x uniform tile depth of the V-cycle), keeps the fastest and returns it in *chosen (may be NULL) with its
  * mean solve time in *best_ms (may be NULL).  Uses only the grid's scratch
  * buffers: the state is untouched.  Synchronises. */
 uf_status uf_autotune(uf_grid* g, int reps, uf_tuning* chosen, double* best_ms);

@@ -69,7 +69,10 @@ struct LaunchMap {
 };
 
 // Launch kinds: one work list each (march levels: one per level).
-enum MapKind { MAP_CFL = 0, MAP_CELL, MAP_FACE, MAP_CHUNK, MAP_TAIL, MAP_ADV, MAP_MARCH0 };
+// MAP_DIR: the march tiles of the finest level, every instance; the V-cycle
+// maps (MAP_TAIL, MAP_MARCH0 ..) hold the instances that run it, the MAP_SEP
+// ones those with the separable inverse.
+enum MapKind { MAP_CFL = 0, MAP_CELL, MAP_FACE, MAP_CHUNK, MAP_TAIL, MAP_ADV, MAP_DIR, MAP_SEPZ, MAP_SEPY, MAP_SEPX, MAP_MARCH0 };
 constexpr int kMaps = MAP_MARCH0 + uf::MAX_LEVELS;
 
 __device__ __forceinline__ int map_entry(const LaunchMap* __restrict__ m, int w) {
@@ -192,6 +195,16 @@ struct MgP {     // V-cycle level kernels
   uf::SolveState* st;
 };
 
+struct SepP {    // separable inverse
+  uf::Level<float> L;
+  uf::Sep S;
+  float* x;
+  const float *d0, *d1, *q;
+  float* z;
+  double* partials;
+  uf::SolveState* st;
+};
+
 // Minimum resident blocks per SM (second __launch_bounds__ argument): the
 // batch's working set exceeds L2, so these kernels wait on DRAM latency and
 // gain from more resident warps; measured on the 32-instance workload, 4
@@ -292,6 +305,27 @@ __global__ void __launch_bounds__(uf::FT, 4) kb_mg_up(const __grid_constant__ Ar
   });
 }
 
+template <bool CG>
+__global__ void __launch_bounds__(uf::SEP_T, 2) kb_sep_zf(const __grid_constant__ Args<SepP> A,
+                                                          cudaGraphConditionalHandle cond, int use_cond, int* left) {
+  for_items(&A.m, [&](int i, int, const VBlock& vb) {
+    const SepP& P = A.at[i];
+    uf::sep_zf_body<CG>(P.L, P.S, P.x, P.d0, P.d1, P.q, P.partials, P.st, cond, use_cond, CG ? left : nullptr, vb);
+  });
+}
+__global__ void __launch_bounds__(uf::SEP_T, 2) kb_sep_y(const __grid_constant__ Args<SepP> A, int inverse) {
+  for_items(&A.m, [&](int i, int, const VBlock& vb) { uf::sep_y_body(A.at[i].L, A.at[i].S, inverse, A.at[i].st, vb); });
+}
+__global__ void __launch_bounds__(32 * uf::SEP_X_LINES) kb_sep_x(const __grid_constant__ Args<SepP> A) {
+  for_items(&A.m, [&](int i, int, const VBlock& vb) { uf::sep_x_body(A.at[i].L, A.at[i].S, A.at[i].st, vb); });
+}
+__global__ void __launch_bounds__(uf::SEP_T, 2) kb_sep_zi(const __grid_constant__ Args<SepP> A, int mode) {
+  for_items(&A.m, [&](int i, int, const VBlock& vb) {
+    const SepP& P = A.at[i];
+    uf::sep_zi_body(P.L, P.S, P.z, mode, P.partials, P.st, vb);
+  });
+}
+
 template <typename T>
 __global__ void __launch_bounds__(uf::NT, 6) kb_pressure_commit(const __grid_constant__ Args<CommitP<T>> A) {
   for_plane_items(&A.m, [&](int i, const VBlock& vb) {
@@ -360,6 +394,7 @@ class BatchImpl final : public uf_batch {
   int n_fixed = 0, n_iter = 0, max_levels = 0;
   int sms = 0;
   size_t tail_smem = 0;
+  size_t sepz_smem = 0, sepy_smem = 0;   // largest panels of the separable instances
 
   ~BatchImpl() override {
     if (exec) cudaGraphExecDestroy(exec);
@@ -426,7 +461,7 @@ class BatchImpl final : public uf_batch {
     maps.assign(kMaps, LaunchMap());
     for (auto& m : maps) std::memset(&m, 0, sizeof(m));
     max_levels = 0;
-    tail_smem = 0;
+    tail_smem = sepz_smem = sepy_smem = 0;
     for (int i = 0; i < n; ++i) {
       const View<T>& G = views[i];
       const uf_grid_desc& d = G.d;
@@ -442,6 +477,16 @@ class BatchImpl final : public uf_batch {
                       3 * d.nz + 1);
       add_entry(maps[MAP_CHUNK], i, G.chunk_g[0], G.chunk_g[1], G.chunk_g[2], G.chunk_zc);
       add_entry(maps[MAP_ADV], i, G.adv_g[0], G.adv_g[1], G.adv_g[2], G.adv_zc);
+      add_entry(maps[MAP_DIR], i, G.march_g[0][0], G.march_g[0][1], G.march_g[0][2], G.march_zc[0]);
+      if (G.sep.on) {
+        const int by = 32 * uf::sep_y_wn(d.ny), P = G.lv[0].P;
+        add_entry(maps[MAP_SEPZ], i, (int)uf::sep_z_blocks(P, d.ny, d.nz), 1, 1, 0);
+        add_entry(maps[MAP_SEPY], i, (P + by - 1) / by, uf::sep_y_split(P, d.ny, d.nz), d.nz, 0);
+        add_entry(maps[MAP_SEPX], i, (d.ny * d.nz + uf::SEP_X_LINES - 1) / uf::SEP_X_LINES, 1, 1, 0);
+        sepz_smem = std::max(sepz_smem, uf::sep_smem(uf::SEP_Z_WN, d.nz));
+        sepy_smem = std::max(sepy_smem, uf::sep_smem(uf::sep_y_wn(d.ny), d.ny));
+        continue;
+      }
       add_entry(maps[MAP_TAIL], i, 1, 1, 1, 0);
       for (int l = 0; l < G.tail_level; ++l)
         add_entry(maps[MAP_MARCH0 + l], i, G.march_g[l][0], G.march_g[l][1], G.march_g[l][2], G.march_zc[l]);
@@ -579,7 +624,7 @@ class BatchImpl final : public uf_batch {
         }
       }
     }
-    {
+    if (items(MAP_TAIL) > 0) {
       auto k = kb_mg_tail<T, SM>;
       L(s, "b_mg_tail", sum_over(MAP_TAIL, [](const View<T>& G) {
           return (double)G.tail.n_coarse * G.tail.n_coarse * 8 + 2 * cells(G, G.tail_level) * tb;
@@ -620,7 +665,48 @@ class BatchImpl final : public uf_batch {
     }
   }
 
+  // The instances with the separable inverse (capi.cu, rec_sep).
+  void rec_sep(cudaStream_t s, int mode, cudaGraphConditionalHandle cond, int use_cond) {
+    if constexpr (std::is_same<T, float>::value) {
+      if (items(MAP_SEPZ) == 0) return;
+      auto fill = [](SepP& P, const View<T>& G) {
+        P.L = G.lv[0];
+        P.S = G.sep;
+        P.x = G.p; P.d0 = G.d0; P.d1 = G.d1; P.q = G.q; P.z = G.z;
+        P.partials = G.partials;
+        P.st = G.st;
+      };
+      const int t = uf::SEP_T;
+      const auto& Az = args<SepP>(MAP_SEPZ, fill);
+      if (mode == 1)
+        L(s, "b_sep_zf_cg", plane_bytes(MAP_SEPZ, 7), [&] {
+          kb_sep_zf<true><<<grid_of(kb_sep_zf<true>, t, sepz_smem, items(MAP_SEPZ)), t, sepz_smem, s>>>(Az, cond, use_cond, d_left);
+        });
+      else
+        L(s, "b_sep_zf", plane_bytes(MAP_SEPZ, 2), [&] {
+          kb_sep_zf<false><<<grid_of(kb_sep_zf<false>, t, sepz_smem, items(MAP_SEPZ)), t, sepz_smem, s>>>(Az, cond, 0, nullptr);
+        });
+      for (int inv = 0; inv < 2; ++inv) {
+        const auto& Ay = args<SepP>(MAP_SEPY, fill);
+        L(s, "b_sep_y", plane_bytes(MAP_SEPY, 2), [&] {
+          kb_sep_y<<<grid_of(kb_sep_y, t, sepy_smem, items(MAP_SEPY)), t, sepy_smem, s>>>(Ay, inv);
+        });
+        if (inv) break;
+        const auto& Ax = args<SepP>(MAP_SEPX, fill);
+        L(s, "b_sep_x", plane_bytes(MAP_SEPX, 3), [&] {
+          kb_sep_x<<<grid_of(kb_sep_x, 32 * uf::SEP_X_LINES, 0, items(MAP_SEPX)), 32 * uf::SEP_X_LINES, 0, s>>>(Ax);
+        });
+      }
+      const auto& Ai = args<SepP>(MAP_SEPZ, fill);
+      L(s, "b_sep_zi", plane_bytes(MAP_SEPZ, 3), [&] {
+        kb_sep_zi<<<grid_of(kb_sep_zi, t, sepz_smem, items(MAP_SEPZ)), t, sepz_smem, s>>>(Ai, mode);
+      });
+    }
+  }
+
   void vcycle(cudaStream_t s, int mode, cudaGraphConditionalHandle cond, int use_cond) {
+    rec_sep(s, mode, cond, use_cond);
+    if (items(MAP_TAIL) == 0) return;
     if (smoother == UF_SMOOTH_RBGS) rec_vcycle<uf::SM_RBGS>(s, mode, cond, use_cond);
     else rec_vcycle<uf::SM_JACOBI>(s, mode, cond, use_cond);
   }
@@ -717,9 +803,9 @@ class BatchImpl final : public uf_batch {
   // one CG iteration: direction + A d, then the V-cycle with the CG update
   void rec_iter(cudaStream_t s, cudaGraphConditionalHandle cond, int use_cond) {
     auto k = kb_cg_dir_q<T>;
-    const auto& A = args<CgP<T>>(MAP_MARCH0, [](CgP<T>& P, const View<T>& G) { P = cg_params(G); });
-    L(s, "b_cg_dir_q", plane_bytes(MAP_MARCH0, 4),
-      [&] { k<<<grid_of(k, uf::FT, 0, items(MAP_MARCH0)), dim3(uf::FT), 0, s>>>(A); });
+    const auto& A = args<CgP<T>>(MAP_DIR, [](CgP<T>& P, const View<T>& G) { P = cg_params(G); });
+    L(s, "b_cg_dir_q", plane_bytes(MAP_DIR, 4),
+      [&] { k<<<grid_of(k, uf::FT, 0, items(MAP_DIR)), dim3(uf::FT), 0, s>>>(A); });
     vcycle(s, 1, cond, use_cond);
   }
 
@@ -896,6 +982,10 @@ class BatchImpl final : public uf_batch {
       };
       UFB_CUDA(lim_static((const void*)kb_advect_fused<T>));
       UFB_CUDA(lim_static((const void*)kb_momentum_fused<T>));
+      UFB_CUDA(lim_static((const void*)kb_sep_zf<false>));
+      UFB_CUDA(lim_static((const void*)kb_sep_zf<true>));
+      UFB_CUDA(lim_static((const void*)kb_sep_zi));
+      UFB_CUDA(lim_static((const void*)kb_sep_y));
       UFB_CUDA(cudaStreamSynchronize(stream));
       uf_status s = capture();
       if (s != UF_OK) return s;

@@ -22,6 +22,7 @@
 #include "advect_fused.cuh"
 #include "momentum_fused.cuh"
 #include "mg_coarse.cuh"
+#include "sep_solve.cuh"
 #include "mesh_kernels.cuh"
 
 namespace {
@@ -139,9 +140,24 @@ struct Plan {
   size_t tail_cr_off;      // byte offset of the coarsest solve's FP64 right-hand side in it
   std::vector<int> tail_off;
   std::vector<size_t> lr, lx, lt, lu;   // lu: scratch of the cluster V-cycle (levels >= 1)
+  bool sep;                             // the separable inverse is available (sep_solve.cuh)
+  size_t sep_y[2], sep_z[2];            // its packed matrices (forward, inverse); the pivots lie in r2
   size_t prof, dt, dtT, scal, state, partials, ainv, boxes, grad;
   size_t total;
 };
+
+// Whether a grid has the separable inverse: FP32 with the default V-cycle
+// settings (a caller who asks for another smoother or transfer gets that
+// V-cycle), sizes whose panels fit one block's shared memory (227 KB: nz x
+// 136 words, ny x 72 or 40 words) and whose x lines fit one warp, and at most
+// kPartials panels per reducing launch.
+bool sep_available(const uf_grid_desc* d) {
+  if (d->precision != UF_F32 || d->precond != UF_PRECOND_MG || d->mg_smoother != UF_SMOOTH_CHEBY ||
+      d->mg_transfer != UF_TRANSFER_LINEAR)
+    return false;
+  return d->nx <= uf::SEP_MAX_NX && d->ny <= 1392 && d->nz <= 400 &&
+         uf::sep_z_blocks(pitch_of(d->nx), d->ny, d->nz) <= (unsigned)kPartials;
+}
 
 Plan make_plan(const uf_grid_desc* d) {
   Plan P;
@@ -206,6 +222,12 @@ Plan make_plan(const uf_grid_desc* d) {
   P.ainv = L.take(sizeof(double) * (size_t)P.coarse_n * P.coarse_n);
   P.boxes = L.take(sizeof(uf::DesignBox) * uf::MAX_BOXES);
   P.grad = L.take(sizeof(double) * 3 * uf::MAX_BOXES);
+  P.sep = sep_available(d);
+  if (P.sep) {
+    auto packed = [](int n) { return (size_t)((n + 15) / 16) * ((n + 7) / 8) * 32 * sizeof(float4); };
+    for (size_t& o : P.sep_y) o = L.take(packed(d->ny));
+    for (size_t& o : P.sep_z) o = L.take(packed(d->nz));
+  }
   P.total = L.off + 256;
   return P;
 }
@@ -334,6 +356,7 @@ class GridImpl final : public uf_grid {
   // pressure store; p holds the solve's correction, then p^{n+1} rounded
   uf::PStore<T> *pd, *gd;
   uf::TailArgs<T> tail;
+  uf::Sep sep{};        // the separable inverse (sep.on = 0: not available)
   T* sol_x = nullptr;   // the solve's unknown (the pressure correction for the step; mu for the adjoint)
   T* sol_b = nullptr;   // its right-hand side
   const uf::PStore<T>* sol_g = nullptr;   // guess of the step's solve (nullptr: warm start in sol_x)
@@ -471,6 +494,18 @@ class GridImpl final : public uf_grid {
       tail.rin = 0;
     }
     UF_CUDA(set_smem_limits());   // every grid: the fused step kernels need more than 48 KB
+    if constexpr (std::is_same<T, float>::value) {
+      if (P.sep) {
+        float4* m[4] = {at<float4>(P.sep_y[0]), at<float4>(P.sep_y[1]), at<float4>(P.sep_z[0]), at<float4>(P.sep_z[1])};
+        for (int q = 0; q < 4; ++q) {
+          const int n = q < 2 ? d.ny : d.nz, bit = q < 2 ? 4 : 16;
+          const int e = (n + 15) / 16 * ((n + 7) / 8) * 32;
+          uf::k_sep_pack<<<(e + 255) / 256, 256, 0, stream>>>(m[q], n, out_mask & bit, out_mask & (2 * bit), q & 1);
+        }
+        sep = uf::Sep{1, m[0], m[1], m[2], m[3], r2, lv[0].x, lv[0].t};
+        UF_CUDA(sep_pivots());
+      }
+    }
     if (d.precond == UF_PRECOND_MG) cluster_ctas = probe_cluster();
     if (d.precond == UF_PRECOND_MG) {
       const LevelDims& cl = P.levels.back();
@@ -558,6 +593,12 @@ class GridImpl final : public uf_grid {
     lim((const void*)uf::k_momentum_fused<T>);
     lim((const void*)uf::k_mg_coarse<T, uf::SM_JACOBI>);
     lim((const void*)uf::k_mg_coarse<T, uf::SM_RBGS>);
+    if (P.sep) {
+      lim((const void*)uf::k_sep_zf<false>);
+      lim((const void*)uf::k_sep_zf<true>);
+      lim((const void*)uf::k_sep_zi<float>);
+      lim((const void*)uf::k_sep_y<float>);
+    }
     return e;
   }
 
@@ -635,7 +676,7 @@ class GridImpl final : public uf_grid {
 
   // First level of the cluster V-cycle (below it, the per-level kernels);
   // tail_level when the cluster kernel is not used.
-  // Automatic (0) is per-level launches: the cluster runs on 16 SMs at most,
+  // Automatic (0) runs no cluster: the cluster runs on 16 SMs at most,
   // and its phases are slower than the per-level kernels on every level but
   // the last one or two before the tail, where the two are about even.
   int coarse_start() const {
@@ -734,7 +775,41 @@ class GridImpl final : public uf_grid {
     }
     for (int l = cs - 1; l >= 0; --l) rec_up<SM>(s, l, mode, om);
   }
+  // The pivots share r2 with the V-cycle (whose residual alternates between r
+  // and r2), so they are formed again whenever the grid leaves the V-cycle.
+  cudaError_t sep_pivots() {
+    if constexpr (std::is_same<T, float>::value) {
+      if (use_sep()) uf::k_sep_pivots<<<(d.ny * d.nz + 63) / 64, 64, 0, stream>>>(lv[0], r2);
+      return cudaGetLastError();
+    }
+    return cudaSuccess;
+  }
+  // The separable inverse takes the V-cycle's place wherever it is available
+  // and the V-cycle's launches were not asked for (uf_tuning.coarse_start).
+  bool use_sep() const { return sep.on && coarse_start_tuned == 0; }
+  void rec_sep(cudaStream_t s, int mode, cudaGraphConditionalHandle cond, int use_cond) {
+    if constexpr (std::is_same<T, float>::value) {
+      const unsigned gz = uf::sep_z_blocks(lv[0].P, d.ny, d.nz);
+      const size_t sz = uf::sep_smem(uf::SEP_Z_WN, d.nz), sy = uf::sep_smem(uf::sep_y_wn(d.ny), d.ny);
+      const int by = 32 * uf::sep_y_wn(d.ny);
+      const dim3 gy((lv[0].P + by - 1) / by, uf::sep_y_split(lv[0].P, d.ny, d.nz), d.nz);
+      const unsigned gx = (unsigned)((d.ny * d.nz + uf::SEP_X_LINES - 1) / uf::SEP_X_LINES);
+      if (mode == 1)
+        L(s, "sep_zf_cg", 7 * N() * tb(), [&] {
+          uf::k_sep_zf<true><<<gz, uf::SEP_T, sz, s>>>(lv[0], sep, sol_x, d0, d1, q, partials, st, cond, use_cond);
+        });
+      else
+        L(s, "sep_zf", 2 * N() * tb(), [&] {
+          uf::k_sep_zf<false><<<gz, uf::SEP_T, sz, s>>>(lv[0], sep, nullptr, nullptr, nullptr, nullptr, partials, st, cond, 0);
+        });
+      L(s, "sep_y", 2 * N() * tb(), [&] { uf::k_sep_y<float><<<gy, uf::SEP_T, sy, s>>>(lv[0], sep, 0, st); });
+      L(s, "sep_x", 3 * N() * tb(), [&] { uf::k_sep_x<float><<<gx, 32 * uf::SEP_X_LINES, 0, s>>>(lv[0], sep, st); });
+      L(s, "sep_y", 2 * N() * tb(), [&] { uf::k_sep_y<float><<<gy, uf::SEP_T, sy, s>>>(lv[0], sep, 1, st); });
+      L(s, "sep_zi", 3 * N() * tb(), [&] { uf::k_sep_zi<float><<<gz, uf::SEP_T, sz, s>>>(lv[0], sep, z, mode, partials, st); });
+    }
+  }
   void rec_vcycle(cudaStream_t s, int mode, cudaGraphConditionalHandle cond, int use_cond) {
+    if (use_sep()) return rec_sep(s, mode, cond, use_cond);
     if (d.mg_smoother == UF_SMOOTH_RBGS) rec_vcycle_sm<uf::SM_RBGS>(s, mode, cond, use_cond);
     else rec_vcycle_sm<uf::SM_JACOBI>(s, mode, cond, use_cond);
   }
@@ -1446,7 +1521,7 @@ class GridImpl final : public uf_grid {
     advect_grid(&azc);
     t->advect_zc = azc;
     t->unfused = unfused;
-    t->coarse_start = coarse_start() < P.tail_level ? coarse_start() : -1;
+    t->coarse_start = use_sep() ? 0 : coarse_start() < P.tail_level ? coarse_start() : -1;
     if (levels) *levels = P.nl;
     return UF_OK;
   }
@@ -1466,13 +1541,15 @@ class GridImpl final : public uf_grid {
     unfused = t ? t->unfused : 0;
     coarse_start_tuned = t ? t->coarse_start : 0;
     for (int l = 0; l < uf::MAX_LEVELS; ++l) march_zc_tuned[l] = t ? t->march_zc[l] : 0;
+    UF_CUDA(sep_pivots());
     return set_tail_level(t && t->tail_level > 0 ? t->tail_level : P.auto_tail_level);
   }
 
   // Autotuner: candidates = tail level (automatic and up to two levels
   // deeper) x a uniform tile depth (automatic, 2, 4, 8) x per-level launches
   // or the cluster V-cycle over the last level above the tail (where the
-  // device co-schedules the cluster); each is timed over
+  // device co-schedules the cluster), after the automatic choice where that
+  // is the separable inverse; each is timed over
   // `reps` solves of a synthetic right-hand side from a zero guess, with the
   // unknown and the right-hand side in scratch buffers (ut, uh) that no step
   // keeps between steps.
@@ -1494,6 +1571,7 @@ class GridImpl final : public uf_grid {
       int lt, zc, cs;
     };
     std::vector<Cand> cands;
+    if (sep.on) cands.push_back({P.auto_tail_level, 0, 0});
     for (int lt = P.auto_tail_level; lt <= std::min(P.nl - 1, P.auto_tail_level + 2); ++lt)
       for (int zc : {0, 2, 4, 8}) {
         cands.push_back({lt, zc, -1});
@@ -1625,6 +1703,8 @@ class GridImpl final : public uf_grid {
     V.dt = dt;
     V.dtT = dtT;
     V.sw = smooth_weights();
+    V.sep = sep;
+    V.sep.on = use_sep();
   }
 
   // ------------------------------------------------------------ entry points

@@ -10,6 +10,7 @@
 #include "../../include/uf.h"
 #include "mg_fused.cuh"
 #include "momentum_fused.cuh"
+#include "sep_solve.cuh"
 
 // Launch geometry and buffers of one grid, as its own graphs use them; the
 // batch replays the same blocks (same z chunks, same tail level), so a grid
@@ -40,6 +41,7 @@ struct GridView {
   double* dt;
   T* dtT;
   uf::SmoothW<T> sw;               // smoother weights
+  uf::Sep sep;                     // separable inverse (sep.on: in use instead of the V-cycle)
 };
 
 // An NVTX range (host side) for the lifetime of a scope.

@@ -498,22 +498,7 @@ __device__ __forceinline__ void mg_down_body(const Level<T>& F, const Level<T>& 
       double tot[1];
       reduce_partials_sum<FT, 1>(partials, tot, sh, vb.n);
       if (tid == 0) {
-        const double rr = tot[0];
-        st->rr = rr;
-        st->iter = it0 + 1;
-        st->total_iters += 1;
-        if (!(rr == rr) || isinf(rr)) {
-          st->status = DEV_NAN;
-          if (st->sticky == 0) st->sticky = DEV_NAN;
-          st->converged = 1;
-        } else if (rr <= st->tol2 * st->bb) {
-          st->converged = 1;
-        } else if (it0 + 1 >= st->max_iter) {
-          st->status = DEV_NOT_CONVERGED;
-          if (st->sticky == 0) st->sticky = DEV_NOT_CONVERGED;
-          st->converged = 1;
-        }
-        if (st->converged) signal_converged(cond, use_cond, left);
+        finish_rr(st, tot[0], it0, cond, use_cond, left);
         st->ticket[3] = 0u;
       }
     }

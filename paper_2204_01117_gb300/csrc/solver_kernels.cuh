@@ -276,6 +276,27 @@ __global__ void __launch_bounds__(NT) k_cg_update(Level<T> L, T* __restrict__ x,
   }
 }
 
+// Ends CG iteration it0 with the new ||r||^2: counts it and sets the
+// convergence flag (tolerance, iteration cap, or a non-finite residual).
+__device__ __forceinline__ void finish_rr(SolveState* st, double rr, int it0, cudaGraphConditionalHandle cond,
+                                          int use_cond, int* left) {
+  st->rr = rr;
+  st->iter = it0 + 1;
+  st->total_iters += 1;
+  if (!(rr == rr) || isinf(rr)) {
+    st->status = DEV_NAN;
+    if (st->sticky == 0) st->sticky = DEV_NAN;
+    st->converged = 1;
+  } else if (rr <= st->tol2 * st->bb) {
+    st->converged = 1;
+  } else if (it0 + 1 >= st->max_iter) {
+    st->status = DEV_NOT_CONVERGED;
+    if (st->sticky == 0) st->sticky = DEV_NOT_CONVERGED;
+    st->converged = 1;
+  }
+  if (st->converged) signal_converged(cond, use_cond, left);
+}
+
 // Finishes a preconditioner application: rz_new = r.z; mode 0 (set-up) stores
 // it, mode 1 (iteration) also forms beta = rz_new / rz_old.
 __device__ __forceinline__ void finish_rz(SolveState* st, double rz_new, int mode) {
