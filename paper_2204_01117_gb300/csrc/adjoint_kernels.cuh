@@ -84,9 +84,10 @@ __device__ __forceinline__ void strain_sq_adj(T* lu, T* lv, T* lw, const T* __re
   const int im = i > 0 ? i - 1 : i, ip = i < p.nx - 1 ? i + 1 : i;
   const int jm = j > 0 ? j - 1 : j, jp = j < p.ny - 1 ? j + 1 : j;
   const int km = k > 0 ? k - 1 : k, kp = k < p.nz - 1 ? k + 1 : k;
-  const T sx = (ip > im) ? ih / T(ip - im) : T(0);
-  const T sy = (jp > jm) ? ih / T(jp - jm) : T(0);
-  const T sz = (kp > km) ? ih / T(kp - km) : T(0);
+  const T hh = T(0.5) * ih;
+  const T sx = ip - im == 2 ? hh : (ip > im ? ih : T(0));
+  const T sy = jp - jm == 2 ? hh : (jp > jm ? ih : T(0));
+  const T sz = kp - km == 2 ? hh : (kp > km ? ih : T(0));
   const T sxx = (u[idx_u(p, i + 1, j, k)] - u[idx_u(p, i, j, k)]) * ih;
   const T syy = (v[idx_v(p, i, j + 1, k)] - v[idx_v(p, i, j, k)]) * ih;
   const T szz = (w[idx_c(p, i, j, k + 1)] - w[idx_c(p, i, j, k)]) * ih;
@@ -117,11 +118,11 @@ __device__ __forceinline__ void strain_sq_adj(T* lu, T* lv, T* lw, const T* __re
 // limited_nut with its partial derivatives (the forward's branch decides).
 template <typename T>
 __device__ __forceinline__ T limited_nut_d(const StepParams<T>& p, T kv, T omv, T S2, T dt, T& dk, T& dom, T& dS2) {
-  const T strain_om = p.C_lim * sqrt(S2) / sqrt(p.C_mu * T(0.5));
+  const T strain_om = p.S_lim * sqrt(S2);
   const bool om_branch = !(strain_om > omv);   // fmax(omv, strain_om) returns omv unless strain_om is larger
   const T om_t = om_branch ? omv : strain_om;
   const T raw = kv / om_t;
-  const T lim = p.h * p.h / (T(6) * dt) - p.nu;
+  const T lim = nut_cap(p, dt);
   dk = dom = dS2 = T(0);
   const T nut = fmin(raw, lim);
   if (!(nut > T(0))) return T(0);
@@ -129,7 +130,7 @@ __device__ __forceinline__ T limited_nut_d(const StepParams<T>& p, T kv, T omv, 
     dk = T(1) / om_t;
     const T d_omt = -kv / (om_t * om_t);
     if (om_branch) dom = d_omt;
-    else if (S2 > T(0)) dS2 = d_omt * (p.C_lim / sqrt(p.C_mu * T(0.5))) * T(0.5) / sqrt(S2);
+    else if (S2 > T(0)) dS2 = d_omt * p.S_lim * T(0.5) / sqrt(S2);
   }
   return nut;
 }

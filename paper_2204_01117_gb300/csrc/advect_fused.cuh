@@ -13,16 +13,32 @@
 // and the clamp to the range of the forward sample's 8 values then read
 // both from shared memory.  Per plane: two barriers (see advect_fused_body).
 //
+// The kernel is bound by the instructions it issues (shared-memory reads
+// among them), so the common case is stripped to what it needs.  A thread
+// forms phi^ of its own point of every component, keeping the displacements
+// and ranges in registers for the backward step of the next plane, and of
+// one fixed point of the halo (84 points x 3 components on 252 threads).
+// While every displacement is below one cell the sample's cell follows from
+// the signs of the displacements, its corners are staged, and only blocks and
+// planes at the lattice's ends can clamp (EDGE).  The CFL time step keeps
+// every displacement below cfl cells (FAR = false); a fixed time step need
+// not, and a sample that leaves the cell then goes through the general
+// functions below, each a call, which costs registers and moves even where
+// it is never made: a kernel of its own (FAR = true).  Measured, FP32 and
+// CFL time step, against general samples for all points, spread over the
+// threads by component: 256 x 256 x 64 375 -> 172 us (310 M -> 135 M warp
+// instructions, 1030 a cell), 512 x 512 x 128 2734 -> 1069 us; issue slots
+// 72 % busy at 3 blocks per SM.
+//
 // Every value is formed by the same expressions as the two-kernel form
-// (k_advect_forward, k_advect_backward) from the same inputs: displacement(),
-// axis_cell() and trilerp() are shared, only the memory the corners come
-// from differs.  The results are bit for bit those of the two kernels.
+// (k_advect_forward, k_advect_backward) from the same inputs; only the
+// memory the corners come from differs.  The results are bit for bit those
+// of the two kernels.
 //
 // A sample whose corners are not all in the staged window reads global
 // memory instead (a displacement of a cell or more, possible with a fixed
 // time step); a backward sample whose corners are not all in the phi^ window
-// recomputes phi^ at its corners from global memory.  With the CFL time
-// step the displacement stays below half a cell and neither happens.
+// recomputes phi^ at its corners from global memory.
 //
 // Tape (the adjoint's recompute sweep): when A.uh is not null, phi^ at every
 // lattice point the block owns is also written to A.uh, A.vh, A.wh.
@@ -39,26 +55,38 @@ namespace uf {
 constexpr int MX = 32, MY = 8, MT = MX * MY;                    // owned column, threads per block
 constexpr int MWX = MX + 4, MWY = MY + 4, MWP = MWX * MWY;      // window of the fields (halo 2)
 constexpr int MHX = MX + 2, MHY = MY + 2, MHP = MHX * MHY;      // window of phi^ (halo 1)
+constexpr int MHALO = MHP - MT;                                 // its points outside the column
+static_assert(3 * MHALO <= MT, "one halo point per thread");
 // ring depths (planes): 5 and 3 are live; powers of two make the slot of plane
 // kk (kk >= -2) a bit mask instead of a division
 constexpr int MFR = 8, MHR = 4;
+constexpr int CF = MFR * MWP, CH = MHR * MHP;   // from one component's ring to the next
 static_assert((MFR & (MFR - 1)) == 0 && (MHR & (MHR - 1)) == 0, "ring depths are powers of two");
 #ifndef UF_ADVECT_MINB
-#define UF_ADVECT_MINB 2   // resident blocks per SM the register budget is sized for
+#define UF_ADVECT_MINB 3   // resident blocks per SM the register budget is sized for
 #endif
 
 template <typename T>
-constexpr size_t advect_fused_smem() {
+constexpr size_t advect_fused_smem_total() {
   return sizeof(T) * 3 * ((size_t)MFR * MWP + (size_t)MHR * MHP);
+}
+
+// The block's shared memory: the rings of the fields ([3][MFR][MWP]), then
+// those of phi^ ([3][MHR][MHP]).  A place in it is a byte offset into this
+// one array: a 32-bit address that takes constant distances as immediates.
+template <typename T>
+__device__ __forceinline__ T* adv_sm(int place) {
+  extern __shared__ __align__(16) unsigned char adv_smem[];
+  return reinterpret_cast<T*>(adv_smem + place);
 }
 
 // Staged planes [zlo, zhi] of a W x H window with lattice origin (ox, oy),
 // held in a ring of R planes (R a power of two: plane kk in slot kk & (R - 1)).
 template <typename T, int W, int H, int R>
 struct Win {
-  const T* ring;
+  int ring;   // place (bytes) of its first plane
   int ox, oy, zlo, zhi;
-  __device__ __forceinline__ const T* plane(int kk) const { return ring + (kk & (R - 1)) * (W * H); }
+  __device__ __forceinline__ const T* plane(int kk) const { return adv_sm<T>(ring) + (kk & (R - 1)) * (W * H); }
   __device__ __forceinline__ bool holds(int i0, int i1, int j0, int j1, int k0, int k1) const {
     return i0 >= ox && i1 < ox + W && j0 >= oy && j1 < oy + H && k0 >= zlo && k1 <= zhi;
   }
@@ -69,45 +97,11 @@ struct Win {
     f[0] = p0[r0 + x0]; f[1] = p0[r0 + x1]; f[2] = p0[r1 + x0]; f[3] = p0[r1 + x1];
     f[4] = p1[r0 + x0]; f[5] = p1[r0 + x1]; f[6] = p1[r1 + x0]; f[7] = p1[r1 + x1];
   }
-  __device__ __forceinline__ T at(int i, int j, int kk) const { return plane(kk)[(i - ox) + W * (j - oy)]; }
 };
-
-// Trilinear sample of a lattice field whose window is staged (global
-// memory for corners outside the window).
-template <typename T, bool RANGE, int W, int H, int R>
-__device__ __forceinline__ T wsample(const T* __restrict__ g, Lattice L, const Win<T, W, H, R>& win, int ia, T oa,
-                                     int ib, T ob, int ic, T oc, T* mn = nullptr, T* mx = nullptr) {
-  int i0, i1, j0, j1, k0, k1;
-  T ta, tb, tc;
-  axis_cell(ia, oa, L.Lx, i0, i1, ta);
-  axis_cell(ib, ob, L.Ly, j0, j1, tb);
-  axis_cell(ic, oc, L.Lz, k0, k1, tc);
-  T f[8];
-  if (win.holds(i0, i1, j0, j1, k0, k1)) win.corners(i0, i1, j0, j1, k0, k1, f);
-  else corners_global(g, L, i0, i1, j0, j1, k0, k1, f);
-  return trilerp<T, RANGE>(f, ta, tb, tc, mn, mx);
-}
-
-// The three staged component windows of the fields.
-template <typename T>
-struct FWins {
-  Win<T, MWX, MWY, MFR> c[3];
-};
-
-// phi^ at a lattice point from global memory only (the fallback of a
-// backward sample that leaves the phi^ window): the forward step of
-// advect_forward_body.
-template <typename T>
-__device__ __noinline__ T fh_global(const AdvectArgs<T>& A, int q, Lattice L, const T* __restrict__ F, int i, int j,
-                                    int k, T s) {
-  T d[3];
-  displacement(A, q, i, j, k, s, d);
-  return sample<T, false>(F, L, i, -d[0], j, -d[1], k, -d[2]);
-}
 
 // Per-component accessors (Q known at compile time).
 template <int Q, typename T>
-__device__ __forceinline__ Lattice lat_of(const AdvectArgs<T>& A) { return Q == 0 ? A.Lu : (Q == 1 ? A.Lv : A.Lw); }
+__device__ __forceinline__ const Lattice& lat_of(const AdvectArgs<T>& A) { return Q == 0 ? A.Lu : (Q == 1 ? A.Lv : A.Lw); }
 template <int Q, typename T>
 __device__ __forceinline__ const T* field_of(const AdvectArgs<T>& A) { return Q == 0 ? A.u : (Q == 1 ? A.v : A.w); }
 template <int Q, typename T>
@@ -124,209 +118,398 @@ __device__ __forceinline__ void cp_async_elem(T* dst, const T* src) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::); }
 
-// Starts the copy of plane kk of the three fields into its ring slot: the
-// window positions tid and tid + MT of each component that lie on its lattice.
+// A thread's two positions of the staged window (t, t + MT): offsets within
+// a lattice plane (the u lattice; v, w and cells share theirs) and which
+// lattices hold them (bits 0..2: u, v, w).
+struct StagePos {
+  int u[2], c[2], ok[2];
+};
 template <typename T>
-__device__ __forceinline__ void stage_plane(const AdvectArgs<T>& A, T* sF, int i0, int j0, int kk) {
-  if (kk < 0) return;
-  const int slot = kk & (MFR - 1);
+__device__ __forceinline__ StagePos stage_pos(const AdvectArgs<T>& A, int i0, int j0) {
+  StagePos S;
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const int t = threadIdx.x + h * MT;
-    if (t >= MWP) break;
     const int gx = i0 - 2 + t % MWX, gy = j0 - 2 + t / MWX;
-    if (gx < 0 || gy < 0) continue;
+    const bool in = t < MWP && gx >= 0 && gy >= 0;
+    S.u[h] = gx + A.Lu.P * gy;
+    S.c[h] = gx + A.Lv.P * gy;
+    S.ok[h] = !in ? 0 : (gx < A.Lu.Lx && gy < A.Lu.Ly ? 1 : 0) | (gx < A.Lv.Lx && gy < A.Lv.Ly ? 2 : 0) |
+                            (gx < A.Lw.Lx && gy < A.Lw.Ly ? 4 : 0);
+  }
+  return S;
+}
+// Starts the copy of plane kk of the three fields into its ring slot.
+template <typename T>
+__device__ __forceinline__ void stage_plane(const AdvectArgs<T>& A, const StagePos& S, int kk) {
+  if (kk < 0 || kk > A.nz) return;
+  T* dst = adv_sm<T>(0) + (kk & (MFR - 1)) * MWP + threadIdx.x;
+  const T* su = A.u + (size_t)kk * ((size_t)A.Lu.P * A.Lu.Ly);
+  const T* sv = A.v + (size_t)kk * ((size_t)A.Lv.P * A.Lv.Ly);
+  const T* sw = A.w + (size_t)kk * ((size_t)A.Lw.P * A.Lw.Ly);
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      const Lattice L = q == 0 ? A.Lu : (q == 1 ? A.Lv : A.Lw);
-      const T* F = q == 0 ? A.u : (q == 1 ? A.v : A.w);
-      if (gx < L.Lx && gy < L.Ly && kk < L.Lz)
-        cp_async_elem(sF + (q * MFR + slot) * MWP + t, F + (size_t)kk * ((size_t)L.P * L.Ly) + gx + (size_t)L.P * gy);
+  for (int h = 0; h < 2; ++h) {
+    if (kk < A.nz) {
+      if (S.ok[h] & 1) cp_async_elem(dst + h * MT, su + S.u[h]);
+      if (S.ok[h] & 2) cp_async_elem(dst + MFR * MWP + h * MT, sv + S.c[h]);
     }
+    if (S.ok[h] & 4) cp_async_elem(dst + 2 * MFR * MWP + h * MT, sw + S.c[h]);
   }
 }
 
-// Trilinear sample whose corners are all staged (the cross-component
-// samples at half-cell offsets: within one cell of a point of the phi^
-// window, whose planes the window always holds).
-template <typename T, int W, int H, int R>
-__device__ __forceinline__ T ssample(Lattice L, const Win<T, W, H, R>& win, int ia, T oa, int ib, T ob, int ic, T oc) {
+// ------------------------------------------------- displacements < 1 cell --
+// The cell of a sample at (index + off), |off| < 1, relative to the index: o
+// = -1 below it, 0 above, and the weight t -- what axis_cell gives.  At the
+// lattice's first (last) point a sample outside clamps to it.
+template <bool EDGE, typename T>
+__device__ __forceinline__ bool axis_near(T off, bool first, bool last, bool thin, T& t) {   // true: o = -1
+  const bool below = off < T(0);
+  t = below ? off + T(1) : off;
+  if (!EDGE) return below;
+  if (first && below) { t = T(0); return false; }
+  if (last && !below) { t = thin ? T(0) : T(1); return !thin; }
+  return below;
+}
+// Where a point lies on its lattice (EDGE only): the ends along each axis,
+// and a lattice one point high.
+struct Ends {
+  bool x0, x1, y0, y1, z0, z1, thin;
+};
+__device__ __forceinline__ Ends ends_of(const Lattice& L, int gi, int gj, int k) {
+  return Ends{gi == 0, gi == L.Lx - 1, gj == 0, gj == L.Ly - 1, k == 0, k == L.Lz - 1, L.Lz < 2};
+}
+// Trilinear sample around a staged point; pm, pc, pp: the point's place in
+// the planes below, its own and above.
+template <bool EDGE, bool RANGE, int W, typename T>
+__device__ __forceinline__ T near_sample(int pm, int pc, int pp, T ox, T oy, T oz, const Ends& E, T* mn, T* mx) {
+  T ta, tb, tc;
+  const bool bx = axis_near<EDGE>(ox, E.x0, E.x1, false, ta);
+  const bool by = axis_near<EDGE>(oy, E.y0, E.y1, false, tb);
+  const bool bz = axis_near<EDGE>(oz, E.z0, E.z1, E.thin, tc);
+  constexpr int B = sizeof(T);
+  const int o = (bx ? -B : 0) + (by ? -W * B : 0);
+  const T* q0 = adv_sm<T>((bz ? pm : pc) + o);
+  const T* q1 = adv_sm<T>((bz || (EDGE && E.thin) ? pc : pp) + o);
+  const T f[8] = {q0[0], q0[1], q0[W], q0[W + 1], q1[0], q1[1], q1[W], q1[W + 1]};
+  return trilerp<T, RANGE>(f, ta, tb, tc, mn, mx);
+}
+template <typename T>
+__device__ __forceinline__ bool below_one(const T (&d)[3]) {
+  return max3(fabs(d[0]), fabs(d[1]), fabs(d[2])) < T(1);   // (a single NaN passes: its sample's corners are still the point's own)
+}
+
+// What a point's forward step leaves for its backward step: displacement and
+// range of the forward sample's 8 values.
+template <typename T>
+struct Kept {
+  T d[3], mn, mx;
+};
+
+// Forward sample with a displacement of a cell or more (or not a number):
+// the general sample, from the staged window where it holds the corners.
+// (By value: an address passed to a function that is not inlined would keep
+// the range of every point in local memory.)
+template <typename T>
+struct Sampled {
+  T val, mn, mx;
+};
+template <typename T>
+__device__ __noinline__ Sampled<T> fwd_far(const T* __restrict__ F, Lattice L, Win<T, MWX, MWY, MFR> Wn, int i, int j, int k,
+                                           T dx, T dy, T dz) {
   int i0, i1, j0, j1, k0, k1;
   T ta, tb, tc;
-  axis_cell(ia, oa, L.Lx, i0, i1, ta);
-  axis_cell(ib, ob, L.Ly, j0, j1, tb);
-  axis_cell(ic, oc, L.Lz, k0, k1, tc);
+  axis_cell(i, -dx, L.Lx, i0, i1, ta);
+  axis_cell(j, -dy, L.Ly, j0, j1, tb);
+  axis_cell(k, -dz, L.Lz, k0, k1, tc);
   T f[8];
-  win.corners(i0, i1, j0, j1, k0, k1, f);
-  return trilerp<T, false>(f, ta, tb, tc, nullptr, nullptr);
+  if (Wn.holds(i0, i1, j0, j1, k0, k1)) Wn.corners(i0, i1, j0, j1, k0, k1, f);
+  else corners_global(F, L, i0, i1, j0, j1, k0, k1, f);
+  Sampled<T> r;
+  r.val = trilerp<T, true>(f, ta, tb, tc, &r.mn, &r.mx);
+  return r;
 }
-
-// Displacement at a point of the phi^ window, the expressions of
-// displacement() with the corners from the staged windows.
-template <int Q, typename T>
-__device__ __forceinline__ void displacement_s(const AdvectArgs<T>& A, const FWins<T>& Wn, int i, int j, int k, T s,
-                                               T d[3]) {
-  if (Q == 0) {   // u point (i, j+1/2, k+1/2)
-    d[0] = s * Wn.c[0].at(i, j, k);
-    d[1] = s * ssample(A.Lv, Wn.c[1], i, T(-0.5), j, T(0.5), k, T(0));
-    d[2] = s * ssample(A.Lw, Wn.c[2], i, T(-0.5), j, T(0), k, T(0.5));
-  } else if (Q == 1) {   // v point (i+1/2, j, k+1/2)
-    d[0] = s * ssample(A.Lu, Wn.c[0], i, T(0.5), j, T(-0.5), k, T(0));
-    d[1] = s * Wn.c[1].at(i, j, k);
-    d[2] = s * ssample(A.Lw, Wn.c[2], i, T(0), j, T(-0.5), k, T(0.5));
-  } else {   // w point (i+1/2, j+1/2, k)
-    d[0] = s * ssample(A.Lu, Wn.c[0], i, T(0.5), j, T(0), k, T(-0.5));
-    d[1] = s * ssample(A.Lv, Wn.c[1], i, T(0), j, T(0.5), k, T(-0.5));
-    d[2] = s * Wn.c[2].at(i, j, k);
-  }
-}
-
-// Per owned point and component, what the phi^ phase leaves for the
-// backward step of the next plane: the displacement and the range of the
-// forward sample's 8 values (the forward value itself is phi^ there).
-// Ring of 2 planes: [plane & 1][component][value][MT].
-constexpr int MKEEP = 5;
+// phi^ at a lattice point from global memory only: the forward step of
+// advect_forward_body.
 template <typename T>
-constexpr size_t advect_keep_elems() { return (size_t)2 * 3 * MKEEP * MT; }
-
-// phi^ of component Q at window position t (lattice point (gi, gj, m));
-// stored in its ring slot (0 off the lattice), kept for owned points, taped.
-template <int Q, typename T>
-__device__ __forceinline__ void fhat_point(const AdvectArgs<T>& A, const FWins<T>& Wn, T* sH, T* sK, int m, int t,
-                                           T s, int i0, int j0, int k0, int kend) {
-  const Lattice L = lat_of<Q>(A);
-  const int gi = i0 - 1 + t % MHX, gj = j0 - 1 + t / MHX;
-  T val = T(0);
-  if (gi >= 0 && gj >= 0 && m >= 0 && gi < L.Lx && gj < L.Ly && m < L.Lz) {
-    T d[3], mn, mx;
-    displacement_s<Q>(A, Wn, gi, gj, m, s, d);
-    val = wsample<T, true>(field_of<Q>(A), L, Wn.c[Q], gi, -d[0], gj, -d[1], m, -d[2], &mn, &mx);
-    const bool inx = gi >= i0 && gi < i0 + MX, iny = gj >= j0 && gj < j0 + MY;
-    if (inx && iny) {
-      T* kp = sK + ((m & 1) * 3 + Q) * MKEEP * MT + (gi - i0) + MX * (gj - j0);
-      kp[0] = d[0]; kp[MT] = d[1]; kp[2 * MT] = d[2]; kp[3 * MT] = mn; kp[4 * MT] = mx;
-    }
-    T* tape = fhat_of<Q>(A);
-    if (tape) {
-      // owned: inside the column, or the lattice's last point beyond it
-      const bool ox = inx || (gi >= i0 + MX && i0 + MX >= A.nx);
-      const bool oy = iny || (gj >= j0 + MY && j0 + MY >= A.ny);
-      const bool oz = (m >= k0 && m < kend) || (m >= kend && kend == A.nz);
-      if (ox && oy && oz) tape[(size_t)gi + (size_t)L.P * ((size_t)gj + (size_t)L.Ly * m)] = val;
-    }
-  }
-  sH[(Q * MHR + (m & (MHR - 1))) * MHP + t] = val;
+__device__ __noinline__ T fh_global(const AdvectArgs<T>& A, int q, Lattice L, const T* __restrict__ F, int i, int j,
+                                    int k, T s) {
+  T d[3];
+  displacement(A, q, i, j, k, s, d);
+  return sample<T, false>(F, L, i, -d[0], j, -d[1], k, -d[2]);
 }
-
-// phi^ on plane m over the halo-1 window: 3 x MHP items (component,
-// position) spread evenly over the threads.
+// Backward sample with a displacement of a cell or more: from the phi^
+// window where it holds the corners, else phi^ is formed there again.
 template <typename T>
-__device__ __forceinline__ void fhat_plane(const AdvectArgs<T>& A, T* sF, T* sH, T* sK, int m, int zlo, int zhi, T s,
-                                           int i0, int j0, int k0, int kend) {
-  FWins<T> Wn;
-#pragma unroll
-  for (int q = 0; q < 3; ++q) Wn.c[q] = Win<T, MWX, MWY, MFR>{sF + q * MFR * MWP, i0 - 2, j0 - 2, zlo, zhi};
-#pragma unroll 1
-  for (int it = threadIdx.x; it < 3 * MHP; it += MT) {
-    if (it < MHP) fhat_point<0>(A, Wn, sH, sK, m, it, s, i0, j0, k0, kend);
-    else if (it < 2 * MHP) fhat_point<1>(A, Wn, sH, sK, m, it - MHP, s, i0, j0, k0, kend);
-    else fhat_point<2>(A, Wn, sH, sK, m, it - 2 * MHP, s, i0, j0, k0, kend);
-  }
-}
-
-// Backward step, correction and clamp of component Q at the owned point
-// (gi, gj, k): phi* = phi^ + (phi - phi^(x + dt u(x)))/2, clamped.
-template <int Q, typename T>
-__device__ __forceinline__ void maccormack_point(const AdvectArgs<T>& A, const T* sF, const T* sH, const T* sK,
-                                                 int gi, int gj, int k, T s, int i0, int j0) {
-  const bool interior = Q == 0 ? (gi > 0 && gi < A.nx && gj < A.ny)
-                               : (Q == 1 ? (gi < A.nx && gj > 0 && gj < A.ny) : (gi < A.nx && gj < A.ny && k > 0 && k < A.nz));
-  if (!interior) return;
-  const Lattice L = lat_of<Q>(A);
-  const int o = (gi - i0) + MX * (gj - j0);
-  const T* kp = sK + ((k & 1) * 3 + Q) * MKEEP * MT + o;
-  const T d0 = kp[0], d1 = kp[MT], d2 = kp[2 * MT], mn = kp[3 * MT], mx = kp[4 * MT];
-  const Win<T, MHX, MHY, MHR> Hw{sH + Q * MHR * MHP, i0 - 1, j0 - 1, k - 1, k + 1};
-  const T fwd = Hw.at(gi, gj, k);
+__device__ __noinline__ T bwd_far(const AdvectArgs<T>& A, int q, Lattice L, const T* __restrict__ F,
+                                  Win<T, MHX, MHY, MHR> Hw, int i, int j, int k, T dx, T dy, T dz, T s) {
   int a0, a1, b0, b1, c0, c1;
   T ta, tb, tc;
-  axis_cell(gi, d0, L.Lx, a0, a1, ta);
-  axis_cell(gj, d1, L.Ly, b0, b1, tb);
-  axis_cell(k, d2, L.Lz, c0, c1, tc);
+  axis_cell(i, dx, L.Lx, a0, a1, ta);
+  axis_cell(j, dy, L.Ly, b0, b1, tb);
+  axis_cell(k, dz, L.Lz, c0, c1, tc);
   T f[8];
   if (Hw.holds(a0, a1, b0, b1, c0, c1)) {
     Hw.corners(a0, a1, b0, b1, c0, c1, f);
   } else {
-    const T* F = field_of<Q>(A);
-    f[0] = fh_global(A, Q, L, F, a0, b0, c0, s); f[1] = fh_global(A, Q, L, F, a1, b0, c0, s);
-    f[2] = fh_global(A, Q, L, F, a0, b1, c0, s); f[3] = fh_global(A, Q, L, F, a1, b1, c0, s);
-    f[4] = fh_global(A, Q, L, F, a0, b0, c1, s); f[5] = fh_global(A, Q, L, F, a1, b0, c1, s);
-    f[6] = fh_global(A, Q, L, F, a0, b1, c1, s); f[7] = fh_global(A, Q, L, F, a1, b1, c1, s);
+    for (int e = 0; e < 8; ++e) f[e] = fh_global(A, q, L, F, e & 1 ? a1 : a0, e & 2 ? b1 : b0, e & 4 ? c1 : c0, s);
   }
-  const T bwd = trilerp<T, false>(f, ta, tb, tc, nullptr, nullptr);
-  const T own = sF[(Q * MFR + (k & (MFR - 1))) * MWP + (gi - i0 + 2) + MWX * (gj - j0 + 2)];
-  const T r = fwd + T(0.5) * (own - bwd);
-  out_of<Q>(A)[(size_t)gi + (size_t)L.P * ((size_t)gj + (size_t)L.Ly * k)] = fmin(fmax(r, mn), mx);
+  return trilerp<T, false>(f, ta, tb, tc, nullptr, nullptr);
 }
 
-// Eddy viscosity of cell (gi, gj, k) (the expressions of
+// A block's march: where it is and its shared memory.
+template <typename T>
+struct Advance {
+  int i0, j0, k0, kend;
+  T s;     // dt / h
+  static constexpr int B = sizeof(T);
+  // place of position b of plane kk in the window of component 0; the others lie CF (CH) values further on
+  __device__ __forceinline__ int F(int kk, int b) const { return ((kk & (MFR - 1)) * MWP + b) * B; }
+  __device__ __forceinline__ int H(int kk, int h) const { return (3 * CF + (kk & (MHR - 1)) * MHP + h) * B; }
+};
+// A point's place in three staged planes of the fields, and the pairs of
+// faces around it: the sums of displacement(), each along its component's
+// own axis.
+template <typename T>
+struct Near {
+  int m, c, p;   // planes k - 1, k, k + 1
+  __device__ __forceinline__ T at(int q, int e) const { return adv_sm<T>(q)[e]; }   // e values past place q
+  __device__ __forceinline__ T u2(int q) const { return add_rn(at(q, 0), at(q, 1)); }
+  __device__ __forceinline__ T v2(int q) const { return add_rn(at(q, CF), at(q, CF + MWX)); }
+  __device__ __forceinline__ T w2(int o) const { return add_rn(at(c + o, 2 * CF), at(p + o, 2 * CF)); }
+};
+// Neighbour offsets of displacement(): the pair below and the pair above a
+// face along x and y; along z the planes (EDGE: beyond the lattice's end the
+// last pair).
+template <bool EDGE, int B>
+struct Around {   // in bytes
+  int xl, xh, yl, yh;
+  __device__ __forceinline__ Around(int gi, int gj, int nx, int ny)
+      : xl(EDGE && gi == 0 ? 0 : -B), xh(EDGE && gi == nx ? -B : 0), yl(EDGE && gj == 0 ? 0 : -MWX * B),
+        yh(EDGE && gj == ny ? -MWX * B : 0) {}
+};
+
+template <int Q, typename T>
+__device__ __forceinline__ bool on_lattice(const AdvectArgs<T>& A, int gi, int gj, int m) {
+  const Lattice& L = lat_of<Q>(A);
+  return gi >= 0 && gj >= 0 && m >= 0 && gi < L.Lx && gj < L.Ly && m < L.Lz;
+}
+
+// phi^ at lattice point (gi, gj, m) of component q from its displacement.
+template <bool EDGE, bool FAR, typename T>
+__device__ __forceinline__ T forward_at(const AdvectArgs<T>& A, const Advance<T>& M, const Lattice& L, const T* F, int q, const Near<T>& N,
+                                        int gi, int gj, int m, Kept<T>& K) {
+  constexpr int B = sizeof(T);
+  if (!FAR || below_one(K.d))
+    return near_sample<EDGE, true, MWX>(N.m + q * CF * B, N.c + q * CF * B, N.p + q * CF * B, -K.d[0], -K.d[1], -K.d[2], ends_of(L, gi, gj, m), &K.mn,
+                                        &K.mx);
+  const Sampled<T> r = fwd_far(F, L, Win<T, MWX, MWY, MFR>{q * CF * B, M.i0 - 2, M.j0 - 2, max(m, M.k0) - 2, m + 1}, gi, gj, m,
+                               K.d[0], K.d[1], K.d[2]);
+  K.mn = r.mn;
+  K.mx = r.mx;
+  return r.val;
+}
+// Writes phi^ of an owned lattice point to the tape: inside the column, or
+// the lattice's last point beyond it.
+template <typename T>
+__device__ __forceinline__ void tape_point(const AdvectArgs<T>& A, const Advance<T>& M, T* tape, const Lattice& L, int gi, int gj, int m, T val) {
+  const bool ox = (gi >= M.i0 && gi < M.i0 + MX) || (gi >= M.i0 + MX && M.i0 + MX >= A.nx);
+  const bool oy = (gj >= M.j0 && gj < M.j0 + MY) || (gj >= M.j0 + MY && M.j0 + MY >= A.ny);
+  const bool oz = (m >= M.k0 && m < M.kend) || (m >= M.kend && M.kend == A.nz);
+  if (ox && oy && oz) tape[(size_t)gi + (size_t)L.P * ((size_t)gj + (size_t)L.Ly * m)] = val;
+}
+
+// A thread's places: its own point and its halo point.
+struct Places {
+  int gi, gj, b, h;        // own point, its place in the two windows
+  int hq, hi, hj, hb, hh;  // halo point: component (3: none), lattice point, places
+};
+
+// phi^ on plane m: the thread's own point of every component (kept in K) and
+// its halo point; stored (0 off the lattice), taped.  All loads come before
+// the first store, so that the faces the components share are read once.
+template <bool EDGE, bool FAR, typename T>
+__device__ __forceinline__ void fhat_plane(const AdvectArgs<T>& A, const Advance<T>& M, const Places& X, int m, Kept<T> (&K)[3]) {
+  const T s = M.s, s4 = T(0.25) * s;
+  const int za = EDGE ? max(m - 1, 0) : m - 1, zc = EDGE ? min(m, A.nz - 1) : m;   // cell planes below and above the w point
+  {
+    const Near<T> N{M.F(m - 1, X.b), M.F(m, X.b), M.F(m + 1, X.b)};
+    const Around<EDGE, sizeof(T)> o(X.gi, X.gj, A.nx, A.ny);
+    const int a = EDGE ? M.F(za, X.b) : N.m, c = EDGE ? M.F(zc, X.b) : N.c;
+    const bool on0 = !EDGE || on_lattice<0>(A, X.gi, X.gj, m), on1 = !EDGE || on_lattice<1>(A, X.gi, X.gj, m),
+               on2 = !EDGE || on_lattice<2>(A, X.gi, X.gj, m);
+    T val[3] = {T(0), T(0), T(0)};
+    if (on0) {
+      K[0].d[0] = s * N.at(N.c, 0);
+      K[0].d[1] = s4 * add_rn(N.v2(N.c + o.xl), N.v2(N.c + o.xh));
+      K[0].d[2] = s4 * add_rn(N.w2(o.xl), N.w2(o.xh));
+      val[0] = forward_at<EDGE, FAR>(A, M, A.Lu, A.u, 0, N, X.gi, X.gj, m, K[0]);
+    }
+    if (on1) {
+      K[1].d[0] = s4 * add_rn(N.u2(N.c + o.yl), N.u2(N.c + o.yh));
+      K[1].d[1] = s * N.at(N.c, CF);
+      K[1].d[2] = s4 * add_rn(N.w2(o.yl), N.w2(o.yh));
+      val[1] = forward_at<EDGE, FAR>(A, M, A.Lv, A.v, 1, N, X.gi, X.gj, m, K[1]);
+    }
+    if (on2) {
+      K[2].d[0] = s4 * add_rn(N.u2(a), N.u2(c));
+      K[2].d[1] = s4 * add_rn(N.v2(a), N.v2(c));
+      K[2].d[2] = s * N.at(N.c, 2 * CF);
+      val[2] = forward_at<EDGE, FAR>(A, M, A.Lw, A.w, 2, N, X.gi, X.gj, m, K[2]);
+    }
+    T* h = adv_sm<T>(M.H(m, X.h));
+    h[0] = val[0];
+    h[CH] = val[1];
+    h[2 * CH] = val[2];
+    if (A.uh) {
+      if (on0 && m >= 0) tape_point(A, M, A.uh, A.Lu, X.gi, X.gj, m, val[0]);
+      if (on1 && m >= 0) tape_point(A, M, A.vh, A.Lv, X.gi, X.gj, m, val[1]);
+      if (on2 && m >= 0) tape_point(A, M, A.wh, A.Lw, X.gi, X.gj, m, val[2]);
+    }
+  }
+  if (X.hq < 3) {
+    const Near<T> N{M.F(m - 1, X.hb), M.F(m, X.hb), M.F(m + 1, X.hb)};
+    const Around<EDGE, sizeof(T)> o(X.hi, X.hj, A.nx, A.ny);
+    const Lattice& L = X.hq == 0 ? A.Lu : (X.hq == 1 ? A.Lv : A.Lw);
+    T val = T(0);
+    if (!EDGE || (X.hi >= 0 && X.hj >= 0 && m >= 0 && X.hi < L.Lx && X.hj < L.Ly && m < L.Lz)) {
+      Kept<T> K1;
+      const T own = s * N.at(N.c, X.hq * CF);
+      if (X.hq == 0) {
+        K1.d[0] = own;
+        K1.d[1] = s4 * add_rn(N.v2(N.c + o.xl), N.v2(N.c + o.xh));
+        K1.d[2] = s4 * add_rn(N.w2(o.xl), N.w2(o.xh));
+      } else if (X.hq == 1) {
+        K1.d[0] = s4 * add_rn(N.u2(N.c + o.yl), N.u2(N.c + o.yh));
+        K1.d[1] = own;
+        K1.d[2] = s4 * add_rn(N.w2(o.yl), N.w2(o.yh));
+      } else {
+        const int a = EDGE ? M.F(za, X.hb) : N.m, c = EDGE ? M.F(zc, X.hb) : N.c;
+        K1.d[0] = s4 * add_rn(N.u2(a), N.u2(c));
+        K1.d[1] = s4 * add_rn(N.v2(a), N.v2(c));
+        K1.d[2] = own;
+      }
+      const T* F = X.hq == 0 ? A.u : (X.hq == 1 ? A.v : A.w);
+      val = forward_at<EDGE, FAR>(A, M, L, F, X.hq, N, X.hi, X.hj, m, K1);
+      if (A.uh) tape_point(A, M, X.hq == 0 ? A.uh : (X.hq == 1 ? A.vh : A.wh), L, X.hi, X.hj, m, val);
+    }
+    adv_sm<T>(M.H(m, X.hh))[X.hq * CH] = val;
+  }
+}
+
+// Backward step, correction and clamp of component Q at the thread's own
+// point on plane k: phi* = phi^ + (phi - phi^(x + dt u(x)))/2, clamped.  f:
+// the point in the staged plane k; hm, hc, hp: in the phi^ planes around it.
+template <int Q, bool EDGE, bool FAR, typename T>
+__device__ __forceinline__ void maccormack_point(const AdvectArgs<T>& A, const Advance<T>& M, const Places& X, int k, int f, int hm,
+                                                 int hc, int hp, const Kept<T>& K) {
+  const int gi = X.gi, gj = X.gj;
+  if (EDGE) {
+    const bool interior = Q == 0 ? (gi > 0 && gi < A.nx && gj < A.ny)
+                                 : (Q == 1 ? (gi < A.nx && gj > 0 && gj < A.ny) : (gi < A.nx && gj < A.ny && k > 0 && k < A.nz));
+    if (!interior) return;
+  }
+  const Lattice& L = lat_of<Q>(A);
+  constexpr int B = sizeof(T);
+  T bwd;
+  if (!FAR || below_one(K.d))
+    bwd = near_sample<EDGE, false, MHX>(hm + Q * CH * B, hc + Q * CH * B, hp + Q * CH * B, K.d[0], K.d[1], K.d[2], ends_of(L, gi, gj, k),
+                                        (T*)nullptr, (T*)nullptr);
+  else
+    bwd = bwd_far(A, Q, L, field_of<Q>(A), Win<T, MHX, MHY, MHR>{(3 * CF + Q * CH) * B, M.i0 - 1, M.j0 - 1, k - 1, k + 1}, gi, gj, k, K.d[0],
+                  K.d[1], K.d[2], M.s);
+  const T fwd = adv_sm<T>(hc)[Q * CH], own = adv_sm<T>(f)[Q * CF];
+  const T r = fwd + T(0.5) * (own - bwd);
+  (out_of<Q>(A) + (size_t)k * ((size_t)L.P * L.Ly))[gi + L.P * gj] = fmin(fmax(r, K.mn), K.mx);
+}
+template <bool EDGE, bool FAR, typename T>
+__device__ __forceinline__ void maccormack_plane(const AdvectArgs<T>& A, const Advance<T>& M, const Places& X, int k,
+                                                 const Kept<T> (&K)[3]) {
+  const int f = M.F(k, X.b), hm = M.H(k - 1, X.h), hc = M.H(k, X.h), hp = M.H(k + 1, X.h);
+  maccormack_point<0, EDGE, FAR>(A, M, X, k, f, hm, hc, hp, K[0]);
+  maccormack_point<1, EDGE, FAR>(A, M, X, k, f, hm, hc, hp, K[1]);
+  maccormack_point<2, EDGE, FAR>(A, M, X, k, f, hm, hc, hp, K[2]);
+}
+
+// Eddy viscosity of the thread's cell on plane k (the expressions of
 // eddy_viscosity_body) with the faces strain_sq reads taken from the staged
 // windows: planes k-1 .. k+2 of the fields are complete here.
-template <typename T>
-__device__ __forceinline__ void eddy_point(const AdvectArgs<T>& A, const T* sF, int gi, int gj, int k, int i0, int j0) {
-  auto at = [&](int q, int a, int b, int c) {
-    return sF[(q * MFR + (c & (MFR - 1))) * MWP + (a - i0 + 2) + MWX * (b - j0 + 2)];
-  };
-  const T S2 = strain_sq_acc<T>(
-      A.sp, gi, gj, k, [&](int a, int b, int c) { return at(0, a, b, c); },
-      [&](int a, int b, int c) { return at(1, a, b, c); }, [&](int a, int b, int c) { return at(2, a, b, c); });
-  const size_t c = idx_c(A.sp, gi, gj, k);
-  A.nut[c] = limited_nut(A.sp, A.kf[c], A.om[c], S2, *A.dtT);
-}
-
-template <typename T>
-constexpr size_t advect_fused_smem_total() {
-  return advect_fused_smem<T>() + sizeof(T) * advect_keep_elems<T>();
+template <bool EDGE, typename T>
+__device__ __forceinline__ void eddy_point(const AdvectArgs<T>& A, const Advance<T>& M, const Places& X, int k, const T* kf,
+                                           const T* om, T cap) {
+  const int fm = M.F(k - 1, X.b), fc = M.F(k, X.b), fp = M.F(k + 1, X.b);
+  const T S2 = strain_sq_acc<EDGE, T>(
+      A.sp, X.gi, X.gj, k, [&](int q, int dx, int dy, int dz) { return adv_sm<T>(dz == 0 ? fc : (dz < 0 ? fm : fp))[q * CF + dx + MWX * dy]; });
+  const size_t plane = (size_t)k * ((size_t)A.Lw.P * A.Lw.Ly);   // (cells share the w lattice's rows)
+  const int c = X.gi + A.Lw.P * X.gj;
+  (A.nut + plane)[c] = limited_nut(A.sp, (kf + plane)[c], (om + plane)[c], S2, cap);
 }
 
 // Pipeline per output plane k:  wait for plane k+2 of the fields, sync,
-// start the copy of plane k+3 (into the slot of k-2, which no one reads any
+// start the copy of plane k+3 (into the slot of k-5, which no one reads any
 // more), phi^ of plane k+1, sync, phi* of plane k.  The phi^ phase reads
-// the fields on planes [k-1, k+2].
-template <typename T>
-__device__ __forceinline__ void advect_fused_body(const AdvectArgs<T>& A, int zc, const VBlock& vb) {
-  extern __shared__ __align__(16) unsigned char adv_smem[];
-  T* sF = reinterpret_cast<T*>(adv_smem);   // [3][MFR][MWP]
-  T* sH = sF + 3 * MFR * MWP;               // [3][MHR][MHP]
-  T* sK = sH + 3 * MHR * MHP;               // [2][3][MKEEP][MT]
-  const int i0 = vb.x * MX, j0 = vb.y * MY, k0 = vb.z * zc;
-  const int kend = min(A.nz, k0 + zc);
-  const T s = *A.dtT * A.inv_h;
-  for (int kk = k0 - 2; kk <= k0 + 2; ++kk) stage_plane(A, sF, i0, j0, kk);
+// the fields on planes [k-1, k+2].  kf, om: k and omega of the eddy
+// viscosity (where A.nut is set).
+template <bool FAR, typename T>
+__device__ __forceinline__ void advect_fused_body(const AdvectArgs<T>& A, int zc, const T* kf, const T* om, const VBlock& vb) {
+  Advance<T> M;
+  M.i0 = vb.x * MX;
+  M.j0 = vb.y * MY;
+  M.k0 = vb.z * zc;
+  M.kend = min(A.nz, M.k0 + zc);
+  M.s = *A.dtT * A.inv_h;
+  const StagePos S = stage_pos(A, M.i0, M.j0);
+  for (int kk = M.k0 - 2; kk <= M.k0 + 2; ++kk) stage_plane(A, S, kk);
   cp_async_commit();
+  Places X;
+  {
+    const int t = threadIdx.x, tx = t % MX, ty = t / MX;
+    X.gi = M.i0 + tx;
+    X.gj = M.j0 + ty;
+    X.b = (tx + 2) + MWX * (ty + 2);
+    X.h = (tx + 1) + MHX * (ty + 1);
+    X.hq = t / MHALO;
+    const int e = t % MHALO;   // first row, last row, then the two side columns
+    const int wx = e < MHX ? e : (e < 2 * MHX ? e - MHX : ((e & 1) ? MHX - 1 : 0));
+    const int wy = e < MHX ? 0 : (e < 2 * MHX ? MHY - 1 : 1 + (e - 2 * MHX) / 2);
+    X.hi = M.i0 - 1 + wx;
+    X.hj = M.j0 - 1 + wy;
+    X.hb = (wx + 1) + MWX * (wy + 1);
+    X.hh = wx + MHX * wy;
+  }
+  // every point of the phi^ window, its samples and its faces inside all three lattices along x and y
+  const bool inner = M.i0 >= 2 && M.i0 + MX <= A.nx - 2 && M.j0 >= 2 && M.j0 + MY <= A.ny - 2;
+  auto edge = [&](int m) { return !inner || m < 1 || m > A.nz - 2; };
+  const T cap = A.nut ? nut_cap(A.sp, *A.dtT) : T(0);
+  Kept<T> K[3], N[3];
   cp_async_wait_all();
   __syncthreads();
-  fhat_plane(A, sF, sH, sK, k0 - 1, k0 - 2, k0 + 2, s, i0, j0, k0, kend);
-  fhat_plane(A, sF, sH, sK, k0, k0 - 2, k0 + 2, s, i0, j0, k0, kend);
-  const int gi = i0 + (int)threadIdx.x % MX, gj = j0 + (int)threadIdx.x / MX;
-  for (int k = k0; k < kend; ++k) {
+  for (int m = M.k0 - 1; m <= M.k0; ++m) {
+    if (edge(m)) fhat_plane<true, FAR>(A, M, X, m, K);
+    else fhat_plane<false, FAR>(A, M, X, m, K);
+  }
+  for (int k = M.k0; k < M.kend; ++k) {
     cp_async_wait_all();
     __syncthreads();
-    stage_plane(A, sF, i0, j0, k + 3);
+    stage_plane(A, S, k + 3);
     cp_async_commit();
-    fhat_plane(A, sF, sH, sK, k + 1, k - 1, k + 2, s, i0, j0, k0, kend);
+    if (edge(k + 1)) fhat_plane<true, FAR>(A, M, X, k + 1, N);
+    else fhat_plane<false, FAR>(A, M, X, k + 1, N);
     __syncthreads();
-    maccormack_point<0>(A, sF, sH, sK, gi, gj, k, s, i0, j0);
-    maccormack_point<1>(A, sF, sH, sK, gi, gj, k, s, i0, j0);
-    maccormack_point<2>(A, sF, sH, sK, gi, gj, k, s, i0, j0);
-    if (A.nut && gi < A.nx && gj < A.ny) eddy_point(A, sF, gi, gj, k, i0, j0);
+    if (edge(k)) maccormack_plane<true, FAR>(A, M, X, k, K);
+    else maccormack_plane<false, FAR>(A, M, X, k, K);
+    if (A.nut && X.gi < A.nx && X.gj < A.ny) {
+      if (edge(k)) eddy_point<true>(A, M, X, k, kf, om, cap);
+      else eddy_point<false>(A, M, X, k, kf, om, cap);
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q) K[q] = N[q];
   }
   cp_async_wait_all();
 }
 
-template <typename T>
-__global__ void __launch_bounds__(MT, UF_ADVECT_MINB) k_advect_fused(const __grid_constant__ AdvectArgs<T> A, int zc) {
-  advect_fused_body<T>(A, zc, vblock());
+template <typename T, bool FAR>
+__global__ void __launch_bounds__(MT, FAR ? 2 : UF_ADVECT_MINB) k_advect_fused(const __grid_constant__ AdvectArgs<T> A, int zc) {
+  advect_fused_body<FAR, T>(A, zc, A.kf, A.om, vblock());
 }
 
 }  // namespace uf

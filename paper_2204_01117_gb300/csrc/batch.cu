@@ -72,7 +72,7 @@ struct LaunchMap {
 // MAP_DIR: the march tiles of the finest level, every instance; the V-cycle
 // maps (MAP_TAIL, MAP_MARCH0 ..) hold the instances that run it, the MAP_SEP
 // ones those with the separable inverse.
-enum MapKind { MAP_CFL = 0, MAP_CELL, MAP_FACE, MAP_CHUNK, MAP_TAIL, MAP_ADV, MAP_DIR, MAP_SEPZ, MAP_SEPY, MAP_SEPX, MAP_MARCH0 };
+enum MapKind { MAP_CFL = 0, MAP_CELL, MAP_FACE, MAP_CHUNK, MAP_TAIL, MAP_ADV, MAP_ADV_FAR, MAP_DIR, MAP_SEPZ, MAP_SEPY, MAP_SEPX, MAP_MARCH0 };
 constexpr int kMaps = MAP_MARCH0 + uf::MAX_LEVELS;
 
 __device__ __forceinline__ int map_entry(const LaunchMap* __restrict__ m, int w) {
@@ -145,7 +145,7 @@ struct CflP {
   T* dtT;
 };
 template <typename T>
-struct CellP {   // eddy viscosity, k-omega
+struct CellP {   // k-omega
   uf::StepParams<T> sp;
   const T *u, *v, *w;
   T* nut;
@@ -155,6 +155,8 @@ struct CellP {   // eddy viscosity, k-omega
 template <typename T>
 struct AdvP {
   uf::AdvectArgs<T> a;
+  const T* kb[2];
+  const T* ob[2];
 };
 template <typename T>
 struct MomP {    // fused diffusion + drag + BCs + pressure right-hand side
@@ -218,19 +220,15 @@ __global__ void __launch_bounds__(256) kb_cfl(const __grid_constant__ Args<CflP<
   });
 }
 
-template <typename T>
-__global__ void __launch_bounds__(uf::NT, 6) kb_eddy(const __grid_constant__ Args<CellP<T>> A,
-                                                  const int* __restrict__ par) {
-  for_plane_items(&A.m, [&](int i, const VBlock& vb) {
-    const CellP<T>& P = A.at[i];
+// (with the eddy viscosity, from the current k and omega)
+template <typename T, bool FAR>
+__global__ void __launch_bounds__(uf::MT, FAR ? 2 : UF_ADVECT_MINB) kb_advect_fused(const __grid_constant__ Args<AdvP<T>> A,
+                                                                                    const int* __restrict__ par) {
+  for_items(&A.m, [&](int i, int zc, const VBlock& vb) {
+    const AdvP<T>& P = A.at[i];
     const int a = par[i];
-    uf::eddy_viscosity_body<T>(P.sp, P.u, P.v, P.w, P.kb[a], P.ob[a], P.nut, vb);
+    uf::advect_fused_body<FAR, T>(P.a, zc, P.kb[a], P.ob[a], vb);
   });
-}
-
-template <typename T>
-__global__ void __launch_bounds__(uf::MT, UF_ADVECT_MINB) kb_advect_fused(const __grid_constant__ Args<AdvP<T>> A) {
-  for_items(&A.m, [&](int i, int zc, const VBlock& vb) { uf::advect_fused_body<T>(A.at[i].a, zc, vb); });
 }
 
 template <typename T>
@@ -462,6 +460,15 @@ class BatchImpl final : public uf_batch {
     for (auto& m : maps) std::memset(&m, 0, sizeof(m));
     max_levels = 0;
     tail_smem = sepz_smem = sepy_smem = 0;
+    // planes per item of the fused advection: the values do not depend on it,
+    // and a batch needs no more items than a few per resident block
+    int adv_zc = 16;
+    for (const int c : {16, 8, 4, 2, 1}) {
+      long long total = 0;
+      for (int i = 0; i < n; ++i) total += (long long)views[i].adv_g[0] * views[i].adv_g[1] * ((views[i].d.nz + c - 1) / c);
+      adv_zc = c;
+      if (total >= 3LL * 2 * sms) break;
+    }
     for (int i = 0; i < n; ++i) {
       const View<T>& G = views[i];
       const uf_grid_desc& d = G.d;
@@ -476,7 +483,8 @@ class BatchImpl final : public uf_batch {
       add_plane_entry(maps[MAP_FACE], i, (d.nx + 1 + uf::BX - 1) / uf::BX, (d.ny + 1 + uf::BY - 1) / uf::BY,
                       3 * d.nz + 1);
       add_entry(maps[MAP_CHUNK], i, G.chunk_g[0], G.chunk_g[1], G.chunk_g[2], G.chunk_zc);
-      add_entry(maps[MAP_ADV], i, G.adv_g[0], G.adv_g[1], G.adv_g[2], G.adv_zc);
+      add_entry(maps[G.adv_far ? MAP_ADV_FAR : MAP_ADV], i, G.adv_g[0], G.adv_g[1],
+                G.adv_auto ? (d.nz + adv_zc - 1) / adv_zc : G.adv_g[2], G.adv_auto ? adv_zc : G.adv_zc);
       add_entry(maps[MAP_DIR], i, G.march_g[0][0], G.march_g[0][1], G.march_g[0][2], G.march_zc[0]);
       if (G.sep.on) {
         const int by = 32 * uf::sep_y_wn(d.ny), P = G.lv[0].P;
@@ -758,21 +766,18 @@ class BatchImpl final : public uf_batch {
       });
       L(s, "b_cfl_dt", plane_bytes(MAP_CFL, 3), [&] { k<<<grid_of(k, 256, 0, items(MAP_CFL)), 256, 0, s>>>(A); });
     }
-    {
-      auto k = kb_eddy<T>;
-      const auto& A = args<CellP<T>>(MAP_CELL, [](CellP<T>& P, const View<T>& G) { P = cell_params(G); });
-      L(s, "b_eddy_viscosity", plane_bytes(MAP_CELL, 6),
-        [&] { k<<<grid_of(k, uf::NT, 0, items(MAP_CELL)), blk, 0, s>>>(A, d_par); });
-    }
-    {   // both MacCormack passes (the fused kernel of the single grids, bit for bit the two-pass form)
-      auto k = kb_advect_fused<T>;
-      const auto& A = args<AdvP<T>>(MAP_ADV, [](AdvP<T>& P, const View<T>& G) {
+    for (int far = 0; far < 2; ++far) {   // eddy viscosity and both MacCormack passes, CFL and fixed time steps apart
+      const int kind = MAP_ADV + far;
+      if (items(kind) == 0) continue;
+      auto k = far ? kb_advect_fused<T, true> : kb_advect_fused<T, false>;
+      const auto& A = args<AdvP<T>>(kind, [](AdvP<T>& P, const View<T>& G) {
         P.a = G.adv;
         P.a.uh = P.a.vh = P.a.wh = nullptr;   // no tape
+        P.a.nut = G.nut;
+        for (int q = 0; q < 2; ++q) { P.kb[q] = G.kb[q]; P.ob[q] = G.ob[q]; }
       });
       const size_t sm = uf::advect_fused_smem_total<T>();
-      L(s, "b_advect_fused", plane_bytes(MAP_ADV, 6),
-        [&] { k<<<grid_of(k, uf::MT, sm, items(MAP_ADV)), uf::MT, sm, s>>>(A); });
+      L(s, "b_advect_fused", plane_bytes(kind, 9), [&] { k<<<grid_of(k, uf::MT, sm, items(kind)), uf::MT, sm, s>>>(A, d_par); });
     }
     {   // diffusion, drag, velocity BCs and the pressure right-hand side in one pass
       auto k = kb_momentum_fused<T>;
@@ -980,7 +985,8 @@ class BatchImpl final : public uf_batch {
           e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
         return e;
       };
-      UFB_CUDA(lim_static((const void*)kb_advect_fused<T>));
+      UFB_CUDA(lim_static((const void*)kb_advect_fused<T, false>));
+      UFB_CUDA(lim_static((const void*)kb_advect_fused<T, true>));
       UFB_CUDA(lim_static((const void*)kb_momentum_fused<T>));
       UFB_CUDA(lim_static((const void*)kb_sep_zf<false>));
       UFB_CUDA(lim_static((const void*)kb_sep_zf<true>));

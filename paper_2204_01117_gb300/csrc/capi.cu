@@ -428,6 +428,7 @@ class GridImpl final : public uf_grid {
     sp.rho = (T)d.rho; sp.nu = (T)d.nu;
     sp.C_mu = (T)d.C_mu; sp.alpha = (T)d.alpha; sp.beta = (T)d.beta; sp.sigma = (T)d.sigma;
     sp.sigma_star = (T)d.sigma_star; sp.C_lim = (T)d.C_lim;
+    sp.S_lim = (T)(d.C_lim / std::sqrt(0.5 * d.C_mu));
     sp.k_min = (T)d.k_min; sp.om_min = (T)d.omega_min;
     const double uin = inflow_speed(d, d.z_ref);
     const double kin = 1.5 * (d.I * uin) * (d.I * uin);
@@ -589,7 +590,8 @@ class GridImpl final : public uf_grid {
     };
     lim((const void*)uf::k_mg_tail<T, uf::SM_JACOBI>);
     lim((const void*)uf::k_mg_tail<T, uf::SM_RBGS>);
-    lim((const void*)uf::k_advect_fused<T>);
+    lim((const void*)uf::k_advect_fused<T, false>);
+    lim((const void*)uf::k_advect_fused<T, true>);
     lim((const void*)uf::k_momentum_fused<T>);
     lim((const void*)uf::k_mg_coarse<T, uf::SM_JACOBI>);
     lim((const void*)uf::k_mg_coarse<T, uf::SM_RBGS>);
@@ -933,11 +935,32 @@ class GridImpl final : public uf_grid {
     return A;
   }
 
-  // Fused advection: 32 x 8 columns, zc planes per block (16 unless tuned).
+  // Whether a displacement may reach a cell: every face velocity is at most
+  // the maximum the CFL time step was formed from, so |dt u / h| <= cfl up to
+  // rounding (the margin).
+  bool advect_far() const { return d.fixed_dt > 0 || !(d.cfl <= 0.999); }
+
+  // Fused advection: 32 x 8 columns, zc planes per block.  Automatic: at most
+  // 16.  A block forms 1.7 planes' worth of halo besides its own (512 x 512 x
+  // 128: 2715 us at 1 plane, 1388 at 4, 1069 at 16), and a last wave that is
+  // not full costs about half of what it leaves idle (256 x 256 x 64, 456
+  // blocks resident: 12 planes = 2.99 waves 172 us, 16 = 2.25 waves 186 us;
+  // 48 x 40 x 16: 1 plane 12 us, 16 planes 47 us); the depth with the least
+  // product of the two.
   dim3 advect_grid(int* zc) const {
-    const int z = advect_zc_tuned > 0 ? advect_zc_tuned : 16;
+    const int bx = (d.nx + uf::MX - 1) / uf::MX, by = (d.ny + uf::MY - 1) / uf::MY;
+    int z = advect_zc_tuned;
+    if (z <= 0) {
+      const double resident = 152.0 * (sizeof(T) == 8 ? 1 : advect_far() ? 2 : UF_ADVECT_MINB);
+      double best = 1e300;
+      for (int c : {16, 12, 8, 6, 4, 3, 2, 1}) {
+        const double waves = (double)bx * by * d.nz / c / resident;
+        const double cost = (1.0 + 1.7 / c) * (1.0 + 0.5 * (std::ceil(waves) / waves - 1.0));
+        if (cost < best) { best = cost; z = c; }
+      }
+    }
     *zc = z;
-    return dim3((d.nx + uf::MX - 1) / uf::MX, (d.ny + uf::MY - 1) / uf::MY, (d.nz + z - 1) / z);
+    return dim3(bx, by, (d.nz + z - 1) / z);
   }
 
   void rec_momentum(cudaStream_t s, const T* kin, const T* oin) {
@@ -959,7 +982,8 @@ class GridImpl final : public uf_grid {
       int zc;
       const dim3 gf = advect_grid(&zc);
       L(s, "advect_fused", 2 * faces + 3 * cells, [&] {
-        uf::k_advect_fused<T><<<gf, uf::MT, uf::advect_fused_smem_total<T>(), s>>>(Af, zc);
+        if (advect_far()) uf::k_advect_fused<T, true><<<gf, uf::MT, uf::advect_fused_smem_total<T>(), s>>>(Af, zc);
+        else uf::k_advect_fused<T, false><<<gf, uf::MT, uf::advect_fused_smem_total<T>(), s>>>(Af, zc);
       });
     } else {
       L(s, "eddy_viscosity", faces + 3 * cells,
@@ -1517,9 +1541,7 @@ class GridImpl final : public uf_grid {
       march_grid(l, &zc);
       t->march_zc[l] = d.precond == UF_PRECOND_MG ? zc : 0;
     }
-    int azc;
-    advect_grid(&azc);
-    t->advect_zc = azc;
+    t->advect_zc = advect_zc_tuned > 0 ? advect_zc_tuned : 16;
     t->unfused = unfused;
     t->coarse_start = use_sep() ? 0 : coarse_start() < P.tail_level ? coarse_start() : -1;
     if (levels) *levels = P.nl;
@@ -1697,6 +1719,8 @@ class GridImpl final : public uf_grid {
     const dim3 ga = advect_grid(&azc);
     V.adv_g[0] = ga.x; V.adv_g[1] = ga.y; V.adv_g[2] = ga.z;
     V.adv_zc = azc;
+    V.adv_far = advect_far();
+    V.adv_auto = advect_zc_tuned <= 0;
     V.dt_blocks = kDtBlocks;
     V.st = st;
     V.partials = partials;

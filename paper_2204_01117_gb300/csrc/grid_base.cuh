@@ -35,6 +35,8 @@ struct GridView {
   int march_zc[uf::MAX_LEVELS];    // z planes per block
   int chunk_g[3], chunk_zc;        // z-chunked reductions over the cells (and the fused momentum pass)
   int adv_g[3], adv_zc;            // blocks and z planes per block of the fused advection
+  int adv_auto;                    // adv_zc is the automatic choice for the grid alone
+  int adv_far;                     // a displacement may reach a cell (k_advect_fused)
   int dt_blocks;                   // blocks of the CFL reduction
   uf::SolveState* st;
   double* partials;

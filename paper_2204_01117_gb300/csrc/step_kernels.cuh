@@ -76,31 +76,34 @@ __global__ void __launch_bounds__(256) k_cfl_dt(const T* __restrict__ u, size_t 
 // stored: diagonal terms from the two faces of the cell, off-diagonal terms
 // from central differences of cell-averaged velocities (one-sided at the
 // domain edge, zero for an extent of 1).
-// uf(a, b, c), vf, wf: the face velocities; from global memory (strain_sq)
-// or from staged windows (the fused advection), with the same result: the
-// sum of squares is spelled with explicitly rounded operations, the rest
-// has nothing the compiler could fuse.
-template <typename T, typename UF, typename VF, typename WF>
-__device__ __forceinline__ T strain_sq_acc(const StepParams<T>& p, int i, int j, int k, UF uf, VF vf, WF wf) {
+// f(q, dx, dy, dz): velocity component q at the face (i + dx, j + dy, k + dz)
+// of its lattice; from global memory (strain_sq) or from staged windows (the
+// fused advection), with the same result: the sum of squares is spelled with
+// explicitly rounded operations, the rest has nothing the compiler could
+// fuse.
+// EDGE = false: the cell has neighbours on all sides.
+template <bool EDGE, typename T, typename F>
+__device__ __forceinline__ T strain_sq_acc(const StepParams<T>& p, int i, int j, int k, F f) {
   const T ih = p.inv_h;
-  auto uc = [&](int a, int b, int c) { return T(0.5) * (uf(a, b, c) + uf(a + 1, b, c)); };
-  auto vc = [&](int a, int b, int c) { return T(0.5) * (vf(a, b, c) + vf(a, b + 1, c)); };
-  auto wc = [&](int a, int b, int c) { return T(0.5) * (wf(a, b, c) + wf(a, b, c + 1)); };
-  const int im = i > 0 ? i - 1 : i, ip = i < p.nx - 1 ? i + 1 : i;
-  const int jm = j > 0 ? j - 1 : j, jp = j < p.ny - 1 ? j + 1 : j;
-  const int km = k > 0 ? k - 1 : k, kp = k < p.nz - 1 ? k + 1 : k;
-  const T sx = (ip > im) ? ih / T(ip - im) : T(0);
-  const T sy = (jp > jm) ? ih / T(jp - jm) : T(0);
-  const T sz = (kp > km) ? ih / T(kp - km) : T(0);
-  const T sxx = (uf(i + 1, j, k) - uf(i, j, k)) * ih;
-  const T syy = (vf(i, j + 1, k) - vf(i, j, k)) * ih;
-  const T szz = (wf(i, j, k + 1) - wf(i, j, k)) * ih;
-  const T du_dy = (uc(i, jp, k) - uc(i, jm, k)) * sy;
-  const T du_dz = (uc(i, j, kp) - uc(i, j, km)) * sz;
-  const T dv_dx = (vc(ip, j, k) - vc(im, j, k)) * sx;
-  const T dv_dz = (vc(i, j, kp) - vc(i, j, km)) * sz;
-  const T dw_dx = (wc(ip, j, k) - wc(im, j, k)) * sx;
-  const T dw_dy = (wc(i, jp, k) - wc(i, jm, k)) * sy;
+  auto uc = [&](int a, int b, int c) { return T(0.5) * (f(0, a, b, c) + f(0, a + 1, b, c)); };
+  auto vc = [&](int a, int b, int c) { return T(0.5) * (f(1, a, b, c) + f(1, a, b + 1, c)); };
+  auto wc = [&](int a, int b, int c) { return T(0.5) * (f(2, a, b, c) + f(2, a, b, c + 1)); };
+  const int im = !EDGE || i > 0 ? -1 : 0, ip = !EDGE || i < p.nx - 1 ? 1 : 0;
+  const int jm = !EDGE || j > 0 ? -1 : 0, jp = !EDGE || j < p.ny - 1 ? 1 : 0;
+  const int km = !EDGE || k > 0 ? -1 : 0, kp = !EDGE || k < p.nz - 1 ? 1 : 0;
+  const T hh = T(0.5) * ih;   // the spacing is one or two cells
+  const T sx = ip - im == 2 ? hh : (ip > im ? ih : T(0));
+  const T sy = jp - jm == 2 ? hh : (jp > jm ? ih : T(0));
+  const T sz = kp - km == 2 ? hh : (kp > km ? ih : T(0));
+  const T sxx = (f(0, 1, 0, 0) - f(0, 0, 0, 0)) * ih;
+  const T syy = (f(1, 0, 1, 0) - f(1, 0, 0, 0)) * ih;
+  const T szz = (f(2, 0, 0, 1) - f(2, 0, 0, 0)) * ih;
+  const T du_dy = (uc(0, jp, 0) - uc(0, jm, 0)) * sy;
+  const T du_dz = (uc(0, 0, kp) - uc(0, 0, km)) * sz;
+  const T dv_dx = (vc(ip, 0, 0) - vc(im, 0, 0)) * sx;
+  const T dv_dz = (vc(0, 0, kp) - vc(0, 0, km)) * sz;
+  const T dw_dx = (wc(ip, 0, 0) - wc(im, 0, 0)) * sx;
+  const T dw_dy = (wc(0, jp, 0) - wc(0, jm, 0)) * sy;
   const T sxy = T(0.5) * (du_dy + dv_dx), sxz = T(0.5) * (du_dz + dw_dx), syz = T(0.5) * (dv_dz + dw_dy);
   const T diag = fma_rn(szz, szz, fma_rn(syy, syy, mul_rn(sxx, sxx)));
   const T off = fma_rn(syz, syz, fma_rn(sxz, sxz, mul_rn(sxy, sxy)));
@@ -109,18 +112,20 @@ __device__ __forceinline__ T strain_sq_acc(const StepParams<T>& p, int i, int j,
 template <typename T>
 __device__ __forceinline__ T strain_sq(const T* __restrict__ u, const T* __restrict__ v, const T* __restrict__ w,
                                        const StepParams<T>& p, int i, int j, int k) {
-  return strain_sq_acc<T>(
-      p, i, j, k, [&](int a, int b, int c) { return u[idx_u(p, a, b, c)]; },
-      [&](int a, int b, int c) { return v[idx_v(p, a, b, c)]; }, [&](int a, int b, int c) { return w[idx_c(p, a, b, c)]; });
+  return strain_sq_acc<true, T>(p, i, j, k, [&](int q, int dx, int dy, int dz) {
+    return q == 0 ? u[idx_u(p, i + dx, j + dy, k + dz)] : (q == 1 ? v[idx_v(p, i + dx, j + dy, k + dz)] : w[idx_c(p, i + dx, j + dy, k + dz)]);
+  });
 }
 
 // k-omega eddy viscosity with the strain limiter on omega (Sec. 3) and the
 // von Neumann viscosity limiter h^2/(6 dt) - nu, clamped at zero.
 template <typename T>
-__device__ __forceinline__ T limited_nut(const StepParams<T>& p, T kv, T omv, T S2, T dt) {
-  const T om_t = fmax(omv, p.C_lim * sqrt(S2) / sqrt(p.C_mu * T(0.5)));
+__device__ __forceinline__ T nut_cap(const StepParams<T>& p, T dt) { return p.h * p.h / (T(6) * dt) - p.nu; }
+template <typename T>   // cap: nut_cap of the time step
+__device__ __forceinline__ T limited_nut(const StepParams<T>& p, T kv, T omv, T S2, T cap) {
+  const T om_t = fmax(omv, p.S_lim * sqrt(S2));
   T nut = kv / om_t;
-  nut = fmin(nut, p.h * p.h / (T(6) * dt) - p.nu);
+  nut = fmin(nut, cap);
   return nut > T(0) ? nut : T(0);
 }
 
@@ -133,7 +138,7 @@ __device__ __forceinline__ void eddy_viscosity_body(const StepParams<T>& p, cons
   if (i >= p.nx || j >= p.ny) return;
   const T dt = *p.dtT;
   const size_t c = idx_c(p, i, j, k);
-  nut[c] = limited_nut(p, kf[c], om[c], strain_sq(u, v, w, p, i, j, k), dt);
+  nut[c] = limited_nut(p, kf[c], om[c], strain_sq(u, v, w, p, i, j, k), nut_cap(p, dt));
 }
 
 template <typename T>
@@ -187,11 +192,23 @@ __device__ __forceinline__ bool axis_inside(int base, T off, int n) {
 // weights (ta, tb, tc), as nested lerps along x, then y, then z; optionally
 // the range of the 8 values.  Every semi-Lagrangian sample of the step goes
 // through this one expression, whatever memory the corners come from.
+__device__ __forceinline__ float min3(float a, float b, float c) {
+  float r;
+  asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float r;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+__device__ __forceinline__ double min3(double a, double b, double c) { return fmin(fmin(a, b), c); }
+__device__ __forceinline__ double max3(double a, double b, double c) { return fmax(fmax(a, b), c); }
 template <typename T, bool RANGE>
 __device__ __forceinline__ T trilerp(const T (&f)[8], T ta, T tb, T tc, T* mn, T* mx) {
   if (RANGE) {
-    *mn = fmin(fmin(fmin(f[0], f[1]), fmin(f[2], f[3])), fmin(fmin(f[4], f[5]), fmin(f[6], f[7])));
-    *mx = fmax(fmax(fmax(f[0], f[1]), fmax(f[2], f[3])), fmax(fmax(f[4], f[5]), fmax(f[6], f[7])));
+    *mn = fmin(min3(min3(f[0], f[1], f[2]), f[3], f[4]), min3(f[5], f[6], f[7]));
+    *mx = fmax(max3(max3(f[0], f[1], f[2]), f[3], f[4]), max3(f[5], f[6], f[7]));
   }
   const T x00 = lerp_(f[0], f[1], ta), x10 = lerp_(f[2], f[3], ta);
   const T x01 = lerp_(f[4], f[5], ta), x11 = lerp_(f[6], f[7], ta);
@@ -249,21 +266,33 @@ struct AdvectArgs {
 };
 
 // Displacement in lattice units (dt/h * velocity) at a lattice point of
-// component q, every component sampled from time level n.
+// component q, every component sampled from time level n; s = dt/h.  The
+// other two components are the mean of their four faces around the point (a
+// trilinear sample half a cell off along two axes), the pairs of faces along
+// the component's own axis summed first; beyond the lattice's ends the last
+// pair counts twice (the sample clamps).
 template <typename T>
 __device__ __forceinline__ void displacement(const AdvectArgs<T>& A, int q, int i, int j, int k, T s, T d[3]) {
+  auto at = [&](const T* F, const Lattice& L, int a, int b, int c) { return F[(size_t)a + (size_t)L.P * ((size_t)b + (size_t)L.Ly * c)]; };
+  auto u2 = [&](int a, int b, int c) { return add_rn(at(A.u, A.Lu, a, b, c), at(A.u, A.Lu, a + 1, b, c)); };
+  auto v2 = [&](int a, int b, int c) { return add_rn(at(A.v, A.Lv, a, b, c), at(A.v, A.Lv, a, b + 1, c)); };
+  auto w2 = [&](int a, int b, int c) { return add_rn(at(A.w, A.Lw, a, b, c), at(A.w, A.Lw, a, b, c + 1)); };
+  const T s4 = T(0.25) * s;
   if (q == 0) {   // u point (i, j+1/2, k+1/2)
-    d[0] = s * A.u[(size_t)i + (size_t)A.Lu.P * ((size_t)j + (size_t)A.Lu.Ly * k)];
-    d[1] = s * sample<T, false>(A.v, A.Lv, i, T(-0.5), j, T(0.5), k, T(0));
-    d[2] = s * sample<T, false>(A.w, A.Lw, i, T(-0.5), j, T(0), k, T(0.5));
+    const int a = max(i - 1, 0), b = min(i, A.nx - 1);
+    d[0] = s * at(A.u, A.Lu, i, j, k);
+    d[1] = s4 * add_rn(v2(a, j, k), v2(b, j, k));
+    d[2] = s4 * add_rn(w2(a, j, k), w2(b, j, k));
   } else if (q == 1) {   // v point (i+1/2, j, k+1/2)
-    d[0] = s * sample<T, false>(A.u, A.Lu, i, T(0.5), j, T(-0.5), k, T(0));
-    d[1] = s * A.v[(size_t)i + (size_t)A.Lv.P * ((size_t)j + (size_t)A.Lv.Ly * k)];
-    d[2] = s * sample<T, false>(A.w, A.Lw, i, T(0), j, T(-0.5), k, T(0.5));
+    const int a = max(j - 1, 0), b = min(j, A.ny - 1);
+    d[0] = s4 * add_rn(u2(i, a, k), u2(i, b, k));
+    d[1] = s * at(A.v, A.Lv, i, j, k);
+    d[2] = s4 * add_rn(w2(i, a, k), w2(i, b, k));
   } else {   // w point (i+1/2, j+1/2, k)
-    d[0] = s * sample<T, false>(A.u, A.Lu, i, T(0.5), j, T(0), k, T(-0.5));
-    d[1] = s * sample<T, false>(A.v, A.Lv, i, T(0), j, T(0.5), k, T(-0.5));
-    d[2] = s * A.w[(size_t)i + (size_t)A.Lw.P * ((size_t)j + (size_t)A.Lw.Ly * k)];
+    const int a = max(k - 1, 0), b = min(k, A.nz - 1);
+    d[0] = s4 * add_rn(u2(i, j, a), u2(i, j, b));
+    d[1] = s4 * add_rn(v2(i, j, a), v2(i, j, b));
+    d[2] = s * at(A.w, A.Lw, i, j, k);
   }
 }
 
@@ -668,7 +697,7 @@ __device__ __forceinline__ void turbulence_body(const StepParams<T>& p, const T*
   const size_t c = idx_c(p, i, j, k);
   const T kc = ki[c], oc = oi[c];
   const T S2 = strain_sq(u, v, w, p, i, j, k);
-  const T nut = limited_nut(p, kc, oc, S2, dt);
+  const T nut = limited_nut(p, kc, oc, S2, nut_cap(p, dt));
   const T vel[3] = {T(0.5) * (u[idx_u(p, i, j, k)] + u[idx_u(p, i + 1, j, k)]),
                     T(0.5) * (v[idx_v(p, i, j, k)] + v[idx_v(p, i, j + 1, k)]),
                     T(0.5) * (w[idx_c(p, i, j, k)] + w[idx_c(p, i, j, k + 1)])};

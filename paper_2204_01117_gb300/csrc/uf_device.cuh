@@ -37,6 +37,7 @@ struct StepParams {
   T dirx, diry;            // horizontal wind direction (cos, sin)
   T rho, nu;
   T C_mu, alpha, beta, sigma, sigma_star, C_lim;
+  T S_lim;                 // C_lim / sqrt(C_mu / 2), the strain limiter's factor
   T k_min, om_min, k_in, om_in;
   const T* prof;           // inflow speed at the nz cell-centre heights
   const double* dt;        // device scalar: the step's time step (FP64)
