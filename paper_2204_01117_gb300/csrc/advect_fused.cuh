@@ -323,6 +323,23 @@ struct Places {
   int gi, gj, b, h;        // own point, its place in the two windows
   int hq, hi, hj, hb, hh;  // halo point: component (3: none), lattice point, places
 };
+__device__ __forceinline__ Places block_places(int i0, int j0) {
+  Places X;
+  const int t = threadIdx.x, tx = t % MX, ty = t / MX;
+  X.gi = i0 + tx;
+  X.gj = j0 + ty;
+  X.b = (tx + 2) + MWX * (ty + 2);
+  X.h = (tx + 1) + MHX * (ty + 1);
+  X.hq = t / MHALO;
+  const int e = t % MHALO;   // first row, last row, then the two side columns
+  const int wx = e < MHX ? e : (e < 2 * MHX ? e - MHX : ((e & 1) ? MHX - 1 : 0));
+  const int wy = e < MHX ? 0 : (e < 2 * MHX ? MHY - 1 : 1 + (e - 2 * MHX) / 2);
+  X.hi = i0 - 1 + wx;
+  X.hj = j0 - 1 + wy;
+  X.hb = (wx + 1) + MWX * (wy + 1);
+  X.hh = wx + MHX * wy;
+  return X;
+}
 
 // phi^ on plane m: the thread's own point of every component (kept in K) and
 // its halo point; stored (0 off the lattice), taped.  All loads come before
@@ -444,10 +461,10 @@ __device__ __forceinline__ void eddy_point(const AdvectArgs<T>& A, const Advance
   (A.nut + plane)[c] = limited_nut(A.sp, (kf + plane)[c], (om + plane)[c], S2, cap);
 }
 
-// Pipeline per output plane k:  wait for plane k+2 of the fields, sync,
-// start the copy of plane k+3 (into the slot of k-5, which no one reads any
-// more), phi^ of plane k+1, sync, phi* of plane k.  The phi^ phase reads
-// the fields on planes [k-1, k+2].  kf, om: k and omega of the eddy
+// Pipeline per plane m of phi^:  wait for plane m+1 of the fields, sync,
+// start the copy of plane m+2 (into the slot of m-6, which no one reads any
+// more), phi^ of plane m, sync, phi* of plane m-1.  The phi^ phase reads
+// the fields on planes [m-2, m+1].  kf, om: k and omega of the eddy
 // viscosity (where A.nut is set).
 template <bool FAR, typename T>
 __device__ __forceinline__ void advect_fused_body(const AdvectArgs<T>& A, int zc, const T* kf, const T* om, const VBlock& vb) {
@@ -458,48 +475,32 @@ __device__ __forceinline__ void advect_fused_body(const AdvectArgs<T>& A, int zc
   M.kend = min(A.nz, M.k0 + zc);
   M.s = *A.dtT * A.inv_h;
   const StagePos S = stage_pos(A, M.i0, M.j0);
-  for (int kk = M.k0 - 2; kk <= M.k0 + 2; ++kk) stage_plane(A, S, kk);
+  for (int kk = M.k0 - 2; kk <= M.k0; ++kk) stage_plane(A, S, kk);
   cp_async_commit();
-  Places X;
-  {
-    const int t = threadIdx.x, tx = t % MX, ty = t / MX;
-    X.gi = M.i0 + tx;
-    X.gj = M.j0 + ty;
-    X.b = (tx + 2) + MWX * (ty + 2);
-    X.h = (tx + 1) + MHX * (ty + 1);
-    X.hq = t / MHALO;
-    const int e = t % MHALO;   // first row, last row, then the two side columns
-    const int wx = e < MHX ? e : (e < 2 * MHX ? e - MHX : ((e & 1) ? MHX - 1 : 0));
-    const int wy = e < MHX ? 0 : (e < 2 * MHX ? MHY - 1 : 1 + (e - 2 * MHX) / 2);
-    X.hi = M.i0 - 1 + wx;
-    X.hj = M.j0 - 1 + wy;
-    X.hb = (wx + 1) + MWX * (wy + 1);
-    X.hh = wx + MHX * wy;
-  }
+  const Places X = block_places(M.i0, M.j0);
   // every point of the phi^ window, its samples and its faces inside all three lattices along x and y
   const bool inner = M.i0 >= 2 && M.i0 + MX <= A.nx - 2 && M.j0 >= 2 && M.j0 + MY <= A.ny - 2;
   auto edge = [&](int m) { return !inner || m < 1 || m > A.nz - 2; };
   const T cap = A.nut ? nut_cap(A.sp, *A.dtT) : T(0);
   Kept<T> K[3], N[3];
-  cp_async_wait_all();
-  __syncthreads();
-  for (int m = M.k0 - 1; m <= M.k0; ++m) {
-    if (edge(m)) fhat_plane<true, FAR>(A, M, X, m, K);
-    else fhat_plane<false, FAR>(A, M, X, m, K);
-  }
-  for (int k = M.k0; k < M.kend; ++k) {
+  // m: the plane of phi^; phi* follows one plane behind.  (One copy of each
+  // phase's code in the loop: the kernel is sensitive to its code size.)
+  for (int m = M.k0 - 1; m <= M.kend; ++m) {
+    const int k = m - 1;
     cp_async_wait_all();
     __syncthreads();
-    stage_plane(A, S, k + 3);
+    stage_plane(A, S, m + 2);
     cp_async_commit();
-    if (edge(k + 1)) fhat_plane<true, FAR>(A, M, X, k + 1, N);
-    else fhat_plane<false, FAR>(A, M, X, k + 1, N);
-    __syncthreads();
-    if (edge(k)) maccormack_plane<true, FAR>(A, M, X, k, K);
-    else maccormack_plane<false, FAR>(A, M, X, k, K);
-    if (A.nut && X.gi < A.nx && X.gj < A.ny) {
-      if (edge(k)) eddy_point<true>(A, M, X, k, kf, om, cap);
-      else eddy_point<false>(A, M, X, k, kf, om, cap);
+    if (edge(m)) fhat_plane<true, FAR>(A, M, X, m, N);
+    else fhat_plane<false, FAR>(A, M, X, m, N);
+    if (m > M.k0) {
+      __syncthreads();
+      if (edge(k)) maccormack_plane<true, FAR>(A, M, X, k, K);
+      else maccormack_plane<false, FAR>(A, M, X, k, K);
+      if (A.nut && X.gi < A.nx && X.gj < A.ny) {
+        if (edge(k)) eddy_point<true>(A, M, X, k, kf, om, cap);
+        else eddy_point<false>(A, M, X, k, kf, om, cap);
+      }
     }
 #pragma unroll
     for (int q = 0; q < 3; ++q) K[q] = N[q];

@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(uf::MT, FAR ? 2 : UF_ADVECT_MINB) kb_advect_fu
 }
 
 template <typename T>
-__global__ void __launch_bounds__(uf::MT) kb_momentum_fused(const __grid_constant__ Args<MomP<T>> A) {
+__global__ void __launch_bounds__(uf::MT, sizeof(T) == 8 ? 2 : UF_MOMENTUM_MINB) kb_momentum_fused(const __grid_constant__ Args<MomP<T>> A) {
   for_items(&A.m, [&](int i, int, const VBlock& vb) { uf::momentum_fused_body<T>(A.at[i].M, vb); });
 }
 

@@ -5,16 +5,28 @@
 // One z-marching kernel per 32 x 8 column of cells replaces k_diffuse,
 // k_drag_bc and k_pressure_rhs.  Per block, in shared memory:
 //   * the advected velocity (u~, v~, w~), nu_t and the drag coefficient c on
-//     the column plus a halo of 2 (36 x 12, a ring of 5 planes), copied one
+//     the column plus a halo of 2 (36 x 12, a ring of 4 planes), copied one
 //     plane ahead with cp.async;
 //   * the diffused velocity u2 of the three components on the column plus a
 //     halo of 1 (34 x 10, a ring of 2 planes);
 //   * the dragged velocity u3 of the plane's x and y faces, for the fluxes.
-// Per plane k: u2 on plane k+1, sync, u3 on the faces of plane k (u, v) and
-// on the w faces of plane k+1, sync, b of plane k and ||b||^2.
+// Per plane k: u2 on plane k+1 and b of plane k-1 with ||b||^2, sync, u3 on
+// the faces of plane k (u, v) and on the w faces of plane k+1, sync.
 //
-// Boundary faces of u~ and u2 (never stored between sub-steps) come from
-// the BC rules at the moment they are read, as in the unfused kernels.
+// Bound by the instructions it issues, as the advection, and built like it:
+// a thread forms u2 of its own three faces, with their values on the planes
+// below and at its own in registers, and of one fixed halo face; only blocks
+// and planes that touch the domain's ends ask where a value comes from a
+// boundary rule (EDGE), and they write the boundary faces of u2 down, so that
+// the drag reads faces alike everywhere;
+// where the drag coefficient is zero (open air, most of a city) the face
+// keeps its value, which is what the drag expression gives.  Measured at
+// 256 x 256 x 64, FP32, against loops over the general expressions: 235 -> 141
+// us (197 M -> 118 M warp instructions), 512 x 512 x 128 1493 -> 777 us; the
+// code of one variant more in the loop body cost 30 us in instruction fetch.
+//
+// Boundary faces of u~ and u2 are never stored between sub-steps; they come
+// from the BC rules, as in the unfused kernels.
 // Every value is formed by the expressions of k_diffuse, k_drag_bc and
 // k_pressure_rhs; the block and z-chunk decomposition is that of
 // k_pressure_rhs (chunk_grid), so ||b||^2 is summed in the same order.  The
@@ -27,10 +39,13 @@
 
 namespace uf {
 
-constexpr int DR = 5;   // ring of staged planes
+constexpr int DR = 4;   // ring of staged planes: k .. k+2 live, k+3 on its way
 constexpr int UR = 2;   // ring of u2 planes
 // staged fields, in this order, each [DR][MWP]
 constexpr int DF_U = 0, DF_V = 1, DF_W = 2, DF_NUT = 3, DF_C = 4, DF_N = 5;
+#ifndef UF_MOMENTUM_MINB
+#define UF_MOMENTUM_MINB 4   // resident blocks per SM the register budget is sized for
+#endif
 
 template <typename T>
 struct MomentumArgs {
@@ -57,299 +72,354 @@ constexpr size_t momentum_fused_smem() {
   return sizeof(T) * ((size_t)DF_N * DR * MWP + (size_t)3 * UR * MHP + (size_t)(MX + 1) * MY + (size_t)MX * (MY + 1));
 }
 
-// Shared-memory view of one block's planes.
+// One block's planes in its shared memory, as places (byte offsets).
+template <typename T>
+__device__ __forceinline__ T* mom_sm(int place) {
+  extern __shared__ __align__(16) unsigned char mom_smem[];
+  return reinterpret_cast<T*>(mom_smem + place);
+}
 template <typename T>
 struct MView {
-  T* sD;    // [DF_N][DR][MWP]
-  T* sU2;   // [3][UR][MHP]
-  T* sU3;   // (MX+1) x MY  u3 of the plane's x faces
-  T* sV3;   // MX x (MY+1)  u3 of the plane's y faces
-  int i0, j0;
-  __device__ __forceinline__ const T* D(int f, int k) const {   // plane k of staged field f
-    return sD + (f * DR + (k + 4 * DR) % DR) * MWP;
-  }
-  __device__ __forceinline__ T* U2(int q, int k) const { return sU2 + (q * UR + (k & 1)) * MHP; }
-  // window indices of lattice point (i, j)
-  __device__ __forceinline__ int sidx(int i, int j) const { return (i - i0 + 2) + MWX * (j - j0 + 2); }
-  __device__ __forceinline__ int hidx(int i, int j) const { return (i - i0 + 1) + MHX * (j - j0 + 1); }
+  static constexpr int B = sizeof(T);
+  static constexpr int U2_0 = DF_N * DR * MWP, U3_0 = U2_0 + 3 * UR * MHP, V3_0 = U3_0 + (MX + 1) * MY;
+  int i0, j0, k0, kend;
+  __device__ __forceinline__ int D(int f, int k) const { return (f * DR + (k & (DR - 1))) * MWP * B; }     // plane k of staged field f
+  __device__ __forceinline__ int U2(int q, int k) const { return (U2_0 + (q * UR + (k & 1)) * MHP) * B; }
+  __device__ __forceinline__ T* sU3() const { return mom_sm<T>(U3_0 * B); }   // (MX+1) x MY: u3 of the plane's x faces
+  __device__ __forceinline__ T* sV3() const { return mom_sm<T>(V3_0 * B); }   // MX x (MY+1): u3 of the plane's y faces
 };
 
-// Diffusion of one interior face (the expressions of diffuse_body).  Fm,
-// Fc, Fp: planes k-1, k, k+1 of the component's staged u~; Nm, Nc: planes
-// k-1, k of nu_t; s: the face's index in the staged window.  Boundary
-// faces of u~ come from the BC rules (inflow value, the adjacent interior
-// face at an outlet, 0 at a wall).
-template <int Q, typename T>
-__device__ __forceinline__ T diffuse_at(const StepParams<T>& p, T c, const T* Fm, const T* Fc, const T* Fp,
-                                        const T* Nm, const T* Nc, int s, int i, int j, int k) {
-  const int nx = p.nx, ny = p.ny, nz = p.nz;
-  const T x0 = Fc[s];
-  if (Q == 0) {
-    const T inflow = p.prof[k] * p.dirx;
-    const T xm = i - 1 == 0 ? normal_face(p.side[0], Fc[s], inflow) : Fc[s - 1];
-    const T xp = i + 1 == nx ? normal_face(p.side[1], Fc[s], inflow) : Fc[s + 1];
-    const T ym = j > 0 ? Fc[s - MWX] : tangential_ghost(p.side[2], x0, inflow);
-    const T yp = j < ny - 1 ? Fc[s + MWX] : tangential_ghost(p.side[3], x0, inflow);
-    const T zm = k > 0 ? Fm[s] : tangential_ghost(p.side[4], x0, T(0));
-    const T zp = k < nz - 1 ? Fp[s] : tangential_ghost(p.side[5], x0, T(0));
-    const T lap = xm + xp + ym + yp + zm + zp - T(6) * x0;
-    const T nf = T(0.5) * (Nc[s - 1] + Nc[s]);
-    return x0 + c * (p.nu + nf) * lap;
-  } else if (Q == 1) {
-    const T inflow = p.prof[k] * p.diry;
-    const T xm = i > 0 ? Fc[s - 1] : tangential_ghost(p.side[0], x0, inflow);
-    const T xp = i < nx - 1 ? Fc[s + 1] : tangential_ghost(p.side[1], x0, inflow);
-    const T ym = j - 1 == 0 ? normal_face(p.side[2], Fc[s], inflow) : Fc[s - MWX];
-    const T yp = j + 1 == ny ? normal_face(p.side[3], Fc[s], inflow) : Fc[s + MWX];
-    const T zm = k > 0 ? Fm[s] : tangential_ghost(p.side[4], x0, T(0));
-    const T zp = k < nz - 1 ? Fp[s] : tangential_ghost(p.side[5], x0, T(0));
-    const T lap = xm + xp + ym + yp + zm + zp - T(6) * x0;
-    const T nf = T(0.5) * (Nc[s - MWX] + Nc[s]);
-    return x0 + c * (p.nu + nf) * lap;
-  } else {
-    const T xm = i > 0 ? Fc[s - 1] : tangential_ghost(p.side[0], x0, T(0));
-    const T xp = i < nx - 1 ? Fc[s + 1] : tangential_ghost(p.side[1], x0, T(0));
-    const T ym = j > 0 ? Fc[s - MWX] : tangential_ghost(p.side[2], x0, T(0));
-    const T yp = j < ny - 1 ? Fc[s + MWX] : tangential_ghost(p.side[3], x0, T(0));
-    const T zm = k - 1 == 0 ? T(0) : Fm[s];
-    const T zp = k + 1 == nz ? T(0) : Fp[s];
-    const T lap = xm + xp + ym + yp + zm + zp - T(6) * x0;
-    const T nf = T(0.5) * (Nm[s] + Nc[s]);
-    return x0 + c * (p.nu + nf) * lap;
-  }
-}
-
-// u2 read at a face with the BC rules on boundary faces; U, Vp, W: the u2
-// plane of the u, v or w lattice, h: the face's index in the halo-1 window.
+// Starts the copy of plane kk of the five staged fields into its ring slot
+// (S: the thread's two window positions, stage_pos).
 template <typename T>
-__device__ __forceinline__ T u2f(const StepParams<T>& p, const T* U, int h, int i, int k) {
-  if (i == 0) return normal_face(p.side[0], U[h + 1], p.prof[k] * p.dirx);
-  if (i == p.nx) return normal_face(p.side[1], U[h - 1], p.prof[k] * p.dirx);
-  return U[h];
-}
-template <typename T>
-__device__ __forceinline__ T v2f(const StepParams<T>& p, const T* Vp, int h, int j, int k) {
-  if (j == 0) return normal_face(p.side[2], Vp[h + MHX], p.prof[k] * p.diry);
-  if (j == p.ny) return normal_face(p.side[3], Vp[h - MHX], p.prof[k] * p.diry);
-  return Vp[h];
-}
-template <typename T>
-__device__ __forceinline__ T w2f(const StepParams<T>& p, const T* W, int h, int k) {
-  return (k == 0 || k == p.nz) ? T(0) : W[h];
-}
-
-// Drag of one interior face of u2 (the expressions of drag_u/v/w).  u and v
-// faces of plane k: A = u2 planes at k, B = at k + 1, C0 = c at plane k.
-// w faces of plane k: A = u2 planes at k, B = at k - 1, C0 = c at k - 1,
-// C1 = c at k.  h, s: the face's index in the halo-1 and staged windows.
-template <int Q, typename T>
-__device__ __forceinline__ T drag_at(const StepParams<T>& p, T dt, const T* const* A, const T* const* B, const T* C0,
-                                     const T* C1, int h, int s, int i, int j, int k) {
-  if (Q == 0) {
-    const T q = A[0][h];
-    const T vb = T(0.25) * (v2f(p, A[1], h - 1, j, k) + v2f(p, A[1], h, j, k) + v2f(p, A[1], h - 1 + MHX, j + 1, k) +
-                            v2f(p, A[1], h + MHX, j + 1, k));
-    const T wb = T(0.25) * (w2f(p, A[2], h - 1, k) + w2f(p, A[2], h, k) + w2f(p, B[2], h - 1, k + 1) +
-                            w2f(p, B[2], h, k + 1));
-    const T sp = sqrt(q * q + vb * vb + wb * wb);
-    const T cf = T(0.5) * (C0[s - 1] + C0[s]);
-    return fmax(T(0), T(1) - dt * cf * sp) * q;
-  } else if (Q == 1) {
-    const T q = A[1][h];
-    const T ub = T(0.25) * (u2f(p, A[0], h - MHX, i, k) + u2f(p, A[0], h + 1 - MHX, i + 1, k) + u2f(p, A[0], h, i, k) +
-                            u2f(p, A[0], h + 1, i + 1, k));
-    const T wb = T(0.25) * (w2f(p, A[2], h - MHX, k) + w2f(p, A[2], h, k) + w2f(p, B[2], h - MHX, k + 1) +
-                            w2f(p, B[2], h, k + 1));
-    const T sp = sqrt(ub * ub + q * q + wb * wb);
-    const T cf = T(0.5) * (C0[s - MWX] + C0[s]);
-    return fmax(T(0), T(1) - dt * cf * sp) * q;
-  } else {
-    const T q = A[2][h];
-    const T ub = T(0.25) * (u2f(p, B[0], h, i, k - 1) + u2f(p, B[0], h + 1, i + 1, k - 1) + u2f(p, A[0], h, i, k) +
-                            u2f(p, A[0], h + 1, i + 1, k));
-    const T vb = T(0.25) * (v2f(p, B[1], h, j, k - 1) + v2f(p, B[1], h + MHX, j + 1, k - 1) + v2f(p, A[1], h, j, k) +
-                            v2f(p, A[1], h + MHX, j + 1, k));
-    const T sp = sqrt(ub * ub + vb * vb + q * q);
-    const T cf = T(0.5) * (C0[s] + C1[s]);
-    return fmax(T(0), T(1) - dt * cf * sp) * q;
-  }
-}
-
-// u3 of a u / v face (boundary faces from the BC rule on the dragged
-// interior neighbour, as drag_bc_body) and of a w face.  The face whose drag
-// is formed is chosen first, so the drag expression is inlined once.
-template <typename T>
-__device__ __forceinline__ T u3_at(const StepParams<T>& p, T dt, const T* const* A, const T* const* B, const T* C0,
-                                   int h, int s, int i, int j, int k) {
-  const int sh = i == 0 ? 1 : (i == p.nx ? -1 : 0);
-  const T dr = drag_at<0>(p, dt, A, B, C0, C0, h + sh, s + sh, i + sh, j, k);
-  if (sh == 0) return dr;
-  return normal_face(p.side[i == 0 ? 0 : 1], dr, p.prof[k] * p.dirx);
-}
-template <typename T>
-__device__ __forceinline__ T v3_at(const StepParams<T>& p, T dt, const T* const* A, const T* const* B, const T* C0,
-                                   int h, int s, int i, int j, int k) {
-  const int sh = j == 0 ? 1 : (j == p.ny ? -1 : 0);
-  const T dr = drag_at<1>(p, dt, A, B, C0, C0, h + sh * MHX, s + sh * MWX, i, j + sh, k);
-  if (sh == 0) return dr;
-  return normal_face(p.side[j == 0 ? 2 : 3], dr, p.prof[k] * p.diry);
-}
-template <typename T>
-__device__ __forceinline__ T w3_at(const StepParams<T>& p, T dt, const T* const* A, const T* const* B, const T* C0,
-                                   const T* C1, int h, int s, int i, int j, int k) {
-  return (k == 0 || k == p.nz) ? T(0) : drag_at<2>(p, dt, A, B, C0, C1, h, s, i, j, k);
-}
-
-// Starts the copy of plane kk of the five staged fields into its ring slot.
-template <typename T>
-__device__ __forceinline__ void stage_momentum(const MomentumArgs<T>& M, T* sD, int i0, int j0, int kk) {
+__device__ __forceinline__ void stage_momentum(const MomentumArgs<T>& M, const MView<T>& V, const StagePos& S, int kk) {
   const StepParams<T>& p = M.p;
   if (kk < 0 || kk > p.nz) return;
-  const int slot = (kk + 4 * DR) % DR;
+  T* dst = mom_sm<T>(V.D(0, kk)) + threadIdx.x;
+  const size_t pc = (size_t)kk * ((size_t)p.Pc * p.ny);
+  const T* su = M.ut + (size_t)kk * ((size_t)p.Pu * p.ny);
+  const T* sv = M.vt + (size_t)kk * ((size_t)p.Pc * (p.ny + 1));
+  const T *sw = M.wt + pc, *sn = M.nut + pc, *sc = M.cc + pc;
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
-    const int t = threadIdx.x + h * MT;
-    if (t >= MWP) break;
-    const int gx = i0 - 2 + t % MWX, gy = j0 - 2 + t / MWX;
-    if (gx < 0 || gy < 0) continue;
+    T* d = dst + h * MT;
     if (kk < p.nz) {
-      if (gx <= p.nx && gy < p.ny) cp_async_elem(sD + (DF_U * DR + slot) * MWP + t, M.ut + idx_u(p, gx, gy, kk));
-      if (gx < p.nx && gy <= p.ny) cp_async_elem(sD + (DF_V * DR + slot) * MWP + t, M.vt + idx_v(p, gx, gy, kk));
-      if (gx < p.nx && gy < p.ny) {
-        cp_async_elem(sD + (DF_NUT * DR + slot) * MWP + t, M.nut + idx_c(p, gx, gy, kk));
-        cp_async_elem(sD + (DF_C * DR + slot) * MWP + t, M.cc + idx_c(p, gx, gy, kk));
+      if (S.ok[h] & 1) cp_async_elem(d + DF_U * DR * MWP, su + S.u[h]);
+      if (S.ok[h] & 2) cp_async_elem(d + DF_V * DR * MWP, sv + S.c[h]);
+      if (S.ok[h] & 4) {
+        cp_async_elem(d + DF_NUT * DR * MWP, sn + S.c[h]);
+        cp_async_elem(d + DF_C * DR * MWP, sc + S.c[h]);
       }
     }
-    if (gx < p.nx && gy < p.ny) cp_async_elem(sD + (DF_W * DR + slot) * MWP + t, M.wt + idx_c(p, gx, gy, kk));
+    if (S.ok[h] & 4) cp_async_elem(d + DF_W * DR * MWP, sw + S.c[h]);
   }
 }
 
-// u2 of the three components on plane m over the halo-1 window; only
-// interior faces are formed (boundary faces come from the BC rules).
+// Diffusion of one interior face (the expressions of diffuse_body) from its
+// six neighbours.
 template <typename T>
-__device__ __forceinline__ void u2_plane(const MomentumArgs<T>& M, const MView<T>& V, T c, int m, int k0, int kend) {
-  const StepParams<T>& p = M.p;
-  if (m < 0 || m > p.nz) return;
-  const T* Nm = V.D(DF_NUT, m - 1);
-  const T* Nc = V.D(DF_NUT, m);
-#pragma unroll 1
-  for (int it = threadIdx.x; it < 3 * MHP; it += MT) {
-    const int q = it >= 2 * MHP ? 2 : (it >= MHP ? 1 : 0), t = it - q * MHP;
-    const int wx = t % MHX, wy = t / MHX;
-    const int gi = V.i0 - 1 + wx, gj = V.j0 - 1 + wy;
-    if (gi < 0 || gj < 0) continue;
-    const int s = (wx + 1) + MWX * (wy + 1);
-    const int f = DF_U + q;
-    const T* Fm = V.D(f, m - 1);
-    const T* Fc = V.D(f, m);
-    const T* Fp = V.D(f, m + 1);
-    T val;
-    if (q == 0) {
-      if (!(gi > 0 && gi < p.nx && gj < p.ny && m < p.nz)) continue;
-      val = diffuse_at<0>(p, c, Fm, Fc, Fp, Nm, Nc, s, gi, gj, m);
-    } else if (q == 1) {
-      if (!(gi < p.nx && gj > 0 && gj < p.ny && m < p.nz)) continue;
-      val = diffuse_at<1>(p, c, Fm, Fc, Fp, Nm, Nc, s, gi, gj, m);
-    } else {
-      if (!(gi < p.nx && gj < p.ny && m > 0 && m < p.nz)) continue;
-      val = diffuse_at<2>(p, c, Fm, Fc, Fp, Nm, Nc, s, gi, gj, m);
+__device__ __forceinline__ T diffuse_face(const StepParams<T>& p, T c, T x0, T xm, T xp, T ym, T yp, T zm, T zp, T n0, T n1) {
+  const T lap = xm + xp + ym + yp + zm + zp - T(6) * x0;
+  const T nf = T(0.5) * (n0 + n1);
+  return x0 + c * (p.nu + nf) * lap;
+}
+// ... of a face with all its neighbours inside; f: its place in the plane.
+template <typename T>
+__device__ __forceinline__ T diffuse_inner(const StepParams<T>& p, T c, const T* f, T x0, T zm, T zp, T n0, T n1) {
+  return diffuse_face(p, c, x0, f[-1], f[1], f[-MWX], f[MWX], zm, zp, n0, n1);
+}
+// u2 of component Q at lattice point (i, j, m) near the domain's ends, b its
+// place in the staged window; in: the component's inflow value of the plane.
+// A boundary face takes its rule's value (at an outlet that of the adjacent
+// interior face, formed here too), so that whoever reads u2 finds every face.
+// 0 off the lattice.
+template <int Q, typename T>
+__device__ __forceinline__ T u2_edge(const StepParams<T>& p, const MView<T>& V, T c, int b, int i, int j, int m, T in) {
+  const int nx = p.nx, ny = p.ny, nz = p.nz;
+  if (i < 0 || j < 0 || m < 0 || i >= nx + (Q == 0) || j >= ny + (Q == 1) || m >= nz + (Q == 2)) return T(0);
+  if (Q == 2 && (m == 0 || m == nz)) return T(0);
+  int rule = NOSLIP + 1;   // of a boundary face
+  if (Q == 0) {
+    if (i == 0) { rule = p.side[0]; i += 1; b += 1; }
+    else if (i == nx) { rule = p.side[1]; i -= 1; b -= 1; }
+  }
+  if (Q == 1) {
+    if (j == 0) { rule = p.side[2]; j += 1; b += MWX; }
+    else if (j == ny) { rule = p.side[3]; j -= 1; b -= MWX; }
+  }
+  const T *f = mom_sm<T>(V.D(Q, m)) + b, *n = mom_sm<T>(V.D(DF_NUT, m)) + b;
+  const T x0 = f[0];
+  T xm = f[-1], xp = f[1], ym = f[-MWX], yp = f[MWX], zm = mom_sm<T>(V.D(Q, m - 1))[b], zp = mom_sm<T>(V.D(Q, m + 1))[b];
+  // along its own axis the neighbour may be a boundary face, along the others a ghost
+  if (Q == 0) {
+    if (i == 1) xm = normal_face(p.side[0], x0, in);
+    if (i == nx - 1) xp = normal_face(p.side[1], x0, in);
+  } else {
+    if (i == 0) xm = tangential_ghost(p.side[0], x0, in);
+    if (i == nx - 1) xp = tangential_ghost(p.side[1], x0, in);
+  }
+  if (Q == 1) {
+    if (j == 1) ym = normal_face(p.side[2], x0, in);
+    if (j == ny - 1) yp = normal_face(p.side[3], x0, in);
+  } else {
+    if (j == 0) ym = tangential_ghost(p.side[2], x0, in);
+    if (j == ny - 1) yp = tangential_ghost(p.side[3], x0, in);
+  }
+  if (Q == 2) {
+    if (m == 1) zm = T(0);
+    if (m == nz - 1) zp = T(0);
+  } else {
+    if (m == 0) zm = tangential_ghost(p.side[4], x0, T(0));
+    if (m == nz - 1) zp = tangential_ghost(p.side[5], x0, T(0));
+  }
+  const T n0 = Q == 0 ? n[-1] : (Q == 1 ? n[-MWX] : mom_sm<T>(V.D(DF_NUT, m - 1))[b]);
+  const T val = diffuse_face(p, c, x0, xm, xp, ym, yp, zm, zp, n0, n[0]);
+  return rule > NOSLIP ? val : normal_face(rule, val, in);
+}
+template <int Q, typename T>
+__device__ __forceinline__ void tape_u2(const MomentumArgs<T>& M, const MView<T>& V, int i, int j, int m, T val) {
+  // the column's own interior faces
+  if (m < V.k0 || m >= V.kend || i >= M.p.nx || j >= M.p.ny || (Q == 0 ? i : (Q == 1 ? j : m)) == 0) return;
+  if (Q == 0) M.u2t[idx_u(M.p, i, j, m)] = val;
+  else if (Q == 1) M.v2t[idx_v(M.p, i, j, m)] = val;
+  else M.w2t[idx_c(M.p, i, j, m)] = val;
+}
+
+// A thread's own staged values on the planes m - 1 and m (u~, v~, w~, nu_t),
+// rolled along the march.
+template <typename T>
+struct OwnColumn {
+  T below[4], here[4];
+  __device__ __forceinline__ void start(const MView<T>& V, int b, int m) {   // before u2_plane(m)
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+      below[f] = mom_sm<T>(V.D(f, m - 1))[b];
+      here[f] = mom_sm<T>(V.D(f, m))[b];
     }
-    V.U2(q, m)[t] = val;
-    if (M.u2t) {   // tape of the owned interior faces
-      const bool ox = gi >= V.i0 && gi < V.i0 + MX, oy = gj >= V.j0 && gj < V.j0 + MY, oz = m >= k0 && m < kend;
-      if (ox && oy && oz) {
-        if (q == 0) M.u2t[idx_u(p, gi, gj, m)] = val;
-        else if (q == 1) M.v2t[idx_v(p, gi, gj, m)] = val;
-        else M.w2t[idx_c(p, gi, gj, m)] = val;
-      }
+  }
+};
+
+// u2 on plane m: the thread's own faces and its halo face.
+template <bool EDGE, typename T>
+__device__ __forceinline__ void u2_plane(const MomentumArgs<T>& M, const MView<T>& V, const Places& X, OwnColumn<T>& O, T c, int m) {
+  const StepParams<T>& p = M.p;
+  constexpr int FS = DR * MWP, US = UR * MHP;   // from one field (component) to the next
+  const T* fc = mom_sm<T>(V.D(0, m)) + X.b;
+  const T* fp = mom_sm<T>(V.D(0, m + 1)) + X.b;
+  T* u2 = mom_sm<T>(V.U2(0, m));
+  T next[4];
+#pragma unroll
+  for (int f = 0; f < 4; ++f) next[f] = fp[f * FS];
+  if (EDGE) {
+    const T prof = m >= 0 && m < p.nz ? p.prof[m] : T(0);
+    const T inu = prof * p.dirx, inv = prof * p.diry;
+    const T a = u2_edge<0>(p, V, c, X.b, X.gi, X.gj, m, inu);
+    const T b = u2_edge<1>(p, V, c, X.b, X.gi, X.gj, m, inv);
+    const T w = u2_edge<2>(p, V, c, X.b, X.gi, X.gj, m, T(0));
+    T h = 0;
+    if (X.hq == 0) h = u2_edge<0>(p, V, c, X.hb, X.hi, X.hj, m, inu);
+    else if (X.hq == 1) h = u2_edge<1>(p, V, c, X.hb, X.hi, X.hj, m, inv);
+    else if (X.hq == 2) h = u2_edge<2>(p, V, c, X.hb, X.hi, X.hj, m, T(0));
+    u2[X.h] = a;
+    u2[US + X.h] = b;
+    u2[2 * US + X.h] = w;
+    if (X.hq < 3) u2[X.hq * US + X.hh] = h;
+    if (M.u2t) {
+      tape_u2<0>(M, V, X.gi, X.gj, m, a);
+      tape_u2<1>(M, V, X.gi, X.gj, m, b);
+      tape_u2<2>(M, V, X.gi, X.gj, m, w);
+    }
+  } else {
+    const T* n = fc + 3 * FS;
+    const T a = diffuse_inner(p, c, fc, O.here[0], O.below[0], next[0], n[-1], O.here[3]);
+    const T b = diffuse_inner(p, c, fc + FS, O.here[1], O.below[1], next[1], n[-MWX], O.here[3]);
+    const T w = diffuse_inner(p, c, fc + 2 * FS, O.here[2], O.below[2], next[2], O.below[3], O.here[3]);
+    T h = 0;
+    if (X.hq < 3) {
+      const T* g = mom_sm<T>(V.D(0, m)) + X.hq * FS + X.hb;
+      const T *gm = mom_sm<T>(V.D(0, m - 1)) + X.hb, *gp = mom_sm<T>(V.D(0, m + 1)) + X.hb;
+      const T* gn = mom_sm<T>(V.D(DF_NUT, m)) + X.hb;
+      h = diffuse_inner(p, c, g, g[0], gm[X.hq * FS], gp[X.hq * FS], X.hq == 2 ? gm[3 * FS] : gn[X.hq == 0 ? -1 : -MWX], gn[0]);
+    }
+    u2[X.h] = a;
+    u2[US + X.h] = b;
+    u2[2 * US + X.h] = w;
+    if (X.hq < 3) u2[X.hq * US + X.hh] = h;
+    if (M.u2t) {
+      tape_u2<0>(M, V, X.gi, X.gj, m, a);
+      tape_u2<1>(M, V, X.gi, X.gj, m, b);
+      tape_u2<2>(M, V, X.gi, X.gj, m, w);
+    }
+  }
+#pragma unroll
+  for (int f = 0; f < 4; ++f) {
+    O.below[f] = O.here[f];
+    O.here[f] = next[f];
+  }
+}
+
+// Drag of a face away from the domain's ends: q its value, cf the mean drag
+// coefficient, a0..a3 and b0..b3 the four faces around it of the other two
+// components, in the order of drag_at; o: its position among q and the two
+// means (0, 1, 2 for u, v, w).  With cf = 0 the factor is exactly 1.
+template <int O, typename T, typename FA, typename FB>
+__device__ __forceinline__ T drag_inner(T dt, T q, T cf, FA a, FB b) {
+  if (cf == T(0)) return q;
+  const T am = T(0.25) * (a(0) + a(1) + a(2) + a(3));
+  const T bm = T(0.25) * (b(0) + b(1) + b(2) + b(3));
+  const T sp = O == 0 ? sqrt(q * q + am * am + bm * bm) : (O == 1 ? sqrt(am * am + q * q + bm * bm) : sqrt(am * am + bm * bm + q * q));
+  return fmax(T(0), T(1) - dt * cf * sp) * q;
+}
+// u3 of a face away from the ends at places h (u2 window) and s (staged
+// window): an x face and a y face of plane k, a z face of plane k.
+template <typename T>
+__device__ __forceinline__ T u3_inner(const MView<T>& V, T dt, int h, int s, int k) {
+  const T *u = mom_sm<T>(V.U2(0, k)) + h, *v = mom_sm<T>(V.U2(1, k)) + h, *w = mom_sm<T>(V.U2(2, k)) + h, *wp = mom_sm<T>(V.U2(2, k + 1)) + h;
+  const T* C = mom_sm<T>(V.D(DF_C, k)) + s;
+  return drag_inner<0>(dt, u[0], T(0.5) * (C[-1] + C[0]), [&](int e) { return v[-1 + (e & 1) + (e >> 1) * MHX]; },
+                       [&](int e) { return (e < 2 ? w : wp)[-1 + (e & 1)]; });
+}
+template <typename T>
+__device__ __forceinline__ T v3_inner(const MView<T>& V, T dt, int h, int s, int k) {
+  const T *u = mom_sm<T>(V.U2(0, k)) + h, *v = mom_sm<T>(V.U2(1, k)) + h, *w = mom_sm<T>(V.U2(2, k)) + h, *wp = mom_sm<T>(V.U2(2, k + 1)) + h;
+  const T* C = mom_sm<T>(V.D(DF_C, k)) + s;
+  return drag_inner<1>(dt, v[0], T(0.5) * (C[-MWX] + C[0]), [&](int e) { return u[-MHX + (e & 1) + (e >> 1) * MHX]; },
+                       [&](int e) { return (e < 2 ? w : wp)[-MHX + (e & 1) * MHX]; });
+}
+template <typename T>
+__device__ __forceinline__ T w3_inner(const MView<T>& V, T dt, int h, int s, int k) {
+  const T *u = mom_sm<T>(V.U2(0, k)) + h, *v = mom_sm<T>(V.U2(1, k)) + h, *w = mom_sm<T>(V.U2(2, k)) + h;
+  const T *um = mom_sm<T>(V.U2(0, k - 1)) + h, *vm = mom_sm<T>(V.U2(1, k - 1)) + h;
+  const T c0 = mom_sm<T>(V.D(DF_C, k - 1))[s], c1 = mom_sm<T>(V.D(DF_C, k))[s];
+  return drag_inner<2>(dt, w[0], T(0.5) * (c0 + c1), [&](int e) { return (e < 2 ? um : u)[e & 1]; },
+                       [&](int e) { return (e < 2 ? vm : v)[(e & 1) * MHX]; });
+}
+
+// u3 on the faces of plane k and the w faces of plane k + 1 (only_w: those
+// alone); the x and y faces go to shared memory for the fluxes.  own[]: the
+// thread's own u3, v3 of plane k and w3 of plane k + 1.  The faces on the
+// column's far sides, the row j0 + MY of y faces and the column i0 + MX of x
+// faces, are formed by the first warp and by a lane per row of the second.
+template <bool EDGE, typename T>
+__device__ __forceinline__ void u3_plane(const MomentumArgs<T>& M, const MView<T>& V, const Places& X, T dt, int k, bool only_w,
+                                         T (&own)[3]) {
+  const StepParams<T>& p = M.p;
+  const int t = threadIdx.x, tx = t % MX, ty = t / MX;
+  T *sU = V.sU3(), *sV = V.sV3();
+  T* gu = M.u + (size_t)k * ((size_t)p.Pu * p.ny);
+  T* gv = M.v + (size_t)k * ((size_t)p.Pc * (p.ny + 1));
+  T* gw = M.w + (size_t)(k + 1) * ((size_t)p.Pc * p.ny);
+  const bool own_w = k + 1 < V.kend || k + 1 == p.nz;
+  const T prof = EDGE && k >= 0 ? p.prof[k] : T(0);
+  // x face (i, j) and y face (i, j): places h, b; a boundary face follows its rule on the dragged interior neighbour
+  auto xface = [&](int h, int b, int i) {
+    const int sh = EDGE ? (i == 0 ? 1 : (i == p.nx ? -1 : 0)) : 0;
+    const T r = u3_inner(V, dt, h + sh, b + sh, k);
+    return EDGE && sh ? normal_face(p.side[i == 0 ? 0 : 1], r, prof * p.dirx) : r;
+  };
+  auto yface = [&](int h, int b, int j) {
+    const int sh = EDGE ? (j == 0 ? 1 : (j == p.ny ? -1 : 0)) : 0;
+    const T r = v3_inner(V, dt, h + sh * MHX, b + sh * MWX, k);
+    return EDGE && sh ? normal_face(p.side[j == 0 ? 2 : 3], r, prof * p.diry) : r;
+  };
+  const int gi = X.gi, gj = X.gj;
+  const bool in_x = !EDGE || gi < p.nx, in_y = !EDGE || gj < p.ny;
+  if (in_x && in_y) {
+    own[2] = EDGE && (k + 1 == 0 || k + 1 == p.nz) ? T(0) : w3_inner(V, dt, X.h, X.b, k + 1);
+    if (own_w) gw[gi + p.Pc * gj] = own[2];
+  }
+  if (only_w) return;
+  if (!EDGE || (gi <= p.nx && in_y)) {
+    own[0] = xface(X.h, X.b, gi);
+    sU[tx + (MX + 1) * ty] = own[0];
+    gu[gi + p.Pu * gj] = own[0];
+  }
+  if (!EDGE || (in_x && gj <= p.ny)) {
+    own[1] = yface(X.h, X.b, gj);
+    sV[t] = own[1];
+    gv[gi + p.Pc * gj] = own[1];
+  }
+  if (t < MX) {
+    const int j = V.j0 + MY;
+    if (!EDGE || (in_x && j <= p.ny)) {
+      const T val = yface(X.h + MHX * MY, X.b + MWX * MY, j);
+      sV[t + MT] = val;
+      if (EDGE && j == p.ny) gv[gi + p.Pc * j] = val;
+    }
+  } else if (t < MX + MY) {
+    const int i = V.i0 + MX, j = V.j0 + tx;
+    if (!EDGE || (i <= p.nx && j < p.ny)) {
+      const T val = xface(MX + 1 + MHX * (tx + 1), MX + 2 + MWX * (tx + 2), i);
+      sU[MX + (MX + 1) * tx] = val;
+      if (EDGE && i == p.nx) gu[i + p.Pu * j] = val;
     }
   }
 }
 
 template <typename T>
 __device__ __forceinline__ void momentum_fused_body(const MomentumArgs<T>& M, const VBlock& vb) {
-  extern __shared__ __align__(16) unsigned char mom_smem[];
   __shared__ double sh[32];
   __shared__ bool last;
   const StepParams<T>& p = M.p;
   MView<T> V;
-  V.sD = reinterpret_cast<T*>(mom_smem);
-  V.sU2 = V.sD + DF_N * DR * MWP;
-  V.sU3 = V.sU2 + 3 * UR * MHP;
-  V.sV3 = V.sU3 + (MX + 1) * MY;
   V.i0 = vb.x * MX;
   V.j0 = vb.y * MY;
-  const int k0 = vb.z * M.zc, kend = min(p.nz, k0 + M.zc);
-  const int tid = threadIdx.x, tx = tid % MX, ty = tid / MX;
-  const int gi = V.i0 + tx, gj = V.j0 + ty;
-  const bool own_c = gi < p.nx && gj < p.ny;
+  V.k0 = vb.z * M.zc;
+  V.kend = min(p.nz, V.k0 + M.zc);
+  const int k0 = V.k0, kend = V.kend;
+  const int tx = threadIdx.x % MX, ty = threadIdx.x / MX;
+  const Places X = block_places(V.i0, V.j0);
+  const bool own_c = X.gi < p.nx && X.gj < p.ny;
   const T dt = *p.dtT;
   const T c = dt * p.inv_h * p.inv_h;
   const T sc = -p.rho * p.h / *p.dtT;
-  for (int kk = k0 - 2; kk <= k0 + 2; ++kk) stage_momentum(M, V.sD, V.i0, V.j0, kk);
-  cp_async_commit();
-  cp_async_wait_all();
-  __syncthreads();
-  u2_plane(M, V, c, k0 - 1, k0, kend);
-  u2_plane(M, V, c, k0, k0, kend);
-  __syncthreads();
-  const int h_own = V.hidx(gi, gj), s_own = V.sidx(gi, gj);
-  // w3 of the column's bottom face (owned when k0 is this chunk's first plane)
-  T w3lo = T(0);
-  if (own_c) {
-    const T* A[3] = {V.U2(0, k0), V.U2(1, k0), V.U2(2, k0)};
-    const T* B[3] = {V.U2(0, k0 - 1), V.U2(1, k0 - 1), V.U2(2, k0 - 1)};
-    w3lo = w3_at(p, dt, A, B, V.D(DF_C, k0 - 1), V.D(DF_C, k0), h_own, s_own, gi, gj, k0);
-    M.w[idx_c(p, gi, gj, k0)] = w3lo;
+  StagePos S;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int t = threadIdx.x + h * MT, gx = V.i0 - 2 + t % MWX, gy = V.j0 - 2 + t / MWX;
+    const bool in = t < MWP && gx >= 0 && gy >= 0;
+    S.u[h] = gx + p.Pu * gy;
+    S.c[h] = gx + p.Pc * gy;
+    S.ok[h] = !in ? 0 : (gx <= p.nx && gy < p.ny ? 1 : 0) | (gx < p.nx && gy <= p.ny ? 2 : 0) | (gx < p.nx && gy < p.ny ? 4 : 0);
   }
+  // no face of the halo-1 window, nor a neighbour of one, on the domain's x and y ends
+  const bool inner = V.i0 >= 3 && V.i0 + MX + 1 <= p.nx - 1 && V.j0 >= 3 && V.j0 + MY + 1 <= p.ny - 1;
+  auto edge2 = [&](int m) { return !inner || m < 2 || m > p.nz - 2; };          // of u2 on plane m
+  auto edge3 = [&](int k) { return !inner || k < 1 || k + 1 > p.nz - 1; };      // of u3 on plane k and w3 on k + 1
+  for (int kk = k0 - 2; kk <= k0; ++kk) stage_momentum(M, V, S, kk);
+  cp_async_commit();
   DotAcc<T> dacc;
-  for (int k = k0; k < kend; ++k) {
+  T own[3] = {T(0), T(0), T(0)}, w3lo = T(0);
+  OwnColumn<T> O;
+  // b of plane k from the faces in shared memory and the thread's own
+  auto rhs = [&](int k) {
+    // cell_flux: u(i+1)-u(i) + v(j+1)-v(j) + w(k+1)-w(k)
+    const T flux = V.sU3()[(tx + 1) + (MX + 1) * ty] - own[0] + V.sV3()[tx + MX * (ty + 1)] - own[1] + own[2] - w3lo;
+    const T bv = sc * flux;
+    (M.b + (size_t)k * ((size_t)p.Pc * p.ny))[X.gi + p.Pc * X.gj] = bv;
+    dacc.add(bv, bv);
+    w3lo = own[2];
+  };
+  // m: the plane of u2; the faces follow one plane behind, b another one
+  for (int m = k0 - 1; m <= kend; ++m) {
+    const int k = m - 1;
     cp_async_wait_all();
     __syncthreads();
-    stage_momentum(M, V.sD, V.i0, V.j0, k + 3);
+    stage_momentum(M, V, S, m + 2);   // into the slot of m - 2
     cp_async_commit();
-    u2_plane(M, V, c, k + 1, k0, kend);
+    if (m == k0 - 1) O.start(V, X.b, m);
+    if (k > k0 && own_c) rhs(k - 1);
+    if (edge2(m)) u2_plane<true>(M, V, X, O, c, m);
+    else u2_plane<false>(M, V, X, O, c, m);
+    if (m < k0) continue;
     __syncthreads();
-    // u3 of plane k's x faces i0..i0+MX and y faces j0..j0+MY, w3 of plane k+1
-    const T* A[3] = {V.U2(0, k), V.U2(1, k), V.U2(2, k)};
-    const T* B[3] = {V.U2(0, k + 1), V.U2(1, k + 1), V.U2(2, k + 1)};
-    const T* Ck = V.D(DF_C, k);
-    for (int it = tid; it < (MX + 1) * MY; it += MT) {
-      const int fx = it % (MX + 1), fy = it / (MX + 1);
-      const int fi = V.i0 + fx, fj = V.j0 + fy;
-      if (fi <= p.nx && fj < p.ny) {
-        const T val = u3_at(p, dt, A, B, Ck, (fx + 1) + MHX * (fy + 1), (fx + 2) + MWX * (fy + 2), fi, fj, k);
-        V.sU3[it] = val;
-        const bool own = fi < V.i0 + MX || fi == p.nx;
-        if (own) M.u[idx_u(p, fi, fj, k)] = val;
-      }
-    }
-    for (int it = tid; it < MX * (MY + 1); it += MT) {
-      const int fx = it % MX, fy = it / MX;
-      const int fi = V.i0 + fx, fj = V.j0 + fy;
-      if (fi < p.nx && fj <= p.ny) {
-        const T val = v3_at(p, dt, A, B, Ck, (fx + 1) + MHX * (fy + 1), (fx + 2) + MWX * (fy + 2), fi, fj, k);
-        V.sV3[it] = val;
-        const bool own = fj < V.j0 + MY || fj == p.ny;
-        if (own) M.v[idx_v(p, fi, fj, k)] = val;
-      }
-    }
-    T w3hi = T(0);
-    if (own_c) {
-      w3hi = w3_at(p, dt, B, A, Ck, V.D(DF_C, k + 1), h_own, s_own, gi, gj, k + 1);
-      if (k + 1 < kend || k + 1 == p.nz) M.w[idx_c(p, gi, gj, k + 1)] = w3hi;
-    }
-    __syncthreads();
-    if (own_c) {
-      // cell_flux: u(i+1)-u(i) + v(j+1)-v(j) + w(k+1)-w(k)
-      const T flux = V.sU3[(tx + 1) + (MX + 1) * ty] - V.sU3[tx + (MX + 1) * ty] + V.sV3[tx + MX * (ty + 1)] -
-                     V.sV3[tx + MX * ty] + w3hi - w3lo;
-      const T bv = sc * flux;
-      M.b[idx_c(p, gi, gj, k)] = bv;
-      dacc.add(bv, bv);
-    }
-    w3lo = w3hi;
+    // (at m = k0 only the w faces of the column's bottom, for the first flux)
+    if (edge3(k)) u3_plane<true>(M, V, X, dt, k, k < k0, own);
+    else u3_plane<false>(M, V, X, dt, k, k < k0, own);
+    if (k < k0) w3lo = own[2];
   }
+  __syncthreads();
+  if (own_c) rhs(kend - 1);
   cp_async_wait_all();
   double acc = 0.0;
   acc += dacc.value();
@@ -369,7 +439,7 @@ __device__ __forceinline__ void momentum_fused_body(const MomentumArgs<T>& M, co
 }
 
 template <typename T>
-__global__ void __launch_bounds__(MT) k_momentum_fused(const __grid_constant__ MomentumArgs<T> M) {
+__global__ void __launch_bounds__(MT, sizeof(T) == 8 ? 2 : UF_MOMENTUM_MINB) k_momentum_fused(const __grid_constant__ MomentumArgs<T> M) {
   momentum_fused_body<T>(M, vblock());
 }
 
