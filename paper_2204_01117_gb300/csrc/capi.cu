@@ -142,7 +142,7 @@ struct Plan {
   std::vector<size_t> lr, lx, lt, lu;   // lu: scratch of the cluster V-cycle (levels >= 1)
   bool sep;                             // the separable inverse is available (sep_solve.cuh)
   size_t sep_y[2], sep_z[2];            // its packed matrices (forward, inverse); the pivots lie in r2
-  size_t prof, dt, dtT, scal, state, partials, ainv, boxes, grad;
+  size_t prof, dt, dtT, scal, state, partials, ainv, grad;
   size_t total;
 };
 
@@ -220,7 +220,6 @@ Plan make_plan(const uf_grid_desc* d) {
   P.state = L.take(sizeof(uf::SolveState));
   P.partials = L.take(sizeof(double) * kPartials * 2);
   P.ainv = L.take(sizeof(double) * (size_t)P.coarse_n * P.coarse_n);
-  P.boxes = L.take(sizeof(uf::DesignBox) * uf::MAX_BOXES);
   P.grad = L.take(sizeof(double) * 3 * uf::MAX_BOXES);
   P.sep = sep_available(d);
   if (P.sep) {
@@ -1393,25 +1392,26 @@ class GridImpl final : public uf_grid {
   }
 
   // ---------------------------------------------------- design -> phi ----
-  uf_status upload_boxes(int nbox, const double* boxes, const double* theta) {
+  static dim3 design_grid(int nx, int ny, int nz) {
+    return dim3((nx + uf::BX - 1) / uf::BX, (ny + uf::BY - 1) / uf::BY, (nz + uf::DZ - 1) / uf::DZ);
+  }
+  uf_status pack_boxes(int nbox, const double* boxes, const double* theta, uf::DesignBoxes* out) {
     if (nbox < 1 || nbox > uf::MAX_BOXES) return fail(UF_ERR_ARG, "nbox must lie in [1, 64]");
     if (!boxes || !theta) return fail(UF_ERR_ARG, "NULL boxes or theta");
-    std::vector<uf::DesignBox> hb(nbox);
+    std::memset(out, 0, sizeof(*out));
     for (int i = 0; i < nbox; ++i)
-      hb[i] = {boxes[4 * i], boxes[4 * i + 1], boxes[4 * i + 2], boxes[4 * i + 3], theta[3 * i], theta[3 * i + 1],
-               theta[3 * i + 2]};
-    UF_CUDA(cudaMemcpyAsync(at<uf::DesignBox>(P.boxes), hb.data(), sizeof(uf::DesignBox) * nbox, cudaMemcpyHostToDevice,
-                            stream));
-    UF_CUDA(cudaStreamSynchronize(stream));
+      out->b[i] = {boxes[4 * i], boxes[4 * i + 1], boxes[4 * i + 2], boxes[4 * i + 3], theta[3 * i], theta[3 * i + 1],
+                   theta[3 * i + 2]};
     return UF_OK;
   }
   uf_status design_phi(int nbox, const double* boxes, const double* theta, double width, void* out) override {
     if (!(width > 0)) return fail(UF_ERR_ARG, "width must be positive");
-    uf_status s = upload_boxes(nbox, boxes, theta);
+    uf::DesignBoxes hb;
+    uf_status s = pack_boxes(nbox, boxes, theta, &hb);
     if (s != UF_OK) return s;
     T* dst = out ? q : phi;
-    uf::k_design_phi<T><<<plane_grid(d.nx, d.ny, d.nz), dim3(uf::BX, uf::BY), 0, stream>>>(
-        d.nx, d.ny, d.nz, P.Pc, d.h, at<uf::DesignBox>(P.boxes), nbox, width, dst);
+    uf::k_design_phi<T><<<design_grid(d.nx, d.ny, d.nz), dim3(uf::BX, uf::BY), 0, stream>>>(d.nx, d.ny, d.nz, P.Pc, d.h, hb, nbox,
+                                                                                            width, dst);
     UF_CUDA(cudaGetLastError());
     if (out) return copy_out(out, q, d.nx, d.ny, d.nz, P.Pc);
     const size_t n = P.n_c;
@@ -1422,14 +1422,15 @@ class GridImpl final : public uf_grid {
   uf_status design_vjp(int nbox, const double* boxes, const double* theta, double width, const void* lphi_in,
                        double* g_out) override {
     if (!(width > 0) || !g_out) return fail(UF_ERR_ARG, "width must be positive and g_out non-NULL");
-    uf_status s = upload_boxes(nbox, boxes, theta);
+    uf::DesignBoxes hb;
+    uf_status s = pack_boxes(nbox, boxes, theta, &hb);
     if (s != UF_OK) return s;
     s = copy_in(q, d.nx, d.ny, d.nz, P.Pc, lphi_in);
     if (s != UF_OK) return s;
     double* g = at<double>(P.grad);
     UF_CUDA(cudaMemsetAsync(g, 0, sizeof(double) * 3 * nbox, stream));
-    uf::k_design_phi_vjp<T><<<plane_grid(d.nx, d.ny, d.nz), dim3(uf::BX, uf::BY), 0, stream>>>(
-        d.nx, d.ny, d.nz, P.Pc, d.h, at<uf::DesignBox>(P.boxes), nbox, width, q, g);
+    uf::k_design_phi_vjp<T><<<design_grid(d.nx, d.ny, d.nz), dim3(uf::BX, uf::BY), 0, stream>>>(d.nx, d.ny, d.nz, P.Pc, d.h, hb, nbox,
+                                                                                                width, q, g);
     UF_CUDA(cudaGetLastError());
     UF_CUDA(cudaMemcpyAsync(g_out, g, sizeof(double) * 3 * nbox, cudaMemcpyDeviceToHost, stream));
     UF_CUDA(cudaStreamSynchronize(stream));
