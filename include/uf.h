@@ -384,7 +384,9 @@ uf_status uf_design_to_phi(uf_grid* g, int nbox, const double* boxes, const doub
  * decisions are made in FP64 with every operation rounded separately, so
  * they are reproducible.  phi_out == NULL: sets the grid's porosity (as
  * uf_set_porosity); else writes the dense field there (host or device).
- * Allocates and frees device memory for the mesh; synchronises.  Errors:
+ * The mesh goes to the step's scratch arrays where it fits (call between
+ * steps, as uf_set_fields), else to device memory allocated and freed by the
+ * call; synchronises.  Errors:
  * UF_ERR_ARG (NULL arrays, sub outside 1..16, a triangle range outside the
  * mesh, a porosity outside [0, 1], a non-finite vertex). */
 uf_status uf_mesh_to_phi(uf_grid* g, int ntri, const double* tris, int nobj, const int* obj_first,

@@ -2025,27 +2025,47 @@ class GridImpl final : public uf_grid {
         }
       }
     }
-    double* dtri = nullptr;
-    uf::MeshObject* dobj = nullptr;
-    const size_t tb_tri = (size_t)std::max(ntri, 1) * 9 * sizeof(double);
-    const size_t tb_obj = (size_t)std::max(nobj, 1) * sizeof(uf::MeshObject);
-    UF_CUDA(cudaMalloc(&dtri, tb_tri));
-    cudaError_t e = cudaMalloc(&dobj, tb_obj);
-    if (e == cudaSuccess && ntri > 0)
-      e = cudaMemcpyAsync(dtri, tris, (size_t)ntri * 9 * sizeof(double), cudaMemcpyHostToDevice, stream);
+    // the triangles, the objects and the per-triangle tables of the crossing
+    // tests: in the step's scratch arrays (uh .. w2, recomputed by every step)
+    // where they fit, else in memory allocated for the call
+    long long entries = 0;
+    for (int o = 0; o < nobj; ++o) {
+      uf::MeshObject& m = obj[o];
+      if (entries > 0x7fffffffLL - m.count) return fail(UF_ERR_ARG, "too many triangles");
+      m.entry = (int)entries;
+      entries += m.count;
+      const double size = std::max({m.hi[0] - m.lo[0], m.hi[1] - m.lo[1], m.hi[2] - m.lo[2]}) + 2.0 * d.h;
+      m.scale = 1.0 / size;
+    }
+    Layout ML;
+    const size_t o_tri = ML.take((size_t)ntri * 9 * sizeof(double)), o_obj = ML.take((size_t)nobj * sizeof(uf::MeshObject));
+    const size_t o_te = ML.take((size_t)entries * sizeof(uf::MeshTri)), o_tf = ML.take((size_t)entries * sizeof(uf::MeshTriF));
+    char *block = at<char>(P.uh), *owned = nullptr;
+    if (ML.off > P.k0 - P.uh) {
+      UF_CUDA(cudaMalloc(&owned, ML.off));
+      block = owned;
+    }
+    const double* dtri = reinterpret_cast<const double*>(block + o_tri);
+    const uf::MeshObject* dobj = reinterpret_cast<const uf::MeshObject*>(block + o_obj);
+    uf::MeshTri* te = reinterpret_cast<uf::MeshTri*>(block + o_te);
+    uf::MeshTriF* tf = reinterpret_cast<uf::MeshTriF*>(block + o_tf);
+    cudaError_t e = cudaSuccess;
+    if (ntri > 0)
+      e = cudaMemcpyAsync(block + o_tri, tris, (size_t)ntri * 9 * sizeof(double), cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess && nobj > 0)
-      e = cudaMemcpyAsync(dobj, obj.data(), nobj * sizeof(uf::MeshObject), cudaMemcpyHostToDevice, stream);
+      e = cudaMemcpyAsync(block + o_obj, obj.data(), nobj * sizeof(uf::MeshObject), cudaMemcpyHostToDevice, stream);
     T* dst = phi_out ? q : phi;
+    if (e == cudaSuccess && nobj > 0) {
+      uf::k_mesh_prep<128><<<nobj, 128, 0, stream>>>(dtri, dobj, te, tf);
+      e = cudaGetLastError();
+    }
     if (e == cudaSuccess) {
-      const long long cells = (long long)d.nx * d.ny * d.nz;
-      const unsigned blocks = (unsigned)((cells + uf::MESH_WARPS - 1) / uf::MESH_WARPS);
-      uf::k_mesh_phi<T><<<blocks, 32 * uf::MESH_WARPS, 0, stream>>>(d.nx, d.ny, d.nz, P.Pc, d.h, sub, dtri, dobj,
-                                                                     nobj, dst);
+      const dim3 g((d.nx + uf::MESH_BX - 1) / uf::MESH_BX, (d.ny + uf::MESH_BY - 1) / uf::MESH_BY, (d.nz + uf::MESH_BZ - 1) / uf::MESH_BZ);
+      uf::k_mesh_phi<T><<<g, 32 * uf::MESH_WARPS, 0, stream>>>(d.nx, d.ny, d.nz, P.Pc, d.h, sub, te, tf, dobj, nobj, dst);
       e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-    cudaFree(dtri);
-    if (dobj) cudaFree(dobj);
+    if (owned) cudaFree(owned);
     UF_CUDA(e);
     if (phi_out) {
       uf_status s = copy_out(phi_out, q, d.nx, d.ny, d.nz, P.Pc);
