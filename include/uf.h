@@ -60,11 +60,12 @@ typedef enum {
 enum { UF_F32 = 0,   /* FP32 fields, FP64 reductions and coarsest MG solve */
        UF_F64 = 1 }; /* FP64 throughout                                     */
 
-enum { UF_PRECOND_MG = 0,      /* geometric multigrid V-cycle (default); FP32
-                                  grids with the default smoother and transfers
-                                  use the exact inverse by separation of
-                                  variables in its place (uf_tuning.coarse_start
-                                  below): same solution, fewer CG iterations    */
+enum { UF_PRECOND_MG = 0,      /* geometric multigrid V-cycle (default); with
+                                  the default smoother and transfers the exact
+                                  inverse by separation of variables takes its
+                                  place where the sizes allow
+                                  (uf_tuning.coarse_start below): the same
+                                  solution in fewer CG iterations               */
        UF_PRECOND_AI1 = 1,     /* approximate inverse, 1st order (Sec. 3)     */
        UF_PRECOND_JACOBI = 2,
        UF_PRECOND_NONE = 3,
@@ -427,9 +428,10 @@ typedef struct {
                                  BCs and the pressure right-hand side as
                                  three kernels.  Both forms give the same
                                  values bit for bit.  0 = all fused (default) */
-  int coarse_start;           /* 0 = automatic: FP32 grids with the default
+  int coarse_start;           /* 0 = automatic: grids with the default
                                  smoother (CHEBY) and transfers (LINEAR), nx <=
-                                 1024, ny <= 1392 and nz <= 400 run the exact
+                                 1024 and, in FP32, ny <= 1392 and nz <= 400,
+                                 in FP64, ny + nz <= 480, run the exact
                                  inverse of the operator (separation of
                                  variables: cosine transforms along y and z,
                                  tridiagonal solves along x) in place of the

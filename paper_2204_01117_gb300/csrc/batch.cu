@@ -197,12 +197,13 @@ struct MgP {     // V-cycle level kernels
   uf::SolveState* st;
 };
 
+template <typename T>
 struct SepP {    // separable inverse
-  uf::Level<float> L;
-  uf::Sep S;
-  float* x;
-  const float *d0, *d1, *q;
-  float* z;
+  uf::Level<T> L;
+  uf::Sep<T> S;
+  T* x;
+  const T *d0, *d1, *q;
+  T* z;
   double* partials;
   uf::SolveState* st;
 };
@@ -303,23 +304,26 @@ __global__ void __launch_bounds__(uf::FT, 4) kb_mg_up(const __grid_constant__ Ar
   });
 }
 
-template <bool CG>
-__global__ void __launch_bounds__(uf::SEP_T, 2) kb_sep_zf(const __grid_constant__ Args<SepP> A,
+template <bool CG, typename T>
+__global__ void __launch_bounds__(uf::SEP_T, 2) kb_sep_zf(const __grid_constant__ Args<SepP<T>> A,
                                                           cudaGraphConditionalHandle cond, int use_cond, int* left) {
   for_items(&A.m, [&](int i, int, const VBlock& vb) {
-    const SepP& P = A.at[i];
+    const SepP<T>& P = A.at[i];
     uf::sep_zf_body<CG>(P.L, P.S, P.x, P.d0, P.d1, P.q, P.partials, P.st, cond, use_cond, CG ? left : nullptr, vb);
   });
 }
-__global__ void __launch_bounds__(uf::SEP_T, 2) kb_sep_y(const __grid_constant__ Args<SepP> A, int inverse) {
+template <typename T>
+__global__ void __launch_bounds__(uf::SEP_T, 2) kb_sep_y(const __grid_constant__ Args<SepP<T>> A, int inverse) {
   for_items(&A.m, [&](int i, int, const VBlock& vb) { uf::sep_y_body(A.at[i].L, A.at[i].S, inverse, A.at[i].st, vb); });
 }
-__global__ void __launch_bounds__(32 * uf::SEP_X_LINES) kb_sep_x(const __grid_constant__ Args<SepP> A) {
+template <typename T>
+__global__ void __launch_bounds__(32 * uf::SEP_X_LINES) kb_sep_x(const __grid_constant__ Args<SepP<T>> A) {
   for_items(&A.m, [&](int i, int, const VBlock& vb) { uf::sep_x_body(A.at[i].L, A.at[i].S, A.at[i].st, vb); });
 }
-__global__ void __launch_bounds__(uf::SEP_T, 2) kb_sep_zi(const __grid_constant__ Args<SepP> A, int mode) {
+template <typename T>
+__global__ void __launch_bounds__(uf::SEP_T, 2) kb_sep_zi(const __grid_constant__ Args<SepP<T>> A, int mode) {
   for_items(&A.m, [&](int i, int, const VBlock& vb) {
-    const SepP& P = A.at[i];
+    const SepP<T>& P = A.at[i];
     uf::sep_zi_body(P.L, P.S, P.z, mode, P.partials, P.st, vb);
   });
 }
@@ -487,12 +491,12 @@ class BatchImpl final : public uf_batch {
                 G.adv_auto ? (d.nz + adv_zc - 1) / adv_zc : G.adv_g[2], G.adv_auto ? adv_zc : G.adv_zc);
       add_entry(maps[MAP_DIR], i, G.march_g[0][0], G.march_g[0][1], G.march_g[0][2], G.march_zc[0]);
       if (G.sep.on) {
-        const int by = 32 * uf::sep_y_wn(d.ny), P = G.lv[0].P;
-        add_entry(maps[MAP_SEPZ], i, (int)uf::sep_z_blocks(P, d.ny, d.nz), 1, 1, 0);
-        add_entry(maps[MAP_SEPY], i, (P + by - 1) / by, uf::sep_y_split(P, d.ny, d.nz), d.nz, 0);
+        const int wn = uf::sep_y_wn<T>(d.ny), by = 32 * wn, P = G.lv[0].P;
+        add_entry(maps[MAP_SEPZ], i, (int)uf::sep_z_blocks<T>(P, d.ny, d.nz), 1, 1, 0);
+        add_entry(maps[MAP_SEPY], i, (P + by - 1) / by, uf::sep_y_split<T>(P, d.ny, d.nz), d.nz, 0);
         add_entry(maps[MAP_SEPX], i, (d.ny * d.nz + uf::SEP_X_LINES - 1) / uf::SEP_X_LINES, 1, 1, 0);
-        sepz_smem = std::max(sepz_smem, uf::sep_smem(uf::SEP_Z_WN, d.nz));
-        sepy_smem = std::max(sepy_smem, uf::sep_smem(uf::sep_y_wn(d.ny), d.ny));
+        sepz_smem = std::max(sepz_smem, uf::sep_smem<T>(uf::SEP_Z_WN<T>, d.nz));
+        sepy_smem = std::max(sepy_smem, uf::sep_smem<T>(wn, d.ny));
         continue;
       }
       add_entry(maps[MAP_TAIL], i, 1, 1, 1, 0);
@@ -675,41 +679,40 @@ class BatchImpl final : public uf_batch {
 
   // The instances with the separable inverse (capi.cu, rec_sep).
   void rec_sep(cudaStream_t s, int mode, cudaGraphConditionalHandle cond, int use_cond) {
-    if constexpr (std::is_same<T, float>::value) {
-      if (items(MAP_SEPZ) == 0) return;
-      auto fill = [](SepP& P, const View<T>& G) {
-        P.L = G.lv[0];
-        P.S = G.sep;
-        P.x = G.p; P.d0 = G.d0; P.d1 = G.d1; P.q = G.q; P.z = G.z;
-        P.partials = G.partials;
-        P.st = G.st;
-      };
-      const int t = uf::SEP_T;
-      const auto& Az = args<SepP>(MAP_SEPZ, fill);
-      if (mode == 1)
-        L(s, "b_sep_zf_cg", plane_bytes(MAP_SEPZ, 7), [&] {
-          kb_sep_zf<true><<<grid_of(kb_sep_zf<true>, t, sepz_smem, items(MAP_SEPZ)), t, sepz_smem, s>>>(Az, cond, use_cond, d_left);
-        });
-      else
-        L(s, "b_sep_zf", plane_bytes(MAP_SEPZ, 2), [&] {
-          kb_sep_zf<false><<<grid_of(kb_sep_zf<false>, t, sepz_smem, items(MAP_SEPZ)), t, sepz_smem, s>>>(Az, cond, 0, nullptr);
-        });
-      for (int inv = 0; inv < 2; ++inv) {
-        const auto& Ay = args<SepP>(MAP_SEPY, fill);
-        L(s, "b_sep_y", plane_bytes(MAP_SEPY, 2), [&] {
-          kb_sep_y<<<grid_of(kb_sep_y, t, sepy_smem, items(MAP_SEPY)), t, sepy_smem, s>>>(Ay, inv);
-        });
-        if (inv) break;
-        const auto& Ax = args<SepP>(MAP_SEPX, fill);
-        L(s, "b_sep_x", plane_bytes(MAP_SEPX, 3), [&] {
-          kb_sep_x<<<grid_of(kb_sep_x, 32 * uf::SEP_X_LINES, 0, items(MAP_SEPX)), 32 * uf::SEP_X_LINES, 0, s>>>(Ax);
-        });
-      }
-      const auto& Ai = args<SepP>(MAP_SEPZ, fill);
-      L(s, "b_sep_zi", plane_bytes(MAP_SEPZ, 3), [&] {
-        kb_sep_zi<<<grid_of(kb_sep_zi, t, sepz_smem, items(MAP_SEPZ)), t, sepz_smem, s>>>(Ai, mode);
+    if (items(MAP_SEPZ) == 0) return;
+    auto fill = [](SepP<T>& P, const View<T>& G) {
+      P.L = G.lv[0];
+      P.S = G.sep;
+      P.x = G.p; P.d0 = G.d0; P.d1 = G.d1; P.q = G.q; P.z = G.z;
+      P.partials = G.partials;
+      P.st = G.st;
+    };
+    const int t = uf::SEP_T;
+    const auto& A = args<SepP<T>>(MAP_SEPZ, fill);
+    auto zf = kb_sep_zf<false, T>;
+    auto zfc = kb_sep_zf<true, T>;
+    if (mode == 1)
+      L(s, "b_sep_zf_cg", plane_bytes(MAP_SEPZ, 7),
+        [&] { zfc<<<grid_of(zfc, t, sepz_smem, items(MAP_SEPZ)), t, sepz_smem, s>>>(A, cond, use_cond, d_left); });
+    else
+      L(s, "b_sep_zf", plane_bytes(MAP_SEPZ, 2),
+        [&] { zf<<<grid_of(zf, t, sepz_smem, items(MAP_SEPZ)), t, sepz_smem, s>>>(A, cond, 0, nullptr); });
+    for (int inv = 0; inv < 2; ++inv) {
+      const auto& Ay = args<SepP<T>>(MAP_SEPY, fill);
+      auto y = kb_sep_y<T>;
+      L(s, "b_sep_y", plane_bytes(MAP_SEPY, 2),
+        [&] { y<<<grid_of(y, t, sepy_smem, items(MAP_SEPY)), t, sepy_smem, s>>>(Ay, inv); });
+      if (inv) break;
+      const auto& Ax = args<SepP<T>>(MAP_SEPX, fill);
+      auto xs = kb_sep_x<T>;
+      L(s, "b_sep_x", plane_bytes(MAP_SEPX, 3), [&] {
+        xs<<<grid_of(xs, 32 * uf::SEP_X_LINES, 0, items(MAP_SEPX)), 32 * uf::SEP_X_LINES, 0, s>>>(Ax);
       });
     }
+    const auto& Ai = args<SepP<T>>(MAP_SEPZ, fill);
+    auto zi = kb_sep_zi<T>;
+    L(s, "b_sep_zi", plane_bytes(MAP_SEPZ, 3),
+      [&] { zi<<<grid_of(zi, t, sepz_smem, items(MAP_SEPZ)), t, sepz_smem, s>>>(Ai, mode); });
   }
 
   void vcycle(cudaStream_t s, int mode, cudaGraphConditionalHandle cond, int use_cond) {
@@ -988,10 +991,12 @@ class BatchImpl final : public uf_batch {
       UFB_CUDA(lim_static((const void*)kb_advect_fused<T, false>));
       UFB_CUDA(lim_static((const void*)kb_advect_fused<T, true>));
       UFB_CUDA(lim_static((const void*)kb_momentum_fused<T>));
-      UFB_CUDA(lim_static((const void*)kb_sep_zf<false>));
-      UFB_CUDA(lim_static((const void*)kb_sep_zf<true>));
-      UFB_CUDA(lim_static((const void*)kb_sep_zi));
-      UFB_CUDA(lim_static((const void*)kb_sep_y));
+      auto zf = kb_sep_zf<false, T>;
+      auto zfc = kb_sep_zf<true, T>;
+      UFB_CUDA(lim_static((const void*)zf));
+      UFB_CUDA(lim_static((const void*)zfc));
+      UFB_CUDA(lim_static((const void*)kb_sep_zi<T>));
+      UFB_CUDA(lim_static((const void*)kb_sep_y<T>));
       UFB_CUDA(cudaStreamSynchronize(stream));
       uf_status s = capture();
       if (s != UF_OK) return s;

@@ -146,17 +146,25 @@ struct Plan {
   size_t total;
 };
 
-// Whether a grid has the separable inverse: FP32 with the default V-cycle
-// settings (a caller who asks for another smoother or transfer gets that
-// V-cycle), sizes whose panels fit one block's shared memory (227 KB: nz x
-// 136 words, ny x 72 or 40 words) and whose x lines fit one warp, and at most
-// kPartials panels per reducing launch.
+// Whether a grid has the separable inverse: the default V-cycle settings (a
+// caller who asks for another smoother or transfer gets that V-cycle), sizes
+// whose panels fit one block's shared memory (227 KB: FP32 nz x 136 words, ny
+// x 72 or 40 words; FP64 32 doubles per cell of either axis) and whose x lines
+// fit one warp, and at most kPartials panels per reducing launch.  FP64:
+// the transforms cost 8 (ny + nz) FP64 operations a cell and application, the
+// V-cycle's fourteen iterations about 4 ns a cell at any size; with two
+// applications that is even near ny + nz = 550 (one step with the V-cycle and
+// with the inverse: 64 x 32 x 16 2.72 and 0.20 ms, 128 x 96 x 40 6.6 and 1.35,
+// 256 x 256 x 64 26.6 and 10.9, 128 x 330 x 64 24.6 and 7.9).
+constexpr int kSep64Sum = 480;
 bool sep_available(const uf_grid_desc* d) {
-  if (d->precision != UF_F32 || d->precond != UF_PRECOND_MG || d->mg_smoother != UF_SMOOTH_CHEBY ||
-      d->mg_transfer != UF_TRANSFER_LINEAR)
+  if (d->precond != UF_PRECOND_MG || d->mg_smoother != UF_SMOOTH_CHEBY || d->mg_transfer != UF_TRANSFER_LINEAR ||
+      d->nx > uf::SEP_MAX_NX)
     return false;
-  return d->nx <= uf::SEP_MAX_NX && d->ny <= 1392 && d->nz <= 400 &&
-         uf::sep_z_blocks(pitch_of(d->nx), d->ny, d->nz) <= (unsigned)kPartials;
+  const int P = pitch_of(d->nx);
+  if (d->precision == UF_F64)
+    return d->ny + d->nz <= kSep64Sum && uf::sep_z_blocks<double>(P, d->ny, d->nz) <= (unsigned)kPartials;
+  return d->ny <= 1392 && d->nz <= 400 && uf::sep_z_blocks<float>(P, d->ny, d->nz) <= (unsigned)kPartials;
 }
 
 Plan make_plan(const uf_grid_desc* d) {
@@ -223,7 +231,9 @@ Plan make_plan(const uf_grid_desc* d) {
   P.grad = L.take(sizeof(double) * 3 * uf::MAX_BOXES);
   P.sep = sep_available(d);
   if (P.sep) {
-    auto packed = [](int n) { return (size_t)((n + 15) / 16) * ((n + 7) / 8) * 32 * sizeof(float4); };
+    auto packed = [&](int n) {
+      return d->precision == UF_F64 ? uf::sep_mat_count<double>(n) * sizeof(double) : uf::sep_mat_count<float>(n) * sizeof(float4);
+    };
     for (size_t& o : P.sep_y) o = L.take(packed(d->ny));
     for (size_t& o : P.sep_z) o = L.take(packed(d->nz));
   }
@@ -355,7 +365,7 @@ class GridImpl final : public uf_grid {
   // pressure store; p holds the solve's correction, then p^{n+1} rounded
   uf::PStore<T> *pd, *gd;
   uf::TailArgs<T> tail;
-  uf::Sep sep{};        // the separable inverse (sep.on = 0: not available)
+  uf::Sep<T> sep{};     // the separable inverse (sep.on = 0: not available)
   T* sol_x = nullptr;   // the solve's unknown (the pressure correction for the step; mu for the adjoint)
   T* sol_b = nullptr;   // its right-hand side
   const uf::PStore<T>* sol_g = nullptr;   // guess of the step's solve (nullptr: warm start in sol_x)
@@ -494,17 +504,17 @@ class GridImpl final : public uf_grid {
       tail.rin = 0;
     }
     UF_CUDA(set_smem_limits());   // every grid: the fused step kernels need more than 48 KB
-    if constexpr (std::is_same<T, float>::value) {
-      if (P.sep) {
-        float4* m[4] = {at<float4>(P.sep_y[0]), at<float4>(P.sep_y[1]), at<float4>(P.sep_z[0]), at<float4>(P.sep_z[1])};
-        for (int q = 0; q < 4; ++q) {
-          const int n = q < 2 ? d.ny : d.nz, bit = q < 2 ? 4 : 16;
-          const int e = (n + 15) / 16 * ((n + 7) / 8) * 32;
-          uf::k_sep_pack<<<(e + 255) / 256, 256, 0, stream>>>(m[q], n, out_mask & bit, out_mask & (2 * bit), q & 1);
-        }
-        sep = uf::Sep{1, m[0], m[1], m[2], m[3], r2, lv[0].x, lv[0].t};
-        UF_CUDA(sep_pivots());
+    if (P.sep) {
+      using Mat = typename uf::Sep<T>::Mat;
+      Mat* m[4] = {at<Mat>(P.sep_y[0]), at<Mat>(P.sep_y[1]), at<Mat>(P.sep_z[0]), at<Mat>(P.sep_z[1])};
+      for (int q = 0; q < 4; ++q) {
+        const int n = q < 2 ? d.ny : d.nz, bit = q < 2 ? 4 : 16;
+        const unsigned nb = (unsigned)((uf::sep_mat_count<T>(n) + 255) / 256);
+        uf::k_sep_pack<T><<<nb, 256, 0, stream>>>(m[q], n, out_mask & bit, out_mask & (2 * bit), q & 1);
       }
+      UF_CUDA(cudaGetLastError());
+      sep = uf::Sep<T>{1, m[0], m[1], m[2], m[3], r2, lv[0].x, lv[0].t};
+      UF_CUDA(sep_pivots());
     }
     if (d.precond == UF_PRECOND_MG) cluster_ctas = probe_cluster();
     if (d.precond == UF_PRECOND_MG) {
@@ -595,10 +605,10 @@ class GridImpl final : public uf_grid {
     lim((const void*)uf::k_mg_coarse<T, uf::SM_JACOBI>);
     lim((const void*)uf::k_mg_coarse<T, uf::SM_RBGS>);
     if (P.sep) {
-      lim((const void*)uf::k_sep_zf<false>);
-      lim((const void*)uf::k_sep_zf<true>);
-      lim((const void*)uf::k_sep_zi<float>);
-      lim((const void*)uf::k_sep_y<float>);
+      lim((const void*)uf::k_sep_zf<false, T>);
+      lim((const void*)uf::k_sep_zf<true, T>);
+      lim((const void*)uf::k_sep_zi<T>);
+      lim((const void*)uf::k_sep_y<T>);
     }
     return e;
   }
@@ -779,35 +789,30 @@ class GridImpl final : public uf_grid {
   // The pivots share r2 with the V-cycle (whose residual alternates between r
   // and r2), so they are formed again whenever the grid leaves the V-cycle.
   cudaError_t sep_pivots() {
-    if constexpr (std::is_same<T, float>::value) {
-      if (use_sep()) uf::k_sep_pivots<<<(d.ny * d.nz + 63) / 64, 64, 0, stream>>>(lv[0], r2);
-      return cudaGetLastError();
-    }
-    return cudaSuccess;
+    if (use_sep()) uf::k_sep_pivots<T><<<(d.ny * d.nz + 63) / 64, 64, 0, stream>>>(lv[0], r2);
+    return cudaGetLastError();
   }
   // The separable inverse takes the V-cycle's place wherever it is available
   // and the V-cycle's launches were not asked for (uf_tuning.coarse_start).
   bool use_sep() const { return sep.on && coarse_start_tuned == 0; }
   void rec_sep(cudaStream_t s, int mode, cudaGraphConditionalHandle cond, int use_cond) {
-    if constexpr (std::is_same<T, float>::value) {
-      const unsigned gz = uf::sep_z_blocks(lv[0].P, d.ny, d.nz);
-      const size_t sz = uf::sep_smem(uf::SEP_Z_WN, d.nz), sy = uf::sep_smem(uf::sep_y_wn(d.ny), d.ny);
-      const int by = 32 * uf::sep_y_wn(d.ny);
-      const dim3 gy((lv[0].P + by - 1) / by, uf::sep_y_split(lv[0].P, d.ny, d.nz), d.nz);
-      const unsigned gx = (unsigned)((d.ny * d.nz + uf::SEP_X_LINES - 1) / uf::SEP_X_LINES);
-      if (mode == 1)
-        L(s, "sep_zf_cg", 7 * N() * tb(), [&] {
-          uf::k_sep_zf<true><<<gz, uf::SEP_T, sz, s>>>(lv[0], sep, sol_x, d0, d1, q, partials, st, cond, use_cond);
-        });
-      else
-        L(s, "sep_zf", 2 * N() * tb(), [&] {
-          uf::k_sep_zf<false><<<gz, uf::SEP_T, sz, s>>>(lv[0], sep, nullptr, nullptr, nullptr, nullptr, partials, st, cond, 0);
-        });
-      L(s, "sep_y", 2 * N() * tb(), [&] { uf::k_sep_y<float><<<gy, uf::SEP_T, sy, s>>>(lv[0], sep, 0, st); });
-      L(s, "sep_x", 3 * N() * tb(), [&] { uf::k_sep_x<float><<<gx, 32 * uf::SEP_X_LINES, 0, s>>>(lv[0], sep, st); });
-      L(s, "sep_y", 2 * N() * tb(), [&] { uf::k_sep_y<float><<<gy, uf::SEP_T, sy, s>>>(lv[0], sep, 1, st); });
-      L(s, "sep_zi", 3 * N() * tb(), [&] { uf::k_sep_zi<float><<<gz, uf::SEP_T, sz, s>>>(lv[0], sep, z, mode, partials, st); });
-    }
+    const int wn = uf::sep_y_wn<T>(d.ny), by = 32 * wn;
+    const unsigned gz = uf::sep_z_blocks<T>(lv[0].P, d.ny, d.nz);
+    const size_t sz = uf::sep_smem<T>(uf::SEP_Z_WN<T>, d.nz), sy = uf::sep_smem<T>(wn, d.ny);
+    const dim3 gy((lv[0].P + by - 1) / by, uf::sep_y_split<T>(lv[0].P, d.ny, d.nz), d.nz);
+    const unsigned gx = (unsigned)((d.ny * d.nz + uf::SEP_X_LINES - 1) / uf::SEP_X_LINES);
+    if (mode == 1)
+      L(s, "sep_zf_cg", 7 * N() * tb(), [&] {
+        uf::k_sep_zf<true, T><<<gz, uf::SEP_T, sz, s>>>(lv[0], sep, sol_x, d0, d1, q, partials, st, cond, use_cond);
+      });
+    else
+      L(s, "sep_zf", 2 * N() * tb(), [&] {
+        uf::k_sep_zf<false, T><<<gz, uf::SEP_T, sz, s>>>(lv[0], sep, nullptr, nullptr, nullptr, nullptr, partials, st, cond, 0);
+      });
+    L(s, "sep_y", 2 * N() * tb(), [&] { uf::k_sep_y<T><<<gy, uf::SEP_T, sy, s>>>(lv[0], sep, 0, st); });
+    L(s, "sep_x", 3 * N() * tb(), [&] { uf::k_sep_x<T><<<gx, 32 * uf::SEP_X_LINES, 0, s>>>(lv[0], sep, st); });
+    L(s, "sep_y", 2 * N() * tb(), [&] { uf::k_sep_y<T><<<gy, uf::SEP_T, sy, s>>>(lv[0], sep, 1, st); });
+    L(s, "sep_zi", 3 * N() * tb(), [&] { uf::k_sep_zi<T><<<gz, uf::SEP_T, sz, s>>>(lv[0], sep, z, mode, partials, st); });
   }
   void rec_vcycle(cudaStream_t s, int mode, cudaGraphConditionalHandle cond, int use_cond) {
     if (use_sep()) return rec_sep(s, mode, cond, use_cond);

@@ -43,7 +43,7 @@ struct GridView {
   double* dt;
   T* dtT;
   uf::SmoothW<T> sw;               // smoother weights
-  uf::Sep sep;                     // separable inverse (sep.on: in use instead of the V-cycle)
+  uf::Sep<T> sep;                  // separable inverse (sep.on: in use instead of the V-cycle)
 };
 
 // An NVTX range (host side) for the lifetime of a scope.

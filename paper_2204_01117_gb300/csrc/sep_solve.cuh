@@ -1,5 +1,6 @@
 // Exact inverse of the finest-level pressure operator by separation of
-// variables, the default preconditioner of FP32 grids (capi.cu, use_sep()).
+// variables, the default preconditioner where its sizes allow (capi.cu,
+// sep_available, use_sep).
 //
 // The operator of Sec. 3 has constant coefficients (buildings act through
 // drag), so A = Tx + Ty + Tz with one tridiagonal matrix per axis: -1, 2, -1
@@ -39,48 +40,73 @@ constexpr int SEP_T = 256;        // threads of the transform kernels (8 warps)
 constexpr int SEP_X_LINES = 8;    // lines (warps) per block of the x solve
 constexpr int SEP_MAX_NX = 1024;  // 32 lanes x 32 values per line
 
-// Separable solver of one grid.  Matrices are packed in the order in which
-// the lanes of a warp read the A operand of mma.m16n8k8: one float4 per lane
-// and 16 x 8 tile, tiles row by row, zero beyond the matrix.
+// FP64 grids do the same on the FP64 pipe, 1/64 of the FP32 rate on this
+// chip: the products are then what a pass costs, and a rule on the sizes
+// keeps the V-cycle where they would outweigh the iterations saved
+// (sep_available in capi.cu, with both sides measured).
+template <typename T>
+struct SepMat { using type = float4; };   // FP32: see below
+template <>
+struct SepMat<double> { using type = double; };
+
+// Separable solver of one grid.  FP32 matrices are packed in the order in
+// which the lanes of a warp read the A operand of mma.m16n8k8: one float4 per
+// lane and 16 x 8 tile, tiles row by row, zero beyond the matrix.  FP64
+// matrices are stored column by column, each padded with zeros to an even
+// number of rows.
+template <typename T>
 struct Sep {
+  using Mat = typename SepMat<T>::type;
   long long on;        // 0: this grid uses the V-cycle (8 bytes: no padding, the struct is compared bytewise)
-  const float4* yf;    // forward: row m = mode, column j = cell
-  const float4* yi;    // inverse (transpose)
-  const float4* zf;
-  const float4* zi;
-  const float* piv;    // 1 / pivot of the x systems, one row of P per (y mode, z mode)
-  float* t;            // scratch (padded cell arrays): z transforms and the y transform back write t,
-  float* u;            // the y transform writes u, the x solve works on it in place
+  const Mat* yf;    // forward: row m = mode, column j = cell
+  const Mat* yi;    // inverse (transpose)
+  const Mat* zf;
+  const Mat* zi;
+  const T* piv;    // 1 / pivot of the x systems, one row of P per (y mode, z mode)
+  T* t;                // scratch (padded cell arrays): z transforms and the y transform back write t,
+  T* u;                // the y transform writes u, the x solve works on it in place
 };
 
-// Panel geometry: a warp owns 32 rows x 32 columns of the result, a block
-// WM x WN warps; the panel of the field ([K][32 WN], the whole contracted
-// axis) stays in shared memory with a row pitch of 8 mod 32 words, which
-// gives the 32 lanes of a B fragment (4 rows x 8 columns) 32 banks.
-template <int WN>
-constexpr int SEP_PITCH = 32 * WN + 8;
-inline size_t sep_smem(int wn, int n) { return sizeof(float) * (size_t)((n + 7) / 8 * 8) * (32 * wn + 8); }
-// Columns of a y panel: 64 while it fits (n <= 768), else 32.
+// Panel geometry.  The whole contracted axis of a set of columns of the field
+// stays in shared memory.  FP32: a warp owns 32 rows x 32 columns of the
+// result, a block (8 / WN) x WN warps; the row pitch of 8 mod 32 words gives
+// the 32 lanes of a B fragment (4 rows x 8 columns) 32 banks.  FP64: panels of
+// 32 columns (WN = 1); a warp owns 4 rows.
+template <typename T, int WN>
+constexpr int SEP_PITCH = sizeof(T) == 4 ? 32 * WN + 8 : 32;
+// Columns of a y panel in units of 32: two while it fits (n <= 768), else one.
 constexpr int SEP_Y_WIDE = 768;
-#ifndef UF_SEP_Y_BLOCKS
-#define UF_SEP_Y_BLOCKS 304   // two resident blocks on each of 152 SMs
-#endif
-constexpr int SEP_Y_BLOCKS = UF_SEP_Y_BLOCKS;
-inline int sep_y_wn(int ny) { return ny <= SEP_Y_WIDE ? 2 : 1; }
-constexpr int SEP_Z_WN = 4;
+template <typename T>
+__host__ __device__ inline int sep_y_wn(int ny) { return sizeof(T) == 4 && ny <= SEP_Y_WIDE ? 2 : 1; }
+template <typename T>
+constexpr int SEP_Z_WN = sizeof(T) == 4 ? 4 : 1;
+template <typename T>
+inline size_t sep_smem(int wn, int n) { return sizeof(T) * (size_t)((n + 7) / 8 * 8) * (sizeof(T) == 4 ? 32 * wn + 8 : 32); }
 // Columns (x, y) of a z panel, and the blocks that cover the plane.  One cell
 // in z has nothing to transform: the threads just share the columns out.
-__host__ __device__ inline int sep_z_cols(int nz) { return nz > 1 ? 32 * SEP_Z_WN : 4 * SEP_T; }
-inline unsigned sep_z_blocks(int P, int ny, int nz) { return (unsigned)(((size_t)P * ny + sep_z_cols(nz) - 1) / sep_z_cols(nz)); }
+template <typename T>
+__host__ __device__ inline int sep_z_cols(int nz) { return nz > 1 ? 32 * SEP_Z_WN<T> : (int)(16 / sizeof(T)) * SEP_T; }
+template <typename T>
+inline unsigned sep_z_blocks(int P, int ny, int nz) {
+  return (unsigned)(((size_t)P * ny + sep_z_cols<T>(nz) - 1) / sep_z_cols<T>(nz));
+}
 // Blocks that share a y panel, each taking every split-th round of result
 // rows: a quasi-2D grid has fewer panels than SMs (512 x 768 x 1: 8, one pass
-// 97 us unsplit).
+// 97 us unsplit, 27 us split).
+constexpr int SEP_Y_BLOCKS = 304;   // two resident blocks on each of 152 SMs
+template <typename T>
 __host__ __device__ inline int sep_y_split(int P, int ny, int nz) {
-  const int wn = ny <= SEP_Y_WIDE ? 2 : 1;
-  const int panels = (P + 32 * wn - 1) / (32 * wn) * nz, rounds = (ny + 32 * (8 / wn) - 1) / (32 * (8 / wn));
+  const int wn = sep_y_wn<T>(ny), rows = sizeof(T) == 4 ? 32 * (8 / wn) : 32;   // of a round
+  const int panels = (P + 32 * wn - 1) / (32 * wn) * nz, rounds = (ny + rows - 1) / rows;
   const int want = (SEP_Y_BLOCKS + panels - 1) / panels;
   return want < rounds ? want : rounds;
 }
+// 16 bytes of a field.
+template <typename T>
+struct alignas(16) SepVec {
+  static constexpr int N = 16 / sizeof(T);
+  T e[N];
+};
 
 // x = hi + lo (+ below 2^-22 |x|): hi rounded to TF32's 11 bits, lo cut to them.
 __device__ __forceinline__ void tf32_split(float x, uint32_t& hi, uint32_t& lo) {
@@ -97,10 +123,10 @@ __device__ __forceinline__ void mma_tf32(float (&c)[4], const uint32_t (&a)[4], 
 // Result rows of the block's panel: A (M x K packed) times sB ([K][pitch]),
 // rounds part, part + parts, ... of 32 WM rows.
 // put(row, column of the panel (even), value, next value).
-template <int WM, int WN, typename Put>
+template <int WN, typename Put>
 __device__ __forceinline__ void sep_gemm(const float4* __restrict__ A, int M, int K, const float* sB, int part, int parts,
                                          Put put) {
-  constexpr int PB = SEP_PITCH<WN>;
+  constexpr int PB = SEP_PITCH<float, WN>, WM = 8 / WN;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3, wm = warp / WN, wn = warp % WN;
   const int KT = (K + 7) / 8, MT16 = (M + 15) / 16;
@@ -157,62 +183,92 @@ __device__ __forceinline__ void sep_gemm(const float4* __restrict__ A, int M, in
   }
 }
 
+// FP64: lane l owns columns 2 (l % 16), + 1 and rows 2 (l / 16), + 1 of its
+// warp's four (A: column by column, MP rows each).
+template <int WN, typename Put>
+__device__ __forceinline__ void sep_gemm(const double* __restrict__ A, int M, int K, const double* sB, int part, int parts,
+                                         Put put) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, col = 2 * (lane & 15), MP = (M + 1) & ~1;
+  for (int r0 = 4 * warp + 32 * part; r0 < M; r0 += 32 * parts) {
+    const int row = r0 + 2 * (lane >> 4);
+    const double* a = A + (row < M ? row : 0);
+    double c00 = 0, c01 = 0, c10 = 0, c11 = 0;
+#pragma unroll 4
+    for (int k = 0; k < K; ++k) {
+      const double2 av = __ldg(reinterpret_cast<const double2*>(a + (size_t)k * MP));
+      const double2 bv = *reinterpret_cast<const double2*>(sB + k * 32 + col);
+      c00 = fma(av.x, bv.x, c00);
+      c01 = fma(av.x, bv.y, c01);
+      c10 = fma(av.y, bv.x, c10);
+      c11 = fma(av.y, bv.y, c11);
+    }
+    if (row < M) put(row, col, c00, c01);
+    if (row + 1 < M) put(row + 1, col, c10, c11);
+  }
+}
+
+__device__ __forceinline__ void sep_put2(float* o, float a, float b) { *reinterpret_cast<float2*>(o) = make_float2(a, b); }
+__device__ __forceinline__ void sep_put2(double* o, double a, double b) { *reinterpret_cast<double2*>(o) = make_double2(a, b); }
+__device__ __forceinline__ float2 sep_get2(const float* o) { return *reinterpret_cast<const float2*>(o); }
+__device__ __forceinline__ double2 sep_get2(const double* o) { return *reinterpret_cast<const double2*>(o); }
+
 // ------------------------------------------------------- z transforms ----
 // A panel is 128 consecutive columns (x, y) of the P x ny plane with every z
 // in shared memory, so each cell is read once.  CG = true (inside the CG
 // loop): the panel's load is also the CG update x += alpha d, r -= alpha q
 // with ||r||^2 and the convergence test.  Columns in the row padding
 // (x >= nx) are forced to zero.
-template <bool CG>
-__device__ __forceinline__ void sep_zf_body(const Level<float>& L, const Sep& S, float* __restrict__ x, const float* d0,
-                                            const float* d1, const float* __restrict__ q, double* partials,
-                                            SolveState* st, cudaGraphConditionalHandle cond, int use_cond, int* left,
-                                            const VBlock& vb) {
-  extern __shared__ __align__(16) float sep_sm[];
+template <bool CG, typename T>
+__device__ __forceinline__ void sep_zf_body(const Level<T>& L, const Sep<T>& S, T* __restrict__ x, const T* d0, const T* d1,
+                                            const T* __restrict__ q, double* partials, SolveState* st,
+                                            cudaGraphConditionalHandle cond, int use_cond, int* left, const VBlock& vb) {
+  extern __shared__ __align__(16) unsigned char sep_raw[];
+  T* sep_sm = reinterpret_cast<T*>(sep_raw);
   __shared__ double sh[32];
   __shared__ bool last;
   if (st->converged) return;
-  constexpr int BN = 32 * SEP_Z_WN, PB = SEP_PITCH<SEP_Z_WN>, VR = BN / 4;
+  using V = SepVec<T>;
+  constexpr int WN = SEP_Z_WN<T>, BN = 32 * WN, PB = SEP_PITCH<T, WN>, VR = BN / V::N;
   static_assert(SEP_T % VR == 0, "a thread keeps its columns");
   const size_t PS = (size_t)L.P * L.ny;
-  const bool flat = L.nz == 1;   // one cell in z: the identity, a thread per 4 columns
-  const int row0 = flat ? 0 : threadIdx.x / VR, col0 = 4 * (flat ? threadIdx.x : threadIdx.x % VR);
-  const size_t c = (size_t)vb.x * sep_z_cols(L.nz) + col0;
+  const bool flat = L.nz == 1;   // one cell in z: the identity, a thread per 16 bytes
+  const int row0 = flat ? 0 : threadIdx.x / VR, col0 = V::N * (flat ? threadIdx.x : threadIdx.x % VR);
+  const size_t c = (size_t)vb.x * sep_z_cols<T>(L.nz) + col0;
   const bool in = c < PS;
-  const int i = (int)(c % L.P);
-  const bool k0 = i < L.nx, k1 = i + 1 < L.nx, k2 = i + 2 < L.nx, k3 = i + 3 < L.nx;
+  const int left_x = L.nx - (int)(c % L.P);   // how many of the values lie inside the domain
   const int it0 = st->iter;
-  const float alpha = CG ? (float)st->alpha : 0.f;
-  const float* dn = (it0 & 1) ? d0 : d1;
-  DotAcc<float> dacc;
+  const T alpha = CG ? (T)st->alpha : T(0);
+  const T* dn = (it0 & 1) ? d0 : d1;
+  DotAcc<T> dacc;
   const int KP = flat ? 1 : (L.nz + 7) / 8 * 8;
 #pragma unroll 2
   for (int k = row0; k < KP; k += SEP_T / VR) {
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    V v = {};
     if (in && k < L.nz) {
       const size_t o = (size_t)k * PS + c;
-      v = *reinterpret_cast<const float4*>(L.r + o);
+      v = *reinterpret_cast<const V*>(L.r + o);
       if (CG) {
-        const float4 qv = *reinterpret_cast<const float4*>(q + o);
-        const float4 dv = *reinterpret_cast<const float4*>(dn + o);
-        float4 xv = *reinterpret_cast<const float4*>(x + o);
-        v.x = k0 ? v.x - alpha * qv.x : 0.f; v.y = k1 ? v.y - alpha * qv.y : 0.f;
-        v.z = k2 ? v.z - alpha * qv.z : 0.f; v.w = k3 ? v.w - alpha * qv.w : 0.f;
-        xv.x = k0 ? xv.x + alpha * dv.x : 0.f; xv.y = k1 ? xv.y + alpha * dv.y : 0.f;
-        xv.z = k2 ? xv.z + alpha * dv.z : 0.f; xv.w = k3 ? xv.w + alpha * dv.w : 0.f;
-        *reinterpret_cast<float4*>(L.r + o) = v;
-        *reinterpret_cast<float4*>(x + o) = xv;
-        dacc.add(v.x, v.x); dacc.add(v.y, v.y); dacc.add(v.z, v.z); dacc.add(v.w, v.w);
+        const V qv = *reinterpret_cast<const V*>(q + o);
+        const V dv = *reinterpret_cast<const V*>(dn + o);
+        V xv = *reinterpret_cast<const V*>(x + o);
+#pragma unroll
+        for (int e = 0; e < V::N; ++e) {
+          v.e[e] = e < left_x ? v.e[e] - alpha * qv.e[e] : T(0);
+          xv.e[e] = e < left_x ? xv.e[e] + alpha * dv.e[e] : T(0);
+          dacc.add(v.e[e], v.e[e]);
+        }
+        *reinterpret_cast<V*>(L.r + o) = v;
+        *reinterpret_cast<V*>(x + o) = xv;
       }
     }
-    if (!flat) *reinterpret_cast<float4*>(sep_sm + k * PB + col0) = v;
-    else if (in) *reinterpret_cast<float4*>(S.t + c) = v;
+    if (!flat) *reinterpret_cast<V*>(sep_sm + k * PB + col0) = v;
+    else if (in) *reinterpret_cast<V*>(S.t + c) = v;
   }
   if (!flat) {
     __syncthreads();
     const size_t cb = (size_t)vb.x * BN;
-    sep_gemm<8 / SEP_Z_WN, SEP_Z_WN>(S.zf, L.nz, L.nz, sep_sm, 0, 1, [&](int row, int col, float a, float b) {
-      if (cb + col < PS) *reinterpret_cast<float2*>(S.t + (size_t)row * PS + cb + col) = make_float2(a, b);
+    sep_gemm<WN>(S.zf, L.nz, L.nz, sep_sm, 0, 1, [&](int row, int col, T a, T b) {
+      if (cb + col < PS) sep_put2(S.t + (size_t)row * PS + cb + col, a, b);
     });
   }
   if (CG) {
@@ -229,41 +285,44 @@ __device__ __forceinline__ void sep_zf_body(const Level<float>& L, const Sep& S,
 }
 
 // Back along z: z = Qz^T t, and r.z (CG beta in mode 1).
-__device__ __forceinline__ void sep_zi_body(const Level<float>& L, const Sep& S, float* __restrict__ z, int mode,
-                                            double* partials, SolveState* st, const VBlock& vb) {
-  extern __shared__ __align__(16) float sep_sm[];
+template <typename T>
+__device__ __forceinline__ void sep_zi_body(const Level<T>& L, const Sep<T>& S, T* __restrict__ z, int mode, double* partials,
+                                            SolveState* st, const VBlock& vb) {
+  extern __shared__ __align__(16) unsigned char sep_raw[];
+  T* sep_sm = reinterpret_cast<T*>(sep_raw);
   __shared__ double sh[32];
   __shared__ bool last;
   if (st->converged) return;
-  constexpr int BN = 32 * SEP_Z_WN, PB = SEP_PITCH<SEP_Z_WN>, VR = BN / 4;
+  using V = SepVec<T>;
+  constexpr int WN = SEP_Z_WN<T>, BN = 32 * WN, PB = SEP_PITCH<T, WN>, VR = BN / V::N;
   const size_t PS = (size_t)L.P * L.ny;
   const bool flat = L.nz == 1;
-  const int col0 = 4 * (flat ? threadIdx.x : threadIdx.x % VR);
-  const size_t c = (size_t)vb.x * sep_z_cols(L.nz) + col0;
-  DotAcc<float> dacc;
-  auto put = [&](size_t o, float a, float b) {
-    const float2 rv = *reinterpret_cast<const float2*>(L.r + o);
-    *reinterpret_cast<float2*>(z + o) = make_float2(a, b);
+  const int col0 = V::N * (flat ? threadIdx.x : threadIdx.x % VR);
+  const size_t c = (size_t)vb.x * sep_z_cols<T>(L.nz) + col0;
+  DotAcc<T> dacc;
+  auto put = [&](size_t o, T a, T b) {
+    const auto rv = sep_get2(L.r + o);
+    sep_put2(z + o, a, b);
     dacc.add(rv.x, a);
     dacc.add(rv.y, b);
   };
   if (flat) {
     if (c < PS) {
-      const float4 v = *reinterpret_cast<const float4*>(S.t + c);
-      put(c, v.x, v.y);
-      put(c + 2, v.z, v.w);
+      const V v = *reinterpret_cast<const V*>(S.t + c);
+#pragma unroll
+      for (int e = 0; e < V::N; e += 2) put(c + e, v.e[e], v.e[e + 1]);
     }
   } else {
     const int KP = (L.nz + 7) / 8 * 8;
 #pragma unroll 4
     for (int k = threadIdx.x / VR; k < KP; k += SEP_T / VR) {
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (c < PS && k < L.nz) v = *reinterpret_cast<const float4*>(S.t + (size_t)k * PS + c);
-      *reinterpret_cast<float4*>(sep_sm + k * PB + col0) = v;
+      V v = {};
+      if (c < PS && k < L.nz) v = *reinterpret_cast<const V*>(S.t + (size_t)k * PS + c);
+      *reinterpret_cast<V*>(sep_sm + k * PB + col0) = v;
     }
     __syncthreads();
     const size_t cb = (size_t)vb.x * BN;
-    sep_gemm<8 / SEP_Z_WN, SEP_Z_WN>(S.zi, L.nz, L.nz, sep_sm, 0, 1, [&](int row, int col, float a, float b) {
+    sep_gemm<WN>(S.zi, L.nz, L.nz, sep_sm, 0, 1, [&](int row, int col, T a, T b) {
       if (cb + col < PS) put((size_t)row * PS + cb + col, a, b);
     });
   }
@@ -281,34 +340,37 @@ __device__ __forceinline__ void sep_zi_body(const Level<float>& L, const Sep& S,
 // --------------------------------------------------------- y transforms --
 // One panel of 32 WN columns of a z plane, every y; blocks vb.y of `split`
 // share the panel's result rows.
-template <int WN>
-__device__ __forceinline__ void sep_y_panel(const Level<float>& L, const float4* A, const float* __restrict__ src,
-                                            float* __restrict__ dst, int split, const VBlock& vb) {
-  extern __shared__ __align__(16) float sep_sm[];
-  constexpr int BN = 32 * WN, PB = SEP_PITCH<WN>, VR = BN / 4;
-  const int x0 = vb.x * BN, xv = 4 * (threadIdx.x % VR);
+template <int WN, typename T>
+__device__ __forceinline__ void sep_y_panel(const Level<T>& L, const typename Sep<T>::Mat* A, const T* __restrict__ src,
+                                            T* __restrict__ dst, int split, const VBlock& vb) {
+  extern __shared__ __align__(16) unsigned char sep_raw[];
+  T* sep_sm = reinterpret_cast<T*>(sep_raw);
+  using V = SepVec<T>;
+  constexpr int BN = 32 * WN, PB = SEP_PITCH<T, WN>, VR = BN / V::N;
+  const int x0 = vb.x * BN, xv = V::N * (threadIdx.x % VR);
   const size_t base = (size_t)vb.z * L.P * L.ny + x0;
   const bool in = x0 + xv < L.P;
   const int KP = (L.ny + 7) / 8 * 8;
 #pragma unroll 4
   for (int j = threadIdx.x / VR; j < KP; j += SEP_T / VR) {
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (in && j < L.ny) v = *reinterpret_cast<const float4*>(src + base + (size_t)j * L.P + xv);
-    *reinterpret_cast<float4*>(sep_sm + j * PB + xv) = v;
+    V v = {};
+    if (in && j < L.ny) v = *reinterpret_cast<const V*>(src + base + (size_t)j * L.P + xv);
+    *reinterpret_cast<V*>(sep_sm + j * PB + xv) = v;
   }
   __syncthreads();
-  sep_gemm<8 / WN, WN>(A, L.ny, L.ny, sep_sm, vb.y, split, [&](int row, int col, float a, float b) {
-    if (x0 + col < L.P) *reinterpret_cast<float2*>(dst + base + (size_t)row * L.P + col) = make_float2(a, b);
+  sep_gemm<WN>(A, L.ny, L.ny, sep_sm, vb.y, split, [&](int row, int col, T a, T b) {
+    if (x0 + col < L.P) sep_put2(dst + base + (size_t)row * L.P + col, a, b);
   });
 }
-__device__ __forceinline__ void sep_y_body(const Level<float>& L, const Sep& S, int inverse, const SolveState* st,
+template <typename T>
+__device__ __forceinline__ void sep_y_body(const Level<T>& L, const Sep<T>& S, int inverse, const SolveState* st,
                                            const VBlock& vb) {
   if (st->converged) return;
-  const float4* A = inverse ? S.yi : S.yf;
-  const float* src = inverse ? S.u : S.t;
-  float* dst = inverse ? S.t : S.u;
-  const int split = sep_y_split(L.P, L.ny, L.nz);
-  if (L.ny <= SEP_Y_WIDE) sep_y_panel<2>(L, A, src, dst, split, vb);
+  const auto* A = inverse ? S.yi : S.yf;
+  const T* src = inverse ? S.u : S.t;
+  T* dst = inverse ? S.t : S.u;
+  const int split = sep_y_split<T>(L.P, L.ny, L.nz);
+  if (sizeof(T) == 4 && L.ny <= SEP_Y_WIDE) sep_y_panel<sizeof(T) == 4 ? 2 : 1>(L, A, src, dst, split, vb);
   else sep_y_panel<1>(L, A, src, dst, split, vb);
 }
 
@@ -319,55 +381,59 @@ __device__ __forceinline__ void sep_y_body(const Level<float>& L, const Sep& S, 
 // recurrence is a scan of the affine maps of the lanes (Blelloch 1990), so a
 // line takes 10 shuffle steps instead of 2 nx dependent ones.  In the row
 // padding e = 0, which makes the solution 0 there.
-template <int E>
-__device__ __forceinline__ void sep_x_line(float* __restrict__ row, const float* __restrict__ piv, int P) {
+template <int E, typename T>
+__device__ __forceinline__ void sep_x_line(T* __restrict__ row, const T* __restrict__ piv, int P) {
+  using V = SepVec<T>;
   const int lane = threadIdx.x & 31;
-  float f[E], e[E];
-  if (E >= 4) {
+  T f[E], e[E];
+  if (E >= V::N) {
 #pragma unroll
-    for (int m = 0; m < E; m += 4) {
+    for (int m = 0; m < E; m += V::N) {
       const int i = lane * E + m;
-      float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+      V a = {}, b = {};
       if (i < P) {
-        a = *reinterpret_cast<const float4*>(row + i);
-        b = *reinterpret_cast<const float4*>(piv + i);
+        a = *reinterpret_cast<const V*>(row + i);
+        b = *reinterpret_cast<const V*>(piv + i);
       }
-      f[m] = a.x; f[m + 1] = a.y; f[m + 2] = a.z; f[m + 3] = a.w;
-      e[m] = b.x; e[m + 1] = b.y; e[m + 2] = b.z; e[m + 3] = b.w;
+#pragma unroll
+      for (int q = 0; q < V::N && m + q < E; ++q) {
+        f[m + q] = a.e[q];
+        e[m + q] = b.e[q];
+      }
     }
   } else {
 #pragma unroll
     for (int m = 0; m < E; ++m) {
       const int i = lane * E + m;
-      f[m] = i < P ? row[i] : 0.f;
-      e[m] = i < P ? piv[i] : 0.f;
+      f[m] = i < P ? row[i] : T(0);
+      e[m] = i < P ? piv[i] : T(0);
     }
   }
   // forward
-  float ep = __shfl_up_sync(0xffffffffu, e[E - 1], 1);
-  if (lane == 0) ep = 0.f;
-  float a = ep, b = f[0];   // the lane's map: last y = a * (y of the lane before) + b
+  T ep = __shfl_up_sync(0xffffffffu, e[E - 1], 1);
+  if (lane == 0) ep = T(0);
+  T a = ep, b = f[0];   // the lane's map: last y = a * (y of the lane before) + b
 #pragma unroll
   for (int m = 1; m < E; ++m) {
-    b = fmaf(e[m - 1], b, f[m]);
+    b = fma(e[m - 1], b, f[m]);
     a *= e[m - 1];
   }
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const float a2 = __shfl_up_sync(0xffffffffu, a, o), b2 = __shfl_up_sync(0xffffffffu, b, o);
+    const T a2 = __shfl_up_sync(0xffffffffu, a, o), b2 = __shfl_up_sync(0xffffffffu, b, o);
     if (lane >= o) {
-      b = fmaf(a, b2, b);
+      b = fma(a, b2, b);
       a *= a2;
     }
   }
-  float cin = __shfl_up_sync(0xffffffffu, b, 1);
-  if (lane == 0) cin = 0.f;
-  f[0] = fmaf(ep, cin, f[0]);
+  T cin = __shfl_up_sync(0xffffffffu, b, 1);
+  if (lane == 0) cin = T(0);
+  f[0] = fma(ep, cin, f[0]);
 #pragma unroll
-  for (int m = 1; m < E; ++m) f[m] = fmaf(e[m - 1], f[m - 1], f[m]);
+  for (int m = 1; m < E; ++m) f[m] = fma(e[m - 1], f[m - 1], f[m]);
   // backward
-  a = 1.f;
-  b = 0.f;
+  a = T(1);
+  b = T(0);
 #pragma unroll
   for (int m = E - 1; m >= 0; --m) {
     b = e[m] * (f[m] + b);
@@ -375,21 +441,24 @@ __device__ __forceinline__ void sep_x_line(float* __restrict__ row, const float*
   }
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const float a2 = __shfl_down_sync(0xffffffffu, a, o), b2 = __shfl_down_sync(0xffffffffu, b, o);
+    const T a2 = __shfl_down_sync(0xffffffffu, a, o), b2 = __shfl_down_sync(0xffffffffu, b, o);
     if (lane + o < 32) {
-      b = fmaf(a, b2, b);
+      b = fma(a, b2, b);
       a *= a2;
     }
   }
   cin = __shfl_down_sync(0xffffffffu, b, 1);
-  if (lane == 31) cin = 0.f;
+  if (lane == 31) cin = T(0);
 #pragma unroll
   for (int m = E - 1; m >= 0; --m) cin = f[m] = e[m] * (f[m] + cin);
-  if (E >= 4) {
+  if (E >= V::N) {
 #pragma unroll
-    for (int m = 0; m < E; m += 4) {
+    for (int m = 0; m < E; m += V::N) {
       const int i = lane * E + m;
-      if (i < P) *reinterpret_cast<float4*>(row + i) = make_float4(f[m], f[m + 1], f[m + 2], f[m + 3]);
+      V a;
+#pragma unroll
+      for (int q = 0; q < V::N && m + q < E; ++q) a.e[q] = f[m + q];
+      if (i < P) *reinterpret_cast<V*>(row + i) = a;
     }
   } else {
 #pragma unroll
@@ -397,12 +466,13 @@ __device__ __forceinline__ void sep_x_line(float* __restrict__ row, const float*
       if (lane * E + m < P) row[lane * E + m] = f[m];
   }
 }
-__device__ __forceinline__ void sep_x_body(const Level<float>& L, const Sep& S, const SolveState* st, const VBlock& vb) {
+template <typename T>
+__device__ __forceinline__ void sep_x_body(const Level<T>& L, const Sep<T>& S, const SolveState* st, const VBlock& vb) {
   if (st->converged) return;
   const int line = vb.x * SEP_X_LINES + (threadIdx.x >> 5);
   if (line >= L.ny * L.nz) return;
-  float* row = S.u + (size_t)line * L.P;
-  const float* piv = S.piv + (size_t)line * L.P;
+  T* row = S.u + (size_t)line * L.P;
+  const T* piv = S.piv + (size_t)line * L.P;
   if (L.P <= 64) sep_x_line<2>(row, piv, L.P);
   else if (L.P <= 128) sep_x_line<4>(row, piv, L.P);
   else if (L.P <= 256) sep_x_line<8>(row, piv, L.P);
@@ -411,23 +481,23 @@ __device__ __forceinline__ void sep_x_body(const Level<float>& L, const Sep& S, 
 }
 
 // -------------------------------------------------------------- kernels --
-template <bool CG>
-__global__ void __launch_bounds__(SEP_T, 2) k_sep_zf(Level<float> L, Sep S, float* __restrict__ x, const float* d0,
-                                                     const float* d1, const float* __restrict__ q, double* partials,
-                                                     SolveState* st, cudaGraphConditionalHandle cond, int use_cond) {
+template <bool CG, typename T>
+__global__ void __launch_bounds__(SEP_T, 2) k_sep_zf(Level<T> L, Sep<T> S, T* __restrict__ x, const T* d0, const T* d1,
+                                                     const T* __restrict__ q, double* partials, SolveState* st,
+                                                     cudaGraphConditionalHandle cond, int use_cond) {
   sep_zf_body<CG>(L, S, x, d0, d1, q, partials, st, cond, use_cond, nullptr, vblock());
 }
 template <typename T>
-__global__ void __launch_bounds__(SEP_T, 2) k_sep_zi(Level<T> L, Sep S, float* __restrict__ z, int mode,
-                                                            double* partials, SolveState* st) {
+__global__ void __launch_bounds__(SEP_T, 2) k_sep_zi(Level<T> L, Sep<T> S, T* __restrict__ z, int mode, double* partials,
+                                                     SolveState* st) {
   sep_zi_body(L, S, z, mode, partials, st, vblock());
 }
 template <typename T>
-__global__ void __launch_bounds__(SEP_T, 2) k_sep_y(Level<T> L, Sep S, int inverse, const SolveState* st) {
+__global__ void __launch_bounds__(SEP_T, 2) k_sep_y(Level<T> L, Sep<T> S, int inverse, const SolveState* st) {
   sep_y_body(L, S, inverse, st, vblock());
 }
 template <typename T>
-__global__ void __launch_bounds__(32 * SEP_X_LINES) k_sep_x(Level<T> L, Sep S, const SolveState* st) {
+__global__ void __launch_bounds__(32 * SEP_X_LINES) k_sep_x(Level<T> L, Sep<T> S, const SolveState* st) {
   sep_x_body(L, S, st, vblock());
 }
 
@@ -446,19 +516,28 @@ __device__ __forceinline__ double sep_eig(int m, int n, bool out_lo, bool out_hi
   const double s = (!out_lo && !out_hi) ? sinpi(m / (2.0 * n)) : sinpi((2 * m + 1) / (2.0 * (2 * n + 1)));
   return 4.0 * s * s;
 }
-// Packed matrix of an axis: forward (row mode, column cell) or its transpose.
-template <typename V>
-__global__ void k_sep_pack(V* A, int n, int out_lo, int out_hi, int transpose) {
-  const int KT = (n + 7) / 8, MT16 = (n + 15) / 16;
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= MT16 * KT * 32) return;
-  const int lane = e & 31, tile = e >> 5, g = lane >> 2, t = lane & 3;
-  const int r0 = (tile / KT) * 16 + g, c0 = (tile % KT) * 8 + t;
-  auto val = [&](int r, int c) {
-    if (r >= n || c >= n) return 0.f;
-    return (float)(transpose ? sep_mode(c, r, n, out_lo, out_hi) : sep_mode(r, c, n, out_lo, out_hi));
-  };
-  A[e] = make_float4(val(r0, c0), val(r0 + 8, c0), val(r0, c0 + 4), val(r0 + 8, c0 + 4));
+// Matrix of an axis: forward (row mode, column cell) or its transpose.
+__device__ __forceinline__ double sep_entry(int r, int c, int n, int out_lo, int out_hi, int transpose) {
+  if (r >= n || c >= n) return 0.0;
+  return transpose ? sep_mode(c, r, n, out_lo, out_hi) : sep_mode(r, c, n, out_lo, out_hi);
+}
+template <typename T>
+__host__ __device__ inline size_t sep_mat_count(int n) {   // elements of Sep<T>::Mat
+  return sizeof(T) == 4 ? (size_t)((n + 15) / 16) * ((n + 7) / 8) * 32 : (size_t)n * ((n + 1) & ~1);
+}
+template <typename T>
+__global__ void k_sep_pack(typename Sep<T>::Mat* A, int n, int out_lo, int out_hi, int transpose) {
+  const size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (e >= sep_mat_count<T>(n)) return;
+  if constexpr (sizeof(T) == 4) {
+    const int KT = (n + 7) / 8, lane = (int)(e & 31), tile = (int)(e >> 5), g = lane >> 2, t = lane & 3;
+    const int r0 = (tile / KT) * 16 + g, c0 = (tile % KT) * 8 + t;
+    auto val = [&](int r, int c) { return (float)sep_entry(r, c, n, out_lo, out_hi, transpose); };
+    A[e] = make_float4(val(r0, c0), val(r0 + 8, c0), val(r0, c0 + 4), val(r0 + 8, c0 + 4));
+  } else {
+    const int NP = (n + 1) & ~1;
+    A[e] = sep_entry((int)(e % NP), (int)(e / NP), n, out_lo, out_hi, transpose);
+  }
 }
 // Reciprocal pivots of the x systems, one line per thread, in FP64.
 template <typename T>
@@ -467,14 +546,14 @@ __global__ void k_sep_pivots(Level<T> L, T* piv) {
   if (line >= L.ny * L.nz) return;
   const double lam = sep_eig(line % L.ny, L.ny, L.out_mask & 4, L.out_mask & 8) +
                      sep_eig(line / L.ny, L.nz, L.out_mask & 16, L.out_mask & 32);
-  float* row = piv + (size_t)line * L.P;
+  T* row = piv + (size_t)line * L.P;
   double e = 0.0;
   for (int i = 0; i < L.nx; ++i) {
     double d = 2.0 + lam;
     if (i == 0 && !(L.out_mask & 1)) d -= 1.0;
     if (i == L.nx - 1 && !(L.out_mask & 2)) d -= 1.0;
     e = 1.0 / (d - e);
-    row[i] = (float)e;
+    row[i] = (T)e;
   }
 }
 

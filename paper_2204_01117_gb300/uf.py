@@ -668,9 +668,9 @@ class Grid:
         advect_zc: z planes per block of the fused advection; unfused: bit
         mask of fused kernels to run as their separate sub-step kernels
         (1: advection, 2: diffusion + drag + BCs + pressure right-hand side;
-        True: all); coarse_start: 0 automatic (FP32 grids with the default
-        smoother and transfers: the separable inverse instead of the
-        V-cycle), -1 the V-cycle with per-level launches, > 0 its first MG
+        True: all); coarse_start: 0 automatic (with the default smoother and
+        transfers, where the sizes allow: the separable inverse instead of
+        the V-cycle), -1 the V-cycle with per-level launches, > 0 its first MG
         level in the one-launch cluster form.  Every choice gives the same
         values (the separable inverse: to the solver's tolerance)."""
         t = Tuning()
