@@ -72,7 +72,7 @@ struct LaunchMap {
 // MAP_DIR: the march tiles of the finest level, every instance; the V-cycle
 // maps (MAP_TAIL, MAP_MARCH0 ..) hold the instances that run it, the MAP_SEP
 // ones those with the separable inverse.
-enum MapKind { MAP_CFL = 0, MAP_CELL, MAP_FACE, MAP_CHUNK, MAP_TAIL, MAP_ADV, MAP_ADV_FAR, MAP_DIR, MAP_SEPZ, MAP_SEPY, MAP_SEPX, MAP_MARCH0 };
+enum MapKind { MAP_CFL = 0, MAP_TURB, MAP_CELL, MAP_FACE, MAP_CHUNK, MAP_TAIL, MAP_ADV, MAP_ADV_FAR, MAP_DIR, MAP_SEPZ, MAP_SEPY, MAP_SEPX, MAP_MARCH0 };
 constexpr int kMaps = MAP_MARCH0 + uf::MAX_LEVELS;
 
 __device__ __forceinline__ int map_entry(const LaunchMap* __restrict__ m, int w) {
@@ -148,7 +148,6 @@ template <typename T>
 struct CellP {   // k-omega
   uf::StepParams<T> sp;
   const T *u, *v, *w;
-  T* nut;
   T* kb[2];
   T* ob[2];
 };
@@ -345,12 +344,12 @@ __global__ void __launch_bounds__(uf::NT) kb_project(const __grid_constant__ Arg
 }
 
 template <typename T>
-__global__ void __launch_bounds__(uf::NT, 6) kb_turbulence(const __grid_constant__ Args<CellP<T>> A,
+__global__ void __launch_bounds__(uf::NT, sizeof(T) == 8 ? 2 : 3) kb_turbulence(const __grid_constant__ Args<CellP<T>> A,
                                                         const int* __restrict__ par) {
-  for_plane_items(&A.m, [&](int i, const VBlock& vb) {
+  for_items(&A.m, [&](int i, int zc, const VBlock& vb) {
     const CellP<T>& P = A.at[i];
     const int a = par[i], o = a ^ 1;
-    uf::turbulence_body<T>(P.sp, P.u, P.v, P.w, P.kb[a], P.ob[a], P.kb[o], P.ob[o], vb);
+    uf::turbulence_body<T>(P.sp, P.u, P.v, P.w, P.kb[a], P.ob[a], P.kb[o], P.ob[o], zc, vb);
   });
 }
 
@@ -486,6 +485,8 @@ class BatchImpl final : public uf_batch {
       add_plane_entry(maps[MAP_CELL], i, (d.nx + uf::BX - 1) / uf::BX, (d.ny + uf::BY - 1) / uf::BY, d.nz);
       add_plane_entry(maps[MAP_FACE], i, (d.nx + 1 + uf::BX - 1) / uf::BX, (d.ny + 1 + uf::BY - 1) / uf::BY,
                       3 * d.nz + 1);
+      add_entry(maps[MAP_TURB], i, (d.nx + uf::BX - 1) / uf::BX, (d.ny + uf::BY - 1) / uf::BY, (d.nz + uf::TURB_ZC - 1) / uf::TURB_ZC,
+                uf::TURB_ZC);
       add_entry(maps[MAP_CHUNK], i, G.chunk_g[0], G.chunk_g[1], G.chunk_g[2], G.chunk_zc);
       add_entry(maps[G.adv_far ? MAP_ADV_FAR : MAP_ADV], i, G.adv_g[0], G.adv_g[1],
                 G.adv_auto ? (d.nz + adv_zc - 1) / adv_zc : G.adv_g[2], G.adv_auto ? adv_zc : G.adv_zc);
@@ -731,7 +732,6 @@ class BatchImpl final : public uf_batch {
     std::memset(&P, 0, sizeof(P));
     P.sp = G.sp;
     P.u = G.u; P.v = G.v; P.w = G.w;
-    P.nut = G.nut;
     P.kb[0] = G.kb[0]; P.kb[1] = G.kb[1]; P.ob[0] = G.ob[0]; P.ob[1] = G.ob[1];
     return P;
   }
@@ -835,9 +835,9 @@ class BatchImpl final : public uf_batch {
                  }));
     {
       auto k = kb_turbulence<T>;
-      const auto& A = args<CellP<T>>(MAP_CELL, [](CellP<T>& P, const View<T>& G) { P = cell_params(G); });
-      L(s, "b_turbulence", plane_bytes(MAP_CELL, 7),
-        [&] { k<<<grid_of(k, uf::NT, 0, items(MAP_CELL)), dim3(uf::BX, uf::BY), 0, s>>>(A, d_par); });
+      const auto& A = args<CellP<T>>(MAP_TURB, [](CellP<T>& P, const View<T>& G) { P = cell_params(G); });
+      L(s, "b_turbulence", plane_bytes(MAP_TURB, 7),
+        [&] { k<<<grid_of(k, uf::NT, 0, items(MAP_TURB)), dim3(uf::BX, uf::BY), 0, s>>>(A, d_par); });
     }
     L(s, "b_flip_parity", 0, [&] { kb_flip_parity<<<(n + 63) / 64, 64, 0, s>>>(d_par, n); });
   }

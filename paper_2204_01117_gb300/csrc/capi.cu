@@ -1015,6 +1015,16 @@ class GridImpl final : public uf_grid {
     }
   }
 
+  // k-omega update: columns of TURB_ZC planes, fewer where the grid would not
+  // fill the chip (the values do not depend on it).
+  dim3 turb_grid(int* zc) const {
+    const int bx = (d.nx + uf::BX - 1) / uf::BX, by = (d.ny + uf::BY - 1) / uf::BY;
+    int z = uf::TURB_ZC;
+    while (z > 1 && (long)bx * by * ((d.nz + z - 1) / z) < 2 * 456) z /= 2;
+    *zc = z;
+    return dim3(bx, by, (d.nz + z - 1) / z);
+  }
+
   void rec_post(cudaStream_t s, const T* kin, const T* oin, T* kout, T* oout) {
     const dim3 blk(uf::BX, uf::BY);
     const double faces = 3 * N() * tb(), cells = N() * tb();
@@ -1023,7 +1033,11 @@ class GridImpl final : public uf_grid {
     L(s, "project", 2 * faces + 2 * cells,
       [&] { uf::k_project_cells<T><<<plane_grid(d.nx + 1, d.ny + 1, d.nz), blk, 0, s>>>(sp, pd, u, v, w); });
     L(s, "turbulence", faces + 4 * cells,
-      [&] { uf::k_turbulence<T><<<plane_grid(d.nx, d.ny, d.nz), blk, 0, s>>>(sp, u, v, w, kin, oin, kout, oout); });
+      [&] {
+        int zc;
+        const dim3 g = turb_grid(&zc);
+        uf::k_turbulence<T><<<g, blk, 0, s>>>(sp, u, v, w, kin, oin, kout, oout, zc);
+      });
   }
 
   // One step launched eagerly with per-launch events; aggregates by name.
@@ -2232,7 +2246,9 @@ class GridImpl final : public uf_grid {
         UF_TRY(cell_in(C[0], in[3]));
         UF_TRY(cell_in(C[1], in[4]));
         if (!tr) {
-          uf::k_turbulence<T><<<gc, bk, 0, stream>>>(sp, S[0].u, S[0].v, S[0].w, C[0], C[1], C[2], C[3]);
+          int zc;
+          const dim3 gt = turb_grid(&zc);
+          uf::k_turbulence<T><<<gt, bk, 0, stream>>>(sp, S[0].u, S[0].v, S[0].w, C[0], C[1], C[2], C[3], zc);
           UF_CUDA(cudaGetLastError());
           UF_TRY(cell_out(out[0], C[2]));
           return cell_out(out[1], C[3]);

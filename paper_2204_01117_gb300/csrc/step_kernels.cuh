@@ -686,55 +686,106 @@ __global__ void __launch_bounds__(NT) k_project_cells(StepParams<T> p, const PSt
 // 2 alpha |S|^2 - beta omega^2 with P_k = 2 nu_t |S|^2, |S|^2 = S_ij S_ij of
 // the projected velocity.  Ghosts: inlet values on inlet sides, zero
 // gradient elsewhere.  Floors k_min, omega_min.
+// A thread marches a column over zc planes.  What the next plane needs again
+// (its own faces' means, the w faces above, k and omega) stays in registers,
+// so a cell takes 27 loads instead of 46; a neighbour beyond the domain is
+// the cell itself (an offset of zero), which is the one-sided difference of
+// the strain and the zero gradient of k and omega, and only an inlet replaces
+// it.  Bound by instruction issue; measured at 256 x 256 x 64, FP32, against
+// one thread per cell: 86 -> 70 us.
+constexpr int TURB_ZC = 8;   // planes per thread of the single-grid launches
 template <typename T>
 __device__ __forceinline__ void turbulence_body(const StepParams<T>& p, const T* __restrict__ u,
                                                 const T* __restrict__ v, const T* __restrict__ w,
                                                 const T* __restrict__ ki, const T* __restrict__ oi,
-                                                T* __restrict__ ko, T* __restrict__ oo, const VBlock& vb) {
-  const int i = vb.x * BX + threadIdx.x, j = vb.y * BY + threadIdx.y, k = vb.z;
-  if (i >= p.nx || j >= p.ny) return;
-  const T dt = *p.dtT;
-  const size_t c = idx_c(p, i, j, k);
-  const T kc = ki[c], oc = oi[c];
-  const T S2 = strain_sq(u, v, w, p, i, j, k);
-  const T nut = limited_nut(p, kc, oc, S2, nut_cap(p, dt));
-  const T vel[3] = {T(0.5) * (u[idx_u(p, i, j, k)] + u[idx_u(p, i + 1, j, k)]),
-                    T(0.5) * (v[idx_v(p, i, j, k)] + v[idx_v(p, i, j + 1, k)]),
-                    T(0.5) * (w[idx_c(p, i, j, k)] + w[idx_c(p, i, j, k + 1)])};
-  const int pos[3] = {i, j, k}, ext[3] = {p.nx, p.ny, p.nz};
-  T adv_k = 0, adv_o = 0, lap_k = T(-6) * kc, lap_o = T(-6) * oc;
-#pragma unroll
-  for (int ax = 0; ax < 3; ++ax) {
-    const size_t stride = ax == 0 ? 1 : (ax == 1 ? (size_t)p.Pc : (size_t)p.Pc * p.ny);
-    const bool has_m = pos[ax] > 0, has_p = pos[ax] < ext[ax] - 1;
-    const int sm = p.side[2 * ax], sp = p.side[2 * ax + 1];
-    const T km = has_m ? ki[c - stride] : (sm == INFLOW ? p.k_in : kc);
-    const T kp = has_p ? ki[c + stride] : (sp == INFLOW ? p.k_in : kc);
-    const T om_m = has_m ? oi[c - stride] : (sm == INFLOW ? p.om_in : oc);
-    const T om_p = has_p ? oi[c + stride] : (sp == INFLOW ? p.om_in : oc);
-    lap_k += km + kp;
-    lap_o += om_m + om_p;
-    if (vel[ax] > T(0)) {
-      adv_k += vel[ax] * (kc - km) * p.inv_h;
-      adv_o += vel[ax] * (oc - om_m) * p.inv_h;
-    } else if (vel[ax] < T(0)) {
-      adv_k += vel[ax] * (kp - kc) * p.inv_h;
-      adv_o += vel[ax] * (om_p - oc) * p.inv_h;
-    }
+                                                T* __restrict__ ko, T* __restrict__ oo, int zc, const VBlock& vb) {
+  const int i = vb.x * BX + threadIdx.x, j = vb.y * BY + threadIdx.y;
+  const int z0 = vb.z * zc, z1 = min(p.nz, z0 + zc);
+  if (i >= p.nx || j >= p.ny || z0 >= z1) return;
+  const T dt = *p.dtT, cap = nut_cap(p, dt), ih = p.inv_h, ih2 = p.inv_h * p.inv_h, hh = T(0.5) * ih;
+  const int Pu = p.Pu, Pc = p.Pc;
+  const size_t su = (size_t)Pu * p.ny, sv = (size_t)Pc * (p.ny + 1), sc = (size_t)Pc * p.ny;   // plane strides
+  const int xm = i > 0 ? -1 : 0, xp = i < p.nx - 1 ? 1 : 0, ym = j > 0 ? -1 : 0, yp = j < p.ny - 1 ? 1 : 0;
+  const T sx = xp - xm == 2 ? hh : (xp > xm ? ih : T(0)), sy = yp - ym == 2 ? hh : (yp > ym ? ih : T(0));
+  const bool in_xm = i == 0 && p.side[0] == INFLOW, in_xp = i == p.nx - 1 && p.side[1] == INFLOW;
+  const bool in_ym = j == 0 && p.side[2] == INFLOW, in_yp = j == p.ny - 1 && p.side[3] == INFLOW;
+  const T *pu = u + idx_u(p, i, j, z0), *pv = v + idx_v(p, i, j, z0), *pw = w + idx_c(p, i, j, z0);
+  size_t c = idx_c(p, i, j, z0);
+  auto mean = [](T a, T b) { return T(0.5) * (a + b); };
+  T u0 = pu[0], u1 = pu[1], v0 = pv[0], v1 = pv[Pc], w0 = pw[0];
+  T wxm0 = pw[xm], wxp0 = pw[xp], wym0 = pw[ym * Pc], wyp0 = pw[yp * Pc];
+  T kc = ki[c], oc = oi[c];
+  T uz = mean(u0, u1), vz = mean(v0, v1), kz = kc, oz = oc;   // one plane below
+  if (z0 > 0) {
+    uz = mean(*(pu - su), *(pu - su + 1));
+    vz = mean(*(pv - sv), *(pv - sv + Pc));
+    kz = ki[c - sc];
+    oz = oi[c - sc];
   }
-  const T ih2 = p.inv_h * p.inv_h;
-  const T Pk = T(2) * nut * S2;
-  const T rk = -adv_k + Pk - p.C_mu * kc * oc + (p.nu + p.sigma_star * nut) * lap_k * ih2;
-  const T ro = -adv_o + T(2) * p.alpha * S2 - p.beta * oc * oc + (p.nu + p.sigma * nut) * lap_o * ih2;
-  ko[c] = fmax(kc + dt * rk, p.k_min);
-  oo[c] = fmax(oc + dt * ro, p.om_min);
+  for (int k = z0; k < z1; ++k) {
+    const bool top = k == p.nz - 1;
+    const T w1 = pw[sc], wxm1 = (pw + sc)[xm], wxp1 = (pw + sc)[xp], wym1 = (pw + sc)[ym * Pc], wyp1 = (pw + sc)[yp * Pc];
+    const T ujm = mean(pu[ym * Pu], pu[ym * Pu + 1]), ujp = mean(pu[yp * Pu], pu[yp * Pu + 1]);
+    const T vim = mean(pv[xm], pv[xm + Pc]), vip = mean(pv[xp], pv[xp + Pc]);
+    T kxm = ki[c + xm], kxp = ki[c + xp], kym = ki[c + (ptrdiff_t)ym * Pc], kyp = ki[c + (ptrdiff_t)yp * Pc];
+    T oxm = oi[c + xm], oxp = oi[c + xp], oym = oi[c + (ptrdiff_t)ym * Pc], oyp = oi[c + (ptrdiff_t)yp * Pc];
+    T un0 = u0, un1 = u1, vn0 = v0, vn1 = v1, kn = kc, on = oc;   // one plane above
+    if (!top) {
+      un0 = pu[su];
+      un1 = (pu + su)[1];
+      vn0 = pv[sv];
+      vn1 = (pv + sv)[Pc];
+      kn = ki[c + sc];
+      on = oi[c + sc];
+    }
+    if (in_xm) { kxm = p.k_in; oxm = p.om_in; }
+    if (in_xp) { kxp = p.k_in; oxp = p.om_in; }
+    if (in_ym) { kym = p.k_in; oym = p.om_in; }
+    if (in_yp) { kyp = p.k_in; oyp = p.om_in; }
+    const T uc = mean(u0, u1), vc = mean(v0, v1), wc = mean(w0, w1), un = mean(un0, un1), vn = mean(vn0, vn1);
+    // S_ij S_ij (the expressions of strain_sq)
+    const bool below = k > 0;
+    const T sz = below && !top ? hh : (below || !top ? ih : T(0));
+    const T sxx = (u1 - u0) * ih, syy = (v1 - v0) * ih, szz = (w1 - w0) * ih;
+    const T sxy = T(0.5) * ((ujp - ujm) * sy + (vip - vim) * sx);
+    const T sxz = T(0.5) * ((un - uz) * sz + (mean(wxp0, wxp1) - mean(wxm0, wxm1)) * sx);
+    const T syz = T(0.5) * ((vn - vz) * sz + (mean(wyp0, wyp1) - mean(wym0, wym1)) * sy);
+    const T diag = fma_rn(szz, szz, fma_rn(syy, syy, mul_rn(sxx, sxx)));
+    const T off = fma_rn(syz, syz, fma_rn(sxz, sxz, mul_rn(sxy, sxy)));
+    const T S2 = fma_rn(T(2), off, diag);
+    const T nut = limited_nut(p, kc, oc, S2, cap);
+    T adv_k = 0, adv_o = 0, lap_k = T(-6) * kc, lap_o = T(-6) * oc;
+    auto axis = [&](T vel, T km, T kp, T om, T op) {
+      lap_k += km + kp;
+      lap_o += om + op;
+      if (vel > T(0)) {
+        adv_k += vel * (kc - km) * ih;
+        adv_o += vel * (oc - om) * ih;
+      } else if (vel < T(0)) {
+        adv_k += vel * (kp - kc) * ih;
+        adv_o += vel * (op - oc) * ih;
+      }
+    };
+    axis(uc, kxm, kxp, oxm, oxp);
+    axis(vc, kym, kyp, oym, oyp);
+    axis(wc, kz, kn, oz, on);
+    const T Pk = T(2) * nut * S2;
+    const T rk = -adv_k + Pk - p.C_mu * kc * oc + (p.nu + p.sigma_star * nut) * lap_k * ih2;
+    const T ro = -adv_o + T(2) * p.alpha * S2 - p.beta * oc * oc + (p.nu + p.sigma * nut) * lap_o * ih2;
+    ko[c] = fmax(kc + dt * rk, p.k_min);
+    oo[c] = fmax(oc + dt * ro, p.om_min);
+    uz = uc; vz = vc; kz = kc; oz = oc;
+    u0 = un0; u1 = un1; v0 = vn0; v1 = vn1; kc = kn; oc = on;
+    w0 = w1; wxm0 = wxm1; wxp0 = wxp1; wym0 = wym1; wyp0 = wyp1;
+    pu += su; pv += sv; pw += sc; c += sc;
+  }
 }
 
 template <typename T>
-__global__ void __launch_bounds__(NT) k_turbulence(StepParams<T> p, const T* __restrict__ u, const T* __restrict__ v,
+__global__ void __launch_bounds__(NT, sizeof(T) == 8 ? 2 : 3) k_turbulence(StepParams<T> p, const T* __restrict__ u, const T* __restrict__ v,
                                                    const T* __restrict__ w, const T* __restrict__ ki,
-                                                   const T* __restrict__ oi, T* __restrict__ ko, T* __restrict__ oo) {
-  turbulence_body<T>(p, u, v, w, ki, oi, ko, oo, vblock());
+                                                   const T* __restrict__ oi, T* __restrict__ ko, T* __restrict__ oo, int zc) {
+  turbulence_body<T>(p, u, v, w, ki, oi, ko, oo, zc, vblock());
 }
 
 
