@@ -82,23 +82,6 @@ __device__ __forceinline__ T level_apply(const Level<T>& L, int i, int j, int k,
   return acc;
 }
 
-// level_apply on the pressure store: the same stencil, with each
-// neighbour difference taken on the stored pairs (ps_diff).
-template <typename T>
-__device__ __forceinline__ T level_apply_store(const Level<T>& L, int i, int j, int k, const PStore<T>* __restrict__ g) {
-  const PStore<T> gc = g[lidx(L, i, j, k)];
-  const T xc = (T)ps_value(gc);
-  auto d = [&](int a, int b2, int c2) { return (T)ps_diff(gc, g[lidx(L, a, b2, c2)]); };
-  T acc = 0;
-  if (i > 0) acc += L.wx * d(i - 1, j, k); else if (L.out_mask & 1) acc += L.wx * xc;
-  if (i < L.nx - 1) acc += L.wx * d(i + 1, j, k); else if (L.out_mask & 2) acc += L.wx * xc;
-  if (j > 0) acc += L.wy * d(i, j - 1, k); else if (L.out_mask & 4) acc += L.wy * xc;
-  if (j < L.ny - 1) acc += L.wy * d(i, j + 1, k); else if (L.out_mask & 8) acc += L.wy * xc;
-  if (k > 0) acc += L.wz * d(i, j, k - 1); else if (L.out_mask & 16) acc += L.wz * xc;
-  if (k < L.nz - 1) acc += L.wz * d(i, j, k + 1); else if (L.out_mask & 32) acc += L.wz * xc;
-  return acc;
-}
-
 // Cell loop of a 32x8 thread tile over the z planes [z0, z1) of a block.
 #define UF_CELL_LOOP_VB(L, vb)                                              \
   const int i = (vb).x * BX + threadIdx.x, j = (vb).y * BY + threadIdx.y;   \
@@ -135,17 +118,44 @@ __device__ __forceinline__ void cg_init_body(const Level<T>& L, const T* __restr
   const bool zero_rhs = st->bb == 0.0;
   double acc = 0.0;
   DotAcc<T> dacc;
-  if (inside) {
+  if (inside && !zero_rhs && g) {
+    // level_apply on the pressure store, each neighbour difference taken on
+    // the stored pairs (ps_diff); the column's own values roll along z in
+    // registers (256 x 256 x 64: 57 -> 49 us)
+    const int SY = L.P;
+    const size_t SZ = (size_t)L.P * L.ny;
+    size_t c = lidx(L, i, j, z0);
+    const PStore<T>* gp = g + c;
+    T* __restrict__ r = L.r;
+    const bool x0 = i > 0, x1 = i < L.nx - 1, y0 = j > 0, y1 = j < L.ny - 1;
+    PStore<T> gm = z0 > 0 ? *(gp - SZ) : gp[0], gc = gp[0];
+#pragma unroll 2
+    for (int k = z0; k < z1; ++k) {
+      const PStore<T> gxm = x0 ? *(gp - 1) : gc, gxp = x1 ? gp[1] : gc, gym = y0 ? *(gp - SY) : gc, gyp = y1 ? gp[SY] : gc;
+      const PStore<T> gn = k < L.nz - 1 ? gp[SZ] : gc;
+      const T bv = b[c], xc = (T)ps_value(gc);
+      T ax = 0;
+      if (x0) ax += L.wx * (T)ps_diff(gc, gxm); else if (L.out_mask & 1) ax += L.wx * xc;
+      if (x1) ax += L.wx * (T)ps_diff(gc, gxp); else if (L.out_mask & 2) ax += L.wx * xc;
+      if (y0) ax += L.wy * (T)ps_diff(gc, gym); else if (L.out_mask & 4) ax += L.wy * xc;
+      if (y1) ax += L.wy * (T)ps_diff(gc, gyp); else if (L.out_mask & 8) ax += L.wy * xc;
+      if (k > 0) ax += L.wz * (T)ps_diff(gc, gm); else if (L.out_mask & 16) ax += L.wz * xc;
+      if (k < L.nz - 1) ax += L.wz * (T)ps_diff(gc, gn); else if (L.out_mask & 32) ax += L.wz * xc;
+      const T rv = bv - ax;
+      x[c] = T(0);
+      r[c] = rv;
+      dacc.add(rv, rv);
+      gm = gc;
+      gc = gn;
+      gp += SZ;
+      c += SZ;
+    }
+  } else if (inside) {
     for (int k = z0; k < z1; ++k) {
       const size_t c = lidx(L, i, j, k);
       if (zero_rhs) {
         x[c] = T(0);
         L.r[c] = T(0);
-      } else if (g) {
-        const T rv = b[c] - level_apply_store(L, i, j, k, g);
-        x[c] = T(0);
-        L.r[c] = rv;
-        dacc.add(rv, rv);
       } else {
         const T ax = level_apply(L, i, j, k, [&](int a, int b2, int c2) { return x[lidx(L, a, b2, c2)]; });
         const T rv = b[c] - ax;
