@@ -337,9 +337,9 @@ __global__ void __launch_bounds__(uf::NT, 6) kb_pressure_commit(const __grid_con
 
 template <typename T>
 __global__ void __launch_bounds__(uf::NT) kb_project(const __grid_constant__ Args<ProjP<T>> A) {
-  for_plane_items(&A.m, [&](int i, const VBlock& vb) {
+  for_items(&A.m, [&](int i, int, const VBlock& vb) {
     const ProjP<T>& P = A.at[i];
-    uf::project_body<T>(P.sp, P.pr, P.u, P.v, P.w, vb);
+    uf::project_cells_body<T>(P.sp, P.pr, P.u, P.v, P.w, vb);
   });
 }
 
@@ -483,8 +483,8 @@ class BatchImpl final : public uf_batch {
         add_entry(maps[MAP_CFL], i, blocks, 1, 1, 0);
       }
       add_plane_entry(maps[MAP_CELL], i, (d.nx + uf::BX - 1) / uf::BX, (d.ny + uf::BY - 1) / uf::BY, d.nz);
-      add_plane_entry(maps[MAP_FACE], i, (d.nx + 1 + uf::BX - 1) / uf::BX, (d.ny + 1 + uf::BY - 1) / uf::BY,
-                      3 * d.nz + 1);
+      add_entry(maps[MAP_FACE], i, (d.nx + 1 + uf::BX - 1) / uf::BX, (d.ny + 1 + uf::BY - 1) / uf::BY,
+                (d.nz + uf::PROJ_ZC - 1) / uf::PROJ_ZC, uf::PROJ_ZC);
       add_entry(maps[MAP_TURB], i, (d.nx + uf::BX - 1) / uf::BX, (d.ny + uf::BY - 1) / uf::BY, (d.nz + uf::TURB_ZC - 1) / uf::TURB_ZC,
                 uf::TURB_ZC);
       add_entry(maps[MAP_CHUNK], i, G.chunk_g[0], G.chunk_g[1], G.chunk_g[2], G.chunk_zc);
