@@ -231,8 +231,13 @@ Plan make_plan(const uf_grid_desc* d) {
   P.grad = L.take(sizeof(double) * 3 * uf::MAX_BOXES);
   P.sep = sep_available(d);
   if (P.sep) {
-    auto packed = [&](int n) {
-      return d->precision == UF_F64 ? uf::sep_mat_count<double>(n) * sizeof(double) : uf::sep_mat_count<float>(n) * sizeof(float4);
+    auto packed = [&](int n) {   // folded or not
+      size_t b = 0;
+      for (int f = 0; f < 2; ++f) {
+        const uf::SepAxis x{n, f};
+        b = std::max(b, d->precision == UF_F64 ? uf::sep_mat_count<double>(x) * sizeof(double) : uf::sep_mat_count<float>(x) * sizeof(float4));
+      }
+      return b;
     };
     for (size_t& o : P.sep_y) o = L.take(packed(d->ny));
     for (size_t& o : P.sep_z) o = L.take(packed(d->nz));
@@ -508,9 +513,10 @@ class GridImpl final : public uf_grid {
       using Mat = typename uf::Sep<T>::Mat;
       Mat* m[4] = {at<Mat>(P.sep_y[0]), at<Mat>(P.sep_y[1]), at<Mat>(P.sep_z[0]), at<Mat>(P.sep_z[1])};
       for (int q = 0; q < 4; ++q) {
-        const int n = q < 2 ? d.ny : d.nz, bit = q < 2 ? 4 : 16;
-        const unsigned nb = (unsigned)((uf::sep_mat_count<T>(n) + 255) / 256);
-        uf::k_sep_pack<T><<<nb, 256, 0, stream>>>(m[q], n, out_mask & bit, out_mask & (2 * bit), q & 1);
+        const uf::SepAxis x = q < 2 ? uf::sep_axis_y(lv[0]) : uf::sep_axis_z(lv[0]);
+        const int bit = q < 2 ? 4 : 16;
+        const unsigned nb = (unsigned)((uf::sep_mat_count<T>(x) + 255) / 256);
+        uf::k_sep_pack<T><<<nb, 256, 0, stream>>>(m[q], x, out_mask & bit, out_mask & (2 * bit), q & 1);
       }
       UF_CUDA(cudaGetLastError());
       sep = uf::Sep<T>{1, m[0], m[1], m[2], m[3], r2, lv[0].x, lv[0].t};
@@ -798,7 +804,7 @@ class GridImpl final : public uf_grid {
   void rec_sep(cudaStream_t s, int mode, cudaGraphConditionalHandle cond, int use_cond) {
     const int wn = uf::sep_y_wn<T>(d.ny), by = 32 * wn;
     const unsigned gz = uf::sep_z_blocks<T>(lv[0].P, d.ny, d.nz);
-    const size_t sz = uf::sep_smem<T>(uf::SEP_Z_WN<T>, d.nz), sy = uf::sep_smem<T>(wn, d.ny);
+    const size_t sz = uf::sep_smem<T>(uf::SEP_Z_WN<T>, uf::sep_axis_z(lv[0])), sy = uf::sep_smem<T>(wn, uf::sep_axis_y(lv[0]));
     const dim3 gy((lv[0].P + by - 1) / by, uf::sep_y_split<T>(lv[0].P, d.ny, d.nz), d.nz);
     const unsigned gx = (unsigned)((d.ny * d.nz + uf::SEP_X_LINES - 1) / uf::SEP_X_LINES);
     if (mode == 1)

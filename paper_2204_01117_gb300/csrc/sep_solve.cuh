@@ -23,14 +23,21 @@
 // against 4.8e-6).  Measured on a GB300, one time step with the V-cycle and
 // with this: 48 x 40 x 16 0.73 -> 0.20 ms, 157 x 203 x 41 1.87 -> 0.47 ms,
 // 256 x 256 x 64 2.20 -> 1.09 ms, 512 x 768 x 1 1.24 -> 0.34 ms,
-// 512 x 512 x 128 13.0 -> 8.7 ms (where the y transforms, 2 n^2 per column
-// and pass, take 0.41 ms each); the longest axes that fit were all faster.
+// 512 x 512 x 128 13.0 -> 8.7 ms (where the y transforms cost most); the
+// longest axes that fit were all faster.
 //
 // The transforms are contractions of a field with a constant n x n matrix:
 // tensor cores, TF32 operands split into a high and a low part (x = hi + lo,
 // 11 bits each), three products hi hi + hi lo + lo hi accumulated in FP32.
 // The dropped lo lo is below 2^-22 of the product, so a transform is about
 // as accurate as one in plain FP32.
+//
+// The modes of an axis with walls at both ends are even or odd about its
+// middle, so there (always along z; along y for a wind along x) a transform
+// takes the sums and the differences of mirrored cells through two matrices
+// of half the size: half the products (a y transform
+// of 512 x 512 x 128 0.61 -> 0.44 ms, of 256 x 256 x 64 47 -> 38 us; the
+// solves need fewer iterations too, sums of half the length round less).
 #pragma once
 #include "mg_fused.cuh"
 
@@ -53,7 +60,8 @@ struct SepMat<double> { using type = double; };
 // which the lanes of a warp read the A operand of mma.m16n8k8: one float4 per
 // lane and 16 x 8 tile, tiles row by row, zero beyond the matrix.  FP64
 // matrices are stored column by column, each padded with zeros to an even
-// number of rows.
+// number of rows.  A folded axis (SepAxis) has the matrix of its even modes,
+// then that of its odd modes.
 template <typename T>
 struct Sep {
   using Mat = typename SepMat<T>::type;
@@ -80,8 +88,21 @@ template <typename T>
 __host__ __device__ inline int sep_y_wn(int ny) { return sizeof(T) == 4 && ny <= SEP_Y_WIDE ? 2 : 1; }
 template <typename T>
 constexpr int SEP_Z_WN = sizeof(T) == 4 ? 4 : 1;
+// The axis of a transform: its cells (or modes) in one block of panel rows and
+// one matrix, or folded in two, the even one of (n + 1) / 2 rows and the odd
+// one of n / 2 rows, each padded with zero rows to a multiple of 8.
+struct SepAxis {
+  int n, fold;
+  __host__ __device__ int size(int odd) const { return fold ? (n + 1 - odd) / 2 : odd ? 0 : n; }
+  __host__ __device__ int pad(int odd) const { return (size(odd) + 7) / 8 * 8; }
+  __host__ __device__ int rows() const { return pad(0) + pad(1); }
+};
 template <typename T>
-inline size_t sep_smem(int wn, int n) { return sizeof(T) * (size_t)((n + 7) / 8 * 8) * (sizeof(T) == 4 ? 32 * wn + 8 : 32); }
+__host__ __device__ inline SepAxis sep_axis_y(const Level<T>& L) { return {L.ny, !(L.out_mask & 12)}; }
+template <typename T>
+__host__ __device__ inline SepAxis sep_axis_z(const Level<T>& L) { return {L.nz, !(L.out_mask & 48)}; }
+template <typename T>
+inline size_t sep_smem(int wn, const SepAxis& x) { return sizeof(T) * (size_t)x.rows() * (sizeof(T) == 4 ? 32 * wn + 8 : 32); }
 // Columns (x, y) of a z panel, and the blocks that cover the plane.  One cell
 // in z has nothing to transform: the threads just share the columns out.
 template <typename T>
@@ -120,90 +141,196 @@ __device__ __forceinline__ void mma_tf32(float (&c)[4], const uint32_t (&a)[4], 
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// Result rows of the block's panel: A (M x K packed) times sB ([K][pitch]),
-// rounds part, part + parts, ... of 32 WM rows.
-// put(row, column of the panel (even), value, next value).
+// acc[h] += tile row h of A (packed, KT tiles a row) times the 8 KT panel rows at b.
+template <int WN, int TILES>
+__device__ __forceinline__ void sep_mma(float (&acc)[TILES][4][4], const float4* const (&a)[TILES], int KT, const float* b) {
+  constexpr int PB = SEP_PITCH<float, WN>;
+  float4 next[TILES];
+#pragma unroll
+  for (int h = 0; h < TILES; ++h) next[h] = __ldg(a[h]);
+#pragma unroll 2
+  for (int kt = 0; kt < KT; ++kt) {
+    uint32_t hi[TILES][4], lo[TILES][4];
+#pragma unroll
+    for (int h = 0; h < TILES; ++h) {
+      const float4 c = next[h];
+      if (kt + 1 < KT) next[h] = __ldg(a[h] + (size_t)(kt + 1) * 32);
+      tf32_split(c.x, hi[h][0], lo[h][0]);
+      tf32_split(c.y, hi[h][1], lo[h][1]);
+      tf32_split(c.z, hi[h][2], lo[h][2]);
+      tf32_split(c.w, hi[h][3], lo[h][3]);
+    }
+    const float* bk = b + kt * 8 * PB;
+    uint32_t bh[4][2], bl[4][2];
+#pragma unroll
+    for (int n = 0; n < 4; ++n) {
+      tf32_split(bk[n * 8], bh[n][0], bl[n][0]);
+      tf32_split(bk[n * 8 + 4 * PB], bh[n][1], bl[n][1]);
+    }
+    // one product at a time over all accumulators: each waits for its own last product
+#pragma unroll
+    for (int n = 0; n < 4; ++n)
+#pragma unroll
+      for (int h = 0; h < TILES; ++h) mma_tf32(acc[h][n], lo[h], bh[n][0], bh[n][1]);
+#pragma unroll
+    for (int n = 0; n < 4; ++n)
+#pragma unroll
+      for (int h = 0; h < TILES; ++h) mma_tf32(acc[h][n], hi[h], bl[n][0], bl[n][1]);
+#pragma unroll
+    for (int n = 0; n < 4; ++n)
+#pragma unroll
+      for (int h = 0; h < TILES; ++h) mma_tf32(acc[h][n], hi[h], bh[n][0], bh[n][1]);
+  }
+}
+
+// The transform of the block's panel sB ([rows][pitch]) by the matrices A of
+// its axis, result rows in units of a warp: part, part + parts, ... of every
+// round of 8 / WN units.  put(row, column of the panel (even), value, next value).
+//
+// Forward, and both ways of an axis that is not folded: 32 rows a unit, those
+// of the even modes first.
 template <int WN, typename Put>
-__device__ __forceinline__ void sep_gemm(const float4* __restrict__ A, int M, int K, const float* sB, int part, int parts,
+__device__ __forceinline__ void sep_gemm(const float4* __restrict__ A, const SepAxis& x, const float* sB, int part, int parts,
                                          Put put) {
   constexpr int PB = SEP_PITCH<float, WN>, WM = 8 / WN;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3, wm = warp / WN, wn = warp % WN;
-  const int KT = (K + 7) / 8, MT16 = (M + 15) / 16;
-  const float* b = sB + t * PB + wn * 32 + g;
-  for (int m0 = 2 * (wm + WM * part); m0 < MT16; m0 += 2 * WM * parts) {
-    const bool two = m0 + 1 < MT16;
-    const float4* a0 = A + (size_t)m0 * KT * 32 + lane;
-    const float4* a1 = a0 + (two ? (size_t)KT * 32 : 0);
-    float acc[2][4][4];
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-      for (int n = 0; n < 4; ++n)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) acc[h][n][e] = 0.f;
-    float4 n0 = __ldg(a0), n1 = __ldg(a1);
-#pragma unroll 2
-    for (int kt = 0; kt < KT; ++kt) {
-      const float4 c0 = n0, c1 = n1;
-      if (kt + 1 < KT) {
-        n0 = __ldg(a0 + (size_t)(kt + 1) * 32);
-        n1 = __ldg(a1 + (size_t)(kt + 1) * 32);
-      }
-      uint32_t h0[4], l0[4], h1[4], l1[4];
-      tf32_split(c0.x, h0[0], l0[0]); tf32_split(c0.y, h0[1], l0[1]);
-      tf32_split(c0.z, h0[2], l0[2]); tf32_split(c0.w, h0[3], l0[3]);
-      tf32_split(c1.x, h1[0], l1[0]); tf32_split(c1.y, h1[1], l1[1]);
-      tf32_split(c1.z, h1[2], l1[2]); tf32_split(c1.w, h1[3], l1[3]);
-      const float* bk = b + kt * 8 * PB;
-#pragma unroll
-      for (int n = 0; n < 4; ++n) {
-        uint32_t bh0, bl0, bh1, bl1;
-        tf32_split(bk[n * 8], bh0, bl0);
-        tf32_split(bk[n * 8 + 4 * PB], bh1, bl1);
-        mma_tf32(acc[0][n], l0, bh0, bh1);
-        mma_tf32(acc[1][n], l1, bh0, bh1);
-        mma_tf32(acc[0][n], h0, bl0, bl1);
-        mma_tf32(acc[1][n], h1, bl0, bl1);
-        mma_tf32(acc[0][n], h0, bh0, bh1);
-        mma_tf32(acc[1][n], h1, bh0, bh1);
-      }
-    }
+  const int ue = (x.size(0) + 31) / 32, un = ue + (x.size(1) + 31) / 32;
+  for (int un0 = wm + WM * part; un0 < un; un0 += WM * parts) {
+    const int odd = un0 >= ue, M = x.size(odd), KT = x.pad(odd) / 8, m0 = 2 * (odd ? un0 - ue : un0);
+    const bool two = m0 * 16 + 16 < M;
+    const size_t tile = (size_t)m0 * KT + (odd ? (size_t)((x.size(0) + 15) / 16) * (x.pad(0) / 8) : 0);
+    const float4* const a[2] = {A + tile * 32 + lane, A + (tile + (two ? KT : 0)) * 32 + lane};
+    float acc[2][4][4] = {};
+    sep_mma<WN, 2>(acc, a, KT, sB + (t + (odd ? x.pad(0) : 0)) * PB + wn * 32 + g);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int row = (m0 + h) * 16 + g;
-      if (h == 1 && !two) break;
 #pragma unroll
       for (int n = 0; n < 4; ++n) {
         const int col = wn * 32 + n * 8 + 2 * t;
-        if (row < M) put(row, col, acc[h][n][0], acc[h][n][1]);
-        if (row + 8 < M) put(row + 8, col, acc[h][n][2], acc[h][n][3]);
+        if (row < M) put(x.fold ? 2 * row + odd : row, col, acc[h][n][0], acc[h][n][1]);
+        if (row + 8 < M) put(x.fold ? 2 * row + 16 + odd : row + 8, col, acc[h][n][2], acc[h][n][3]);
+      }
+    }
+  }
+}
+// Back along a folded axis: 16 cells and their mirror images a unit, the even
+// modes' sum plus and minus the odd ones'.
+template <int WN, typename Put>
+__device__ __forceinline__ void sep_gemm_back(const float4* __restrict__ A, const SepAxis& x, const float* sB, int part, int parts,
+                                              Put put) {
+  if (!x.fold) return sep_gemm<WN>(A, x, sB, part, parts, put);
+  constexpr int PB = SEP_PITCH<float, WN>, WM = 8 / WN;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int g = lane >> 2, t = lane & 3, wm = warp / WN, wn = warp % WN;
+  const int Me = x.size(0), Mo = x.size(1), KE = x.pad(0) / 8, KO = x.pad(1) / 8;
+  const float* b = sB + t * PB + wn * 32 + g;
+  for (int m = wm + WM * part; m * 16 < Me; m += WM * parts) {
+    float e[1][4][4] = {}, o[1][4][4] = {};
+    const float4* const ae[1] = {A + (size_t)m * KE * 32 + lane};
+    sep_mma<WN, 1>(e, ae, KE, b);
+    if (m * 16 < Mo) {
+      const float4* const ao[1] = {A + ((size_t)((Me + 15) / 16) * KE + (size_t)m * KO) * 32 + lane};
+      sep_mma<WN, 1>(o, ao, KO, b + x.pad(0) * PB);
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int row = m * 16 + g + 8 * h;
+#pragma unroll
+      for (int n = 0; n < 4; ++n) {
+        const int col = wn * 32 + n * 8 + 2 * t;
+        const float e0 = e[0][n][2 * h], e1 = e[0][n][2 * h + 1], o0 = o[0][n][2 * h], o1 = o[0][n][2 * h + 1];
+        if (row < Me) put(row, col, e0 + o0, e1 + o1);
+        if (row < Mo) put(x.n - 1 - row, col, e0 - o0, e1 - o1);
       }
     }
   }
 }
 
 // FP64: lane l owns columns 2 (l % 16), + 1 and rows 2 (l / 16), + 1 of its
-// warp's four (A: column by column, MP rows each).
-template <int WN, typename Put>
-__device__ __forceinline__ void sep_gemm(const double* __restrict__ A, int M, int K, const double* sB, int part, int parts,
-                                         Put put) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, col = 2 * (lane & 15), MP = (M + 1) & ~1;
-  for (int r0 = 4 * warp + 32 * part; r0 < M; r0 += 32 * parts) {
-    const int row = r0 + 2 * (lane >> 4);
-    const double* a = A + (row < M ? row : 0);
-    double c00 = 0, c01 = 0, c10 = 0, c11 = 0;
+// unit's four (A: column by column, an even number of rows each).
+__device__ __forceinline__ void sep_fma(double (&c)[4], const double* __restrict__ A, int row, int M, const double* b) {
+  const int MP = (M + 1) & ~1;
+  const double* a = A + (row < M ? row : 0);
 #pragma unroll 4
-    for (int k = 0; k < K; ++k) {
-      const double2 av = __ldg(reinterpret_cast<const double2*>(a + (size_t)k * MP));
-      const double2 bv = *reinterpret_cast<const double2*>(sB + k * 32 + col);
-      c00 = fma(av.x, bv.x, c00);
-      c01 = fma(av.x, bv.y, c01);
-      c10 = fma(av.y, bv.x, c10);
-      c11 = fma(av.y, bv.y, c11);
+  for (int k = 0; k < M; ++k) {
+    const double2 av = __ldg(reinterpret_cast<const double2*>(a + (size_t)k * MP));
+    const double2 bv = *reinterpret_cast<const double2*>(b + k * 32);
+    c[0] = fma(av.x, bv.x, c[0]);
+    c[1] = fma(av.x, bv.y, c[1]);
+    c[2] = fma(av.y, bv.x, c[2]);
+    c[3] = fma(av.y, bv.y, c[3]);
+  }
+}
+__device__ __forceinline__ size_t sep_mat64(int n) { return (size_t)n * ((n + 1) & ~1); }
+template <int WN, typename Put>
+__device__ __forceinline__ void sep_gemm(const double* __restrict__ A, const SepAxis& x, const double* sB, int part, int parts,
+                                         Put put) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, col = 2 * (lane & 15);
+  const int ue = (x.size(0) + 3) / 4, un = ue + (x.size(1) + 3) / 4;
+  for (int u = warp + 8 * part; u < un; u += 8 * parts) {
+    const int odd = u >= ue, M = x.size(odd), row = 4 * (odd ? u - ue : u) + 2 * (lane >> 4);
+    double c[4] = {};
+    sep_fma(c, A + (odd ? sep_mat64(x.size(0)) : 0), row, M, sB + (odd ? x.pad(0) * 32 : 0) + col);
+    if (row < M) put(x.fold ? 2 * row + odd : row, col, c[0], c[1]);
+    if (row + 1 < M) put(x.fold ? 2 * row + 2 + odd : row + 1, col, c[2], c[3]);
+  }
+}
+template <int WN, typename Put>
+__device__ __forceinline__ void sep_gemm_back(const double* __restrict__ A, const SepAxis& x, const double* sB, int part, int parts,
+                                              Put put) {
+  if (!x.fold) return sep_gemm<WN>(A, x, sB, part, parts, put);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, col = 2 * (lane & 15);
+  const int Me = x.size(0), Mo = x.size(1);
+  for (int u = warp + 8 * part; 4 * u < Me; u += 8 * parts) {
+    const int row = 4 * u + 2 * (lane >> 4);
+    double e[4] = {}, o[4] = {};
+    sep_fma(e, A, row, Me, sB + col);
+    if (row < Mo) sep_fma(o, A + sep_mat64(Me), row, Mo, sB + x.pad(0) * 32 + col);   // (no odd mode reaches the middle cell)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (row + h < Me) put(row + h, col, e[2 * h] + o[2 * h], e[2 * h + 1] + o[2 * h + 1]);
+      if (row + h < Mo) put(x.n - 1 - row - h, col, e[2 * h] - o[2 * h], e[2 * h + 1] - o[2 * h + 1]);
     }
-    if (row < M) put(row, col, c00, c01);
-    if (row + 1 < M) put(row + 1, col, c10, c11);
+  }
+}
+
+// The panel of a transform, 16 bytes a thread: columns col0 .., rows row0,
+// row0 + step, ...  get(i) reads cell (or mode) i of the axis.  Forward, a
+// folded axis stores the sums and then the differences of mirrored cells;
+// back, its even modes and then its odd ones.
+template <typename T, int PB, typename Get>
+__device__ __forceinline__ void sep_panel(T* sm, const SepAxis& x, int row0, int step, int col0, Get get) {
+  using V = SepVec<T>;
+  const int pe = x.pad(0), po = x.pad(1);
+#pragma unroll 2
+  for (int k = row0; k < pe; k += step) {
+    V a = {}, b = {};
+    if (k < x.size(0)) a = get(k);
+    if (k < x.size(1)) {
+      b = get(x.n - 1 - k);
+#pragma unroll
+      for (int e = 0; e < V::N; ++e) {
+        const T s = a.e[e] + b.e[e], d = a.e[e] - b.e[e];
+        a.e[e] = s;
+        b.e[e] = d;
+      }
+    }
+    *reinterpret_cast<V*>(sm + k * PB + col0) = a;
+    if (k < po) *reinterpret_cast<V*>(sm + (pe + k) * PB + col0) = b;
+  }
+}
+template <typename T, int PB, typename Get>
+__device__ __forceinline__ void sep_panel_back(T* sm, const SepAxis& x, int row0, int step, int col0, Get get) {
+  using V = SepVec<T>;
+  const int pe = x.pad(0), rows = x.rows();
+#pragma unroll 4
+  for (int k = row0; k < rows; k += step) {
+    const int odd = k >= pe, m = odd ? k - pe : k;
+    V v = {};
+    if (m < x.size(odd)) v = get(x.fold ? 2 * m + odd : m);
+    *reinterpret_cast<V*>(sm + k * PB + col0) = v;
   }
 }
 
@@ -240,34 +367,35 @@ __device__ __forceinline__ void sep_zf_body(const Level<T>& L, const Sep<T>& S, 
   const T alpha = CG ? (T)st->alpha : T(0);
   const T* dn = (it0 & 1) ? d0 : d1;
   DotAcc<T> dacc;
-  const int KP = flat ? 1 : (L.nz + 7) / 8 * 8;
-#pragma unroll 2
-  for (int k = row0; k < KP; k += SEP_T / VR) {
+  auto get = [&](int k) {
     V v = {};
-    if (in && k < L.nz) {
-      const size_t o = (size_t)k * PS + c;
-      v = *reinterpret_cast<const V*>(L.r + o);
-      if (CG) {
-        const V qv = *reinterpret_cast<const V*>(q + o);
-        const V dv = *reinterpret_cast<const V*>(dn + o);
-        V xv = *reinterpret_cast<const V*>(x + o);
+    if (!in) return v;
+    const size_t o = (size_t)k * PS + c;
+    v = *reinterpret_cast<const V*>(L.r + o);
+    if (CG) {
+      const V qv = *reinterpret_cast<const V*>(q + o);
+      const V dv = *reinterpret_cast<const V*>(dn + o);
+      V xv = *reinterpret_cast<const V*>(x + o);
 #pragma unroll
-        for (int e = 0; e < V::N; ++e) {
-          v.e[e] = e < left_x ? v.e[e] - alpha * qv.e[e] : T(0);
-          xv.e[e] = e < left_x ? xv.e[e] + alpha * dv.e[e] : T(0);
-          dacc.add(v.e[e], v.e[e]);
-        }
-        *reinterpret_cast<V*>(L.r + o) = v;
-        *reinterpret_cast<V*>(x + o) = xv;
+      for (int e = 0; e < V::N; ++e) {
+        v.e[e] = e < left_x ? v.e[e] - alpha * qv.e[e] : T(0);
+        xv.e[e] = e < left_x ? xv.e[e] + alpha * dv.e[e] : T(0);
+        dacc.add(v.e[e], v.e[e]);
       }
+      *reinterpret_cast<V*>(L.r + o) = v;
+      *reinterpret_cast<V*>(x + o) = xv;
     }
-    if (!flat) *reinterpret_cast<V*>(sep_sm + k * PB + col0) = v;
-    else if (in) *reinterpret_cast<V*>(S.t + c) = v;
-  }
-  if (!flat) {
+    return v;
+  };
+  if (flat) {
+    const V v = get(0);
+    if (in) *reinterpret_cast<V*>(S.t + c) = v;
+  } else {
+    const SepAxis ax = sep_axis_z(L);
+    sep_panel<T, PB>(sep_sm, ax, row0, SEP_T / VR, col0, get);
     __syncthreads();
     const size_t cb = (size_t)vb.x * BN;
-    sep_gemm<WN>(S.zf, L.nz, L.nz, sep_sm, 0, 1, [&](int row, int col, T a, T b) {
+    sep_gemm<WN>(S.zf, ax, sep_sm, 0, 1, [&](int row, int col, T a, T b) {
       if (cb + col < PS) sep_put2(S.t + (size_t)row * PS + cb + col, a, b);
     });
   }
@@ -313,16 +441,15 @@ __device__ __forceinline__ void sep_zi_body(const Level<T>& L, const Sep<T>& S, 
       for (int e = 0; e < V::N; e += 2) put(c + e, v.e[e], v.e[e + 1]);
     }
   } else {
-    const int KP = (L.nz + 7) / 8 * 8;
-#pragma unroll 4
-    for (int k = threadIdx.x / VR; k < KP; k += SEP_T / VR) {
+    const SepAxis ax = sep_axis_z(L);
+    sep_panel_back<T, PB>(sep_sm, ax, threadIdx.x / VR, SEP_T / VR, col0, [&](int k) {
       V v = {};
-      if (c < PS && k < L.nz) v = *reinterpret_cast<const V*>(S.t + (size_t)k * PS + c);
-      *reinterpret_cast<V*>(sep_sm + k * PB + col0) = v;
-    }
+      if (c < PS) v = *reinterpret_cast<const V*>(S.t + (size_t)k * PS + c);
+      return v;
+    });
     __syncthreads();
     const size_t cb = (size_t)vb.x * BN;
-    sep_gemm<WN>(S.zi, L.nz, L.nz, sep_sm, 0, 1, [&](int row, int col, T a, T b) {
+    sep_gemm_back<WN>(S.zi, ax, sep_sm, 0, 1, [&](int row, int col, T a, T b) {
       if (cb + col < PS) put((size_t)row * PS + cb + col, a, b);
     });
   }
@@ -341,37 +468,42 @@ __device__ __forceinline__ void sep_zi_body(const Level<T>& L, const Sep<T>& S, 
 // One panel of 32 WN columns of a z plane, every y; blocks vb.y of `split`
 // share the panel's result rows.
 template <int WN, typename T>
-__device__ __forceinline__ void sep_y_panel(const Level<T>& L, const typename Sep<T>::Mat* A, const T* __restrict__ src,
-                                            T* __restrict__ dst, int split, const VBlock& vb) {
+__device__ __forceinline__ void sep_y_panel(const Level<T>& L, const Sep<T>& S, int inverse, int split, const VBlock& vb) {
   extern __shared__ __align__(16) unsigned char sep_raw[];
   T* sep_sm = reinterpret_cast<T*>(sep_raw);
   using V = SepVec<T>;
   constexpr int BN = 32 * WN, PB = SEP_PITCH<T, WN>, VR = BN / V::N;
-  const int x0 = vb.x * BN, xv = V::N * (threadIdx.x % VR);
+  const SepAxis ax = sep_axis_y(L);
+  const int x0 = vb.x * BN, xv = V::N * (threadIdx.x % VR), row0 = threadIdx.x / VR;
   const size_t base = (size_t)vb.z * L.P * L.ny + x0;
   const bool in = x0 + xv < L.P;
-  const int KP = (L.ny + 7) / 8 * 8;
-#pragma unroll 4
-  for (int j = threadIdx.x / VR; j < KP; j += SEP_T / VR) {
+  const T* __restrict__ src = (inverse ? S.u : S.t) + base;
+  T* __restrict__ dst = (inverse ? S.t : S.u) + base;
+  auto get = [&](int j) {
     V v = {};
-    if (in && j < L.ny) v = *reinterpret_cast<const V*>(src + base + (size_t)j * L.P + xv);
-    *reinterpret_cast<V*>(sep_sm + j * PB + xv) = v;
+    if (in) v = *reinterpret_cast<const V*>(src + (size_t)j * L.P + xv);
+    return v;
+  };
+  auto put = [&](int row, int col, T a, T b) {
+    if (x0 + col < L.P) sep_put2(dst + (size_t)row * L.P + col, a, b);
+  };
+  if (inverse) {
+    sep_panel_back<T, PB>(sep_sm, ax, row0, SEP_T / VR, xv, get);
+    __syncthreads();
+    sep_gemm_back<WN>(S.yi, ax, sep_sm, vb.y, split, put);
+  } else {
+    sep_panel<T, PB>(sep_sm, ax, row0, SEP_T / VR, xv, get);
+    __syncthreads();
+    sep_gemm<WN>(S.yf, ax, sep_sm, vb.y, split, put);
   }
-  __syncthreads();
-  sep_gemm<WN>(A, L.ny, L.ny, sep_sm, vb.y, split, [&](int row, int col, T a, T b) {
-    if (x0 + col < L.P) sep_put2(dst + base + (size_t)row * L.P + col, a, b);
-  });
 }
 template <typename T>
 __device__ __forceinline__ void sep_y_body(const Level<T>& L, const Sep<T>& S, int inverse, const SolveState* st,
                                            const VBlock& vb) {
   if (st->converged) return;
-  const auto* A = inverse ? S.yi : S.yf;
-  const T* src = inverse ? S.u : S.t;
-  T* dst = inverse ? S.t : S.u;
   const int split = sep_y_split<T>(L.P, L.ny, L.nz);
-  if (sizeof(T) == 4 && L.ny <= SEP_Y_WIDE) sep_y_panel<sizeof(T) == 4 ? 2 : 1>(L, A, src, dst, split, vb);
-  else sep_y_panel<1>(L, A, src, dst, split, vb);
+  if (sizeof(T) == 4 && L.ny <= SEP_Y_WIDE) sep_y_panel<sizeof(T) == 4 ? 2 : 1>(L, S, inverse, split, vb);
+  else sep_y_panel<1>(L, S, inverse, split, vb);
 }
 
 // -------------------------------------------------------------- x solve --
@@ -516,27 +648,34 @@ __device__ __forceinline__ double sep_eig(int m, int n, bool out_lo, bool out_hi
   const double s = (!out_lo && !out_hi) ? sinpi(m / (2.0 * n)) : sinpi((2 * m + 1) / (2.0 * (2 * n + 1)));
   return 4.0 * s * s;
 }
-// Matrix of an axis: forward (row mode, column cell) or its transpose.
-__device__ __forceinline__ double sep_entry(int r, int c, int n, int out_lo, int out_hi, int transpose) {
-  if (r >= n || c >= n) return 0.0;
-  return transpose ? sep_mode(c, r, n, out_lo, out_hi) : sep_mode(r, c, n, out_lo, out_hi);
-}
 template <typename T>
-__host__ __device__ inline size_t sep_mat_count(int n) {   // elements of Sep<T>::Mat
+__host__ __device__ inline size_t sep_block_count(int n) {   // elements of Sep<T>::Mat of an n x n matrix
   return sizeof(T) == 4 ? (size_t)((n + 15) / 16) * ((n + 7) / 8) * 32 : (size_t)n * ((n + 1) & ~1);
 }
 template <typename T>
-__global__ void k_sep_pack(typename Sep<T>::Mat* A, int n, int out_lo, int out_hi, int transpose) {
-  const size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (e >= sep_mat_count<T>(n)) return;
+__host__ __device__ inline size_t sep_mat_count(const SepAxis& x) { return sep_block_count<T>(x.size(0)) + sep_block_count<T>(x.size(1)); }
+// Matrices of an axis: forward (row mode, column cell) or transposed.  The
+// halves of a folded axis: modes 0, 2, .. and 1, 3, .. at its first cells.
+template <typename T>
+__global__ void k_sep_pack(typename Sep<T>::Mat* A, SepAxis x, int out_lo, int out_hi, int transpose) {
+  size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (e >= sep_mat_count<T>(x)) return;
+  A += e;
+  const size_t ne = sep_block_count<T>(x.size(0));
+  const int odd = e >= ne, m = x.size(odd);
+  if (odd) e -= ne;
+  auto val = [&](int r, int c) {
+    if (r >= m || c >= m) return 0.0;
+    const int mode = transpose ? c : r;
+    return sep_mode(x.fold ? 2 * mode + odd : mode, transpose ? r : c, x.n, out_lo, out_hi);
+  };
   if constexpr (sizeof(T) == 4) {
-    const int KT = (n + 7) / 8, lane = (int)(e & 31), tile = (int)(e >> 5), g = lane >> 2, t = lane & 3;
+    const int KT = (m + 7) / 8, lane = (int)(e & 31), tile = (int)(e >> 5), g = lane >> 2, t = lane & 3;
     const int r0 = (tile / KT) * 16 + g, c0 = (tile % KT) * 8 + t;
-    auto val = [&](int r, int c) { return (float)sep_entry(r, c, n, out_lo, out_hi, transpose); };
-    A[e] = make_float4(val(r0, c0), val(r0 + 8, c0), val(r0, c0 + 4), val(r0 + 8, c0 + 4));
+    *A = make_float4((float)val(r0, c0), (float)val(r0 + 8, c0), (float)val(r0, c0 + 4), (float)val(r0 + 8, c0 + 4));
   } else {
-    const int NP = (n + 1) & ~1;
-    A[e] = sep_entry((int)(e % NP), (int)(e / NP), n, out_lo, out_hi, transpose);
+    const int MP = (m + 1) & ~1;
+    *A = val((int)(e % MP), (int)(e / MP));
   }
 }
 // Reciprocal pivots of the x systems, one line per thread, in FP64.

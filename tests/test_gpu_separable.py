@@ -43,7 +43,9 @@ def direct_solve(b, deg):
 @pytest.mark.parametrize("dims, deg", [((2, 2, 1), 0.0), ((5, 3, 2), 200.0), ((33, 45, 9), 300.0), ((64, 70, 1), 180.0),
                                        ((97, 16, 17), 90.0), ((130, 65, 70), 45.0), ((260, 9, 5), 270.0), ((513, 12, 3), 0.0),
                                        ((1024, 4, 2), 135.0), ((6, 769, 2), 30.0), ((40, 768, 1), 90.0), ((7, 1392, 1), 10.0),
-                                       ((9, 8, 400), 60.0)])
+                                       ((9, 8, 400), 60.0),
+                                       # folded in y too: odd halves, one cell past a 16-row tile, the widest panel
+                                       ((40, 37, 21), 0.0), ((12, 33, 34), 180.0), ((32, 761, 3), 0.0), ((8, 1391, 1), 180.0)])
 @pytest.mark.parametrize("precision", ["f32", "f64"])
 def test_solve_matches_direct(dims, deg, precision):
     nx, ny, nz = dims
