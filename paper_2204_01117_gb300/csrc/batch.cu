@@ -72,7 +72,7 @@ struct LaunchMap {
 // MAP_DIR: the march tiles of the finest level, every instance; the V-cycle
 // maps (MAP_TAIL, MAP_MARCH0 ..) hold the instances that run it, the MAP_SEP
 // ones those with the separable inverse.
-enum MapKind { MAP_CFL = 0, MAP_TURB, MAP_CELL, MAP_FACE, MAP_CHUNK, MAP_TAIL, MAP_ADV, MAP_ADV_FAR, MAP_DIR, MAP_SEPZ, MAP_SEPY, MAP_SEPX, MAP_MARCH0 };
+enum MapKind { MAP_CFL = 0, MAP_TURB, MAP_CELL, MAP_FACE, MAP_CHUNK, MAP_INIT, MAP_TAIL, MAP_ADV, MAP_ADV_FAR, MAP_DIR, MAP_SEPZ, MAP_SEPY, MAP_SEPX, MAP_MARCH0 };
 constexpr int kMaps = MAP_MARCH0 + uf::MAX_LEVELS;
 
 __device__ __forceinline__ int map_entry(const LaunchMap* __restrict__ m, int w) {
@@ -200,6 +200,8 @@ template <typename T>
 struct SepP {    // separable inverse
   uf::Level<T> L;
   uf::Sep<T> S;
+  const T* b;
+  const uf::PStore<T>* g;
   T* x;
   const T *d0, *d1, *q;
   T* z;
@@ -303,12 +305,20 @@ __global__ void __launch_bounds__(uf::FT, 4) kb_mg_up(const __grid_constant__ Ar
   });
 }
 
-template <bool CG, typename T>
-__global__ void __launch_bounds__(uf::SEP_T, 2) kb_sep_zf(const __grid_constant__ Args<SepP<T>> A,
-                                                          cudaGraphConditionalHandle cond, int use_cond, int* left) {
+template <typename T>
+__global__ void __launch_bounds__(uf::SEP_T, 2) kb_sep_init(const __grid_constant__ Args<SepP<T>> A,
+                                                            cudaGraphConditionalHandle cond, int use_cond, int* left) {
   for_items(&A.m, [&](int i, int, const VBlock& vb) {
     const SepP<T>& P = A.at[i];
-    uf::sep_zf_body<CG>(P.L, P.S, P.x, P.d0, P.d1, P.q, P.partials, P.st, cond, use_cond, CG ? left : nullptr, vb);
+    uf::sep_init_body(P.L, P.S, P.b, P.x, P.g, P.partials, P.st, cond, use_cond, left, vb);
+  });
+}
+template <typename T>
+__global__ void __launch_bounds__(uf::SEP_T, 2) kb_sep_update(const __grid_constant__ Args<SepP<T>> A,
+                                                              cudaGraphConditionalHandle cond, int use_cond, int* left) {
+  for_items(&A.m, [&](int i, int, const VBlock& vb) {
+    const SepP<T>& P = A.at[i];
+    uf::sep_update_body(P.L, P.S, P.x, P.d0, P.d1, P.q, P.partials, P.st, cond, use_cond, left, vb);
   });
 }
 template <typename T>
@@ -320,10 +330,10 @@ __global__ void __launch_bounds__(32 * uf::SEP_X_LINES) kb_sep_x(const __grid_co
   for_items(&A.m, [&](int i, int, const VBlock& vb) { uf::sep_x_body(A.at[i].L, A.at[i].S, A.at[i].st, vb); });
 }
 template <typename T>
-__global__ void __launch_bounds__(uf::SEP_T, 2) kb_sep_zi(const __grid_constant__ Args<SepP<T>> A, int mode) {
+__global__ void __launch_bounds__(uf::SEP_T, 2) kb_sep_zi(const __grid_constant__ Args<SepP<T>> A) {
   for_items(&A.m, [&](int i, int, const VBlock& vb) {
     const SepP<T>& P = A.at[i];
-    uf::sep_zi_body(P.L, P.S, P.z, mode, P.partials, P.st, vb);
+    uf::sep_zi_body(P.L, P.S, P.z, P.partials, P.st, vb);
   });
 }
 
@@ -500,6 +510,7 @@ class BatchImpl final : public uf_batch {
         sepy_smem = std::max(sepy_smem, uf::sep_smem<T>(wn, uf::sep_axis_y(G.lv[0])));
         continue;
       }
+      add_entry(maps[MAP_INIT], i, G.chunk_g[0], G.chunk_g[1], G.chunk_g[2], G.chunk_zc);
       add_entry(maps[MAP_TAIL], i, 1, 1, 1, 0);
       for (int l = 0; l < G.tail_level; ++l)
         add_entry(maps[MAP_MARCH0 + l], i, G.march_g[l][0], G.march_g[l][1], G.march_g[l][2], G.march_zc[l]);
@@ -678,46 +689,46 @@ class BatchImpl final : public uf_batch {
     }
   }
 
-  // The instances with the separable inverse (capi.cu, rec_sep).
-  void rec_sep(cudaStream_t s, int mode, cudaGraphConditionalHandle cond, int use_cond) {
+  // The instances with the separable inverse (capi.cu, rec_sep_first and rec_sep_rest).
+  static void fill_sep(SepP<T>& P, const View<T>& G) {
+    P.L = G.lv[0];
+    P.S = G.sep;
+    P.b = G.b; P.g = G.gd;
+    P.x = G.p; P.d0 = G.d0; P.d1 = G.d1; P.q = G.q; P.z = G.z;
+    P.partials = G.partials;
+    P.st = G.st;
+  }
+  void rec_sep_first(cudaStream_t s, bool update, cudaGraphConditionalHandle cond, int use_cond) {
     if (items(MAP_SEPZ) == 0) return;
-    auto fill = [](SepP<T>& P, const View<T>& G) {
-      P.L = G.lv[0];
-      P.S = G.sep;
-      P.x = G.p; P.d0 = G.d0; P.d1 = G.d1; P.q = G.q; P.z = G.z;
-      P.partials = G.partials;
-      P.st = G.st;
-    };
     const int t = uf::SEP_T;
-    const auto& A = args<SepP<T>>(MAP_SEPZ, fill);
-    auto zf = kb_sep_zf<false, T>;
-    auto zfc = kb_sep_zf<true, T>;
-    if (mode == 1)
-      L(s, "b_sep_zf_cg", plane_bytes(MAP_SEPZ, 7),
-        [&] { zfc<<<grid_of(zfc, t, sepz_smem, items(MAP_SEPZ)), t, sepz_smem, s>>>(A, cond, use_cond, d_left); });
-    else
-      L(s, "b_sep_zf", plane_bytes(MAP_SEPZ, 2),
-        [&] { zf<<<grid_of(zf, t, sepz_smem, items(MAP_SEPZ)), t, sepz_smem, s>>>(A, cond, 0, nullptr); });
+    const auto& A = args<SepP<T>>(MAP_SEPZ, fill_sep);
+    auto k = update ? kb_sep_update<T> : kb_sep_init<T>;
+    L(s, update ? "b_sep_update" : "b_sep_init", plane_bytes(MAP_SEPZ, update ? 7 : 6),
+      [&] { k<<<grid_of(k, t, sepz_smem, items(MAP_SEPZ)), t, sepz_smem, s>>>(A, cond, use_cond, d_left); });
+  }
+  void rec_sep_rest(cudaStream_t s) {
+    if (items(MAP_SEPZ) == 0) return;
+    const int t = uf::SEP_T;
     for (int inv = 0; inv < 2; ++inv) {
-      const auto& Ay = args<SepP<T>>(MAP_SEPY, fill);
+      const auto& Ay = args<SepP<T>>(MAP_SEPY, fill_sep);
       auto y = kb_sep_y<T>;
       L(s, "b_sep_y", plane_bytes(MAP_SEPY, 2),
         [&] { y<<<grid_of(y, t, sepy_smem, items(MAP_SEPY)), t, sepy_smem, s>>>(Ay, inv); });
       if (inv) break;
-      const auto& Ax = args<SepP<T>>(MAP_SEPX, fill);
+      const auto& Ax = args<SepP<T>>(MAP_SEPX, fill_sep);
       auto xs = kb_sep_x<T>;
       L(s, "b_sep_x", plane_bytes(MAP_SEPX, 3), [&] {
         xs<<<grid_of(xs, 32 * uf::SEP_X_LINES, 0, items(MAP_SEPX)), 32 * uf::SEP_X_LINES, 0, s>>>(Ax);
       });
     }
-    const auto& Ai = args<SepP<T>>(MAP_SEPZ, fill);
+    const auto& Ai = args<SepP<T>>(MAP_SEPZ, fill_sep);
     auto zi = kb_sep_zi<T>;
     L(s, "b_sep_zi", plane_bytes(MAP_SEPZ, 3),
-      [&] { zi<<<grid_of(zi, t, sepz_smem, items(MAP_SEPZ)), t, sepz_smem, s>>>(Ai, mode); });
+      [&] { zi<<<grid_of(zi, t, sepz_smem, items(MAP_SEPZ)), t, sepz_smem, s>>>(Ai); });
   }
 
   void vcycle(cudaStream_t s, int mode, cudaGraphConditionalHandle cond, int use_cond) {
-    rec_sep(s, mode, cond, use_cond);
+    if (mode == 1) rec_sep_first(s, true, cond, use_cond);
     if (items(MAP_TAIL) == 0) return;
     if (smoother == UF_SMOOTH_RBGS) rec_vcycle<uf::SM_RBGS>(s, mode, cond, use_cond);
     else rec_vcycle<uf::SM_JACOBI>(s, mode, cond, use_cond);
@@ -799,17 +810,20 @@ class BatchImpl final : public uf_batch {
         [&] { k<<<grid_of(k, uf::MT, sm, items(MAP_CHUNK)), uf::MT, sm, s>>>(A); });
     }
     L(s, "b_begin_solve", 0, [&] { kb_begin_solve<<<1, 32, 0, s>>>(d_left, n); });
-    {
+    if (items(MAP_INIT) > 0) {
       auto k = kb_cg_init<T>;
-      const auto& A = args<CgP<T>>(MAP_CHUNK, [](CgP<T>& P, const View<T>& G) { P = cg_params(G); });
-      L(s, "b_cg_init", plane_bytes(MAP_CHUNK, 5),
-        [&] { k<<<grid_of(k, uf::NT, 0, items(MAP_CHUNK)), blk, 0, s>>>(A, cond, use_cond, d_left); });
+      const auto& A = args<CgP<T>>(MAP_INIT, [](CgP<T>& P, const View<T>& G) { P = cg_params(G); });
+      L(s, "b_cg_init", plane_bytes(MAP_INIT, 5),
+        [&] { k<<<grid_of(k, uf::NT, 0, items(MAP_INIT)), blk, 0, s>>>(A, cond, use_cond, d_left); });
     }
+    rec_sep_first(s, false, cond, use_cond);
     vcycle(s, 0, cond, use_cond);
   }
 
-  // one CG iteration: direction + A d, then the V-cycle with the CG update
+  // one CG iteration: what is left of the separable inverse, direction + A d,
+  // then the V-cycle or the inverse's first transform with the CG update
   void rec_iter(cudaStream_t s, cudaGraphConditionalHandle cond, int use_cond) {
+    rec_sep_rest(s);
     auto k = kb_cg_dir_q<T>;
     const auto& A = args<CgP<T>>(MAP_DIR, [](CgP<T>& P, const View<T>& G) { P = cg_params(G); });
     L(s, "b_cg_dir_q", plane_bytes(MAP_DIR, 4),
@@ -991,10 +1005,8 @@ class BatchImpl final : public uf_batch {
       UFB_CUDA(lim_static((const void*)kb_advect_fused<T, false>));
       UFB_CUDA(lim_static((const void*)kb_advect_fused<T, true>));
       UFB_CUDA(lim_static((const void*)kb_momentum_fused<T>));
-      auto zf = kb_sep_zf<false, T>;
-      auto zfc = kb_sep_zf<true, T>;
-      UFB_CUDA(lim_static((const void*)zf));
-      UFB_CUDA(lim_static((const void*)zfc));
+      UFB_CUDA(lim_static((const void*)kb_sep_init<T>));
+      UFB_CUDA(lim_static((const void*)kb_sep_update<T>));
       UFB_CUDA(lim_static((const void*)kb_sep_zi<T>));
       UFB_CUDA(lim_static((const void*)kb_sep_y<T>));
       UFB_CUDA(cudaStreamSynchronize(stream));

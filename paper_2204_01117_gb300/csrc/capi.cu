@@ -611,8 +611,8 @@ class GridImpl final : public uf_grid {
     lim((const void*)uf::k_mg_coarse<T, uf::SM_JACOBI>);
     lim((const void*)uf::k_mg_coarse<T, uf::SM_RBGS>);
     if (P.sep) {
-      lim((const void*)uf::k_sep_zf<false, T>);
-      lim((const void*)uf::k_sep_zf<true, T>);
+      lim((const void*)uf::k_sep_init<T>);
+      lim((const void*)uf::k_sep_update<T>);
       lim((const void*)uf::k_sep_zi<T>);
       lim((const void*)uf::k_sep_y<T>);
     }
@@ -801,27 +801,35 @@ class GridImpl final : public uf_grid {
   // The separable inverse takes the V-cycle's place wherever it is available
   // and the V-cycle's launches were not asked for (uf_tuning.coarse_start).
   bool use_sep() const { return sep.on && coarse_start_tuned == 0; }
-  void rec_sep(cudaStream_t s, int mode, cudaGraphConditionalHandle cond, int use_cond) {
+  // Its z transform closes an iteration (with the CG update and the
+  // convergence test, so an unconverged residual is already transformed) and
+  // the rest opens the next one: the loop ends without launches that find
+  // nothing to do (four of 2 us each where the whole inverse followed the
+  // update).
+  void rec_sep_first(cudaStream_t s, bool update, cudaGraphConditionalHandle cond, int use_cond) {
+    const unsigned gz = uf::sep_z_blocks<T>(lv[0].P, d.ny, d.nz);
+    const size_t sz = uf::sep_smem<T>(uf::SEP_Z_WN<T>, uf::sep_axis_z(lv[0]));
+    if (update)
+      L(s, "sep_update", 7 * N() * tb(), [&] {
+        uf::k_sep_update<T><<<gz, uf::SEP_T, sz, s>>>(lv[0], sep, sol_x, d0, d1, q, partials, st, cond, use_cond);
+      });
+    else
+      L(s, "sep_init", N() * (4 * tb() + (sol_g ? 2 * tb() : 0.0)), [&] {
+        uf::k_sep_init<T><<<gz, uf::SEP_T, sz, s>>>(lv[0], sep, sol_b, sol_x, sol_g, partials, st, cond, use_cond);
+      });
+  }
+  void rec_sep_rest(cudaStream_t s) {
     const int wn = uf::sep_y_wn<T>(d.ny), by = 32 * wn;
     const unsigned gz = uf::sep_z_blocks<T>(lv[0].P, d.ny, d.nz);
     const size_t sz = uf::sep_smem<T>(uf::SEP_Z_WN<T>, uf::sep_axis_z(lv[0])), sy = uf::sep_smem<T>(wn, uf::sep_axis_y(lv[0]));
     const dim3 gy((lv[0].P + by - 1) / by, uf::sep_y_split<T>(lv[0].P, d.ny, d.nz), d.nz);
     const unsigned gx = (unsigned)((d.ny * d.nz + uf::SEP_X_LINES - 1) / uf::SEP_X_LINES);
-    if (mode == 1)
-      L(s, "sep_zf_cg", 7 * N() * tb(), [&] {
-        uf::k_sep_zf<true, T><<<gz, uf::SEP_T, sz, s>>>(lv[0], sep, sol_x, d0, d1, q, partials, st, cond, use_cond);
-      });
-    else
-      L(s, "sep_zf", 2 * N() * tb(), [&] {
-        uf::k_sep_zf<false, T><<<gz, uf::SEP_T, sz, s>>>(lv[0], sep, nullptr, nullptr, nullptr, nullptr, partials, st, cond, 0);
-      });
     L(s, "sep_y", 2 * N() * tb(), [&] { uf::k_sep_y<T><<<gy, uf::SEP_T, sy, s>>>(lv[0], sep, 0, st); });
     L(s, "sep_x", 3 * N() * tb(), [&] { uf::k_sep_x<T><<<gx, 32 * uf::SEP_X_LINES, 0, s>>>(lv[0], sep, st); });
     L(s, "sep_y", 2 * N() * tb(), [&] { uf::k_sep_y<T><<<gy, uf::SEP_T, sy, s>>>(lv[0], sep, 1, st); });
-    L(s, "sep_zi", 3 * N() * tb(), [&] { uf::k_sep_zi<T><<<gz, uf::SEP_T, sz, s>>>(lv[0], sep, z, mode, partials, st); });
+    L(s, "sep_zi", 3 * N() * tb(), [&] { uf::k_sep_zi<T><<<gz, uf::SEP_T, sz, s>>>(lv[0], sep, z, partials, st); });
   }
   void rec_vcycle(cudaStream_t s, int mode, cudaGraphConditionalHandle cond, int use_cond) {
-    if (use_sep()) return rec_sep(s, mode, cond, use_cond);
     if (d.mg_smoother == UF_SMOOTH_RBGS) rec_vcycle_sm<uf::SM_RBGS>(s, mode, cond, use_cond);
     else rec_vcycle_sm<uf::SM_JACOBI>(s, mode, cond, use_cond);
   }
@@ -847,11 +855,13 @@ class GridImpl final : public uf_grid {
   }
 
   void rec_setup_precond(cudaStream_t s, cudaGraphConditionalHandle cond, int use_cond) {
+    if (use_sep()) return;   // (rec_cg_init)
     if (d.precond == UF_PRECOND_MG) rec_vcycle(s, 0, 0, 0);
     else rec_precond(s, 0, cond, use_cond);
   }
 
   void rec_cg_init(cudaStream_t s, cudaGraphConditionalHandle cond, int use_cond) {
+    if (use_sep()) return rec_sep_first(s, false, cond, use_cond);
     int zc;
     dim3 g = chunk_grid(lv[0].nx, lv[0].ny, lv[0].nz, &zc);
     L(s, "cg_init", N() * (3 * tb() + (sol_g ? 2 * tb() : 0.0)), [&] {
@@ -863,10 +873,12 @@ class GridImpl final : public uf_grid {
     if (d.precond == UF_PRECOND_MG) {
       int zc;
       const dim3 g = march_grid(0, &zc);
+      if (use_sep()) rec_sep_rest(s);
       L(s, "cg_dir_q", 4 * N() * tb(), [&] {
         uf::k_cg_dir_q<T><<<g, uf::FT, 0, s>>>(lv[0], zc, z, d0, d1, q, partials, st);
       });
-      rec_vcycle(s, 1, cond, use_cond);
+      if (use_sep()) rec_sep_first(s, true, cond, use_cond);
+      else rec_vcycle(s, 1, cond, use_cond);
       return;
     }
     int zc;

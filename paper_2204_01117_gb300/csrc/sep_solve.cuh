@@ -10,7 +10,7 @@
 // 4 sin^2(theta_m / 2)); what remains is one tridiagonal system along x per
 // pair of modes.  z = A^-1 r is therefore
 //   z transform, y transform, x solve, y transform back, z transform back
-// (k_sep_zf, k_sep_y, k_sep_x, k_sep_y, k_sep_zi).  (Lynch, Rice and Thomas,
+// (k_sep_init or k_sep_update, k_sep_y, k_sep_x, k_sep_y, k_sep_zi).  (Lynch, Rice and Thomas,
 // "Direct solution of partial difference equations by tensor product
 // methods", Numer. Math. 6, 1964.)
 //
@@ -300,11 +300,11 @@ __device__ __forceinline__ void sep_gemm_back(const double* __restrict__ A, cons
 // row0 + step, ...  get(i) reads cell (or mode) i of the axis.  Forward, a
 // folded axis stores the sums and then the differences of mirrored cells;
 // back, its even modes and then its odd ones.
-template <typename T, int PB, typename Get>
+template <typename T, int PB, int UNROLL, typename Get>
 __device__ __forceinline__ void sep_panel(T* sm, const SepAxis& x, int row0, int step, int col0, Get get) {
   using V = SepVec<T>;
   const int pe = x.pad(0), po = x.pad(1);
-#pragma unroll 2
+#pragma unroll UNROLL
   for (int k = row0; k < pe; k += step) {
     V a = {}, b = {};
     if (k < x.size(0)) a = get(k);
@@ -341,81 +341,179 @@ __device__ __forceinline__ double2 sep_get2(const double* o) { return *reinterpr
 
 // ------------------------------------------------------- z transforms ----
 // A panel is 128 consecutive columns (x, y) of the P x ny plane with every z
-// in shared memory, so each cell is read once.  CG = true (inside the CG
-// loop): the panel's load is also the CG update x += alpha d, r -= alpha q
-// with ||r||^2 and the convergence test.  Columns in the row padding
-// (x >= nx) are forced to zero.
-template <bool CG, typename T>
-__device__ __forceinline__ void sep_zf_body(const Level<T>& L, const Sep<T>& S, T* __restrict__ x, const T* d0, const T* d1,
-                                            const T* __restrict__ q, double* partials, SolveState* st,
-                                            cudaGraphConditionalHandle cond, int use_cond, int* left, const VBlock& vb) {
+// in shared memory, so each cell is read once; what the panel holds is formed
+// while it is loaded: the first residual before the CG loop (sep_init_body),
+// the CG update inside it (sep_update_body), with ||r||^2 and the convergence
+// test.  Columns in the row padding (x >= nx) are zero.
+template <typename T>
+struct SepCols {   // a thread's 16 bytes of every row it loads
+  bool flat;       // one cell in z: the identity, a thread per 16 bytes
+  int row0, col0;
+  size_t PS, c;    // cells of a plane, the first column
+  bool in;
+  int left_x;      // how many of the values lie inside the domain
+  static constexpr int VR = 32 * SEP_Z_WN<T> / SepVec<T>::N;
+  __device__ __forceinline__ SepCols(const Level<T>& L, const VBlock& vb) {
+    static_assert(SEP_T % VR == 0, "a thread keeps its columns");
+    flat = L.nz == 1;
+    row0 = flat ? 0 : threadIdx.x / VR;
+    col0 = SepVec<T>::N * (flat ? threadIdx.x : threadIdx.x % VR);
+    PS = (size_t)L.P * L.ny;
+    c = (size_t)vb.x * sep_z_cols<T>(L.nz) + col0;
+    in = c < PS;
+    left_x = L.nx - (int)(c % L.P);
+  }
+};
+// t = Qz (what get gives: 16 bytes of plane k).
+template <int UNROLL, typename T, typename Get>
+__device__ __forceinline__ void sep_zf(const Level<T>& L, const Sep<T>& S, const SepCols<T>& C, const VBlock& vb, Get get) {
   extern __shared__ __align__(16) unsigned char sep_raw[];
   T* sep_sm = reinterpret_cast<T*>(sep_raw);
+  using V = SepVec<T>;
+  constexpr int WN = SEP_Z_WN<T>, PB = SEP_PITCH<T, WN>;
+  if (C.flat) {
+    const V v = get(0);
+    if (C.in) *reinterpret_cast<V*>(S.t + C.c) = v;
+    return;
+  }
+  const SepAxis ax = sep_axis_z(L);
+  sep_panel<T, PB, UNROLL>(sep_sm, ax, C.row0, SEP_T / C.VR, C.col0, get);
+  __syncthreads();
+  const size_t cb = (size_t)vb.x * 32 * WN;
+  sep_gemm<WN>(S.zf, ax, sep_sm, 0, 1, [&](int row, int col, T a, T b) {
+    if (cb + col < C.PS) sep_put2(S.t + (size_t)row * C.PS + cb + col, a, b);
+  });
+}
+
+__device__ __forceinline__ float sep_diff(float2 a, float2 b) { return ps_diff(a, b); }
+__device__ __forceinline__ float sep_diff(float a, float b) { return a - b; }
+__device__ __forceinline__ double sep_diff(double a, double b) { return a - b; }
+__device__ __forceinline__ float sep_value(float2 a) { return ps_value(a); }
+__device__ __forceinline__ float sep_value(float a) { return a; }
+__device__ __forceinline__ double sep_value(double a) { return a; }
+// A f (level_apply) at 16 bytes' worth of cells of plane k; f holds values or
+// the pressure store's pairs, whose differences are taken on the pairs.
+template <typename E, typename T>
+__device__ __forceinline__ SepVec<T> sep_apply(const Level<T>& L, const SepCols<T>& C, const E* __restrict__ f, int k) {
+  constexpr int N = SepVec<T>::N;
+  struct alignas(16) Row { E e[N]; };
+  const int i0 = L.nx - C.left_x, j = (int)(C.c / L.P);
+  f += (size_t)k * C.PS + C.c;
+  const bool y0 = j > 0, y1 = j < L.ny - 1, z0 = k > 0, z1 = k < L.nz - 1;
+  const Row m = *reinterpret_cast<const Row*>(f);
+  Row ym = m, yp = m, zm = m, zp = m;
+  E xm = m.e[0], xp = m.e[N - 1];
+  if (y0) ym = *reinterpret_cast<const Row*>(f - L.P);
+  if (y1) yp = *reinterpret_cast<const Row*>(f + L.P);
+  if (z0) zm = *reinterpret_cast<const Row*>(f - C.PS);
+  if (z1) zp = *reinterpret_cast<const Row*>(f + C.PS);
+  if (i0 > 0) xm = f[-1];
+  if (C.left_x > N) xp = f[N];
+  SepVec<T> a;
+#pragma unroll
+  for (int e = 0; e < N; ++e) {
+    const T v = (T)sep_value(m.e[e]);
+    T s = 0;
+    if (e > 0 || i0 > 0) s += L.wx * (T)sep_diff(m.e[e], e > 0 ? m.e[e - 1] : xm); else if (L.out_mask & 1) s += L.wx * v;
+    if (e < C.left_x - 1) s += L.wx * (T)sep_diff(m.e[e], e < N - 1 ? m.e[e + 1] : xp); else if (L.out_mask & 2) s += L.wx * v;
+    if (y0) s += L.wy * (T)sep_diff(m.e[e], ym.e[e]); else if (L.out_mask & 4) s += L.wy * v;
+    if (y1) s += L.wy * (T)sep_diff(m.e[e], yp.e[e]); else if (L.out_mask & 8) s += L.wy * v;
+    if (z0) s += L.wz * (T)sep_diff(m.e[e], zm.e[e]); else if (L.out_mask & 16) s += L.wz * v;
+    if (z1) s += L.wz * (T)sep_diff(m.e[e], zp.e[e]); else if (L.out_mask & 32) s += L.wz * v;
+    a.e[e] = s;
+  }
+  return a;
+}
+
+// Set-up of the solve: what k_cg_init does for the V-cycle (r = b - A g and a
+// correction x from zero, or r = b - A x), and its z transform, in one pass
+// (256 x 256 x 64: 68 us for the two kernels, 49 for this; 512 x 512 x 128: 345
+// and 307).
+template <typename T>
+__device__ __forceinline__ void sep_init_body(const Level<T>& L, const Sep<T>& S, const T* __restrict__ b, T* __restrict__ x,
+                                              const PStore<T>* __restrict__ g, double* partials, SolveState* st,
+                                              cudaGraphConditionalHandle cond, int use_cond, int* left, const VBlock& vb) {
   __shared__ double sh[32];
   __shared__ bool last;
-  if (st->converged) return;
   using V = SepVec<T>;
-  constexpr int WN = SEP_Z_WN<T>, BN = 32 * WN, PB = SEP_PITCH<T, WN>, VR = BN / V::N;
-  static_assert(SEP_T % VR == 0, "a thread keeps its columns");
-  const size_t PS = (size_t)L.P * L.ny;
-  const bool flat = L.nz == 1;   // one cell in z: the identity, a thread per 16 bytes
-  const int row0 = flat ? 0 : threadIdx.x / VR, col0 = V::N * (flat ? threadIdx.x : threadIdx.x % VR);
-  const size_t c = (size_t)vb.x * sep_z_cols<T>(L.nz) + col0;
-  const bool in = c < PS;
-  const int left_x = L.nx - (int)(c % L.P);   // how many of the values lie inside the domain
-  const int it0 = st->iter;
-  const T alpha = CG ? (T)st->alpha : T(0);
-  const T* dn = (it0 & 1) ? d0 : d1;
+  const SepCols<T> C(L, vb);
+  const bool zero_rhs = st->bb == 0.0;
   DotAcc<T> dacc;
-  auto get = [&](int k) {
+  sep_zf<1>(L, S, C, vb, [&](int k) {
     V v = {};
-    if (!in) return v;
-    const size_t o = (size_t)k * PS + c;
-    v = *reinterpret_cast<const V*>(L.r + o);
-    if (CG) {
-      const V qv = *reinterpret_cast<const V*>(q + o);
-      const V dv = *reinterpret_cast<const V*>(dn + o);
-      V xv = *reinterpret_cast<const V*>(x + o);
+    if (!C.in) return v;
+    const size_t o = (size_t)k * C.PS + C.c;
+    if (!zero_rhs) {
+      const V bv = *reinterpret_cast<const V*>(b + o);
+      const V a = g ? sep_apply(L, C, g, k) : sep_apply(L, C, (const T*)x, k);
 #pragma unroll
       for (int e = 0; e < V::N; ++e) {
-        v.e[e] = e < left_x ? v.e[e] - alpha * qv.e[e] : T(0);
-        xv.e[e] = e < left_x ? xv.e[e] + alpha * dv.e[e] : T(0);
+        v.e[e] = e < C.left_x ? bv.e[e] - a.e[e] : T(0);
         dacc.add(v.e[e], v.e[e]);
       }
-      *reinterpret_cast<V*>(L.r + o) = v;
-      *reinterpret_cast<V*>(x + o) = xv;
     }
+    if (zero_rhs || g) *reinterpret_cast<V*>(x + o) = V{};
+    *reinterpret_cast<V*>(L.r + o) = v;
     return v;
-  };
-  if (flat) {
-    const V v = get(0);
-    if (in) *reinterpret_cast<V*>(S.t + c) = v;
-  } else {
-    const SepAxis ax = sep_axis_z(L);
-    sep_panel<T, PB>(sep_sm, ax, row0, SEP_T / VR, col0, get);
-    __syncthreads();
-    const size_t cb = (size_t)vb.x * BN;
-    sep_gemm<WN>(S.zf, ax, sep_sm, 0, 1, [&](int row, int col, T a, T b) {
-      if (cb + col < PS) sep_put2(S.t + (size_t)row * PS + cb + col, a, b);
-    });
-  }
-  if (CG) {
-    const double vals[1] = {block_sum<SEP_T>(dacc.value(), sh)};
-    if (publish_partials<1>(partials, &st->ticket[3], vals, &last, vb)) {
-      double tot[1];
-      reduce_partials_sum<SEP_T, 1>(partials, tot, sh, vb.n);
-      if (threadIdx.x == 0) {
-        finish_rr(st, tot[0], it0, cond, use_cond, left);
-        st->ticket[3] = 0u;
-      }
+  });
+  const double vals[1] = {block_sum<SEP_T>(dacc.value(), sh)};
+  if (publish_partials<1>(partials, &st->ticket[1], vals, &last, vb)) {
+    double tot[1];
+    reduce_partials_sum<SEP_T, 1>(partials, tot, sh, vb.n);
+    if (threadIdx.x == 0) {
+      finish_init(st, tot[0], zero_rhs, cond, use_cond, left);
+      st->ticket[1] = 0u;
     }
   }
 }
 
-// Back along z: z = Qz^T t, and r.z (CG beta in mode 1).
+// CG update x += alpha d, r -= alpha q and the z transform of the new r.
 template <typename T>
-__device__ __forceinline__ void sep_zi_body(const Level<T>& L, const Sep<T>& S, T* __restrict__ z, int mode, double* partials,
-                                            SolveState* st, const VBlock& vb) {
+__device__ __forceinline__ void sep_update_body(const Level<T>& L, const Sep<T>& S, T* __restrict__ x, const T* d0, const T* d1,
+                                                const T* __restrict__ q, double* partials, SolveState* st,
+                                                cudaGraphConditionalHandle cond, int use_cond, int* left, const VBlock& vb) {
+  __shared__ double sh[32];
+  __shared__ bool last;
+  if (st->converged) return;
+  using V = SepVec<T>;
+  const SepCols<T> C(L, vb);
+  const int it0 = st->iter;
+  const T alpha = (T)st->alpha;
+  const T* dn = (it0 & 1) ? d0 : d1;
+  DotAcc<T> dacc;
+  sep_zf<2>(L, S, C, vb, [&](int k) {
+    V v = {};
+    if (!C.in) return v;
+    const size_t o = (size_t)k * C.PS + C.c;
+    v = *reinterpret_cast<const V*>(L.r + o);
+    const V qv = *reinterpret_cast<const V*>(q + o);
+    const V dv = *reinterpret_cast<const V*>(dn + o);
+    V xv = *reinterpret_cast<const V*>(x + o);
+#pragma unroll
+    for (int e = 0; e < V::N; ++e) {
+      v.e[e] = e < C.left_x ? v.e[e] - alpha * qv.e[e] : T(0);
+      xv.e[e] = e < C.left_x ? xv.e[e] + alpha * dv.e[e] : T(0);
+      dacc.add(v.e[e], v.e[e]);
+    }
+    *reinterpret_cast<V*>(L.r + o) = v;
+    *reinterpret_cast<V*>(x + o) = xv;
+    return v;
+  });
+  const double vals[1] = {block_sum<SEP_T>(dacc.value(), sh)};
+  if (publish_partials<1>(partials, &st->ticket[3], vals, &last, vb)) {
+    double tot[1];
+    reduce_partials_sum<SEP_T, 1>(partials, tot, sh, vb.n);
+    if (threadIdx.x == 0) {
+      finish_rr(st, tot[0], it0, cond, use_cond, left);
+      st->ticket[3] = 0u;
+    }
+  }
+}
+
+// Back along z: z = Qz^T t, and r.z (from the first iteration on also beta).
+template <typename T>
+__device__ __forceinline__ void sep_zi_body(const Level<T>& L, const Sep<T>& S, T* __restrict__ z, double* partials, SolveState* st,
+                                            const VBlock& vb) {
   extern __shared__ __align__(16) unsigned char sep_raw[];
   T* sep_sm = reinterpret_cast<T*>(sep_raw);
   __shared__ double sh[32];
@@ -458,7 +556,7 @@ __device__ __forceinline__ void sep_zi_body(const Level<T>& L, const Sep<T>& S, 
     double tot[1];
     reduce_partials_sum<SEP_T, 1>(partials, tot, sh, vb.n);
     if (threadIdx.x == 0) {
-      finish_rz(st, tot[0], mode);
+      finish_rz(st, tot[0], st->iter > 0);
       st->ticket[0] = 0u;
     }
   }
@@ -492,7 +590,7 @@ __device__ __forceinline__ void sep_y_panel(const Level<T>& L, const Sep<T>& S, 
     __syncthreads();
     sep_gemm_back<WN>(S.yi, ax, sep_sm, vb.y, split, put);
   } else {
-    sep_panel<T, PB>(sep_sm, ax, row0, SEP_T / VR, xv, get);
+    sep_panel<T, PB, 2>(sep_sm, ax, row0, SEP_T / VR, xv, get);
     __syncthreads();
     sep_gemm<WN>(S.yf, ax, sep_sm, vb.y, split, put);
   }
@@ -613,16 +711,22 @@ __device__ __forceinline__ void sep_x_body(const Level<T>& L, const Sep<T>& S, c
 }
 
 // -------------------------------------------------------------- kernels --
-template <bool CG, typename T>
-__global__ void __launch_bounds__(SEP_T, 2) k_sep_zf(Level<T> L, Sep<T> S, T* __restrict__ x, const T* d0, const T* d1,
-                                                     const T* __restrict__ q, double* partials, SolveState* st,
-                                                     cudaGraphConditionalHandle cond, int use_cond) {
-  sep_zf_body<CG>(L, S, x, d0, d1, q, partials, st, cond, use_cond, nullptr, vblock());
+template <typename T>
+__global__ void __launch_bounds__(SEP_T, 2) k_sep_init(Level<T> L, Sep<T> S, const T* __restrict__ b, T* __restrict__ x,
+                                                       const PStore<T>* __restrict__ g, double* partials, SolveState* st,
+                                                       cudaGraphConditionalHandle cond, int use_cond) {
+  sep_init_body(L, S, b, x, g, partials, st, cond, use_cond, nullptr, vblock());
 }
 template <typename T>
-__global__ void __launch_bounds__(SEP_T, 2) k_sep_zi(Level<T> L, Sep<T> S, T* __restrict__ z, int mode, double* partials,
+__global__ void __launch_bounds__(SEP_T, 2) k_sep_update(Level<T> L, Sep<T> S, T* __restrict__ x, const T* d0, const T* d1,
+                                                         const T* __restrict__ q, double* partials, SolveState* st,
+                                                         cudaGraphConditionalHandle cond, int use_cond) {
+  sep_update_body(L, S, x, d0, d1, q, partials, st, cond, use_cond, nullptr, vblock());
+}
+template <typename T>
+__global__ void __launch_bounds__(SEP_T, 2) k_sep_zi(Level<T> L, Sep<T> S, T* __restrict__ z, double* partials,
                                                      SolveState* st) {
-  sep_zi_body(L, S, z, mode, partials, st, vblock());
+  sep_zi_body(L, S, z, partials, st, vblock());
 }
 template <typename T>
 __global__ void __launch_bounds__(SEP_T, 2) k_sep_y(Level<T> L, Sep<T> S, int inverse, const SolveState* st) {

@@ -103,6 +103,17 @@ __device__ __forceinline__ void signal_converged(cudaGraphConditionalHandle cond
 
 // ------------------------------------------------------------ CG kernels --
 
+// Finishes the set-up of a solve: rr = ||r||^2 of the first residual.
+__device__ __forceinline__ void finish_init(SolveState* st, double rr, bool zero_rhs, cudaGraphConditionalHandle cond, int use_cond,
+                                            int* left) {
+  st->rr = rr;
+  st->rr0 = rr;
+  if (zero_rhs || (st->rule == 0 && rr <= st->tol2 * st->bb)) {
+    st->converged = 1;
+    signal_converged(cond, use_cond, left);
+  }
+}
+
 // r = b - A x from the warm start in x.  With g != nullptr the solve is for
 // the correction to the guess g held in the pressure store (the pressure
 // extrapolated in time, see pressure_commit_body) instead: r = b - A g and
@@ -171,12 +182,7 @@ __device__ __forceinline__ void cg_init_body(const Level<T>& L, const T* __restr
     double tot[1];
     reduce_partials_sum<NT, 1>(partials, tot, sh, vb.n);
     if (thread_linear_id() == 0) {
-      st->rr = tot[0];
-      st->rr0 = tot[0];
-      if (zero_rhs || (st->rule == 0 && tot[0] <= st->tol2 * st->bb)) {
-        st->converged = 1;
-        signal_converged(cond, use_cond, left);
-      }
+      finish_init(st, tot[0], zero_rhs, cond, use_cond, left);
       st->ticket[1] = 0u;
     }
   }
