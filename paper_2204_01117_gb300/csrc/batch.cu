@@ -321,9 +321,9 @@ __global__ void __launch_bounds__(uf::SEP_T, 2) kb_sep_update(const __grid_const
     uf::sep_update_body(P.L, P.S, P.x, P.d0, P.d1, P.q, P.partials, P.st, cond, use_cond, left, vb);
   });
 }
-template <typename T>
-__global__ void __launch_bounds__(uf::SEP_T, 2) kb_sep_y(const __grid_constant__ Args<SepP<T>> A, int inverse) {
-  for_items(&A.m, [&](int i, int, const VBlock& vb) { uf::sep_y_body(A.at[i].L, A.at[i].S, inverse, A.at[i].st, vb); });
+template <bool INVERSE, typename T>
+__global__ void __launch_bounds__(uf::SEP_T, 2) kb_sep_y(const __grid_constant__ Args<SepP<T>> A) {
+  for_items(&A.m, [&](int i, int, const VBlock& vb) { uf::sep_y_body<INVERSE>(A.at[i].L, A.at[i].S, A.at[i].st, vb); });
 }
 template <typename T>
 __global__ void __launch_bounds__(32 * uf::SEP_X_LINES) kb_sep_x(const __grid_constant__ Args<SepP<T>> A) {
@@ -711,9 +711,9 @@ class BatchImpl final : public uf_batch {
     const int t = uf::SEP_T;
     for (int inv = 0; inv < 2; ++inv) {
       const auto& Ay = args<SepP<T>>(MAP_SEPY, fill_sep);
-      auto y = kb_sep_y<T>;
+      auto y = inv ? kb_sep_y<true, T> : kb_sep_y<false, T>;
       L(s, "b_sep_y", plane_bytes(MAP_SEPY, 2),
-        [&] { y<<<grid_of(y, t, sepy_smem, items(MAP_SEPY)), t, sepy_smem, s>>>(Ay, inv); });
+        [&] { y<<<grid_of(y, t, sepy_smem, items(MAP_SEPY)), t, sepy_smem, s>>>(Ay); });
       if (inv) break;
       const auto& Ax = args<SepP<T>>(MAP_SEPX, fill_sep);
       auto xs = kb_sep_x<T>;
@@ -1008,7 +1008,10 @@ class BatchImpl final : public uf_batch {
       UFB_CUDA(lim_static((const void*)kb_sep_init<T>));
       UFB_CUDA(lim_static((const void*)kb_sep_update<T>));
       UFB_CUDA(lim_static((const void*)kb_sep_zi<T>));
-      UFB_CUDA(lim_static((const void*)kb_sep_y<T>));
+      auto yf = kb_sep_y<false, T>;
+      auto yi = kb_sep_y<true, T>;
+      UFB_CUDA(lim_static((const void*)yf));
+      UFB_CUDA(lim_static((const void*)yi));
       UFB_CUDA(cudaStreamSynchronize(stream));
       uf_status s = capture();
       if (s != UF_OK) return s;

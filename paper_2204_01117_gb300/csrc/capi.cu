@@ -614,7 +614,8 @@ class GridImpl final : public uf_grid {
       lim((const void*)uf::k_sep_init<T>);
       lim((const void*)uf::k_sep_update<T>);
       lim((const void*)uf::k_sep_zi<T>);
-      lim((const void*)uf::k_sep_y<T>);
+      lim((const void*)uf::k_sep_y<false, T>);
+      lim((const void*)uf::k_sep_y<true, T>);
     }
     return e;
   }
@@ -824,9 +825,9 @@ class GridImpl final : public uf_grid {
     const size_t sz = uf::sep_smem<T>(uf::SEP_Z_WN<T>, uf::sep_axis_z(lv[0])), sy = uf::sep_smem<T>(wn, uf::sep_axis_y(lv[0]));
     const dim3 gy((lv[0].P + by - 1) / by, uf::sep_y_split<T>(lv[0].P, d.ny, d.nz), d.nz);
     const unsigned gx = (unsigned)((d.ny * d.nz + uf::SEP_X_LINES - 1) / uf::SEP_X_LINES);
-    L(s, "sep_y", 2 * N() * tb(), [&] { uf::k_sep_y<T><<<gy, uf::SEP_T, sy, s>>>(lv[0], sep, 0, st); });
+    L(s, "sep_y", 2 * N() * tb(), [&] { uf::k_sep_y<false, T><<<gy, uf::SEP_T, sy, s>>>(lv[0], sep, st); });
     L(s, "sep_x", 3 * N() * tb(), [&] { uf::k_sep_x<T><<<gx, 32 * uf::SEP_X_LINES, 0, s>>>(lv[0], sep, st); });
-    L(s, "sep_y", 2 * N() * tb(), [&] { uf::k_sep_y<T><<<gy, uf::SEP_T, sy, s>>>(lv[0], sep, 1, st); });
+    L(s, "sep_y", 2 * N() * tb(), [&] { uf::k_sep_y<true, T><<<gy, uf::SEP_T, sy, s>>>(lv[0], sep, st); });
     L(s, "sep_zi", 3 * N() * tb(), [&] { uf::k_sep_zi<T><<<gz, uf::SEP_T, sz, s>>>(lv[0], sep, z, partials, st); });
   }
   void rec_vcycle(cudaStream_t s, int mode, cudaGraphConditionalHandle cond, int use_cond) {

@@ -82,8 +82,8 @@ struct Sep {
 // 32 columns (WN = 1); a warp owns 4 rows.
 template <typename T, int WN>
 constexpr int SEP_PITCH = sizeof(T) == 4 ? 32 * WN + 8 : 32;
-// Columns of a y panel in units of 32: two while it fits (n <= 768), else one.
-constexpr int SEP_Y_WIDE = 768;
+// Columns of a y panel in units of 32: two while they fit with a full queue, else one.
+constexpr int SEP_Y_WIDE = 688;
 template <typename T>
 __host__ __device__ inline int sep_y_wn(int ny) { return sizeof(T) == 4 && ny <= SEP_Y_WIDE ? 2 : 1; }
 template <typename T>
@@ -102,7 +102,19 @@ __host__ __device__ inline SepAxis sep_axis_y(const Level<T>& L) { return {L.ny,
 template <typename T>
 __host__ __device__ inline SepAxis sep_axis_z(const Level<T>& L) { return {L.nz, !(L.out_mask & 48)}; }
 template <typename T>
-inline size_t sep_smem(int wn, const SepAxis& x) { return sizeof(T) * (size_t)x.rows() * (sizeof(T) == 4 ? 32 * wn + 8 : 32); }
+__host__ __device__ inline size_t sep_panel_bytes(int wn, const SepAxis& x) {
+  return sizeof(T) * (size_t)x.rows() * (sizeof(T) == 4 ? 32 * wn + 8 : 32);
+}
+// Behind an FP32 panel lies a queue of matrix tiles for each thread, four deep
+// where a block's shared memory (227 KB) allows, else one.
+constexpr int SEP_QUEUE = 4, SEP_SLOT = 2 * 16 * SEP_T;   // bytes of a slot: two tiles, 16 bytes per thread and tile
+__host__ __device__ inline int sep_queue(int wn, const SepAxis& x) {
+  return sep_panel_bytes<float>(wn, x) + SEP_QUEUE * SEP_SLOT + 1024 <= 227 * 1024 ? SEP_QUEUE : 1;
+}
+template <typename T>
+inline size_t sep_smem(int wn, const SepAxis& x) {
+  return sep_panel_bytes<T>(wn, x) + (sizeof(T) == 4 ? (size_t)sep_queue(wn, x) * SEP_SLOT : 0);
+}
 // Columns (x, y) of a z panel, and the blocks that cover the plane.  One cell
 // in z has nothing to transform: the threads just share the columns out.
 template <typename T>
@@ -129,6 +141,22 @@ struct alignas(16) SepVec {
   T e[N];
 };
 
+__device__ __forceinline__ void sep_put2(float* o, float a, float b) { *reinterpret_cast<float2*>(o) = make_float2(a, b); }
+__device__ __forceinline__ void sep_put2(double* o, double a, double b) { *reinterpret_cast<double2*>(o) = make_double2(a, b); }
+__device__ __forceinline__ float2 sep_get2(const float* o) { return *reinterpret_cast<const float2*>(o); }
+__device__ __forceinline__ double2 sep_get2(const double* o) { return *reinterpret_cast<const double2*>(o); }
+// Results of a transform to rows of `pitch` values, `cols` columns of them.
+template <typename T>
+struct SepStore {
+  T* __restrict__ dst;
+  size_t pitch;
+  long long cols;
+  __device__ __forceinline__ int fetch(int, int) const { return 0; }
+  __device__ __forceinline__ void operator()(int row, int col, T a, T b, int) const {
+    if (col < cols) sep_put2(dst + row * pitch + col, a, b);
+  }
+};
+
 // x = hi + lo (+ below 2^-22 |x|): hi rounded to TF32's 11 bits, lo cut to them.
 __device__ __forceinline__ void tf32_split(float x, uint32_t& hi, uint32_t& lo) {
   hi = (__float_as_uint(x) + 0x1000u) & 0xffffe000u;
@@ -141,108 +169,179 @@ __device__ __forceinline__ void mma_tf32(float (&c)[4], const uint32_t (&a)[4], 
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// acc[h] += tile row h of A (packed, KT tiles a row) times the 8 KT panel rows at b.
-template <int WN, int TILES>
-__device__ __forceinline__ void sep_mma(float (&acc)[TILES][4][4], const float4* const (&a)[TILES], int KT, const float* b) {
-  constexpr int PB = SEP_PITCH<float, WN>;
-  float4 next[TILES];
-#pragma unroll
-  for (int h = 0; h < TILES; ++h) next[h] = __ldg(a[h]);
-#pragma unroll 2
-  for (int kt = 0; kt < KT; ++kt) {
-    uint32_t hi[TILES][4], lo[TILES][4];
-#pragma unroll
-    for (int h = 0; h < TILES; ++h) {
-      const float4 c = next[h];
-      if (kt + 1 < KT) next[h] = __ldg(a[h] + (size_t)(kt + 1) * 32);
-      tf32_split(c.x, hi[h][0], lo[h][0]);
-      tf32_split(c.y, hi[h][1], lo[h][1]);
-      tf32_split(c.z, hi[h][2], lo[h][2]);
-      tf32_split(c.w, hi[h][3], lo[h][3]);
-    }
-    const float* bk = b + kt * 8 * PB;
-    uint32_t bh[4][2], bl[4][2];
-#pragma unroll
-    for (int n = 0; n < 4; ++n) {
-      tf32_split(bk[n * 8], bh[n][0], bl[n][0]);
-      tf32_split(bk[n * 8 + 4 * PB], bh[n][1], bl[n][1]);
-    }
-    // one product at a time over all accumulators: each waits for its own last product
-#pragma unroll
-    for (int n = 0; n < 4; ++n)
-#pragma unroll
-      for (int h = 0; h < TILES; ++h) mma_tf32(acc[h][n], lo[h], bh[n][0], bh[n][1]);
-#pragma unroll
-    for (int n = 0; n < 4; ++n)
-#pragma unroll
-      for (int h = 0; h < TILES; ++h) mma_tf32(acc[h][n], hi[h], bl[n][0], bl[n][1]);
-#pragma unroll
-    for (int n = 0; n < 4; ++n)
-#pragma unroll
-      for (int h = 0; h < TILES; ++h) mma_tf32(acc[h][n], hi[h], bh[n][0], bh[n][1]);
-  }
+__device__ __forceinline__ void sep_copy16(void* to, const void* from, bool on) {   // zeros where not on
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(to)), "l"(from), "r"(on ? 16 : 0)
+               : "memory");
 }
+__device__ __forceinline__ void sep_copy_tile(void* to, const void* from) {   // through L1: other warps want the same
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(to)), "l"(from) : "memory");
+}
+__device__ __forceinline__ void sep_copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void sep_copies_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// The transform of the block's panel sB ([rows][pitch]) by the matrices A of
-// its axis, result rows in units of a warp: part, part + parts, ... of every
-// round of 8 / WN units.  put(row, column of the panel (even), value, next value).
+// The matrix tiles of a warp's work on their way to shared memory, `depth`
+// ahead of its products: segment i (seg(i, a): the KT tiles behind each of a,
+// 0 at the end), segment i + 1, ...  The first leave before the panel is
+// loaded.  A thread copies the 16 bytes of each tile that its own MMAs read, so
+// the queue needs no barrier; a slot is filled again once the products of its
+// last content are issued.  (With one or two blocks of 8 warps per SM nothing
+// else hides L2's latency: plain loads one tile ahead left the tensor pipe 43 %
+// busy at n = 512, two ahead no more.  With the queue, the panel's copies all
+// under way at once and the loads of r batched in the last transform: y of 512 x
+// 512 x 128 443 -> 378 us, back along z 226 -> 151 us; 256 x 256 x 64 38 -> 34
+// and 36 -> 27 us.)
+template <int TILES, typename Seg>
+struct SepQueue {
+  float4* slots;
+  const int depth;
+  int slot = 0, i = 0, at = 0, KT;
+  const float4* a[TILES];
+  Seg seg;
+  __device__ __forceinline__ SepQueue(void* queue, int depth_, Seg seg_)
+      : slots(reinterpret_cast<float4*>(queue) + threadIdx.x), depth(depth_), seg(seg_) {
+    KT = seg(0, a);
+    for (int p = 0; p < depth; ++p) fill(p);
+  }
+  __device__ __forceinline__ void fill(int to) {
+    if (at < KT) {
+#pragma unroll
+      for (int h = 0; h < TILES; ++h) sep_copy_tile(slots + to * (SEP_SLOT / 16) + h * SEP_T, a[h] + (size_t)at * 32);
+      if (++at == KT) {
+        at = 0;
+        KT = seg(++i, a);
+      }
+    }
+    sep_copies_commit();
+  }
+  // acc[h] += the next n tiles of row h times the 8 n panel rows at b.
+  template <int WN>
+  __device__ __forceinline__ void mma(float (&acc)[TILES][4][4], int n_tiles, const float* b) {
+    constexpr int PB = SEP_PITCH<float, WN>;
+#pragma unroll 2
+    for (int kt = 0; kt < n_tiles; ++kt) {
+      if (depth == SEP_QUEUE) sep_copies_wait<SEP_QUEUE - 1>();
+      else sep_copies_wait<0>();
+      uint32_t hi[TILES][4], lo[TILES][4];
+#pragma unroll
+      for (int h = 0; h < TILES; ++h) {
+        const float4 c = slots[slot * (SEP_SLOT / 16) + h * SEP_T];
+        tf32_split(c.x, hi[h][0], lo[h][0]);
+        tf32_split(c.y, hi[h][1], lo[h][1]);
+        tf32_split(c.z, hi[h][2], lo[h][2]);
+        tf32_split(c.w, hi[h][3], lo[h][3]);
+      }
+      const float* bk = b + kt * 8 * PB;
+      uint32_t bh[4][2], bl[4][2];
+#pragma unroll
+      for (int n = 0; n < 4; ++n) {
+        tf32_split(bk[n * 8], bh[n][0], bl[n][0]);
+        tf32_split(bk[n * 8 + 4 * PB], bh[n][1], bl[n][1]);
+      }
+      // one product at a time over all accumulators: each waits for its own last product
+#pragma unroll
+      for (int n = 0; n < 4; ++n)
+#pragma unroll
+        for (int h = 0; h < TILES; ++h) mma_tf32(acc[h][n], lo[h], bh[n][0], bh[n][1]);
+#pragma unroll
+      for (int n = 0; n < 4; ++n)
+#pragma unroll
+        for (int h = 0; h < TILES; ++h) mma_tf32(acc[h][n], hi[h], bl[n][0], bl[n][1]);
+#pragma unroll
+      for (int n = 0; n < 4; ++n)
+#pragma unroll
+        for (int h = 0; h < TILES; ++h) mma_tf32(acc[h][n], hi[h], bh[n][0], bh[n][1]);
+      fill(slot);
+      slot = slot + 1 == depth ? 0 : slot + 1;
+    }
+  }
+};
+
+// The transform of the block's panel sB ([rows][pitch], which panel() loads) by
+// the matrices A of its axis, result rows in units of a warp: part, part +
+// parts, ... of every round of 8 / WN units.  put(row, column of the panel
+// (even), value, next value, what put.fetch(row, column) loaded).
 //
 // Forward, and both ways of an axis that is not folded: 32 rows a unit, those
 // of the even modes first.
-template <int WN, typename Put>
-__device__ __forceinline__ void sep_gemm(const float4* __restrict__ A, const SepAxis& x, const float* sB, int part, int parts,
-                                         Put put) {
+template <int WN, typename Panel, typename Put>
+__device__ __forceinline__ void sep_gemm(const float4* __restrict__ A, const SepAxis& x, float* sB, int part, int parts,
+                                         Panel panel, Put put) {
   constexpr int PB = SEP_PITCH<float, WN>, WM = 8 / WN;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3, wm = warp / WN, wn = warp % WN;
   const int ue = (x.size(0) + 31) / 32, un = ue + (x.size(1) + 31) / 32;
-  for (int un0 = wm + WM * part; un0 < un; un0 += WM * parts) {
-    const int odd = un0 >= ue, M = x.size(odd), KT = x.pad(odd) / 8, m0 = 2 * (odd ? un0 - ue : un0);
-    const bool two = m0 * 16 + 16 < M;
+  auto seg = [&](int i, const float4* (&a)[2]) {
+    const int u = wm + WM * (part + parts * i);
+    if (u >= un) return 0;
+    const int odd = u >= ue, KT = x.pad(odd) / 8, m0 = 2 * (odd ? u - ue : u);
     const size_t tile = (size_t)m0 * KT + (odd ? (size_t)((x.size(0) + 15) / 16) * (x.pad(0) / 8) : 0);
-    const float4* const a[2] = {A + tile * 32 + lane, A + (tile + (two ? KT : 0)) * 32 + lane};
+    a[0] = A + tile * 32 + lane;
+    a[1] = m0 * 16 + 16 < x.size(odd) ? a[0] + (size_t)KT * 32 : a[0];
+    return KT;
+  };
+  SepQueue<2, decltype(seg)> queue(sB + x.rows() * PB, sep_queue(WN, x), seg);
+  panel();
+  __syncthreads();
+  for (int u = wm + WM * part; u < un; u += WM * parts) {
+    const int odd = u >= ue, M = x.size(odd), m0 = 2 * (odd ? u - ue : u);
     float acc[2][4][4] = {};
-    sep_mma<WN, 2>(acc, a, KT, sB + (t + (odd ? x.pad(0) : 0)) * PB + wn * 32 + g);
+    queue.template mma<WN>(acc, x.pad(odd) / 8, sB + (t + (odd ? x.pad(0) : 0)) * PB + wn * 32 + g);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int row = (m0 + h) * 16 + g;
 #pragma unroll
       for (int n = 0; n < 4; ++n) {
         const int col = wn * 32 + n * 8 + 2 * t;
-        if (row < M) put(x.fold ? 2 * row + odd : row, col, acc[h][n][0], acc[h][n][1]);
-        if (row + 8 < M) put(x.fold ? 2 * row + 16 + odd : row + 8, col, acc[h][n][2], acc[h][n][3]);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const int out = x.fold ? 2 * (row + 8 * q) + odd : row + 8 * q;
+          if (row + 8 * q < M) put(out, col, acc[h][n][2 * q], acc[h][n][2 * q + 1], put.fetch(out, col));
+        }
       }
     }
   }
 }
 // Back along a folded axis: 16 cells and their mirror images a unit, the even
 // modes' sum plus and minus the odd ones'.
-template <int WN, typename Put>
-__device__ __forceinline__ void sep_gemm_back(const float4* __restrict__ A, const SepAxis& x, const float* sB, int part, int parts,
-                                              Put put) {
-  if (!x.fold) return sep_gemm<WN>(A, x, sB, part, parts, put);
+template <int WN, typename Panel, typename Put>
+__device__ __forceinline__ void sep_gemm_back(const float4* __restrict__ A, const SepAxis& x, float* sB, int part, int parts,
+                                              Panel panel, Put put) {
+  if (!x.fold) return sep_gemm<WN>(A, x, sB, part, parts, panel, put);
   constexpr int PB = SEP_PITCH<float, WN>, WM = 8 / WN;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3, wm = warp / WN, wn = warp % WN;
   const int Me = x.size(0), Mo = x.size(1), KE = x.pad(0) / 8, KO = x.pad(1) / 8;
+  auto seg = [&](int i, const float4* (&a)[1]) {   // (only the last unit of all can lack odd modes)
+    const int m = wm + WM * (part + parts * (i >> 1)), odd = i & 1;
+    if (m * 16 >= x.size(odd)) return 0;
+    a[0] = A + ((odd ? (size_t)((Me + 15) / 16) * KE : 0) + (size_t)m * (odd ? KO : KE)) * 32 + lane;
+    return odd ? KO : KE;
+  };
+  SepQueue<1, decltype(seg)> queue(sB + x.rows() * PB, sep_queue(WN, x), seg);
+  panel();
+  __syncthreads();
   const float* b = sB + t * PB + wn * 32 + g;
   for (int m = wm + WM * part; m * 16 < Me; m += WM * parts) {
     float e[1][4][4] = {}, o[1][4][4] = {};
-    const float4* const ae[1] = {A + (size_t)m * KE * 32 + lane};
-    sep_mma<WN, 1>(e, ae, KE, b);
-    if (m * 16 < Mo) {
-      const float4* const ao[1] = {A + ((size_t)((Me + 15) / 16) * KE + (size_t)m * KO) * 32 + lane};
-      sep_mma<WN, 1>(o, ao, KO, b + x.pad(0) * PB);
-    }
+    queue.template mma<WN>(e, KE, b);
+    if (m * 16 < Mo) queue.template mma<WN>(o, KO, b + x.pad(0) * PB);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const int row = m * 16 + g + 8 * h;
+      const int row = m * 16 + g + 8 * h, mirror = x.n - 1 - row;
+      decltype(put.fetch(0, 0)) f[4][2] = {};   // what the results meet, all loads before the first use
+#pragma unroll
+      for (int n = 0; n < 4; ++n) {
+        const int col = wn * 32 + n * 8 + 2 * t;
+        if (row < Me) f[n][0] = put.fetch(row, col);
+        if (row < Mo) f[n][1] = put.fetch(mirror, col);
+      }
 #pragma unroll
       for (int n = 0; n < 4; ++n) {
         const int col = wn * 32 + n * 8 + 2 * t;
         const float e0 = e[0][n][2 * h], e1 = e[0][n][2 * h + 1], o0 = o[0][n][2 * h], o1 = o[0][n][2 * h + 1];
-        if (row < Me) put(row, col, e0 + o0, e1 + o1);
-        if (row < Mo) put(x.n - 1 - row, col, e0 - o0, e1 - o1);
+        if (row < Me) put(row, col, e0 + o0, e1 + o1, f[n][0]);
+        if (row < Mo) put(mirror, col, e0 - o0, e1 - o1, f[n][1]);
       }
     }
   }
@@ -264,23 +363,30 @@ __device__ __forceinline__ void sep_fma(double (&c)[4], const double* __restrict
   }
 }
 __device__ __forceinline__ size_t sep_mat64(int n) { return (size_t)n * ((n + 1) & ~1); }
-template <int WN, typename Put>
+template <int WN, typename Panel, typename Put>
 __device__ __forceinline__ void sep_gemm(const double* __restrict__ A, const SepAxis& x, const double* sB, int part, int parts,
-                                         Put put) {
+                                         Panel panel, Put put) {
+  panel();
+  __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, col = 2 * (lane & 15);
   const int ue = (x.size(0) + 3) / 4, un = ue + (x.size(1) + 3) / 4;
   for (int u = warp + 8 * part; u < un; u += 8 * parts) {
     const int odd = u >= ue, M = x.size(odd), row = 4 * (odd ? u - ue : u) + 2 * (lane >> 4);
     double c[4] = {};
     sep_fma(c, A + (odd ? sep_mat64(x.size(0)) : 0), row, M, sB + (odd ? x.pad(0) * 32 : 0) + col);
-    if (row < M) put(x.fold ? 2 * row + odd : row, col, c[0], c[1]);
-    if (row + 1 < M) put(x.fold ? 2 * row + 2 + odd : row + 1, col, c[2], c[3]);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int out = x.fold ? 2 * (row + h) + odd : row + h;
+      if (row + h < M) put(out, col, c[2 * h], c[2 * h + 1], put.fetch(out, col));
+    }
   }
 }
-template <int WN, typename Put>
+template <int WN, typename Panel, typename Put>
 __device__ __forceinline__ void sep_gemm_back(const double* __restrict__ A, const SepAxis& x, const double* sB, int part, int parts,
-                                              Put put) {
-  if (!x.fold) return sep_gemm<WN>(A, x, sB, part, parts, put);
+                                              Panel panel, Put put) {
+  if (!x.fold) return sep_gemm<WN>(A, x, sB, part, parts, panel, put);
+  panel();
+  __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, col = 2 * (lane & 15);
   const int Me = x.size(0), Mo = x.size(1);
   for (int u = warp + 8 * part; 4 * u < Me; u += 8 * parts) {
@@ -290,8 +396,9 @@ __device__ __forceinline__ void sep_gemm_back(const double* __restrict__ A, cons
     if (row < Mo) sep_fma(o, A + sep_mat64(Me), row, Mo, sB + x.pad(0) * 32 + col);   // (no odd mode reaches the middle cell)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      if (row + h < Me) put(row + h, col, e[2 * h] + o[2 * h], e[2 * h + 1] + o[2 * h + 1]);
-      if (row + h < Mo) put(x.n - 1 - row - h, col, e[2 * h] - o[2 * h], e[2 * h + 1] - o[2 * h + 1]);
+      const int mir = x.n - 1 - row - h;
+      if (row + h < Me) put(row + h, col, e[2 * h] + o[2 * h], e[2 * h + 1] + o[2 * h + 1], put.fetch(row + h, col));
+      if (row + h < Mo) put(mir, col, e[2 * h] - o[2 * h], e[2 * h + 1] - o[2 * h + 1], put.fetch(mir, col));
     }
   }
 }
@@ -321,23 +428,21 @@ __device__ __forceinline__ void sep_panel(T* sm, const SepAxis& x, int row0, int
     if (k < po) *reinterpret_cast<V*>(sm + (pe + k) * PB + col0) = b;
   }
 }
-template <typename T, int PB, typename Get>
-__device__ __forceinline__ void sep_panel_back(T* sm, const SepAxis& x, int row0, int step, int col0, Get get) {
-  using V = SepVec<T>;
+// (Back: asynchronous copies, all rows under way at once; mode i of the
+// thread's columns lies at from + i pitch, and counts where `in`.)
+template <typename T, int PB>
+__device__ __forceinline__ void sep_panel_back(T* sm, const SepAxis& x, int row0, int step, int col0, const T* from, size_t pitch,
+                                               bool in) {
   const int pe = x.pad(0), rows = x.rows();
-#pragma unroll 4
+#pragma unroll 2
   for (int k = row0; k < rows; k += step) {
     const int odd = k >= pe, m = odd ? k - pe : k;
-    V v = {};
-    if (m < x.size(odd)) v = get(x.fold ? 2 * m + odd : m);
-    *reinterpret_cast<V*>(sm + k * PB + col0) = v;
+    const bool on = in && m < x.size(odd);
+    sep_copy16(sm + k * PB + col0, from + (on ? (size_t)(x.fold ? 2 * m + odd : m) * pitch : 0), on);
   }
+  sep_copies_commit();
+  sep_copies_wait<0>();
 }
-
-__device__ __forceinline__ void sep_put2(float* o, float a, float b) { *reinterpret_cast<float2*>(o) = make_float2(a, b); }
-__device__ __forceinline__ void sep_put2(double* o, double a, double b) { *reinterpret_cast<double2*>(o) = make_double2(a, b); }
-__device__ __forceinline__ float2 sep_get2(const float* o) { return *reinterpret_cast<const float2*>(o); }
-__device__ __forceinline__ double2 sep_get2(const double* o) { return *reinterpret_cast<const double2*>(o); }
 
 // ------------------------------------------------------- z transforms ----
 // A panel is 128 consecutive columns (x, y) of the P x ny plane with every z
@@ -377,12 +482,9 @@ __device__ __forceinline__ void sep_zf(const Level<T>& L, const Sep<T>& S, const
     return;
   }
   const SepAxis ax = sep_axis_z(L);
-  sep_panel<T, PB, UNROLL>(sep_sm, ax, C.row0, SEP_T / C.VR, C.col0, get);
-  __syncthreads();
+  auto panel = [&] { sep_panel<T, PB, UNROLL>(sep_sm, ax, C.row0, SEP_T / C.VR, C.col0, get); };
   const size_t cb = (size_t)vb.x * 32 * WN;
-  sep_gemm<WN>(S.zf, ax, sep_sm, 0, 1, [&](int row, int col, T a, T b) {
-    if (cb + col < C.PS) sep_put2(S.t + (size_t)row * C.PS + cb + col, a, b);
-  });
+  sep_gemm<WN>(S.zf, ax, sep_sm, 0, 1, panel, SepStore<T>{S.t + cb, C.PS, (long long)(C.PS - cb)});
 }
 
 __device__ __forceinline__ float sep_diff(float2 a, float2 b) { return ps_diff(a, b); }
@@ -510,6 +612,23 @@ __device__ __forceinline__ void sep_update_body(const Level<T>& L, const Sep<T>&
   }
 }
 
+// z and the terms of r.z (rows of `pitch` values, `cols` columns of them).
+template <typename T>
+struct SepStoreDot {
+  const T* __restrict__ r;
+  T* __restrict__ z;
+  size_t pitch;
+  long long cols;
+  DotAcc<T>* dot;
+  using Pair = decltype(sep_get2((const T*)nullptr));
+  __device__ __forceinline__ Pair fetch(int row, int col) const { return col < cols ? sep_get2(r + row * pitch + col) : Pair{}; }
+  __device__ __forceinline__ void operator()(int row, int col, T a, T b, Pair rv) const {
+    if (col >= cols) return;
+    sep_put2(z + row * pitch + col, a, b);
+    dot->add(rv.x, a);
+    dot->add(rv.y, b);
+  }
+};
 // Back along z: z = Qz^T t, and r.z (from the first iteration on also beta).
 template <typename T>
 __device__ __forceinline__ void sep_zi_body(const Level<T>& L, const Sep<T>& S, T* __restrict__ z, double* partials, SolveState* st,
@@ -526,30 +645,18 @@ __device__ __forceinline__ void sep_zi_body(const Level<T>& L, const Sep<T>& S, 
   const int col0 = V::N * (flat ? threadIdx.x : threadIdx.x % VR);
   const size_t c = (size_t)vb.x * sep_z_cols<T>(L.nz) + col0;
   DotAcc<T> dacc;
-  auto put = [&](size_t o, T a, T b) {
-    const auto rv = sep_get2(L.r + o);
-    sep_put2(z + o, a, b);
-    dacc.add(rv.x, a);
-    dacc.add(rv.y, b);
-  };
   if (flat) {
     if (c < PS) {
       const V v = *reinterpret_cast<const V*>(S.t + c);
+      const SepStoreDot<T> put{L.r + c, z + c, PS, V::N, &dacc};
 #pragma unroll
-      for (int e = 0; e < V::N; e += 2) put(c + e, v.e[e], v.e[e + 1]);
+      for (int e = 0; e < V::N; e += 2) put(0, e, v.e[e], v.e[e + 1], put.fetch(0, e));
     }
   } else {
     const SepAxis ax = sep_axis_z(L);
-    sep_panel_back<T, PB>(sep_sm, ax, threadIdx.x / VR, SEP_T / VR, col0, [&](int k) {
-      V v = {};
-      if (c < PS) v = *reinterpret_cast<const V*>(S.t + (size_t)k * PS + c);
-      return v;
-    });
-    __syncthreads();
+    auto panel = [&] { sep_panel_back<T, PB>(sep_sm, ax, threadIdx.x / VR, SEP_T / VR, col0, S.t + (c < PS ? c : 0), PS, c < PS); };
     const size_t cb = (size_t)vb.x * BN;
-    sep_gemm_back<WN>(S.zi, ax, sep_sm, 0, 1, [&](int row, int col, T a, T b) {
-      if (cb + col < PS) put((size_t)row * PS + cb + col, a, b);
-    });
+    sep_gemm_back<WN>(S.zi, ax, sep_sm, 0, 1, panel, SepStoreDot<T>{L.r + cb, z + cb, PS, (long long)(PS - cb), &dacc});
   }
   const double vals[1] = {block_sum<SEP_T>(dacc.value(), sh)};
   if (publish_partials<1>(partials, &st->ticket[0], vals, &last, vb)) {
@@ -565,8 +672,8 @@ __device__ __forceinline__ void sep_zi_body(const Level<T>& L, const Sep<T>& S, 
 // --------------------------------------------------------- y transforms --
 // One panel of 32 WN columns of a z plane, every y; blocks vb.y of `split`
 // share the panel's result rows.
-template <int WN, typename T>
-__device__ __forceinline__ void sep_y_panel(const Level<T>& L, const Sep<T>& S, int inverse, int split, const VBlock& vb) {
+template <int WN, bool INVERSE, typename T>
+__device__ __forceinline__ void sep_y_panel(const Level<T>& L, const Sep<T>& S, int split, const VBlock& vb) {
   extern __shared__ __align__(16) unsigned char sep_raw[];
   T* sep_sm = reinterpret_cast<T*>(sep_raw);
   using V = SepVec<T>;
@@ -575,33 +682,28 @@ __device__ __forceinline__ void sep_y_panel(const Level<T>& L, const Sep<T>& S, 
   const int x0 = vb.x * BN, xv = V::N * (threadIdx.x % VR), row0 = threadIdx.x / VR;
   const size_t base = (size_t)vb.z * L.P * L.ny + x0;
   const bool in = x0 + xv < L.P;
-  const T* __restrict__ src = (inverse ? S.u : S.t) + base;
-  T* __restrict__ dst = (inverse ? S.t : S.u) + base;
+  const T* __restrict__ src = (INVERSE ? S.u : S.t) + base;
+  T* __restrict__ dst = (INVERSE ? S.t : S.u) + base;
   auto get = [&](int j) {
     V v = {};
     if (in) v = *reinterpret_cast<const V*>(src + (size_t)j * L.P + xv);
     return v;
   };
-  auto put = [&](int row, int col, T a, T b) {
-    if (x0 + col < L.P) sep_put2(dst + (size_t)row * L.P + col, a, b);
-  };
-  if (inverse) {
-    sep_panel_back<T, PB>(sep_sm, ax, row0, SEP_T / VR, xv, get);
-    __syncthreads();
-    sep_gemm_back<WN>(S.yi, ax, sep_sm, vb.y, split, put);
+  const SepStore<T> put{dst, (size_t)L.P, L.P - x0};
+  if (INVERSE) {
+    auto panel = [&] { sep_panel_back<T, PB>(sep_sm, ax, row0, SEP_T / VR, xv, src + (in ? xv : 0), (size_t)L.P, in); };
+    sep_gemm_back<WN>(S.yi, ax, sep_sm, vb.y, split, panel, put);
   } else {
-    sep_panel<T, PB, 2>(sep_sm, ax, row0, SEP_T / VR, xv, get);
-    __syncthreads();
-    sep_gemm<WN>(S.yf, ax, sep_sm, vb.y, split, put);
+    auto panel = [&] { sep_panel<T, PB, 4>(sep_sm, ax, row0, SEP_T / VR, xv, get); };
+    sep_gemm<WN>(S.yf, ax, sep_sm, vb.y, split, panel, put);
   }
 }
-template <typename T>
-__device__ __forceinline__ void sep_y_body(const Level<T>& L, const Sep<T>& S, int inverse, const SolveState* st,
-                                           const VBlock& vb) {
+template <bool INVERSE, typename T>
+__device__ __forceinline__ void sep_y_body(const Level<T>& L, const Sep<T>& S, const SolveState* st, const VBlock& vb) {
   if (st->converged) return;
   const int split = sep_y_split<T>(L.P, L.ny, L.nz);
-  if (sizeof(T) == 4 && L.ny <= SEP_Y_WIDE) sep_y_panel<sizeof(T) == 4 ? 2 : 1>(L, S, inverse, split, vb);
-  else sep_y_panel<1>(L, S, inverse, split, vb);
+  if (sizeof(T) == 4 && L.ny <= SEP_Y_WIDE) sep_y_panel<sizeof(T) == 4 ? 2 : 1, INVERSE>(L, S, split, vb);
+  else sep_y_panel<1, INVERSE>(L, S, split, vb);
 }
 
 // -------------------------------------------------------------- x solve --
@@ -728,9 +830,9 @@ __global__ void __launch_bounds__(SEP_T, 2) k_sep_zi(Level<T> L, Sep<T> S, T* __
                                                      SolveState* st) {
   sep_zi_body(L, S, z, partials, st, vblock());
 }
-template <typename T>
-__global__ void __launch_bounds__(SEP_T, 2) k_sep_y(Level<T> L, Sep<T> S, int inverse, const SolveState* st) {
-  sep_y_body(L, S, inverse, st, vblock());
+template <bool INVERSE, typename T>
+__global__ void __launch_bounds__(SEP_T, 2) k_sep_y(Level<T> L, Sep<T> S, const SolveState* st) {
+  sep_y_body<INVERSE>(L, S, st, vblock());
 }
 template <typename T>
 __global__ void __launch_bounds__(32 * SEP_X_LINES) k_sep_x(Level<T> L, Sep<T> S, const SolveState* st) {
