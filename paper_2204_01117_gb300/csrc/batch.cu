@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(uf::NT) kb_cg_init(const __grid_constant__ Arg
 }
 
 template <typename T>
-__global__ void __launch_bounds__(uf::FT) kb_cg_dir_q(const __grid_constant__ Args<CgP<T>> A) {
+__global__ void __launch_bounds__(uf::FT, 4) kb_cg_dir_q(const __grid_constant__ Args<CgP<T>> A) {
   for_items(&A.m, [&](int i, int zc, const VBlock& vb) {
     const CgP<T>& P = A.at[i];
     uf::cg_dir_q_body<T>(P.L, zc, P.z, P.d0, P.d1, P.q, P.partials, P.st, vb);
@@ -500,7 +500,7 @@ class BatchImpl final : public uf_batch {
       add_entry(maps[MAP_CHUNK], i, G.chunk_g[0], G.chunk_g[1], G.chunk_g[2], G.chunk_zc);
       add_entry(maps[G.adv_far ? MAP_ADV_FAR : MAP_ADV], i, G.adv_g[0], G.adv_g[1],
                 G.adv_auto ? (d.nz + adv_zc - 1) / adv_zc : G.adv_g[2], G.adv_auto ? adv_zc : G.adv_zc);
-      add_entry(maps[MAP_DIR], i, G.march_g[0][0], G.march_g[0][1], G.march_g[0][2], G.march_zc[0]);
+      add_entry(maps[MAP_DIR], i, G.dir_g[0], G.dir_g[1], G.dir_g[2], G.dir_zc);
       if (G.sep.on) {
         const int wn = uf::sep_y_wn<T>(d.ny), by = 32 * wn, P = G.lv[0].P;
         add_entry(maps[MAP_SEPZ], i, (int)uf::sep_z_blocks<T>(P, d.ny, d.nz), 1, 1, 0);

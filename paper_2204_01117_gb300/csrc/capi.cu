@@ -639,6 +639,18 @@ class GridImpl final : public uf_grid {
     return dim3(bx, by, (L.nz + z - 1) / z);
   }
 
+  // Direction kernel: DIR_ZC planes per block, fewer where the blocks (four
+  // resident on each of 152 SMs) would not fill the chip, at least two (one
+  // would read three planes for each).
+  dim3 dir_grid(int* zc) const {
+    const unsigned bx = uf::dir_blocks<T>(lv[0].P, d.ny);
+    int z = uf::DIR_ZC;
+    while (z > 2 && (long)bx * ((d.nz + z - 1) / z) < 608) z /= 2;
+    while (z < d.nz && (long long)bx * ((d.nz + z - 1) / z) > kPartials) z *= 2;
+    *zc = z;
+    return dim3(bx, 1, (d.nz + z - 1) / z);
+  }
+
   // Fused V-cycle: down kernels to the tail level, the tail, up kernels.
   // mode 1 (inside the CG loop): the finest down kernel also applies the CG
   // update and the convergence test.
@@ -873,7 +885,7 @@ class GridImpl final : public uf_grid {
   void rec_cg_iter(cudaStream_t s, cudaGraphConditionalHandle cond, int use_cond) {
     if (d.precond == UF_PRECOND_MG) {
       int zc;
-      const dim3 g = march_grid(0, &zc);
+      const dim3 g = dir_grid(&zc);
       if (use_sep()) rec_sep_rest(s);
       L(s, "cg_dir_q", 4 * N() * tb(), [&] {
         uf::k_cg_dir_q<T><<<g, uf::FT, 0, s>>>(lv[0], zc, z, d0, d1, q, partials, st);
@@ -1746,6 +1758,8 @@ class GridImpl final : public uf_grid {
       V.march_g[l][0] = g.x; V.march_g[l][1] = g.y; V.march_g[l][2] = g.z;
       V.march_zc[l] = zc;
     }
+    const dim3 gd = dir_grid(&V.dir_zc);
+    V.dir_g[0] = gd.x; V.dir_g[1] = gd.y; V.dir_g[2] = gd.z;
     V.tail_level = P.tail_level;
     V.tail = tail;
     V.tail.rin = 1;   // batched launches form the tail's right-hand side in the tail

@@ -31,6 +31,7 @@ struct GridView {
   int tail_level;                  // first level of the shared-memory tail
   uf::TailArgs<T> tail;
   size_t tail_smem;
+  int dir_g[3], dir_zc;            // blocks of the CG direction kernel
   int march_g[uf::MAX_LEVELS][3];  // blocks of the z-marching level kernels
   int march_zc[uf::MAX_LEVELS];    // z planes per block
   int chunk_g[3], chunk_zc;        // z-chunked reductions over the cells (and the fused momentum pass)

@@ -967,104 +967,106 @@ __global__ void __launch_bounds__(TAIL_T) k_mg_tail(TailArgs<T> A, SmoothW<T> W,
 
 
 // ------------------------------------------- CG direction + SpMV --------
-// d = z (first iteration) or z + beta d_old, staged per z plane on the tile
-// plus a halo of 1 (ring of 4 planes, one barrier per plane, loads one plane
-// ahead); q = A d on the owned cells; d.q and alpha = rz / d.q.
+// d = z (first iteration) or z + beta d_old; q = A d; d.q and alpha = rz / d.q.
 // q is formed as a sum of differences w (d_c - d_nb): the CG directions turn
 // smooth as the iteration proceeds, and the form D d_c - sum w d_nb would then
 // lose about eps * |D d| to cancellation in FP32 -- an error the recursive
 // residual never sees, which caps the attainable accuracy of the pressure.
 // A Neumann neighbour takes d_c (its term is exactly zero); an outlet
-// neighbour is the staged zero ghost (term w d_c).
+// neighbour is zero (term w d_c).  A thread takes 16 bytes of a row and marches zc
+// planes: the planes below and above stay in registers, the x neighbours come
+// from the lanes beside, and only the rows of the y neighbours are read (and
+// their d formed) again.  Bound by those loads' latency and by memory;
+// measured against a block-wide plane in shared memory with a barrier per
+// plane: 256 x 256 x 64 30 -> 24 us, 512 x 512 x 128 155 -> 113 us.
+template <typename T>
+struct alignas(16) Vec16 {   // 16 bytes of a field
+  static constexpr int N = 16 / sizeof(T);
+  T e[N];
+};
+constexpr int DIR_ZC = 8;   // planes per block at most
+template <typename T>
+__host__ __device__ inline unsigned dir_blocks(int P, int ny) {   // blocks that cover a plane of P x ny cells
+  return (unsigned)(((size_t)P * ny / Vec16<T>::N + FT - 1) / FT);
+}
 template <typename T>
 __device__ __forceinline__ void cg_dir_q_body(const Level<T>& L, int zc, const T* __restrict__ z, T* d0, T* d1,
                                               T* __restrict__ q, double* partials, SolveState* st, const VBlock& vb) {
-  __shared__ T sD[4][XP];
   __shared__ double sh[32];
   __shared__ bool last;
   if (st->converged) return;
-  const int i0 = vb.x * TX, j0 = vb.y * TY, k0 = vb.z * zc;
-  const int kend = min(L.nz, k0 + zc);
-  const int tid = threadIdx.x, tx = tid & (TX - 1), ty = tid / TX;
+  using V = Vec16<T>;
+  constexpr int N = V::N;
+  const int k0 = vb.z * zc, kend = min(L.nz, k0 + zc), lane = threadIdx.x & 31;
+  const size_t PS = (size_t)L.P * L.ny, c = ((size_t)vb.x * FT + threadIdx.x) * N;
+  const int j = (int)(c / L.P), i0 = (int)(c - (size_t)j * L.P), left = L.nx - i0;   // cells of the row from here on
+  const bool in = c < PS && left > 0;
   const int it = st->iter;
-  const T* dold = (it & 1) ? d1 : d0;
-  T* dnew = (it & 1) ? d0 : d1;
+  const T* __restrict__ dold = (it & 1) ? d1 : d0;
+  T* __restrict__ dnew = (it & 1) ? d0 : d1;
   const T beta = it == 0 ? T(0) : (T)st->beta;
-  const size_t PS = (size_t)L.P * L.ny;
-  const PlaneMap mx = plane_map<XX, XY>();
-  PosXY<T> pd[2];
-  int sd[2];
+  auto dir = [&](size_t o) {
+    V a = *reinterpret_cast<const V*>(z + o);
+    if (it != 0) {
+      const V b = *reinterpret_cast<const V*>(dold + o);
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const int xx = h ? mx.x1 : mx.x0, xy = h ? mx.y1 : mx.y0;
-    pd[h] = pos_xy(L, i0 - 1 + xx, j0 - 1 + xy);
-    if (h == 1 && !mx.has1) pd[h].ok = false;
-    sd[h] = xx + XX * xy;
+      for (int e = 0; e < N; ++e) a.e[e] = a.e[e] + beta * b.e[e];
+    }
+    return a;
+  };
+  auto dir1 = [&](size_t o) { return it != 0 ? z[o] + beta * dold[o] : z[o]; };
+  const bool x0 = i0 > 0, y0 = j > 0, y1 = j < L.ny - 1;
+  const bool left_of = in && x0 && lane == 0, right_of = in && left > N && lane == 31;   // beyond the warp
+  size_t o = (size_t)k0 * PS + c;
+  V dm = {}, dc = {};
+  if (in) {
+    dc = dir(o);
+    dm = k0 > 0 ? dir(o - PS) : dc;
   }
-  T pz[2], pdv[2];
-  auto issueD = [&](int k) {
-    const bool kin = (unsigned)k < (unsigned)L.nz;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      pz[h] = 0;
-      pdv[h] = 0;
-      if (kin && pd[h].ok) {
-        const size_t c = (size_t)k * PS + pd[h].off;
-        pz[h] = z[c];
-        if (it != 0) pdv[h] = dold[c];
-      }
-    }
-  };
-  auto commitD = [&](int k) {
-    T* dst = sD[ring4(k)];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      if (h == 1 && !mx.has1) break;
-      dst[sd[h]] = pz[h] + beta * pdv[h];
-    }
-  };
-  const int gi = i0 + tx, gj = j0 + ty;
-  const PosXY<T> po = pos_xy(L, gi, gj);
-  const int b = (tx + 1) + XX * (ty + 1);
-  const bool nxm = gi == 0 && !(L.out_mask & 1), nxp = gi == L.nx - 1 && !(L.out_mask & 2);
-  const bool nym = gj == 0 && !(L.out_mask & 4), nyp = gj == L.ny - 1 && !(L.out_mask & 8);
   DotAcc<T> dacc;
-  issueD(k0 - 1); commitD(k0 - 1);
-  issueD(k0); commitD(k0);
-  issueD(k0 + 1);
-  for (int k = k0; k < kend; ++k) {
-    commitD(k + 1);
-    issueD(k + 2);
-    __syncthreads();
-    if (po.ok) {
-      const T* dm = sD[ring4(k - 1)];
-      const T* dc = sD[ring4(k)];
-      const T* dp = sD[ring4(k + 1)];
-      const T dv = dc[b];
-      const T xm = nxm ? dv : dc[b - 1], xp = nxp ? dv : dc[b + 1];
-      const T ym = nym ? dv : dc[b - XX], yp = nyp ? dv : dc[b + XX];
-      const T zm = (k == 0 && !(L.out_mask & 16)) ? dv : dm[b];
-      const T zp = (k == L.nz - 1 && !(L.out_mask & 32)) ? dv : dp[b];
-      const T qv = L.wx * ((dv - xm) + (dv - xp)) + L.wy * ((dv - ym) + (dv - yp)) + L.wz * ((dv - zm) + (dv - zp));
-      const size_t c = (size_t)k * PS + po.off;
-      dnew[c] = dv;
-      q[c] = qv;
-      dacc.add(dv, qv);
+#pragma unroll 2
+  for (int k = k0; k < kend; ++k, o += PS) {
+    const bool top = k == L.nz - 1;
+    V dp = dc, ym = dc, yp = dc;
+    if (in && !top) dp = dir(o + PS);
+    if (in && y0) ym = dir(o - L.P);
+    if (in && y1) yp = dir(o + L.P);
+    T xm = __shfl_up_sync(0xffffffffu, dc.e[N - 1], 1), xp = __shfl_down_sync(0xffffffffu, dc.e[0], 1);
+    if (left_of) xm = dir1(o - 1);
+    if (right_of) xp = dir1(o + N);
+    if (in) {
+      V qv, dv;
+#pragma unroll
+      for (int e = 0; e < N; ++e) {
+        const bool cell = e < left, last_x = e == left - 1;
+        const T v = dc.e[e];
+        const T a = e > 0 ? dc.e[e > 0 ? e - 1 : 0] : x0 ? xm : (L.out_mask & 1) ? T(0) : v;
+        const T b = last_x ? ((L.out_mask & 2) ? T(0) : v) : e < N - 1 ? dc.e[e < N - 1 ? e + 1 : e] : xp;
+        const T f0 = y0 ? ym.e[e] : (L.out_mask & 4) ? T(0) : v, f1 = y1 ? yp.e[e] : (L.out_mask & 8) ? T(0) : v;
+        const T lo = k > 0 ? dm.e[e] : (L.out_mask & 16) ? T(0) : v, up = !top ? dp.e[e] : (L.out_mask & 32) ? T(0) : v;
+        const T w = L.wx * ((v - a) + (v - b)) + L.wy * ((v - f0) + (v - f1)) + L.wz * ((v - lo) + (v - up));
+        dv.e[e] = cell ? v : T(0);
+        qv.e[e] = cell ? w : T(0);
+        dacc.add(dv.e[e], qv.e[e]);
+      }
+      *reinterpret_cast<V*>(dnew + o) = dv;
+      *reinterpret_cast<V*>(q + o) = qv;
     }
+    dm = dc;
+    dc = dp;
   }
   double acc = block_sum<FT>(dacc.value(), sh);
   const double vals[1] = {acc};
   if (publish_partials<1>(partials, &st->ticket[2], vals, &last, vb)) {
     double tot[1];
     reduce_partials_sum<FT, 1>(partials, tot, sh, vb.n);
-    if (tid == 0) {
+    if (threadIdx.x == 0) {
       st->dq = tot[0];
       st->alpha = st->rz / tot[0];
       st->ticket[2] = 0u;
     }
   }
 }
-
 template <typename T>
 __global__ void __launch_bounds__(FT) k_cg_dir_q(Level<T> L, int zc, const T* __restrict__ z, T* d0, T* d1,
                                                 T* __restrict__ q, double* partials, SolveState* st) {

@@ -134,12 +134,6 @@ __host__ __device__ inline int sep_y_split(int P, int ny, int nz) {
   const int want = (SEP_Y_BLOCKS + panels - 1) / panels;
   return want < rounds ? want : rounds;
 }
-// 16 bytes of a field.
-template <typename T>
-struct alignas(16) SepVec {
-  static constexpr int N = 16 / sizeof(T);
-  T e[N];
-};
 
 __device__ __forceinline__ void sep_put2(float* o, float a, float b) { *reinterpret_cast<float2*>(o) = make_float2(a, b); }
 __device__ __forceinline__ void sep_put2(double* o, double a, double b) { *reinterpret_cast<double2*>(o) = make_double2(a, b); }
@@ -409,7 +403,7 @@ __device__ __forceinline__ void sep_gemm_back(const double* __restrict__ A, cons
 // back, its even modes and then its odd ones.
 template <typename T, int PB, int UNROLL, typename Get>
 __device__ __forceinline__ void sep_panel(T* sm, const SepAxis& x, int row0, int step, int col0, Get get) {
-  using V = SepVec<T>;
+  using V = Vec16<T>;
   const int pe = x.pad(0), po = x.pad(1);
 #pragma unroll UNROLL
   for (int k = row0; k < pe; k += step) {
@@ -457,12 +451,12 @@ struct SepCols {   // a thread's 16 bytes of every row it loads
   size_t PS, c;    // cells of a plane, the first column
   bool in;
   int left_x;      // how many of the values lie inside the domain
-  static constexpr int VR = 32 * SEP_Z_WN<T> / SepVec<T>::N;
+  static constexpr int VR = 32 * SEP_Z_WN<T> / Vec16<T>::N;
   __device__ __forceinline__ SepCols(const Level<T>& L, const VBlock& vb) {
     static_assert(SEP_T % VR == 0, "a thread keeps its columns");
     flat = L.nz == 1;
     row0 = flat ? 0 : threadIdx.x / VR;
-    col0 = SepVec<T>::N * (flat ? threadIdx.x : threadIdx.x % VR);
+    col0 = Vec16<T>::N * (flat ? threadIdx.x : threadIdx.x % VR);
     PS = (size_t)L.P * L.ny;
     c = (size_t)vb.x * sep_z_cols<T>(L.nz) + col0;
     in = c < PS;
@@ -474,7 +468,7 @@ template <int UNROLL, typename T, typename Get>
 __device__ __forceinline__ void sep_zf(const Level<T>& L, const Sep<T>& S, const SepCols<T>& C, const VBlock& vb, Get get) {
   extern __shared__ __align__(16) unsigned char sep_raw[];
   T* sep_sm = reinterpret_cast<T*>(sep_raw);
-  using V = SepVec<T>;
+  using V = Vec16<T>;
   constexpr int WN = SEP_Z_WN<T>, PB = SEP_PITCH<T, WN>;
   if (C.flat) {
     const V v = get(0);
@@ -496,8 +490,8 @@ __device__ __forceinline__ double sep_value(double a) { return a; }
 // A f (level_apply) at 16 bytes' worth of cells of plane k; f holds values or
 // the pressure store's pairs, whose differences are taken on the pairs.
 template <typename E, typename T>
-__device__ __forceinline__ SepVec<T> sep_apply(const Level<T>& L, const SepCols<T>& C, const E* __restrict__ f, int k) {
-  constexpr int N = SepVec<T>::N;
+__device__ __forceinline__ Vec16<T> sep_apply(const Level<T>& L, const SepCols<T>& C, const E* __restrict__ f, int k) {
+  constexpr int N = Vec16<T>::N;
   struct alignas(16) Row { E e[N]; };
   const int i0 = L.nx - C.left_x, j = (int)(C.c / L.P);
   f += (size_t)k * C.PS + C.c;
@@ -511,7 +505,7 @@ __device__ __forceinline__ SepVec<T> sep_apply(const Level<T>& L, const SepCols<
   if (z1) zp = *reinterpret_cast<const Row*>(f + C.PS);
   if (i0 > 0) xm = f[-1];
   if (C.left_x > N) xp = f[N];
-  SepVec<T> a;
+  Vec16<T> a;
 #pragma unroll
   for (int e = 0; e < N; ++e) {
     const T v = (T)sep_value(m.e[e]);
@@ -537,7 +531,7 @@ __device__ __forceinline__ void sep_init_body(const Level<T>& L, const Sep<T>& S
                                               cudaGraphConditionalHandle cond, int use_cond, int* left, const VBlock& vb) {
   __shared__ double sh[32];
   __shared__ bool last;
-  using V = SepVec<T>;
+  using V = Vec16<T>;
   const SepCols<T> C(L, vb);
   const bool zero_rhs = st->bb == 0.0;
   DotAcc<T> dacc;
@@ -577,7 +571,7 @@ __device__ __forceinline__ void sep_update_body(const Level<T>& L, const Sep<T>&
   __shared__ double sh[32];
   __shared__ bool last;
   if (st->converged) return;
-  using V = SepVec<T>;
+  using V = Vec16<T>;
   const SepCols<T> C(L, vb);
   const int it0 = st->iter;
   const T alpha = (T)st->alpha;
@@ -638,7 +632,7 @@ __device__ __forceinline__ void sep_zi_body(const Level<T>& L, const Sep<T>& S, 
   __shared__ double sh[32];
   __shared__ bool last;
   if (st->converged) return;
-  using V = SepVec<T>;
+  using V = Vec16<T>;
   constexpr int WN = SEP_Z_WN<T>, BN = 32 * WN, PB = SEP_PITCH<T, WN>, VR = BN / V::N;
   const size_t PS = (size_t)L.P * L.ny;
   const bool flat = L.nz == 1;
@@ -676,7 +670,7 @@ template <int WN, bool INVERSE, typename T>
 __device__ __forceinline__ void sep_y_panel(const Level<T>& L, const Sep<T>& S, int split, const VBlock& vb) {
   extern __shared__ __align__(16) unsigned char sep_raw[];
   T* sep_sm = reinterpret_cast<T*>(sep_raw);
-  using V = SepVec<T>;
+  using V = Vec16<T>;
   constexpr int BN = 32 * WN, PB = SEP_PITCH<T, WN>, VR = BN / V::N;
   const SepAxis ax = sep_axis_y(L);
   const int x0 = vb.x * BN, xv = V::N * (threadIdx.x % VR), row0 = threadIdx.x / VR;
@@ -715,7 +709,7 @@ __device__ __forceinline__ void sep_y_body(const Level<T>& L, const Sep<T>& S, c
 // padding e = 0, which makes the solution 0 there.
 template <int E, typename T>
 __device__ __forceinline__ void sep_x_line(T* __restrict__ row, const T* __restrict__ piv, int P) {
-  using V = SepVec<T>;
+  using V = Vec16<T>;
   const int lane = threadIdx.x & 31;
   T f[E], e[E];
   if (E >= V::N) {
