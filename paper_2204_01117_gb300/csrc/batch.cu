@@ -504,7 +504,7 @@ class BatchImpl final : public uf_batch {
       if (G.sep.on) {
         const int wn = uf::sep_y_wn<T>(d.ny), by = 32 * wn, P = G.lv[0].P;
         add_entry(maps[MAP_SEPZ], i, (int)uf::sep_z_blocks<T>(P, d.ny, d.nz), 1, 1, 0);
-        add_entry(maps[MAP_SEPY], i, (P + by - 1) / by, uf::sep_y_split<T>(P, d.ny, d.nz), d.nz, 0);
+        add_entry(maps[MAP_SEPY], i, (P + by - 1) / by, uf::sep_y_split(G.lv[0]), d.nz, 0);
         add_entry(maps[MAP_SEPX], i, (d.ny * d.nz + uf::SEP_X_LINES - 1) / uf::SEP_X_LINES, 1, 1, 0);
         sepz_smem = std::max(sepz_smem, uf::sep_smem<T>(uf::SEP_Z_WN<T>, uf::sep_axis_z(G.lv[0])));
         sepy_smem = std::max(sepy_smem, uf::sep_smem<T>(wn, uf::sep_axis_y(G.lv[0])));

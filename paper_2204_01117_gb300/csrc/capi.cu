@@ -641,11 +641,11 @@ class GridImpl final : public uf_grid {
 
   // Direction kernel: DIR_ZC planes per block, fewer where the blocks (four
   // resident on each of 152 SMs) would not fill the chip, at least two (one
-  // would read three planes for each).
+  // would read three planes for each; FP64, bound by its pipe, goes to one).
   dim3 dir_grid(int* zc) const {
     const unsigned bx = uf::dir_blocks<T>(lv[0].P, d.ny);
     int z = uf::DIR_ZC;
-    while (z > 2 && (long)bx * ((d.nz + z - 1) / z) < 608) z /= 2;
+    while (z > (sizeof(T) == 8 ? 1 : 2) && (long)bx * ((d.nz + z - 1) / z) < 608) z /= 2;
     while (z < d.nz && (long long)bx * ((d.nz + z - 1) / z) > kPartials) z *= 2;
     *zc = z;
     return dim3(bx, 1, (d.nz + z - 1) / z);
@@ -835,7 +835,7 @@ class GridImpl final : public uf_grid {
     const int wn = uf::sep_y_wn<T>(d.ny), by = 32 * wn;
     const unsigned gz = uf::sep_z_blocks<T>(lv[0].P, d.ny, d.nz);
     const size_t sz = uf::sep_smem<T>(uf::SEP_Z_WN<T>, uf::sep_axis_z(lv[0])), sy = uf::sep_smem<T>(wn, uf::sep_axis_y(lv[0]));
-    const dim3 gy((lv[0].P + by - 1) / by, uf::sep_y_split<T>(lv[0].P, d.ny, d.nz), d.nz);
+    const dim3 gy((lv[0].P + by - 1) / by, uf::sep_y_split(lv[0]), d.nz);
     const unsigned gx = (unsigned)((d.ny * d.nz + uf::SEP_X_LINES - 1) / uf::SEP_X_LINES);
     L(s, "sep_y", 2 * N() * tb(), [&] { uf::k_sep_y<false, T><<<gy, uf::SEP_T, sy, s>>>(lv[0], sep, st); });
     L(s, "sep_x", 3 * N() * tb(), [&] { uf::k_sep_x<T><<<gx, 32 * uf::SEP_X_LINES, 0, s>>>(lv[0], sep, st); });

@@ -112,7 +112,7 @@ __host__ __device__ inline int sep_queue(int wn, const SepAxis& x) {
   return sep_panel_bytes<float>(wn, x) + SEP_QUEUE * SEP_SLOT + 1024 <= 227 * 1024 ? SEP_QUEUE : 1;
 }
 template <typename T>
-inline size_t sep_smem(int wn, const SepAxis& x) {
+__host__ __device__ inline size_t sep_smem(int wn, const SepAxis& x) {
   return sep_panel_bytes<T>(wn, x) + (sizeof(T) == 4 ? (size_t)sep_queue(wn, x) * SEP_SLOT : 0);
 }
 // Columns (x, y) of a z panel, and the blocks that cover the plane.  One cell
@@ -123,16 +123,22 @@ template <typename T>
 inline unsigned sep_z_blocks(int P, int ny, int nz) {
   return (unsigned)(((size_t)P * ny + sep_z_cols<T>(nz) - 1) / sep_z_cols<T>(nz));
 }
-// Blocks that share a y panel, each taking every split-th round of result
-// rows: a quasi-2D grid has fewer panels than SMs (512 x 768 x 1: 8, one pass
-// 97 us unsplit, 27 us split).
-constexpr int SEP_Y_BLOCKS = 304;   // two resident blocks on each of 152 SMs
+// Blocks that share a y panel, each taking every split-th unit of result rows
+// (sep_gemm).  Whole rounds of units while two blocks per SM have none, and
+// single units where even one per SM would be idle otherwise: a quasi-2D or a
+// small grid has fewer panels than SMs, and a warp's chain of products is what
+// it waits for (512 x 768 x 1: 97 us unsplit, 37 by whole rounds, 31 by units;
+// FP64 128 x 96 x 40: 152 and 120 us).
+constexpr int SEP_SMS = 152;
 template <typename T>
-__host__ __device__ inline int sep_y_split(int P, int ny, int nz) {
-  const int wn = sep_y_wn<T>(ny), rows = sizeof(T) == 4 ? 32 * (8 / wn) : 32;   // of a round
-  const int panels = (P + 32 * wn - 1) / (32 * wn) * nz, rounds = (ny + rows - 1) / rows;
-  const int want = (SEP_Y_BLOCKS + panels - 1) / panels;
-  return want < rounds ? want : rounds;
+__host__ __device__ inline int sep_y_split(const Level<T>& L) {
+  const SepAxis x = sep_axis_y(L);
+  const int wn = sep_y_wn<T>(L.ny), unit = sizeof(T) == 4 ? 32 : 4, round = sizeof(T) == 4 ? 8 / wn : 8;
+  const int units = (x.size(0) + unit - 1) / unit + (x.size(1) + unit - 1) / unit;
+  const int panels = (L.P + 32 * wn - 1) / (32 * wn) * L.nz;
+  const int resident = SEP_SMS * (sep_smem<T>(wn, x) <= 113 * 1024 ? 2 : 1);
+  const int by_round = min((2 * SEP_SMS + panels - 1) / panels, (units + round - 1) / round);
+  return max(by_round, min(resident / panels, units));
 }
 
 __device__ __forceinline__ void sep_put2(float* o, float a, float b) { *reinterpret_cast<float2*>(o) = make_float2(a, b); }
@@ -252,8 +258,8 @@ struct SepQueue {
 };
 
 // The transform of the block's panel sB ([rows][pitch], which panel() loads) by
-// the matrices A of its axis, result rows in units of a warp: part, part +
-// parts, ... of every round of 8 / WN units.  put(row, column of the panel
+// the matrices A of its axis, result rows in units of a warp: the block
+// has units part, part + parts, ...  put(row, column of the panel
 // (even), value, next value, what put.fetch(row, column) loaded).
 //
 // Forward, and both ways of an axis that is not folded: 32 rows a unit, those
@@ -266,7 +272,7 @@ __device__ __forceinline__ void sep_gemm(const float4* __restrict__ A, const Sep
   const int g = lane >> 2, t = lane & 3, wm = warp / WN, wn = warp % WN;
   const int ue = (x.size(0) + 31) / 32, un = ue + (x.size(1) + 31) / 32;
   auto seg = [&](int i, const float4* (&a)[2]) {
-    const int u = wm + WM * (part + parts * i);
+    const int u = part + parts * (wm + WM * i);
     if (u >= un) return 0;
     const int odd = u >= ue, KT = x.pad(odd) / 8, m0 = 2 * (odd ? u - ue : u);
     const size_t tile = (size_t)m0 * KT + (odd ? (size_t)((x.size(0) + 15) / 16) * (x.pad(0) / 8) : 0);
@@ -277,7 +283,7 @@ __device__ __forceinline__ void sep_gemm(const float4* __restrict__ A, const Sep
   SepQueue<2, decltype(seg)> queue(sB + x.rows() * PB, sep_queue(WN, x), seg);
   panel();
   __syncthreads();
-  for (int u = wm + WM * part; u < un; u += WM * parts) {
+  for (int u = part + parts * wm; u < un; u += WM * parts) {
     const int odd = u >= ue, M = x.size(odd), m0 = 2 * (odd ? u - ue : u);
     float acc[2][4][4] = {};
     queue.template mma<WN>(acc, x.pad(odd) / 8, sB + (t + (odd ? x.pad(0) : 0)) * PB + wn * 32 + g);
@@ -307,7 +313,7 @@ __device__ __forceinline__ void sep_gemm_back(const float4* __restrict__ A, cons
   const int g = lane >> 2, t = lane & 3, wm = warp / WN, wn = warp % WN;
   const int Me = x.size(0), Mo = x.size(1), KE = x.pad(0) / 8, KO = x.pad(1) / 8;
   auto seg = [&](int i, const float4* (&a)[1]) {   // (only the last unit of all can lack odd modes)
-    const int m = wm + WM * (part + parts * (i >> 1)), odd = i & 1;
+    const int m = part + parts * (wm + WM * (i >> 1)), odd = i & 1;
     if (m * 16 >= x.size(odd)) return 0;
     a[0] = A + ((odd ? (size_t)((Me + 15) / 16) * KE : 0) + (size_t)m * (odd ? KO : KE)) * 32 + lane;
     return odd ? KO : KE;
@@ -316,7 +322,7 @@ __device__ __forceinline__ void sep_gemm_back(const float4* __restrict__ A, cons
   panel();
   __syncthreads();
   const float* b = sB + t * PB + wn * 32 + g;
-  for (int m = wm + WM * part; m * 16 < Me; m += WM * parts) {
+  for (int m = part + parts * wm; m * 16 < Me; m += WM * parts) {
     float e[1][4][4] = {}, o[1][4][4] = {};
     queue.template mma<WN>(e, KE, b);
     if (m * 16 < Mo) queue.template mma<WN>(o, KO, b + x.pad(0) * PB);
@@ -364,7 +370,7 @@ __device__ __forceinline__ void sep_gemm(const double* __restrict__ A, const Sep
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, col = 2 * (lane & 15);
   const int ue = (x.size(0) + 3) / 4, un = ue + (x.size(1) + 3) / 4;
-  for (int u = warp + 8 * part; u < un; u += 8 * parts) {
+  for (int u = part + parts * warp; u < un; u += 8 * parts) {
     const int odd = u >= ue, M = x.size(odd), row = 4 * (odd ? u - ue : u) + 2 * (lane >> 4);
     double c[4] = {};
     sep_fma(c, A + (odd ? sep_mat64(x.size(0)) : 0), row, M, sB + (odd ? x.pad(0) * 32 : 0) + col);
@@ -383,7 +389,7 @@ __device__ __forceinline__ void sep_gemm_back(const double* __restrict__ A, cons
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, col = 2 * (lane & 15);
   const int Me = x.size(0), Mo = x.size(1);
-  for (int u = warp + 8 * part; 4 * u < Me; u += 8 * parts) {
+  for (int u = part + parts * warp; 4 * u < Me; u += 8 * parts) {
     const int row = 4 * u + 2 * (lane >> 4);
     double e[4] = {}, o[4] = {};
     sep_fma(e, A, row, Me, sB + col);
@@ -695,7 +701,7 @@ __device__ __forceinline__ void sep_y_panel(const Level<T>& L, const Sep<T>& S, 
 template <bool INVERSE, typename T>
 __device__ __forceinline__ void sep_y_body(const Level<T>& L, const Sep<T>& S, const SolveState* st, const VBlock& vb) {
   if (st->converged) return;
-  const int split = sep_y_split<T>(L.P, L.ny, L.nz);
+  const int split = sep_y_split(L);
   if (sizeof(T) == 4 && L.ny <= SEP_Y_WIDE) sep_y_panel<sizeof(T) == 4 ? 2 : 1, INVERSE>(L, S, split, vb);
   else sep_y_panel<1, INVERSE>(L, S, split, vb);
 }
