@@ -2,7 +2,7 @@
 
 One "step" is one full time step of the hot path: CFL dt, eddy viscosity,
 MacCormack advection, diffusion, porosity drag + BCs, pressure right-hand
-side, MG-preconditioned CG pressure solve, projection and the k-omega
+side, preconditioned CG pressure solve, projection and the k-omega
 update, FP32 fields with FP64 reductions.  Inputs are resident in HBM when the
 timed region starts.  The workload is the seeded synthetic urban block (40
 solid boxes + 60 porous canopies, seed = rank, log-law inflow 3 m/s at 10 m);
@@ -52,7 +52,7 @@ NX, NY, NZ = 256, 256, 64
 def workload_config(extra=None):
     cfg = {
         "workload": "urban block 256x256x64, h=2 m, 40 solid boxes + 60 porous canopies (seeded), "
-                    "log-law inflow 3 m/s at 10 m, FP32 fields + FP64 reductions, MG-preconditioned CG",
+                    "log-law inflow 3 m/s at 10 m, FP32 fields + FP64 reductions, preconditioned CG",
         "nx": NX, "ny": NY, "nz": NZ, "cells": NX * NY * NZ,
         "l2": "no flush: per-step working set ~400 MB > 129 MB L2",
     }
@@ -201,20 +201,32 @@ def ncu_traffic(kernel_label: str):
     return None
 
 
+# labels of the kernels inside the CG loop of the default pressure solve
+LOOP_KERNELS = ("sep_y", "sep_x", "sep_zi", "sep_update", "cg_dir_q")
+
+
+def loop_launches(name: str, n: int, prof_iters: int) -> int:
+    """Launches per CG iteration of a kernel that ran n times in a step of
+    prof_iters iterations (0: outside the loop; what n leaves over ran once
+    per step).  After a single iteration the count alone cannot tell."""
+    if prof_iters == 1:
+        return n if name in LOOP_KERNELS else 0
+    return n // prof_iters if prof_iters > 0 else 0
+
+
 def dominant_kernel(kernels: dict, prof_iters: int, mean_iters: float):
     """The kernel with the most time in an average timed step, and its share.
 
     The eagerly profiled step ran prof_iters CG iterations, the timed steps
-    mean_iters on average; as in step_traffic, a kernel that launched at
-    least prof_iters times runs once per iteration plus its fixed launches,
-    so its time per step is its mean launch time x (fixed launches +
-    mean_iters).  (Ranking by the profiled step alone would depend on that
+    mean_iters on average; as in step_traffic, a kernel's time per step is
+    its mean launch time x (fixed launches + loop_launches x mean_iters).  (Ranking by the profiled step alone would depend on that
     one step's iteration count.)  Returns (label, entry, ms per step, share)."""
     per_step = {}
     for name, k in kernels.items():
         n = int(k["launches"])
         avg = float(k["total_ms"]) / max(n, 1)
-        runs = (n - prof_iters + mean_iters) if (prof_iters > 0 and n >= prof_iters) else n
+        m = loop_launches(name, n, prof_iters)
+        runs = n - m * prof_iters + m * mean_iters
         per_step[name] = avg * runs
     name = max(per_step, key=per_step.get)
     return name, kernels[name], per_step[name], per_step[name] / sum(per_step.values())
@@ -227,21 +239,18 @@ def step_traffic(kernels: dict, prof_iters: int, mean_iters: float, ms_per_step:
 
     One counting, per kernel: its bytes per launch (the compulsory reads and
     writes of the launch, from uf_profile_step) times its launches per step.
-    The eagerly profiled step ran prof_iters CG iterations; a kernel that
-    launched at least that many times runs once per iteration (plus a fixed
-    number of set-up launches), the others a fixed number of times per step.
+    The eagerly profiled step ran prof_iters CG iterations; loop_launches of
+    a kernel's launches belong to each, the others run once per step.
     The per-iteration launches are then taken at mean_iters, the mean CG
     iterations of the timed steps, so bytes and time describe the same steps.
     Never raises: a malformed profile gives {"error": ...}."""
     try:
         fixed = per_iter = 0.0
-        for k in kernels.values():
+        for name, k in kernels.items():
             n, b = int(k["launches"]), float(k["bytes_per_launch"])
-            if prof_iters > 0 and n >= prof_iters:
-                fixed += b * (n - prof_iters)
-                per_iter += b
-            else:
-                fixed += b * n
+            m = loop_launches(name, n, prof_iters)
+            fixed += b * (n - m * prof_iters)
+            per_iter += b * m
         total = fixed + per_iter * mean_iters
         gbs = total / (ms_per_step * 1e-3) / 1e9
         return {"bytes": total, "bytes_per_cell": total / cells, "fixed_bytes_per_cell": fixed / cells,
@@ -983,7 +992,7 @@ def run_ours(args):
         "warmup": max(args.warmup, 3), "ms_per_step": ms / args.steps, "higher_is_better": True,
         "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "config": workload_config({"parallelism": f"replicas x{world}", "cg_iters_last_step": st1.cg_iters,
-                                   "precond": "MG V-cycle (2+2 Chebyshev-weighted Jacobi)", "cg_tol": 1e-7}),
+                                   "precond": "separable inverse (cosine transforms along y and z, tridiagonal solves along x)", "cg_tol": 1e-7}),
         "roofline": {"bound": "hbm", "kernel": dom_name, "achieved": achieved, "peak": peak,
                      "unit": "GB/s", "frac": achieved / peak, "traffic": traffic,
                      "peak_source": f"hbm_gbs of {peak_kind}",
@@ -996,14 +1005,15 @@ def run_ours(args):
         "gpu_launches": int(launches),
         "clocks": clk.summary(),
     }
-    # the finest-level CG kernel, the bandwidth-bound one, when another kernel
-    # (the issue-bound fused advection) leads the step
-    cg = kernels.get("mg_down_cg_L0")
-    if cg and dom_name != "mg_down_cg_L0":
+    # the CG update with the inverse's first transform, the bandwidth-bound
+    # kernel of the solve, when another (the issue-bound fused advection) leads
+    # the step
+    cg = kernels.get("sep_update")
+    if cg and dom_name != "sep_update":
         cg_ms = cg["total_ms"] / cg["launches"]
         cg_gbs = cg["bytes_per_launch"] / (cg_ms * 1e-3) / 1e9
-        line["roofline_solver"] = {"bound": "hbm", "kernel": "mg_down_cg_L0", "achieved": cg_gbs, "peak": peak,
-                                   "unit": "GB/s", "frac": cg_gbs / peak, "traffic": ncu_traffic("mg_down_cg_L0"),
+        line["roofline_solver"] = {"bound": "hbm", "kernel": "sep_update", "achieved": cg_gbs, "peak": peak,
+                                   "unit": "GB/s", "frac": cg_gbs / peak, "traffic": ncu_traffic("sep_update"),
                                    "peak_source": f"hbm_gbs of {peak_kind}",
                                    "bytes_per_launch": cg["bytes_per_launch"], "avg_launch_us": cg_ms * 1e3}
     if not args.no_adjoint:
