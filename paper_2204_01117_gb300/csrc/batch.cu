@@ -69,8 +69,8 @@ struct LaunchMap {
 };
 
 // Launch kinds: one work list each (march levels: one per level).
-// MAP_DIR: the march tiles of the finest level, every instance; the V-cycle
-// maps (MAP_TAIL, MAP_MARCH0 ..) hold the instances that run it, the MAP_SEP
+// MAP_DIR: the CG direction, every instance; the V-cycle maps (MAP_INIT,
+// MAP_TAIL, MAP_MARCH0 ..) hold the instances that run it, the MAP_SEP
 // ones those with the separable inverse.
 enum MapKind { MAP_CFL = 0, MAP_TURB, MAP_CELL, MAP_FACE, MAP_CHUNK, MAP_INIT, MAP_TAIL, MAP_ADV, MAP_ADV_FAR, MAP_DIR, MAP_SEPZ, MAP_SEPY, MAP_SEPX, MAP_MARCH0 };
 constexpr int kMaps = MAP_MARCH0 + uf::MAX_LEVELS;
@@ -497,7 +497,7 @@ class BatchImpl final : public uf_batch {
                 (d.nz + uf::PROJ_ZC - 1) / uf::PROJ_ZC, uf::PROJ_ZC);
       add_entry(maps[MAP_TURB], i, (d.nx + uf::BX - 1) / uf::BX, (d.ny + uf::BY - 1) / uf::BY, (d.nz + uf::TURB_ZC - 1) / uf::TURB_ZC,
                 uf::TURB_ZC);
-      add_entry(maps[MAP_CHUNK], i, G.chunk_g[0], G.chunk_g[1], G.chunk_g[2], G.chunk_zc);
+      add_entry(maps[MAP_CHUNK], i, G.mom_g[0], G.mom_g[1], G.mom_g[2], G.mom_zc);
       add_entry(maps[G.adv_far ? MAP_ADV_FAR : MAP_ADV], i, G.adv_g[0], G.adv_g[1],
                 G.adv_auto ? (d.nz + adv_zc - 1) / adv_zc : G.adv_g[2], G.adv_auto ? adv_zc : G.adv_zc);
       add_entry(maps[MAP_DIR], i, G.dir_g[0], G.dir_g[1], G.dir_g[2], G.dir_zc);
@@ -801,7 +801,7 @@ class BatchImpl final : public uf_batch {
         M.ut = G.ut; M.vt = G.vt; M.wt = G.wt; M.nut = G.nut; M.cc = G.cc;
         M.u = G.u; M.v = G.v; M.w = G.w; M.b = G.b;
         M.u2t = M.v2t = M.w2t = nullptr;
-        M.zc = G.chunk_zc;
+        M.zc = G.mom_zc;
         M.partials = G.partials;
         M.st = G.st;
       });

@@ -3,8 +3,9 @@
 //
 // One uf_step replays a CUDA graph captured once per grid (two graphs, one per
 // parity of the k/omega ping-pong buffers).  The pressure CG loop sits in a
-// conditional WHILE node whose body is {direction + SpMV, update + norm,
-// preconditioner}; the update kernel clears the condition when
+// conditional WHILE node whose body is one iteration (preconditioner, direction
+// + SpMV, update + norm, in an order that suits the preconditioner); the update
+// kernel clears the condition when
 // ||r|| <= tol ||b||, when the iteration cap is hit or when the residual is not
 // finite, so the host never polls inside a step.
 #include <cuda_runtime.h>
@@ -149,13 +150,15 @@ struct Plan {
 // Whether a grid has the separable inverse: the default V-cycle settings (a
 // caller who asks for another smoother or transfer gets that V-cycle), sizes
 // whose panels fit one block's shared memory (227 KB: FP32 nz x 136 words, ny
-// x 72 or 40 words; FP64 32 doubles per cell of either axis) and whose x lines
-// fit one warp, and at most kPartials panels per reducing launch.  FP64:
-// the transforms cost 8 (ny + nz) FP64 operations a cell and application, the
-// V-cycle's fourteen iterations about 4 ns a cell at any size; with two
-// applications that is even near ny + nz = 550 (one step with the V-cycle and
-// with the inverse: 64 x 32 x 16 2.72 and 0.20 ms, 128 x 96 x 40 6.6 and 1.35,
-// 256 x 256 x 64 26.6 and 10.9, 128 x 330 x 64 24.6 and 7.9).
+// x 72 or 40 words and at least 8 KB of queue; FP64 32 doubles per cell of
+// either axis) and whose x lines fit one warp, and at most kPartials panels per
+// reducing launch.  FP64: the transforms cost 8 (ny + nz) FP64 operations a cell
+// and application (half along an axis with walls at both ends), the V-cycle's
+// fourteen iterations about 4 ns a cell at any size; with two applications that
+// is even near ny + nz = 550 for the dearest form (one step with the V-cycle
+// and with the inverse, all axes in full: 64 x 32 x 16 2.72 and 0.20 ms, 128 x
+// 96 x 40 6.6 and 1.35, 256 x 256 x 64 26.6 and 10.9, 128 x 330 x 64 24.6 and
+// 7.9).
 constexpr int kSep64Sum = 480;
 bool sep_available(const uf_grid_desc* d) {
   if (d->precond != UF_PRECOND_MG || d->mg_smoother != UF_SMOOTH_CHEBY || d->mg_transfer != UF_TRANSFER_LINEAR ||
@@ -998,6 +1001,29 @@ class GridImpl final : public uf_grid {
     return dim3(bx, by, (d.nz + z - 1) / z);
   }
 
+  // Momentum pass (and the right-hand side of its separate kernels, whose sums
+  // run over the same blocks): 32 x 8 columns, zc planes per block.  A block
+  // works off about two planes more than it has (FP64: 1.2), and few waves leave
+  // the chip idle at their ends: the depth with the least product of the two.
+  // FP32: 512 x 512 x 128 786 us at 64 planes, 737 at 32; 256 x 256 x 64 141 at 8,
+  // 137 at 12; 157 x 203 x 41 74 at 3, 68 at 8; 128 x 128 x 48 59 at 2, 49 at 4; FP64:
+  // 128 x 96 x 40 207 at 1, 129 at 4; the smallest grids want one plane (48 x 40 x
+  // 16 16 us, 25 at 4).
+  dim3 momentum_grid(int* zc) const {
+    const int bx = (d.nx + uf::BX - 1) / uf::BX, by = (d.ny + uf::BY - 1) / uf::BY;
+    const double resident = 152.0 * (sizeof(T) == 8 ? 2 : UF_MOMENTUM_MINB), halo = sizeof(T) == 8 ? 1.2 : 2.0;
+    double best = 1e300;
+    *zc = d.nz;
+    for (int c : {64, 32, 24, 16, 12, 10, 8, 6, 4, 3, 2, 1}) {
+      const int chunks = (d.nz + c - 1) / c;
+      if ((long long)bx * by * chunks > kPartials) break;
+      const double waves = (double)bx * by * chunks / resident;
+      const double cost = (d.nz + halo * chunks) * (waves < 1.0 ? 1.35 / waves : 1.0 + 0.35 / waves);
+      if (cost < best) { best = cost; *zc = c; }
+    }
+    return dim3(bx, by, (d.nz + *zc - 1) / *zc);
+  }
+
   void rec_momentum(cudaStream_t s, const T* kin, const T* oin) {
     const dim3 blk(uf::BX, uf::BY);
     const double faces = 3 * N() * tb(), cells = N() * tb();
@@ -1027,7 +1053,7 @@ class GridImpl final : public uf_grid {
       L(s, "advect_backward", 3 * faces, [&] { uf::k_advect_backward<T><<<ga, blk, 0, s>>>(A); });
     }
     int zc;
-    const dim3 gr = chunk_grid(d.nx, d.ny, d.nz, &zc);
+    const dim3 gr = momentum_grid(&zc);
     if (!(unfused & UF_UNFUSED_MOMENTUM)) {
       // one pass: u~, nu_t, c -> u3 (every face), b
       uf::MomentumArgs<T> M;
@@ -1767,6 +1793,8 @@ class GridImpl final : public uf_grid {
     int zc;
     const dim3 gc = chunk_grid(d.nx, d.ny, d.nz, &zc);
     V.chunk_g[0] = gc.x; V.chunk_g[1] = gc.y; V.chunk_g[2] = gc.z;
+    const dim3 gm = momentum_grid(&V.mom_zc);
+    V.mom_g[0] = gm.x; V.mom_g[1] = gm.y; V.mom_g[2] = gm.z;
     V.chunk_zc = zc;
     int azc;
     const dim3 ga = advect_grid(&azc);

@@ -34,7 +34,8 @@ struct GridView {
   int dir_g[3], dir_zc;            // blocks of the CG direction kernel
   int march_g[uf::MAX_LEVELS][3];  // blocks of the z-marching level kernels
   int march_zc[uf::MAX_LEVELS];    // z planes per block
-  int chunk_g[3], chunk_zc;        // z-chunked reductions over the cells (and the fused momentum pass)
+  int chunk_g[3], chunk_zc;        // z-chunked reductions over the cells
+  int mom_g[3], mom_zc;            // the fused momentum pass
   int adv_g[3], adv_zc;            // blocks and z planes per block of the fused advection
   int adv_auto;                    // adv_zc is the automatic choice for the grid alone
   int adv_far;                     // a displacement may reach a cell (k_advect_fused)
