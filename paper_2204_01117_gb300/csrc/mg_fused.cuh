@@ -5,7 +5,7 @@
 // shared memory, so that two dependent smoothing passes and the residual run
 // without another trip to global memory:
 //
-//   (k_mg_down, k_mg_up and k_cg_dir_q march along z with rolling planes.)
+//   (k_mg_down and k_mg_up march along z with rolling planes.)
 //   k_mg_down  : [finest level: CG update x += a d, r -= a q, ||r||^2]
 //                pre-smoothing from a zero guess, residual, summed
 //                restriction to the next level (under linear transfers: the

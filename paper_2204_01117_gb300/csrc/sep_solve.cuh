@@ -21,7 +21,7 @@
 // so the solution is the same to the same tolerance; its error against 64
 // bits is at most the V-cycle's (512 x 512 x 128, w after two steps: 2.2e-6
 // against 4.8e-6).  Measured on a GB300, one time step with the V-cycle and
-// with this: 48 x 40 x 16 0.73 -> 0.20 ms, 157 x 203 x 41 1.87 -> 0.47 ms,
+// with this in its first form, all else equal: 48 x 40 x 16 0.73 -> 0.20 ms, 157 x 203 x 41 1.87 -> 0.47 ms,
 // 256 x 256 x 64 2.20 -> 1.09 ms, 512 x 768 x 1 1.24 -> 0.34 ms,
 // 512 x 512 x 128 13.0 -> 8.7 ms (where the y transforms cost most); the
 // longest axes that fit were all faster.

@@ -5,13 +5,15 @@
 // inner products and residual norms.
 //
 // Preconditioners:
+//   * the exact inverse by separation of variables (sep_solve.cuh), the default
+//            where its sizes allow.
 //   * MG   - one geometric multigrid V-cycle (cell-centred 2x2x2 agglomeration,
 //            summed restriction R, piecewise-constant prolongation P = R^T,
 //            rediscretised coarse operators, red-black Gauss-Seidel or
 //            damped-Jacobi smoothing, dense FP64 inverse on the coarsest
 //            level); kernels in mg_fused.cuh.  Symmetric and positive
-//            definite, so CG stays CG.  This replaces the paper's
-//            approximate inverse as the default.
+//            definite, so CG stays CG.  The default where the
+//            separable inverse does not apply.
 //   * AI1  - the paper's first-order approximate inverse M^-1 = K^T K,
 //            K = sqrt(2-w) Dbar^-1/2 (I - L Dbar^-1), Dbar = D/w (Sec. 3,
 //            "Approximate Inverse Preconditioner"), applied matrix-free
