@@ -1969,6 +1969,10 @@ class GridImpl final : public uf_grid {
         const dim3 ga = plane_grid(d.nx + 1, d.ny + 1, 3 * d.nz + 1);
         cudaMemsetAsync(pd, 0, P.n_c * sizeof(uf::PStore<T>), s);
         cudaMemsetAsync(gd, 0, P.n_c * sizeof(uf::PStore<T>), s);
+        // the faces below become u, v, w whole, and the CFL maximum runs over
+        // their row padding too: no trace of what else uses the scratch arrays
+        // (field transfers, the autotuner, meshes) may stay in it
+        cudaMemsetAsync(uh, 0, P.ut - P.uh, s);
         uf::k_init_fields<T><<<ga, blk, 0, s>>>(sp, u, v, w, kb[0], ob[0], p);
         rec_count++;
         if (!(d.fixed_dt > 0)) {
