@@ -2144,8 +2144,7 @@ class GridImpl final : public uf_grid {
       e = cudaGetLastError();
     }
     if (e == cudaSuccess) {
-      const dim3 g((d.nx + uf::MESH_BX - 1) / uf::MESH_BX, (d.ny + uf::MESH_BY - 1) / uf::MESH_BY, (d.nz + uf::MESH_BZ - 1) / uf::MESH_BZ);
-      uf::k_mesh_phi<T><<<g, 32 * uf::MESH_WARPS, 0, stream>>>(d.nx, d.ny, d.nz, P.Pc, d.h, sub, te, tf, dobj, nobj, dst);
+      uf::k_mesh_phi<T><<<uf::mesh_blocks(d.nx, d.ny, d.nz), 32 * uf::MESH_WARPS, 0, stream>>>(d.nx, d.ny, d.nz, P.Pc, d.h, sub, te, tf, dobj, nobj, dst);
       e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);

@@ -139,6 +139,9 @@ constexpr int MESH_OPEN = 192;     // undecided triangles of a cell (more: every
 constexpr int MESH_WARPS = 8;
 constexpr int MESH_BX = 8, MESH_BY = 8, MESH_BZ = 4;   // 32 MESH_WARPS cells
 
+inline unsigned mesh_blocks(int nx, int ny, int nz) {   // bricks, x fastest (in one dimension: any nz)
+  return (unsigned)((size_t)((nx + MESH_BX - 1) / MESH_BX) * ((ny + MESH_BY - 1) / MESH_BY) * ((nz + MESH_BZ - 1) / MESH_BZ));
+}
 template <typename T>
 __global__ void __launch_bounds__(32 * MESH_WARPS) k_mesh_phi(int nx, int ny, int nz, int P, double h, int sub,
                                                               const MeshTri* __restrict__ te, const MeshTriF* __restrict__ tf,
@@ -150,7 +153,8 @@ __global__ void __launch_bounds__(32 * MESH_WARPS) k_mesh_phi(int nx, int ny, in
   __shared__ double s_val[MESH_WARPS][32];
   __shared__ double s_off[16];          // sample offsets (a + 1/2) / sub within a cell
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  const int bi = blockIdx.x * MESH_BX, bj = blockIdx.y * MESH_BY, bk = blockIdx.z * MESH_BZ;
+  const unsigned int nbx = (nx + MESH_BX - 1) / MESH_BX, nby = (ny + MESH_BY - 1) / MESH_BY, row = blockIdx.x / nbx;
+  const int bi = (int)(blockIdx.x % nbx) * MESH_BX, bj = (int)(row % nby) * MESH_BY, bk = (int)(row / nby) * MESH_BZ;
   if (t == 0) s_nobj = 0;
   if (t < sub) s_off[t] = __ddiv_rn(__dadd_rn((double)t, 0.5), (double)sub);
   __syncthreads();
