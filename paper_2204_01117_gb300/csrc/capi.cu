@@ -2065,9 +2065,8 @@ class GridImpl final : public uf_grid {
 
   // ---------------------------------------------------- mesh resolver ----
   // Porosity of closed triangle meshes (uf_mesh_to_phi): the mesh and the
-  // objects' bounding boxes are copied to device memory allocated for the
-  // call; the result goes to the grid's porosity (and drag coefficient) or
-  // to phi_out.
+  // objects' bounding boxes are copied to the device (below); the result goes
+  // to the grid's porosity (and drag coefficient) or to phi_out.
   uf_status mesh_to_phi(int ntri, const double* tris, int nobj, const int* first, const int* count,
                         const double* phi_in, int sub, void* phi_out) override {
     if (ntri < 0 || nobj < 0 || (ntri > 0 && !tris) || (nobj > 0 && (!first || !count || !phi_in)))
@@ -2111,40 +2110,49 @@ class GridImpl final : public uf_grid {
     }
     // the triangles, the objects and the per-triangle tables of the crossing
     // tests: in the step's scratch arrays (uh .. w2, recomputed by every step)
-    // where they fit, else in memory allocated for the call
+    // where they fit, else in memory allocated for the call, without the
+    // tables where these outgrow their index or the memory
     long long entries = 0;
     for (int o = 0; o < nobj; ++o) {
       uf::MeshObject& m = obj[o];
-      if (entries > 0x7fffffffLL - m.count) return fail(UF_ERR_ARG, "too many triangles");
-      m.entry = (int)entries;
+      m.entry = (int)std::min(entries, 0x7fffffffLL);
       entries += m.count;
       const double size = std::max({m.hi[0] - m.lo[0], m.hi[1] - m.lo[1], m.hi[2] - m.lo[2]}) + 2.0 * d.h;
       m.scale = 1.0 / size;
     }
+    bool tables = entries <= 0x7fffffffLL;
     Layout ML;
     const size_t o_tri = ML.take((size_t)ntri * 9 * sizeof(double)), o_obj = ML.take((size_t)nobj * sizeof(uf::MeshObject));
+    const size_t bare = ML.off, room = P.k0 - P.uh;
     const size_t o_te = ML.take((size_t)entries * sizeof(uf::MeshTri)), o_tf = ML.take((size_t)entries * sizeof(uf::MeshTriF));
     char *block = at<char>(P.uh), *owned = nullptr;
-    if (ML.off > P.k0 - P.uh) {
-      UF_CUDA(cudaMalloc(&owned, ML.off));
-      block = owned;
+    if (tables && ML.off > room && cudaMalloc(&owned, ML.off) != cudaSuccess) {
+      cudaGetLastError();
+      owned = nullptr;
+      tables = false;
     }
+    if (!tables && bare > room) UF_CUDA(cudaMalloc(&owned, bare));
+    if (owned) block = owned;
     const double* dtri = reinterpret_cast<const double*>(block + o_tri);
     const uf::MeshObject* dobj = reinterpret_cast<const uf::MeshObject*>(block + o_obj);
-    uf::MeshTri* te = reinterpret_cast<uf::MeshTri*>(block + o_te);
-    uf::MeshTriF* tf = reinterpret_cast<uf::MeshTriF*>(block + o_tf);
+    uf::MeshTri* te = tables ? reinterpret_cast<uf::MeshTri*>(block + o_te) : nullptr;
+    uf::MeshTriF* tf = tables ? reinterpret_cast<uf::MeshTriF*>(block + o_tf) : nullptr;
     cudaError_t e = cudaSuccess;
     if (ntri > 0)
       e = cudaMemcpyAsync(block + o_tri, tris, (size_t)ntri * 9 * sizeof(double), cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess && nobj > 0)
       e = cudaMemcpyAsync(block + o_obj, obj.data(), nobj * sizeof(uf::MeshObject), cudaMemcpyHostToDevice, stream);
     T* dst = phi_out ? q : phi;
-    if (e == cudaSuccess && nobj > 0) {
+    if (e == cudaSuccess && nobj > 0 && tables) {
       uf::k_mesh_prep<128><<<nobj, 128, 0, stream>>>(dtri, dobj, te, tf);
       e = cudaGetLastError();
     }
     if (e == cudaSuccess) {
-      uf::k_mesh_phi<T><<<uf::mesh_blocks(d.nx, d.ny, d.nz), 32 * uf::MESH_WARPS, 0, stream>>>(d.nx, d.ny, d.nz, P.Pc, d.h, sub, te, tf, dobj, nobj, dst);
+      const unsigned nb = uf::mesh_blocks(d.nx, d.ny, d.nz);
+      if (tables)
+        uf::k_mesh_phi<T, true><<<nb, 32 * uf::MESH_WARPS, 0, stream>>>(d.nx, d.ny, d.nz, P.Pc, d.h, sub, dtri, te, tf, dobj, nobj, dst);
+      else
+        uf::k_mesh_phi<T, false><<<nb, 32 * uf::MESH_WARPS, 0, stream>>>(d.nx, d.ny, d.nz, P.Pc, d.h, sub, dtri, te, tf, dobj, nobj, dst);
       e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);

@@ -51,8 +51,7 @@ __device__ __forceinline__ double dot3_rn(double ax, double ay, double az, doubl
   return __dadd_rn(__dadd_rn(__dmul_rn(ax, bx), __dmul_rn(ay, by)), __dmul_rn(az, bz));
 }
 
-// Fills an object's table entries (one block per object).
-__device__ __forceinline__ void mesh_prep_tri(const double* v, const MeshObject& m, MeshTri& o, MeshTriF& f) {
+__device__ __forceinline__ double mesh_tri(const double* v, MeshTri& o) {   // the determinant
   for (int a = 0; a < 3; ++a) {
     o.v0[a] = v[a];
     o.e1[a] = __dsub_rn(v[3 + a], v[a]);
@@ -65,6 +64,11 @@ __device__ __forceinline__ void mesh_prep_tri(const double* v, const MeshObject&
   const double det = dot3_rn(o.e1[0], o.e1[1], o.e1[2], o.q[0], o.q[1], o.q[2]);
   o.s = det > 0.0 ? 1.0 : -1.0;
   o.adet = det == 0.0 ? 0.0 : __dmul_rn(det, o.s);
+  return det;
+}
+// Fills an object's table entries (one block per object).
+__device__ __forceinline__ void mesh_prep_tri(const double* v, const MeshObject& m, MeshTri& o, MeshTriF& f) {
+  const double det = mesh_tri(v, o);
   const double c = m.scale, c2 = c * c, g = o.s;
   // w = RAY . (p x e1) = p . (e1 x RAY), t = e2 . (p x e1) = p . (e1 x e2)
   const double w[3] = {o.e1[1] * RAY_Z - o.e1[2] * RAY_Y, o.e1[2] * RAY_X - o.e1[0] * RAY_Z, o.e1[0] * RAY_Y - o.e1[1] * RAY_X};
@@ -134,6 +138,9 @@ __device__ __forceinline__ int ray_bound(float px, float py, float pz, float r, 
 // triangle (1/64 rate) and the serial object list of every cell.  Measured at
 // 256 x 256 x 64 with 100 objects (6500 triangles), the whole call: 23.4 ->
 // 1.15 ms.
+// TABLES = false: a mesh whose tables do not fit (an entry per object and
+// triangle, so objects that share long ranges need many) is tested triangle
+// by triangle.
 constexpr int MESH_LIST = 64;      // objects of a brick (more: every object is visited)
 constexpr int MESH_OPEN = 192;     // undecided triangles of a cell (more: every triangle is tested)
 constexpr int MESH_WARPS = 8;
@@ -142,10 +149,11 @@ constexpr int MESH_BX = 8, MESH_BY = 8, MESH_BZ = 4;   // 32 MESH_WARPS cells
 inline unsigned mesh_blocks(int nx, int ny, int nz) {   // bricks, x fastest (in one dimension: any nz)
   return (unsigned)((size_t)((nx + MESH_BX - 1) / MESH_BX) * ((ny + MESH_BY - 1) / MESH_BY) * ((nz + MESH_BZ - 1) / MESH_BZ));
 }
-template <typename T>
+template <typename T, bool TABLES>
 __global__ void __launch_bounds__(32 * MESH_WARPS) k_mesh_phi(int nx, int ny, int nz, int P, double h, int sub,
-                                                              const MeshTri* __restrict__ te, const MeshTriF* __restrict__ tf,
-                                                              const MeshObject* __restrict__ obj, int nobj, T* __restrict__ phi) {
+                                                              const double* __restrict__ tri, const MeshTri* __restrict__ te,
+                                                              const MeshTriF* __restrict__ tf, const MeshObject* __restrict__ obj,
+                                                              int nobj, T* __restrict__ phi) {
   __shared__ int s_obj[MESH_LIST], s_nobj;
   __shared__ int s_open[MESH_WARPS][MESH_OPEN];          // undecided triangles of the warp's cell, object by object
   __shared__ int s_end[MESH_WARPS][MESH_LIST];           // where each object's end
@@ -183,7 +191,7 @@ __global__ void __launch_bounds__(32 * MESH_WARPS) k_mesh_phi(int nx, int ny, in
     const int src = __ffs(todo) - 1;
     const int ci = __shfl_sync(0xffffffffu, i, src), cj = __shfl_sync(0xffffffffu, j, src), ck = __shfl_sync(0xffffffffu, k, src);
     // bound the triangles over the cell
-    bool exact = all;                                // too much to list: test every triangle
+    bool exact = !TABLES || all;                     // too much to list: test every triangle
     int n = 0;
     for (int q = 0; q < n_obj && !exact; ++q) {
       const MeshObject& m = obj[s_obj[q]];
@@ -225,7 +233,15 @@ __global__ void __launch_bounds__(32 * MESH_WARPS) k_mesh_phi(int nx, int ny, in
         int cross = 0;
         if (exact) {
           if (box && holds(m, ci, cj, ck))
-            for (int f = 0; f < m.count; ++f) cross += te[m.entry + f].adet > 0.0 && ray_crosses(px, py, pz, te[m.entry + f]);
+            for (int f = 0; f < m.count; ++f) {
+              if (TABLES) {
+                cross += te[m.entry + f].adet > 0.0 && ray_crosses(px, py, pz, te[m.entry + f]);
+              } else {
+                MeshTri o;
+                mesh_tri(tri + 9 * ((size_t)m.first + f), o);
+                cross += o.adet > 0.0 && ray_crosses(px, py, pz, o);
+              }
+            }
         } else {
           const int end = s_end[warp][q];
           const unsigned int odd = s_odd[warp][q];
