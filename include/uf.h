@@ -418,9 +418,9 @@ typedef struct {
   int march_zc[UF_MAX_LEVELS];/* z planes per block of level l; 0 = automatic;
                                  otherwise even, 2..64 */
   int advect_zc;              /* z planes per block of the fused MacCormack
-                                 advection; 0 = automatic (16 at most: fewer
-                                 where the grid would leave SMs idle; reported
-                                 as 16), else 1..64 */
+                                 advection; 0 or 16 = automatic (16 at most:
+                                 fewer where the grid would leave SMs idle;
+                                 reported as 16), else 1..64 */
   int unfused;                /* bit mask of the step's fused kernels to run as
                                  their separate sub-step kernels instead:
                                  1 = the advection as its two passes

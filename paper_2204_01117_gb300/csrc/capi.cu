@@ -45,6 +45,7 @@ uf_status fail(uf_status s, const std::string& msg) {
 size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 int pitch_of(int lx) { return (int)round_up((size_t)lx, 32); }
 
+constexpr int kAdvectZc = 16;        // planes per block of the fused advection at most, unless tuned
 constexpr int kPartials = 8192;      // doubles per partials buffer
 constexpr int kDtBlocks = 1024;
 constexpr int kTargetBlocks = 2048;  // blocks of reducing cell kernels
@@ -978,8 +979,9 @@ class GridImpl final : public uf_grid {
   // rounding (the margin).
   bool advect_far() const { return d.fixed_dt > 0 || !(d.cfl <= 0.999); }
 
-  // Fused advection: 32 x 8 columns, zc planes per block.  Automatic: at most
-  // 16.  A block forms 1.7 planes' worth of halo besides its own (512 x 512 x
+  // Fused advection: 32 x 8 columns, zc planes per block.  Automatic (0, and
+  // kAdvectZc, under which get_tuning reports it: a grid that is set to its own
+  // tuning, as the autotuner does, keeps the choice): at most kAdvectZc.  A block forms 1.7 planes' worth of halo besides its own (512 x 512 x
   // 128: 2715 us at 1 plane, 1388 at 4, 1069 at 16), and a last wave that is
   // not full costs about half of what it leaves idle (256 x 256 x 64, 456
   // blocks resident: 12 planes = 2.99 waves 172 us, 16 = 2.25 waves 186 us;
@@ -991,7 +993,7 @@ class GridImpl final : public uf_grid {
     if (z <= 0) {
       const double resident = 152.0 * (sizeof(T) == 8 ? 1 : advect_far() ? 2 : UF_ADVECT_MINB);
       double best = 1e300;
-      for (int c : {16, 12, 8, 6, 4, 3, 2, 1}) {
+      for (int c : {kAdvectZc, 12, 8, 6, 4, 3, 2, 1}) {
         const double waves = (double)bx * by * d.nz / c / resident;
         const double cost = (1.0 + 1.7 / c) * (1.0 + 0.5 * (std::ceil(waves) / waves - 1.0));
         if (cost < best) { best = cost; z = c; }
@@ -1618,7 +1620,7 @@ class GridImpl final : public uf_grid {
       march_grid(l, &zc);
       t->march_zc[l] = d.precond == UF_PRECOND_MG ? zc : 0;
     }
-    t->advect_zc = advect_zc_tuned > 0 ? advect_zc_tuned : 16;
+    t->advect_zc = advect_zc_tuned > 0 ? advect_zc_tuned : kAdvectZc;
     t->unfused = unfused;
     t->coarse_start = use_sep() ? 0 : coarse_start() < P.tail_level ? coarse_start() : -1;
     if (levels) *levels = P.nl;
@@ -1636,7 +1638,7 @@ class GridImpl final : public uf_grid {
       if (t->coarse_start < -1 || t->coarse_start >= UF_MAX_LEVELS) return fail(UF_ERR_ARG, "coarse_start out of range");
     }
     drop_graphs();
-    advect_zc_tuned = t ? t->advect_zc : 0;
+    advect_zc_tuned = t && t->advect_zc != kAdvectZc ? t->advect_zc : 0;
     unfused = t ? t->unfused : 0;
     coarse_start_tuned = t ? t->coarse_start : 0;
     for (int l = 0; l < uf::MAX_LEVELS; ++l) march_zc_tuned[l] = t ? t->march_zc[l] : 0;

@@ -665,10 +665,10 @@ class Grid:
     def set_tuning(self, tail_level: int = 0, march_zc=None, advect_zc: int = 0, unfused: int = 0,
                    coarse_start: int = 0) -> None:
         """0 / None: automatic.  march_zc: per-level z planes per block;
-        advect_zc: z planes per block of the fused advection; unfused: bit
-        mask of fused kernels to run as their separate sub-step kernels
-        (1: advection, 2: diffusion + drag + BCs + pressure right-hand side;
-        True: all); coarse_start: 0 automatic (with the default smoother and
+        advect_zc: z planes per block of the fused advection (0 or 16:
+        automatic); unfused: bit mask of fused kernels to run as their
+        separate sub-step kernels (1: advection, 2: diffusion + drag + BCs +
+        pressure right-hand side; True: all); coarse_start: 0 automatic (with the default smoother and
         transfers, where the sizes allow: the separable inverse instead of
         the V-cycle), -1 the V-cycle with per-level launches, > 0 its first MG
         level in the one-launch cluster form.  Every choice gives the same
