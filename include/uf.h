@@ -505,10 +505,10 @@ uf_status uf_batch_launch_counts(uf_batch* b, int* fixed, int* per_iter);
 uf_status uf_batch_profile_step(uf_batch* b, uf_kernel_time* out, int capacity, int* count);
 
 /* Autotunes per size class: instances with the same number of multigrid
- * levels and cell counts within a factor sqrt(2) (one half-octave bin) share
- * one tuning, chosen by uf_autotune on the first of them; the batch graphs
- * are rebuilt.  classes: number of size classes
- * (may be NULL). */
+ * levels, the same transfers, cell counts within a factor sqrt(2) (one
+ * half-octave bin), and alike in whether the separable inverse is available
+ * to them, share one tuning, chosen by uf_autotune on the first of them; the
+ * batch graphs are rebuilt.  classes: number of size classes (may be NULL). */
 uf_status uf_batch_autotune(uf_batch* b, int reps, int* classes);
 
 uf_status uf_batch_destroy(uf_batch* b);

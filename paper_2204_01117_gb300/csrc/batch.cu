@@ -1059,10 +1059,12 @@ class BatchImpl final : public uf_batch {
     return UF_OK;
   }
 
-  // Size class: the number of multigrid levels and the cell count in
-  // half-octaves (grids within a factor sqrt(2) of each other share one).
+  // Size class: the number of multigrid levels, the cell count in
+  // half-octaves (grids within a factor sqrt(2) of each other share one), and
+  // what decides a grid's solver: whether it has the separable inverse (in use
+  // or not), and its transfers.
   static std::vector<int> size_class(const View<T>& G) {
-    return {G.nl, (int)std::floor(2.0 * std::log2(cells(G, 0)))};
+    return {G.nl, (int)std::floor(2.0 * std::log2(cells(G, 0))), G.sep.yf != nullptr, G.d.mg_transfer};
   }
 
   uf_status autotune(int reps, int* classes) override {
