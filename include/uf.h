@@ -431,7 +431,9 @@ typedef struct {
   int coarse_start;           /* 0 = automatic: grids with the default
                                  smoother (CHEBY) and transfers (LINEAR), nx <=
                                  1024 and, in FP32, ny <= 1392 and nz <= 400,
-                                 in FP64, ny + nz <= 480, run the exact
+                                 in FP64, ny + nz <= 480 and, past nz = 1, at
+                                 most 2^18 cells to a z plane (a row counted
+                                 in full multiples of 32), run the exact
                                  inverse of the operator (separation of
                                  variables: cosine transforms along y and z,
                                  tridiagonal solves along x) in place of the

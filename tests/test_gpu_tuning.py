@@ -73,3 +73,11 @@ def test_a_batch_does_not_share_a_tuning_across_solvers(order):
     for g in b.grids:
         g.init_state()
     b.run(2)
+
+
+# both sides of the rule that uf.h states for coarse_start = 0 (the edges of single axes: test_gpu_separable.py)
+@pytest.mark.parametrize("dims, precision, inverse", [((1024, 256, 4), "f64", True), ((1024, 257, 4), "f64", False),
+                                                      ((993, 257, 4), "f64", False), ((992, 264, 4), "f64", True),
+                                                      ((1024, 257, 1), "f64", True), ((1024, 991, 2), "f32", True)])
+def test_the_stated_size_rule(dims, precision, inverse):
+    assert uf.Grid(*dims, precision=precision).get_tuning()[0]["coarse_start"] == (0 if inverse else -1)
