@@ -201,17 +201,23 @@ def ncu_traffic(kernel_label: str):
     return None
 
 
-# labels of the kernels inside the CG loop of the default pressure solve
+# labels of the kernels inside the CG loop of the default pressure solve, and
+# of those outside the loop of any solve (a batch's have "b_" in front)
 LOOP_KERNELS = ("sep_y", "sep_x", "sep_zi", "sep_update", "cg_dir_q")
+STEP_KERNELS = ("cfl_dt", "eddy_viscosity", "advect_forward", "advect_backward", "advect_fused", "diffuse", "drag_bc",
+                "pressure_rhs", "momentum_fused", "begin_solve", "cg_init", "sep_init", "pressure_commit", "project",
+                "turbulence", "flip_parity")
 
 
 def loop_launches(name: str, n: int, prof_iters: int) -> int:
     """Launches per CG iteration of a kernel that ran n times in a step of
     prof_iters iterations (0: outside the loop; what n leaves over ran once
-    per step).  After a single iteration the count alone cannot tell."""
-    if prof_iters == 1:
-        return n if name in LOOP_KERNELS else 0
-    return n // prof_iters if prof_iters > 0 else 0
+    per step).  The labels decide where they can; of the others (a V-cycle's)
+    the count does, which cannot tell after a single iteration."""
+    label = name.removeprefix("b_")
+    if label in STEP_KERNELS or prof_iters < 1 or (prof_iters == 1 and label not in LOOP_KERNELS):
+        return 0
+    return n // prof_iters
 
 
 def dominant_kernel(kernels: dict, prof_iters: int, mean_iters: float):
