@@ -734,13 +734,14 @@ __device__ __forceinline__ double logistic(double t) { return 1.0 / (1.0 + exp(-
 // widths away.  (FP64 exp and division were what bounded both kernels; the
 // reverse one also added 3 terms per cell and box to shared memory with
 // FP64 atomics.)  Measured at 128 x 128 x 48 with 12 boxes, the map and its
-// transpose together: 11.8 -> 0.54 ms.
+// transpose together: 11.8 -> 0.58 ms.
 constexpr int DZ = 8;
 struct DesignTile {
   double xa[MAX_BOXES][BX], xb[MAX_BOXES][BX], ya[MAX_BOXES][BY], yb[MAX_BOXES][BY], z[MAX_BOXES][DZ];
-  unsigned int mask[2];
+  unsigned int mask[2];      // boxes that reach the tile
+  unsigned int far_mask[2];  // the others, whose chi is not zero throughout for all that
   int list[MAX_BOXES];
-  int n;   // boxes listed, in order
+  int n;   // boxes that reach, in order
 };
 __device__ __forceinline__ void design_tile(DesignTile& t, const DesignBoxes& boxes, int nbox, double h, double wdt, int i0, int j0,
                                             int k0) {
@@ -765,16 +766,20 @@ __device__ __forceinline__ void design_tile(DesignTile& t, const DesignBoxes& bo
   }
   __syncthreads();
   if (tid < MAX_BOXES) {
-    bool reaches = false;
+    bool reaches = false, far = false;
     if (tid < nbox) {
       double mx = 0.0, my = 0.0, mz = 0.0, s = 0.0;   // (s: not a number where any ramp is)
       for (int q = 0; q < BX; ++q) { const double v = t.xa[tid][q] * t.xb[tid][q]; mx = fmax(mx, v); s += v; }
       for (int q = 0; q < BY; ++q) { const double v = t.ya[tid][q] * t.yb[tid][q]; my = fmax(my, v); s += v; }
       for (int q = 0; q < DZ; ++q) { const double v = t.z[tid][q]; mz = fmax(mz, v); s += v; }
       reaches = s != s || mx * my * mz > 0x1p-55;
+      far = !reaches && mx > 0.0 && my > 0.0 && mz > 0.0;
     }
-    const unsigned int m = __ballot_sync(0xffffffffu, reaches);
-    if ((tid & 31) == 0) t.mask[tid >> 5] = m;
+    const unsigned int m = __ballot_sync(0xffffffffu, reaches), f = __ballot_sync(0xffffffffu, far);
+    if ((tid & 31) == 0) {
+      t.mask[tid >> 5] = m;
+      t.far_mask[tid >> 5] = f;
+    }
   }
   __syncthreads();
   if (tid < MAX_BOXES && (t.mask[tid >> 5] >> (tid & 31) & 1u)) {
@@ -810,7 +815,10 @@ __global__ void __launch_bounds__(NT) k_design_phi(int nx, int ny, int nz, int P
 // Vector-Jacobian product: g[3b + {0,1,2}] += sum_cells lphi dphi/d(H, dx, dy)_b.
 // dphi/dchi_b = -prod_{c != b} (1 - chi_c), from products over the boxes
 // before and after b; dchi/dtheta = chi (dlog s/dtheta).  A thread sums its DZ
-// cells, a warp its threads.
+// cells, a warp its threads.  A box that does not reach the tile has factors of
+// exactly 1 there, but its own chi is small, not zero: it drops out of the
+// products and keeps its term (where the tile has a sensitivity that is not
+// finite, also at chi = 0).
 template <typename T>
 __global__ void __launch_bounds__(NT) k_design_phi_vjp(int nx, int ny, int nz, int P, double h,
                                                        const __grid_constant__ DesignBoxes boxes, int nbox, double wdt,
@@ -820,15 +828,31 @@ __global__ void __launch_bounds__(NT) k_design_phi_vjp(int nx, int ny, int nz, i
   design_tile(t, boxes, nbox, h, wdt, i0, j0, k0);
   const int i = i0 + threadIdx.x, j = j0 + threadIdx.y, n = t.n;
   double lam[DZ], pre[DZ];
+  bool wild = false;   // a sensitivity that is not finite
 #pragma unroll
   for (int q = 0; q < DZ; ++q) {
     lam[q] = i < nx && j < ny && k0 + q < nz ? (double)lphi[(size_t)i + (size_t)P * ((size_t)j + (size_t)ny * (k0 + q))] : 0.0;
+    wild |= !isfinite(lam[q]);
     pre[q] = 1.0;   // product over the boxes before r
   }
+  // Adds box b's terms: s1 the thread's sum of (dphi/dchi lam) z over its cells, s2 that of (dphi/dchi lam) z (1 - z).
+  // The warp reduces the three together, halving what a lane holds, and divides once.
+  auto add = [&](int b, double s1, double s2) {
+    const double sxa = t.xa[b][threadIdx.x], sxb = t.xb[b][threadIdx.x], sya = t.ya[b][threadIdx.y], syb = t.yb[b][threadIdx.y];
+    const double a = sxa * sxb * sya * syb, sum = a * s1;
+    const double v0 = a * s2, v1 = sum * (-(1.0 - sxa) + (1.0 - sxb)), v2 = sum * (-(1.0 - sya) + (1.0 - syb));
+    const int lane = threadIdx.x;
+    const bool h = lane & 16, l = lane & 8;
+    const double p = (h ? v2 : v0) + __shfl_xor_sync(0xffffffffu, h ? v0 : v2, 16);
+    const double q = (h ? 0.0 : v1) + __shfl_xor_sync(0xffffffffu, h ? v1 : 0.0, 16);
+    double r = (l ? q : p) + __shfl_xor_sync(0xffffffffu, l ? p : q, 8);   // lanes 0.., 8.., 16..: of v0, v1, v2
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+    if ((lane & 7) == 0 && lane < 24 && r != 0.0) atomicAdd(&g[3 * b + (lane >> 3)], r / wdt);
+  };
   for (int r = 0; r < n; ++r) {
     const int b = t.list[r];
-    const double sxa = t.xa[b][threadIdx.x], sxb = t.xb[b][threadIdx.x], sya = t.ya[b][threadIdx.y], syb = t.yb[b][threadIdx.y];
-    const double a = sxa * sxb * sya * syb;
+    const double a = t.xa[b][threadIdx.x] * t.xb[b][threadIdx.x] * t.ya[b][threadIdx.y] * t.yb[b][threadIdx.y];
     double post[DZ];
 #pragma unroll
     for (int q = 0; q < DZ; ++q) post[q] = 1.0;
@@ -838,22 +862,31 @@ __global__ void __launch_bounds__(NT) k_design_phi_vjp(int nx, int ny, int nz, i
 #pragma unroll
       for (int q = 0; q < DZ; ++q) post[q] *= 1.0 - ac * t.z[bc][q];
     }
-    double sum = 0.0, sumz = 0.0;
+    double s1 = 0.0, s2 = 0.0;
 #pragma unroll
     for (int q = 0; q < DZ; ++q) {
-      const double sz = t.z[b][q], chi = a * sz;
-      const double base = lam[q] != 0.0 ? -(pre[q] * post[q]) * chi * lam[q] : 0.0;
-      sum += base;
-      sumz += base * (1.0 - sz);
-      pre[q] *= 1.0 - chi;
+      const double sz = t.z[b][q];
+      const double base = lam[q] != 0.0 ? -(pre[q] * post[q]) * lam[q] * sz : 0.0;
+      s1 += base;
+      s2 += base * (1.0 - sz);
+      pre[q] *= 1.0 - a * sz;
     }
-    double v[3] = {sumz / wdt, sum * (-(1.0 - sxa) + (1.0 - sxb)) / wdt, sum * (-(1.0 - sya) + (1.0 - syb)) / wdt};
+    add(b, s1, s2);
+  }
+  const bool all = __syncthreads_or(wild);
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
+  for (int q = 0; q < DZ; ++q) lam[q] = lam[q] != 0.0 ? -pre[q] * lam[q] : 0.0;
+  for (int b = 0; b < nbox; ++b) {
+    const unsigned int bit = 1u << (b & 31);
+    if (!((t.far_mask[b >> 5] & bit) || (all && !(t.mask[b >> 5] & bit)))) continue;
+    double s1 = 0.0, s2 = 0.0;
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v[d] += __shfl_xor_sync(0xffffffffu, v[d], o);
-      if (threadIdx.x == 0 && v[d] != 0.0) atomicAdd(&g[3 * b + d], v[d]);
+    for (int q = 0; q < DZ; ++q) {
+      const double sz = t.z[b][q], base = lam[q] * sz;
+      s1 += base;
+      s2 += base * (1.0 - sz);
     }
+    add(b, s1, s2);
   }
 }
 
