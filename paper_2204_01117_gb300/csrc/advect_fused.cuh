@@ -150,10 +150,10 @@ __device__ __forceinline__ void stage_plane(const AdvectArgs<T>& A, const StageP
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     if (kk < A.nz) {
-      if (S.ok[h] & 1) cp_async_elem(dst + h * MT, su + S.u[h]);
-      if (S.ok[h] & 2) cp_async_elem(dst + MFR * MWP + h * MT, sv + S.c[h]);
+      if (S.ok[h] & 1) cp_async_elem(dst + h * MT, UF_PTR(su + S.u[h], A.u, A.Lu.P, A.Lu.Ly, A.Lu.Lz, 1, BA_U));
+      if (S.ok[h] & 2) cp_async_elem(dst + MFR * MWP + h * MT, UF_PTR(sv + S.c[h], A.v, A.Lv.P, A.Lv.Ly, A.Lv.Lz, 1, BA_V));
     }
-    if (S.ok[h] & 4) cp_async_elem(dst + 2 * MFR * MWP + h * MT, sw + S.c[h]);
+    if (S.ok[h] & 4) cp_async_elem(dst + 2 * MFR * MWP + h * MT, UF_PTR(sw + S.c[h], A.w, A.Lw.P, A.Lw.Ly, A.Lw.Lz, 1, BA_CW));
   }
 }
 
@@ -315,6 +315,7 @@ __device__ __forceinline__ void tape_point(const AdvectArgs<T>& A, const Advance
   const bool ox = (gi >= M.i0 && gi < M.i0 + MX) || (gi >= M.i0 + MX && M.i0 + MX >= A.nx);
   const bool oy = (gj >= M.j0 && gj < M.j0 + MY) || (gj >= M.j0 + MY && M.j0 + MY >= A.ny);
   const bool oz = (m >= M.k0 && m < M.kend) || (m >= M.kend && M.kend == A.nz);
+  UF_BOUNDS(!(ox && oy && oz) || (gi < L.Lx && gj < L.Ly && m < L.Lz), BA_LATTICE, gi, gj, m);
   if (ox && oy && oz) tape[(size_t)gi + (size_t)L.P * ((size_t)gj + (size_t)L.Ly * m)] = val;
 }
 
@@ -436,7 +437,8 @@ __device__ __forceinline__ void maccormack_point(const AdvectArgs<T>& A, const A
                   K.d[1], K.d[2], M.s);
   const T fwd = adv_sm<T>(hc)[Q * CH], own = adv_sm<T>(f)[Q * CF];
   const T r = fwd + T(0.5) * (own - bwd);
-  (out_of<Q>(A) + (size_t)k * ((size_t)L.P * L.Ly))[gi + L.P * gj] = fmin(fmax(r, K.mn), K.mx);
+  *UF_PTR(out_of<Q>(A) + (size_t)k * ((size_t)L.P * L.Ly) + (gi + L.P * gj), out_of<Q>(A), L.P, L.Ly, L.Lz, 1, BA_LATTICE) =
+      fmin(fmax(r, K.mn), K.mx);
 }
 template <bool EDGE, bool FAR, typename T>
 __device__ __forceinline__ void maccormack_plane(const AdvectArgs<T>& A, const Advance<T>& M, const Places& X, int k,
@@ -458,7 +460,8 @@ __device__ __forceinline__ void eddy_point(const AdvectArgs<T>& A, const Advance
       A.sp, X.gi, X.gj, k, [&](int q, int dx, int dy, int dz) { return adv_sm<T>(dz == 0 ? fc : (dz < 0 ? fm : fp))[q * CF + dx + MWX * dy]; });
   const size_t plane = (size_t)k * ((size_t)A.Lw.P * A.Lw.Ly);   // (cells share the w lattice's rows)
   const int c = X.gi + A.Lw.P * X.gj;
-  (A.nut + plane)[c] = limited_nut(A.sp, (kf + plane)[c], (om + plane)[c], S2, cap);
+  auto cell = [&](auto* f) { return UF_PTR(f + plane + c, f, A.Lw.P, A.Lw.Ly, A.nz, 1, BA_CW); };
+  *cell(A.nut) = limited_nut(A.sp, *cell(kf), *cell(om), S2, cap);
 }
 
 // Pipeline per plane m of phi^:  wait for plane m+1 of the fields, sync,

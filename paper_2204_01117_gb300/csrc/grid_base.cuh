@@ -58,8 +58,9 @@ struct NvtxRange {
 
 // The message of a bounds-check record (UF_BOUNDS_CHECK builds).
 inline std::string bounds_text(const uf::BoundsHit& h) {
-  static const char* arrays[] = {"u lattice", "v lattice", "cell / w lattice", "multigrid level"};
-  return std::string("index out of its array: ") + (h.array >= 0 && h.array < 4 ? arrays[h.array] : "?") + " at (" +
+  static const char* arrays[] = {"u lattice", "v lattice", "cell / w lattice", "multigrid level", "velocity lattice",
+                                 "transform matrix"};
+  return std::string("index out of its array: ") + (h.array >= 0 && h.array < 6 ? arrays[h.array] : "?") + " at (" +
          std::to_string(h.i) + ", " + std::to_string(h.j) + ", " + std::to_string(h.k) + ")";
 }
 

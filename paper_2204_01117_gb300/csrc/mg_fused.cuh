@@ -1005,16 +1005,17 @@ __device__ __forceinline__ void cg_dir_q_body(const Level<T>& L, int zc, const T
   const T* __restrict__ dold = (it & 1) ? d1 : d0;
   T* __restrict__ dnew = (it & 1) ? d0 : d1;
   const T beta = it == 0 ? T(0) : (T)st->beta;
+  auto in_array = [&](auto* p, const T* base, int width) { return UF_PTR(p, base, L.P, L.ny, L.nz, width, BA_LEVEL); };
   auto dir = [&](size_t o) {
-    V a = *reinterpret_cast<const V*>(z + o);
+    V a = *reinterpret_cast<const V*>(in_array(z + o, z, N));
     if (it != 0) {
-      const V b = *reinterpret_cast<const V*>(dold + o);
+      const V b = *reinterpret_cast<const V*>(in_array(dold + o, dold, N));
 #pragma unroll
       for (int e = 0; e < N; ++e) a.e[e] = a.e[e] + beta * b.e[e];
     }
     return a;
   };
-  auto dir1 = [&](size_t o) { return it != 0 ? z[o] + beta * dold[o] : z[o]; };
+  auto dir1 = [&](size_t o) { return it != 0 ? *in_array(z + o, z, 1) + beta * *in_array(dold + o, dold, 1) : *in_array(z + o, z, 1); };
   const bool x0 = i0 > 0, y0 = j > 0, y1 = j < L.ny - 1;
   const bool left_of = in && x0 && lane == 0, right_of = in && left > N && lane == 31;   // beyond the warp
   size_t o = (size_t)k0 * PS + c;
@@ -1049,8 +1050,8 @@ __device__ __forceinline__ void cg_dir_q_body(const Level<T>& L, int zc, const T
         qv.e[e] = cell ? w : T(0);
         dacc.add(dv.e[e], qv.e[e]);
       }
-      *reinterpret_cast<V*>(dnew + o) = dv;
-      *reinterpret_cast<V*>(q + o) = qv;
+      *reinterpret_cast<V*>(in_array(dnew + o, dnew, N)) = dv;
+      *reinterpret_cast<V*>(in_array(q + o, q, N)) = qv;
     }
     dm = dc;
     dc = dp;

@@ -95,6 +95,7 @@ template <typename T>
 __device__ __forceinline__ void stage_momentum(const MomentumArgs<T>& M, const MView<T>& V, const StagePos& S, int kk) {
   const StepParams<T>& p = M.p;
   if (kk < 0 || kk > p.nz) return;
+  auto cell = [&](const T* at, const T* f) { return UF_PTR(at, f, p.Pc, p.ny, p.nz, 1, BA_CW); };
   T* dst = mom_sm<T>(V.D(0, kk)) + threadIdx.x;
   const size_t pc = (size_t)kk * ((size_t)p.Pc * p.ny);
   const T* su = M.ut + (size_t)kk * ((size_t)p.Pu * p.ny);
@@ -104,14 +105,14 @@ __device__ __forceinline__ void stage_momentum(const MomentumArgs<T>& M, const M
   for (int h = 0; h < 2; ++h) {
     T* d = dst + h * MT;
     if (kk < p.nz) {
-      if (S.ok[h] & 1) cp_async_elem(d + DF_U * DR * MWP, su + S.u[h]);
-      if (S.ok[h] & 2) cp_async_elem(d + DF_V * DR * MWP, sv + S.c[h]);
+      if (S.ok[h] & 1) cp_async_elem(d + DF_U * DR * MWP, UF_PTR(su + S.u[h], M.ut, p.Pu, p.ny, p.nz, 1, BA_U));
+      if (S.ok[h] & 2) cp_async_elem(d + DF_V * DR * MWP, UF_PTR(sv + S.c[h], M.vt, p.Pc, p.ny + 1, p.nz, 1, BA_V));
       if (S.ok[h] & 4) {
-        cp_async_elem(d + DF_NUT * DR * MWP, sn + S.c[h]);
-        cp_async_elem(d + DF_C * DR * MWP, sc + S.c[h]);
+        cp_async_elem(d + DF_NUT * DR * MWP, cell(sn + S.c[h], M.nut));
+        cp_async_elem(d + DF_C * DR * MWP, cell(sc + S.c[h], M.cc));
       }
     }
-    if (S.ok[h] & 4) cp_async_elem(d + DF_W * DR * MWP, sw + S.c[h]);
+    if (S.ok[h] & 4) cp_async_elem(d + DF_W * DR * MWP, UF_PTR(sw + S.c[h], M.wt, p.Pc, p.ny, p.nz + 1, 1, BA_CW));
   }
 }
 
@@ -309,6 +310,8 @@ __device__ __forceinline__ void u3_plane(const MomentumArgs<T>& M, const MView<T
   T* gu = M.u + (size_t)k * ((size_t)p.Pu * p.ny);
   T* gv = M.v + (size_t)k * ((size_t)p.Pc * (p.ny + 1));
   T* gw = M.w + (size_t)(k + 1) * ((size_t)p.Pc * p.ny);
+  auto U = [&](T* at) { return UF_PTR(at, M.u, p.Pu, p.ny, p.nz, 1, BA_U); };
+  auto VV = [&](T* at) { return UF_PTR(at, M.v, p.Pc, p.ny + 1, p.nz, 1, BA_V); };
   const bool own_w = k + 1 < V.kend || k + 1 == p.nz;
   const T prof = EDGE && k >= 0 ? p.prof[k] : T(0);
   // x face (i, j) and y face (i, j): places h, b; a boundary face follows its rule on the dragged interior neighbour
@@ -326,32 +329,32 @@ __device__ __forceinline__ void u3_plane(const MomentumArgs<T>& M, const MView<T
   const bool in_x = !EDGE || gi < p.nx, in_y = !EDGE || gj < p.ny;
   if (in_x && in_y) {
     own[2] = EDGE && (k + 1 == 0 || k + 1 == p.nz) ? T(0) : w3_inner(V, dt, X.h, X.b, k + 1);
-    if (own_w) gw[gi + p.Pc * gj] = own[2];
+    if (own_w) *UF_PTR(gw + (gi + p.Pc * gj), M.w, p.Pc, p.ny, p.nz + 1, 1, BA_CW) = own[2];
   }
   if (only_w) return;
   if (!EDGE || (gi <= p.nx && in_y)) {
     own[0] = xface(X.h, X.b, gi);
     sU[tx + (MX + 1) * ty] = own[0];
-    gu[gi + p.Pu * gj] = own[0];
+    *U(gu + (gi + p.Pu * gj)) = own[0];
   }
   if (!EDGE || (in_x && gj <= p.ny)) {
     own[1] = yface(X.h, X.b, gj);
     sV[t] = own[1];
-    gv[gi + p.Pc * gj] = own[1];
+    *VV(gv + (gi + p.Pc * gj)) = own[1];
   }
   if (t < MX) {
     const int j = V.j0 + MY;
     if (!EDGE || (in_x && j <= p.ny)) {
       const T val = yface(X.h + MHX * MY, X.b + MWX * MY, j);
       sV[t + MT] = val;
-      if (EDGE && j == p.ny) gv[gi + p.Pc * j] = val;
+      if (EDGE && j == p.ny) *VV(gv + (gi + p.Pc * j)) = val;
     }
   } else if (t < MX + MY) {
     const int i = V.i0 + MX, j = V.j0 + tx;
     if (!EDGE || (i <= p.nx && j < p.ny)) {
       const T val = xface(MX + 1 + MHX * (tx + 1), MX + 2 + MWX * (tx + 2), i);
       sU[MX + (MX + 1) * tx] = val;
-      if (EDGE && i == p.nx) gu[i + p.Pu * j] = val;
+      if (EDGE && i == p.nx) *U(gu + (i + p.Pu * j)) = val;
     }
   }
 }
@@ -396,7 +399,7 @@ __device__ __forceinline__ void momentum_fused_body(const MomentumArgs<T>& M, co
     // cell_flux: u(i+1)-u(i) + v(j+1)-v(j) + w(k+1)-w(k)
     const T flux = V.sU3()[(tx + 1) + (MX + 1) * ty] - own[0] + V.sV3()[tx + MX * (ty + 1)] - own[1] + own[2] - w3lo;
     const T bv = sc * flux;
-    (M.b + (size_t)k * ((size_t)p.Pc * p.ny))[X.gi + p.Pc * X.gj] = bv;
+    *UF_PTR(M.b + (size_t)k * ((size_t)p.Pc * p.ny) + (X.gi + p.Pc * X.gj), M.b, p.Pc, p.ny, p.nz, 1, BA_CW) = bv;
     dacc.add(bv, bv);
     w3lo = own[2];
   };

@@ -98,6 +98,12 @@ struct SepAxis {
   __host__ __device__ int rows() const { return pad(0) + pad(1); }
 };
 template <typename T>
+__host__ __device__ inline size_t sep_block_count(int n) {   // elements of Sep<T>::Mat of an n x n matrix
+  return sizeof(T) == 4 ? (size_t)((n + 15) / 16) * ((n + 7) / 8) * 32 : (size_t)n * ((n + 1) & ~1);
+}
+template <typename T>
+__host__ __device__ inline size_t sep_mat_count(const SepAxis& x) { return sep_block_count<T>(x.size(0)) + sep_block_count<T>(x.size(1)); }
+template <typename T>
 __host__ __device__ inline SepAxis sep_axis_y(const Level<T>& L) { return {L.ny, !(L.out_mask & 12)}; }
 template <typename T>
 __host__ __device__ inline SepAxis sep_axis_z(const Level<T>& L) { return {L.nz, !(L.out_mask & 48)}; }
@@ -145,15 +151,19 @@ __device__ __forceinline__ void sep_put2(float* o, float a, float b) { *reinterp
 __device__ __forceinline__ void sep_put2(double* o, double a, double b) { *reinterpret_cast<double2*>(o) = make_double2(a, b); }
 __device__ __forceinline__ float2 sep_get2(const float* o) { return *reinterpret_cast<const float2*>(o); }
 __device__ __forceinline__ double2 sep_get2(const double* o) { return *reinterpret_cast<const double2*>(o); }
+// A pointer into a cell array of the grid (UF_PTR).
+#define SEP_PTR(p, base, L, width) UF_PTR(p, base, (L).P, (L).ny, (L).nz, width, BA_LEVEL)
 // Results of a transform to rows of `pitch` values, `cols` columns of them.
 template <typename T>
 struct SepStore {
   T* __restrict__ dst;
   size_t pitch;
   long long cols;
+  const Level<T>* L;   // (the array dst points into)
+  const T* base;
   __device__ __forceinline__ int fetch(int, int) const { return 0; }
   __device__ __forceinline__ void operator()(int row, int col, T a, T b, int) const {
-    if (col < cols) sep_put2(dst + row * pitch + col, a, b);
+    if (col < cols) sep_put2(SEP_PTR(dst + row * pitch + col, base, *L, 2), a, b);
   }
 };
 
@@ -198,15 +208,19 @@ struct SepQueue {
   int slot = 0, i = 0, at = 0, KT;
   const float4* a[TILES];
   Seg seg;
-  __device__ __forceinline__ SepQueue(void* queue, int depth_, Seg seg_)
-      : slots(reinterpret_cast<float4*>(queue) + threadIdx.x), depth(depth_), seg(seg_) {
+  const float4* A;   // the axis' matrices
+  const SepAxis x;
+  __device__ __forceinline__ SepQueue(void* queue, int depth_, Seg seg_, const float4* A_, const SepAxis& x_)
+      : slots(reinterpret_cast<float4*>(queue) + threadIdx.x), depth(depth_), seg(seg_), A(A_), x(x_) {
     KT = seg(0, a);
     for (int p = 0; p < depth; ++p) fill(p);
   }
   __device__ __forceinline__ void fill(int to) {
     if (at < KT) {
 #pragma unroll
-      for (int h = 0; h < TILES; ++h) sep_copy_tile(slots + to * (SEP_SLOT / 16) + h * SEP_T, a[h] + (size_t)at * 32);
+      for (int h = 0; h < TILES; ++h)
+        sep_copy_tile(slots + to * (SEP_SLOT / 16) + h * SEP_T,
+                      UF_PTR(a[h] + (size_t)at * 32, A, 32, 1, (long long)(sep_mat_count<float>(x) / 32), 1, BA_MATRIX));
       if (++at == KT) {
         at = 0;
         KT = seg(++i, a);
@@ -280,7 +294,7 @@ __device__ __forceinline__ void sep_gemm(const float4* __restrict__ A, const Sep
     a[1] = m0 * 16 + 16 < x.size(odd) ? a[0] + (size_t)KT * 32 : a[0];
     return KT;
   };
-  SepQueue<2, decltype(seg)> queue(sB + x.rows() * PB, sep_queue(WN, x), seg);
+  SepQueue<2, decltype(seg)> queue(sB + x.rows() * PB, sep_queue(WN, x), seg, A, x);
   panel();
   __syncthreads();
   for (int u = part + parts * wm; u < un; u += WM * parts) {
@@ -318,7 +332,7 @@ __device__ __forceinline__ void sep_gemm_back(const float4* __restrict__ A, cons
     a[0] = A + ((odd ? (size_t)((Me + 15) / 16) * KE : 0) + (size_t)m * (odd ? KO : KE)) * 32 + lane;
     return odd ? KO : KE;
   };
-  SepQueue<1, decltype(seg)> queue(sB + x.rows() * PB, sep_queue(WN, x), seg);
+  SepQueue<1, decltype(seg)> queue(sB + x.rows() * PB, sep_queue(WN, x), seg, A, x);
   panel();
   __syncthreads();
   const float* b = sB + t * PB + wn * 32 + g;
@@ -354,7 +368,7 @@ __device__ __forceinline__ void sep_fma(double (&c)[4], const double* __restrict
   const double* a = A + (row < M ? row : 0);
 #pragma unroll 4
   for (int k = 0; k < M; ++k) {
-    const double2 av = __ldg(reinterpret_cast<const double2*>(a + (size_t)k * MP));
+    const double2 av = __ldg(reinterpret_cast<const double2*>(UF_PTR(a + (size_t)k * MP, A, MP, M, 1, 2, BA_MATRIX)));
     const double2 bv = *reinterpret_cast<const double2*>(b + k * 32);
     c[0] = fma(av.x, bv.x, c[0]);
     c[1] = fma(av.x, bv.y, c[1]);
@@ -432,13 +446,13 @@ __device__ __forceinline__ void sep_panel(T* sm, const SepAxis& x, int row0, int
 // thread's columns lies at from + i pitch, and counts where `in`.)
 template <typename T, int PB>
 __device__ __forceinline__ void sep_panel_back(T* sm, const SepAxis& x, int row0, int step, int col0, const T* from, size_t pitch,
-                                               bool in) {
+                                               bool in, const Level<T>& L, const T* base) {
   const int pe = x.pad(0), rows = x.rows();
 #pragma unroll 2
   for (int k = row0; k < rows; k += step) {
     const int odd = k >= pe, m = odd ? k - pe : k;
     const bool on = in && m < x.size(odd);
-    sep_copy16(sm + k * PB + col0, from + (on ? (size_t)(x.fold ? 2 * m + odd : m) * pitch : 0), on);
+    sep_copy16(sm + k * PB + col0, SEP_PTR(from + (on ? (size_t)(x.fold ? 2 * m + odd : m) * pitch : 0), base, L, Vec16<T>::N), on);
   }
   sep_copies_commit();
   sep_copies_wait<0>();
@@ -478,13 +492,13 @@ __device__ __forceinline__ void sep_zf(const Level<T>& L, const Sep<T>& S, const
   constexpr int WN = SEP_Z_WN<T>, PB = SEP_PITCH<T, WN>;
   if (C.flat) {
     const V v = get(0);
-    if (C.in) *reinterpret_cast<V*>(S.t + C.c) = v;
+    if (C.in) *reinterpret_cast<V*>(SEP_PTR(S.t + C.c, S.t, L, V::N)) = v;
     return;
   }
   const SepAxis ax = sep_axis_z(L);
   auto panel = [&] { sep_panel<T, PB, UNROLL>(sep_sm, ax, C.row0, SEP_T / C.VR, C.col0, get); };
   const size_t cb = (size_t)vb.x * 32 * WN;
-  sep_gemm<WN>(S.zf, ax, sep_sm, 0, 1, panel, SepStore<T>{S.t + cb, C.PS, (long long)(C.PS - cb)});
+  sep_gemm<WN>(S.zf, ax, sep_sm, 0, 1, panel, SepStore<T>{S.t + cb, C.PS, (long long)(C.PS - cb), &L, S.t});
 }
 
 __device__ __forceinline__ float sep_diff(float2 a, float2 b) { return ps_diff(a, b); }
@@ -500,17 +514,19 @@ __device__ __forceinline__ Vec16<T> sep_apply(const Level<T>& L, const SepCols<T
   constexpr int N = Vec16<T>::N;
   struct alignas(16) Row { E e[N]; };
   const int i0 = L.nx - C.left_x, j = (int)(C.c / L.P);
+  const E* __restrict__ f0 = f;
   f += (size_t)k * C.PS + C.c;
+  auto row = [&](const E* at) { return *reinterpret_cast<const Row*>(SEP_PTR(at, f0, L, N)); };
   const bool y0 = j > 0, y1 = j < L.ny - 1, z0 = k > 0, z1 = k < L.nz - 1;
-  const Row m = *reinterpret_cast<const Row*>(f);
+  const Row m = row(f);
   Row ym = m, yp = m, zm = m, zp = m;
   E xm = m.e[0], xp = m.e[N - 1];
-  if (y0) ym = *reinterpret_cast<const Row*>(f - L.P);
-  if (y1) yp = *reinterpret_cast<const Row*>(f + L.P);
-  if (z0) zm = *reinterpret_cast<const Row*>(f - C.PS);
-  if (z1) zp = *reinterpret_cast<const Row*>(f + C.PS);
-  if (i0 > 0) xm = f[-1];
-  if (C.left_x > N) xp = f[N];
+  if (y0) ym = row(f - L.P);
+  if (y1) yp = row(f + L.P);
+  if (z0) zm = row(f - C.PS);
+  if (z1) zp = row(f + C.PS);
+  if (i0 > 0) xm = *SEP_PTR(f - 1, f0, L, 1);
+  if (C.left_x > N) xp = *SEP_PTR(f + N, f0, L, 1);
   Vec16<T> a;
 #pragma unroll
   for (int e = 0; e < N; ++e) {
@@ -546,7 +562,7 @@ __device__ __forceinline__ void sep_init_body(const Level<T>& L, const Sep<T>& S
     if (!C.in) return v;
     const size_t o = (size_t)k * C.PS + C.c;
     if (!zero_rhs) {
-      const V bv = *reinterpret_cast<const V*>(b + o);
+      const V bv = *reinterpret_cast<const V*>(SEP_PTR(b + o, b, L, V::N));
       const V a = g ? sep_apply(L, C, g, k) : sep_apply(L, C, (const T*)x, k);
 #pragma unroll
       for (int e = 0; e < V::N; ++e) {
@@ -554,8 +570,8 @@ __device__ __forceinline__ void sep_init_body(const Level<T>& L, const Sep<T>& S
         dacc.add(v.e[e], v.e[e]);
       }
     }
-    if (zero_rhs || g) *reinterpret_cast<V*>(x + o) = V{};
-    *reinterpret_cast<V*>(L.r + o) = v;
+    if (zero_rhs || g) *reinterpret_cast<V*>(SEP_PTR(x + o, x, L, V::N)) = V{};
+    *reinterpret_cast<V*>(SEP_PTR(L.r + o, L.r, L, V::N)) = v;
     return v;
   });
   const double vals[1] = {block_sum<SEP_T>(dacc.value(), sh)};
@@ -587,18 +603,18 @@ __device__ __forceinline__ void sep_update_body(const Level<T>& L, const Sep<T>&
     V v = {};
     if (!C.in) return v;
     const size_t o = (size_t)k * C.PS + C.c;
-    v = *reinterpret_cast<const V*>(L.r + o);
-    const V qv = *reinterpret_cast<const V*>(q + o);
-    const V dv = *reinterpret_cast<const V*>(dn + o);
-    V xv = *reinterpret_cast<const V*>(x + o);
+    v = *reinterpret_cast<const V*>(SEP_PTR(L.r + o, L.r, L, V::N));
+    const V qv = *reinterpret_cast<const V*>(SEP_PTR(q + o, q, L, V::N));
+    const V dv = *reinterpret_cast<const V*>(SEP_PTR(dn + o, dn, L, V::N));
+    V xv = *reinterpret_cast<const V*>(SEP_PTR(x + o, x, L, V::N));
 #pragma unroll
     for (int e = 0; e < V::N; ++e) {
       v.e[e] = e < C.left_x ? v.e[e] - alpha * qv.e[e] : T(0);
       xv.e[e] = e < C.left_x ? xv.e[e] + alpha * dv.e[e] : T(0);
       dacc.add(v.e[e], v.e[e]);
     }
-    *reinterpret_cast<V*>(L.r + o) = v;
-    *reinterpret_cast<V*>(x + o) = xv;
+    *reinterpret_cast<V*>(SEP_PTR(L.r + o, L.r, L, V::N)) = v;
+    *reinterpret_cast<V*>(SEP_PTR(x + o, x, L, V::N)) = xv;
     return v;
   });
   const double vals[1] = {block_sum<SEP_T>(dacc.value(), sh)};
@@ -620,11 +636,13 @@ struct SepStoreDot {
   size_t pitch;
   long long cols;
   DotAcc<T>* dot;
+  const Level<T>* L;   // (the arrays r and z point into)
+  const T *r0, *z0;
   using Pair = decltype(sep_get2((const T*)nullptr));
-  __device__ __forceinline__ Pair fetch(int row, int col) const { return col < cols ? sep_get2(r + row * pitch + col) : Pair{}; }
+  __device__ __forceinline__ Pair fetch(int row, int col) const { return col < cols ? sep_get2(SEP_PTR(r + row * pitch + col, r0, *L, 2)) : Pair{}; }
   __device__ __forceinline__ void operator()(int row, int col, T a, T b, Pair rv) const {
     if (col >= cols) return;
-    sep_put2(z + row * pitch + col, a, b);
+    sep_put2(SEP_PTR(z + row * pitch + col, z0, *L, 2), a, b);
     dot->add(rv.x, a);
     dot->add(rv.y, b);
   }
@@ -647,16 +665,16 @@ __device__ __forceinline__ void sep_zi_body(const Level<T>& L, const Sep<T>& S, 
   DotAcc<T> dacc;
   if (flat) {
     if (c < PS) {
-      const V v = *reinterpret_cast<const V*>(S.t + c);
-      const SepStoreDot<T> put{L.r + c, z + c, PS, V::N, &dacc};
+      const V v = *reinterpret_cast<const V*>(SEP_PTR(S.t + c, S.t, L, V::N));
+      const SepStoreDot<T> put{L.r + c, z + c, PS, V::N, &dacc, &L, L.r, z};
 #pragma unroll
       for (int e = 0; e < V::N; e += 2) put(0, e, v.e[e], v.e[e + 1], put.fetch(0, e));
     }
   } else {
     const SepAxis ax = sep_axis_z(L);
-    auto panel = [&] { sep_panel_back<T, PB>(sep_sm, ax, threadIdx.x / VR, SEP_T / VR, col0, S.t + (c < PS ? c : 0), PS, c < PS); };
+    auto panel = [&] { sep_panel_back<T, PB>(sep_sm, ax, threadIdx.x / VR, SEP_T / VR, col0, S.t + (c < PS ? c : 0), PS, c < PS, L, S.t); };
     const size_t cb = (size_t)vb.x * BN;
-    sep_gemm_back<WN>(S.zi, ax, sep_sm, 0, 1, panel, SepStoreDot<T>{L.r + cb, z + cb, PS, (long long)(PS - cb), &dacc});
+    sep_gemm_back<WN>(S.zi, ax, sep_sm, 0, 1, panel, SepStoreDot<T>{L.r + cb, z + cb, PS, (long long)(PS - cb), &dacc, &L, L.r, z});
   }
   const double vals[1] = {block_sum<SEP_T>(dacc.value(), sh)};
   if (publish_partials<1>(partials, &st->ticket[0], vals, &last, vb)) {
@@ -682,16 +700,18 @@ __device__ __forceinline__ void sep_y_panel(const Level<T>& L, const Sep<T>& S, 
   const int x0 = vb.x * BN, xv = V::N * (threadIdx.x % VR), row0 = threadIdx.x / VR;
   const size_t base = (size_t)vb.z * L.P * L.ny + x0;
   const bool in = x0 + xv < L.P;
-  const T* __restrict__ src = (INVERSE ? S.u : S.t) + base;
-  T* __restrict__ dst = (INVERSE ? S.t : S.u) + base;
+  const T* __restrict__ from = INVERSE ? S.u : S.t;
+  T* __restrict__ to = INVERSE ? S.t : S.u;
+  const T* __restrict__ src = from + base;
+  T* __restrict__ dst = to + base;
   auto get = [&](int j) {
     V v = {};
-    if (in) v = *reinterpret_cast<const V*>(src + (size_t)j * L.P + xv);
+    if (in) v = *reinterpret_cast<const V*>(SEP_PTR(src + (size_t)j * L.P + xv, from, L, V::N));
     return v;
   };
-  const SepStore<T> put{dst, (size_t)L.P, L.P - x0};
+  const SepStore<T> put{dst, (size_t)L.P, L.P - x0, &L, to};
   if (INVERSE) {
-    auto panel = [&] { sep_panel_back<T, PB>(sep_sm, ax, row0, SEP_T / VR, xv, src + (in ? xv : 0), (size_t)L.P, in); };
+    auto panel = [&] { sep_panel_back<T, PB>(sep_sm, ax, row0, SEP_T / VR, xv, src + (in ? xv : 0), (size_t)L.P, in, L, from); };
     sep_gemm_back<WN>(S.yi, ax, sep_sm, vb.y, split, panel, put);
   } else {
     auto panel = [&] { sep_panel<T, PB, 4>(sep_sm, ax, row0, SEP_T / VR, xv, get); };
@@ -803,8 +823,8 @@ __device__ __forceinline__ void sep_x_body(const Level<T>& L, const Sep<T>& S, c
   if (st->converged) return;
   const int line = vb.x * SEP_X_LINES + (threadIdx.x >> 5);
   if (line >= L.ny * L.nz) return;
-  T* row = S.u + (size_t)line * L.P;
-  const T* piv = S.piv + (size_t)line * L.P;
+  T* row = SEP_PTR(S.u + (size_t)line * L.P, S.u, L, L.P);
+  const T* piv = SEP_PTR(S.piv + (size_t)line * L.P, S.piv, L, L.P);
   if (L.P <= 64) sep_x_line<2>(row, piv, L.P);
   else if (L.P <= 128) sep_x_line<4>(row, piv, L.P);
   else if (L.P <= 256) sep_x_line<8>(row, piv, L.P);
@@ -854,12 +874,6 @@ __device__ __forceinline__ double sep_eig(int m, int n, bool out_lo, bool out_hi
   const double s = (!out_lo && !out_hi) ? sinpi(m / (2.0 * n)) : sinpi((2 * m + 1) / (2.0 * (2 * n + 1)));
   return 4.0 * s * s;
 }
-template <typename T>
-__host__ __device__ inline size_t sep_block_count(int n) {   // elements of Sep<T>::Mat of an n x n matrix
-  return sizeof(T) == 4 ? (size_t)((n + 15) / 16) * ((n + 7) / 8) * 32 : (size_t)n * ((n + 1) & ~1);
-}
-template <typename T>
-__host__ __device__ inline size_t sep_mat_count(const SepAxis& x) { return sep_block_count<T>(x.size(0)) + sep_block_count<T>(x.size(1)); }
 // Matrices of an axis: forward (row mode, column cell) or transposed.  The
 // halves of a folded axis: modes 0, 2, .. and 1, 3, .. at its first cells.
 template <typename T>
@@ -891,7 +905,7 @@ __global__ void k_sep_pivots(Level<T> L, T* piv) {
   if (line >= L.ny * L.nz) return;
   const double lam = sep_eig(line % L.ny, L.ny, L.out_mask & 4, L.out_mask & 8) +
                      sep_eig(line / L.ny, L.nz, L.out_mask & 16, L.out_mask & 32);
-  T* row = piv + (size_t)line * L.P;
+  T* row = SEP_PTR(piv + (size_t)line * L.P, piv, L, L.P);
   double e = 0.0;
   for (int i = 0; i < L.nx; ++i) {
     double d = 2.0 + lam;

@@ -141,12 +141,14 @@ __device__ __forceinline__ void cg_init_body(const Level<T>& L, const T* __restr
     const PStore<T>* gp = g + c;
     T* __restrict__ r = L.r;
     const bool x0 = i > 0, x1 = i < L.nx - 1, y0 = j > 0, y1 = j < L.ny - 1;
-    PStore<T> gm = z0 > 0 ? *(gp - SZ) : gp[0], gc = gp[0];
+    auto G = [&](const PStore<T>* at) { return *UF_PTR(at, g, L.P, L.ny, L.nz, 1, BA_LEVEL); };
+    auto cell = [&](auto* p) { return UF_PTR(p + c, p, L.P, L.ny, L.nz, 1, BA_LEVEL); };
+    PStore<T> gc = G(gp), gm = z0 > 0 ? G(gp - SZ) : gc;
 #pragma unroll 2
     for (int k = z0; k < z1; ++k) {
-      const PStore<T> gxm = x0 ? *(gp - 1) : gc, gxp = x1 ? gp[1] : gc, gym = y0 ? *(gp - SY) : gc, gyp = y1 ? gp[SY] : gc;
-      const PStore<T> gn = k < L.nz - 1 ? gp[SZ] : gc;
-      const T bv = b[c], xc = (T)ps_value(gc);
+      const PStore<T> gxm = x0 ? G(gp - 1) : gc, gxp = x1 ? G(gp + 1) : gc, gym = y0 ? G(gp - SY) : gc, gyp = y1 ? G(gp + SY) : gc;
+      const PStore<T> gn = k < L.nz - 1 ? G(gp + SZ) : gc;
+      const T bv = *cell(b), xc = (T)ps_value(gc);
       T ax = 0;
       if (x0) ax += L.wx * (T)ps_diff(gc, gxm); else if (L.out_mask & 1) ax += L.wx * xc;
       if (x1) ax += L.wx * (T)ps_diff(gc, gxp); else if (L.out_mask & 2) ax += L.wx * xc;
@@ -155,8 +157,8 @@ __device__ __forceinline__ void cg_init_body(const Level<T>& L, const T* __restr
       if (k > 0) ax += L.wz * (T)ps_diff(gc, gm); else if (L.out_mask & 16) ax += L.wz * xc;
       if (k < L.nz - 1) ax += L.wz * (T)ps_diff(gc, gn); else if (L.out_mask & 32) ax += L.wz * xc;
       const T rv = bv - ax;
-      x[c] = T(0);
-      r[c] = rv;
+      *cell(x) = T(0);
+      *cell(r) = rv;
       dacc.add(rv, rv);
       gm = gc;
       gc = gn;

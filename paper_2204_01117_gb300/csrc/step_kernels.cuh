@@ -219,6 +219,8 @@ __device__ __forceinline__ T trilerp(const T (&f)[8], T ta, T tb, T tc, T* mn, T
 template <typename T>
 __device__ __forceinline__ void corners_global(const T* __restrict__ F, Lattice L, int i0, int i1, int j0, int j1,
                                                int k0, int k1, T (&f)[8]) {
+  UF_BOUNDS(i0 >= 0 && i0 < L.Lx && j0 >= 0 && j0 < L.Ly && k0 >= 0 && k0 < L.Lz, BA_LATTICE, i0, j0, k0);
+  UF_BOUNDS(i1 >= 0 && i1 < L.Lx && j1 >= 0 && j1 < L.Ly && k1 >= 0 && k1 < L.Lz, BA_LATTICE, i1, j1, k1);
   const size_t r00 = (size_t)L.P * ((size_t)j0 + (size_t)L.Ly * k0);
   const size_t r10 = (size_t)L.P * ((size_t)j1 + (size_t)L.Ly * k0);
   const size_t r01 = (size_t)L.P * ((size_t)j0 + (size_t)L.Ly * k1);
@@ -273,7 +275,10 @@ struct AdvectArgs {
 // pair counts twice (the sample clamps).
 template <typename T>
 __device__ __forceinline__ void displacement(const AdvectArgs<T>& A, int q, int i, int j, int k, T s, T d[3]) {
-  auto at = [&](const T* F, const Lattice& L, int a, int b, int c) { return F[(size_t)a + (size_t)L.P * ((size_t)b + (size_t)L.Ly * c)]; };
+  auto at = [&](const T* F, const Lattice& L, int a, int b, int c) {
+    UF_BOUNDS(a >= 0 && a < L.Lx && b >= 0 && b < L.Ly && c >= 0 && c < L.Lz, BA_LATTICE, a, b, c);
+    return F[(size_t)a + (size_t)L.P * ((size_t)b + (size_t)L.Ly * c)];
+  };
   auto u2 = [&](int a, int b, int c) { return add_rn(at(A.u, A.Lu, a, b, c), at(A.u, A.Lu, a + 1, b, c)); };
   auto v2 = [&](int a, int b, int c) { return add_rn(at(A.v, A.Lv, a, b, c), at(A.v, A.Lv, a, b + 1, c)); };
   auto w2 = [&](int a, int b, int c) { return add_rn(at(A.w, A.Lw, a, b, c), at(A.w, A.Lw, a, b, c + 1)); };
@@ -669,6 +674,10 @@ __device__ __forceinline__ void project_cells_body(const StepParams<T>& p, const
   T* pu = u + ((size_t)k0 * ((size_t)p.Pu * ny) + i + (size_t)p.Pu * j);
   T* pv = v + ((size_t)k0 * ((size_t)p.Pc * (ny + 1)) + i + (size_t)p.Pc * j);
   T* pw = w + c;
+  auto P = [&](const PStore<T>* at) { return *UF_PTR(at, pr, p.Pc, ny, nz, 1, BA_CW); };
+  auto U = [&](T* at) { return UF_PTR(at, u, p.Pu, ny, nz, 1, BA_U); };
+  auto V = [&](T* at) { return UF_PTR(at, v, p.Pc, ny + 1, nz, 1, BA_V); };
+  auto W = [&](T* at) { return UF_PTR(at, w, p.Pc, ny, nz + 1, 1, BA_CW); };
   PStore<T> here[PROJ_ZC], xm[PROJ_ZC], ym[PROJ_ZC], zm[PROJ_ZC];
   T uo[PROJ_ZC], vo[PROJ_ZC], wo[PROJ_ZC];
 #pragma unroll
@@ -678,13 +687,13 @@ __device__ __forceinline__ void project_cells_body(const StepParams<T>& p, const
     here[q] = xm[q] = ym[q] = zm[q] = ps_from(T(0));   // (the ghost cell beyond an outlet: p = 0)
     uo[q] = vo[q] = wo[q] = T(0);
     const PStore<T>* pc = pr + c + (size_t)q * sc;
-    if (on && cell) here[q] = pc[0];
-    if (on && fx && i > 0) xm[q] = *(pc - 1);
-    if (on && fy && j > 0) ym[q] = *(pc - p.Pc);
-    if (on && cell && k >= 1) zm[q] = q ? here[q - 1] : *(pc - sc);
-    if (on && fx) uo[q] = pu[(size_t)q * ((size_t)p.Pu * ny)];
-    if (on && fy) vo[q] = pv[(size_t)q * ((size_t)p.Pc * (ny + 1))];
-    if (on && cell && k >= 1) wo[q] = pw[(size_t)q * sc];
+    if (on && cell) here[q] = P(pc);
+    if (on && fx && i > 0) xm[q] = P(pc - 1);
+    if (on && fy && j > 0) ym[q] = P(pc - p.Pc);
+    if (on && cell && k >= 1) zm[q] = q ? here[q - 1] : P(pc - sc);
+    if (on && fx) uo[q] = *U(pu + (size_t)q * ((size_t)p.Pu * ny));
+    if (on && fy) vo[q] = *V(pv + (size_t)q * ((size_t)p.Pc * (ny + 1)));
+    if (on && cell && k >= 1) wo[q] = *W(pw + (size_t)q * sc);
   }
 #pragma unroll
   for (int q = 0; q < PROJ_ZC; ++q) {
@@ -692,13 +701,13 @@ __device__ __forceinline__ void project_cells_body(const StepParams<T>& p, const
     if (k >= nz) break;
     if (fx) {
       const T dp = i == 0 ? (T)ps_value(here[q]) : (i == nx ? -(T)ps_value(xm[q]) : (T)ps_diff(here[q], xm[q]));
-      pu[(size_t)q * ((size_t)p.Pu * ny)] = uo[q] - g * dp;
+      *U(pu + (size_t)q * ((size_t)p.Pu * ny)) = uo[q] - g * dp;
     }
     if (fy) {
       const T dp = j == 0 ? (T)ps_value(here[q]) : (j == ny ? -(T)ps_value(ym[q]) : (T)ps_diff(here[q], ym[q]));
-      pv[(size_t)q * ((size_t)p.Pc * (ny + 1))] = vo[q] - g * dp;
+      *V(pv + (size_t)q * ((size_t)p.Pc * (ny + 1))) = vo[q] - g * dp;
     }
-    if (cell && k >= 1) pw[(size_t)q * sc] = wo[q] - g * (T)ps_diff(here[q], zm[q]);
+    if (cell && k >= 1) *W(pw + (size_t)q * sc) = wo[q] - g * (T)ps_diff(here[q], zm[q]);
   }
 }
 template <typename T>
@@ -741,31 +750,35 @@ __device__ __forceinline__ void turbulence_body(const StepParams<T>& p, const T*
   const T *pu = u + idx_u(p, i, j, z0), *pv = v + idx_v(p, i, j, z0), *pw = w + idx_c(p, i, j, z0);
   size_t c = idx_c(p, i, j, z0);
   auto mean = [](T a, T b) { return T(0.5) * (a + b); };
-  T u0 = pu[0], u1 = pu[1], v0 = pv[0], v1 = pv[Pc], w0 = pw[0];
-  T wxm0 = pw[xm], wxp0 = pw[xp], wym0 = pw[ym * Pc], wyp0 = pw[yp * Pc];
-  T kc = ki[c], oc = oi[c];
+  auto U = [&](const T* at) { return *UF_PTR(at, u, Pu, p.ny, p.nz, 1, BA_U); };
+  auto V = [&](const T* at) { return *UF_PTR(at, v, Pc, p.ny + 1, p.nz, 1, BA_V); };
+  auto W = [&](const T* at) { return *UF_PTR(at, w, Pc, p.ny, p.nz + 1, 1, BA_CW); };
+  auto C = [&](auto* f, size_t at) { return UF_PTR(f + at, f, Pc, p.ny, p.nz, 1, BA_CW); };
+  T u0 = U(pu), u1 = U(pu + 1), v0 = V(pv), v1 = V(pv + Pc), w0 = W(pw);
+  T wxm0 = W(pw + xm), wxp0 = W(pw + xp), wym0 = W(pw + ym * Pc), wyp0 = W(pw + yp * Pc);
+  T kc = *C(ki, c), oc = *C(oi, c);
   T uz = mean(u0, u1), vz = mean(v0, v1), kz = kc, oz = oc;   // one plane below
   if (z0 > 0) {
-    uz = mean(*(pu - su), *(pu - su + 1));
-    vz = mean(*(pv - sv), *(pv - sv + Pc));
-    kz = ki[c - sc];
-    oz = oi[c - sc];
+    uz = mean(U(pu - su), U(pu - su + 1));
+    vz = mean(V(pv - sv), V(pv - sv + Pc));
+    kz = *C(ki, c - sc);
+    oz = *C(oi, c - sc);
   }
   for (int k = z0; k < z1; ++k) {
     const bool top = k == p.nz - 1;
-    const T w1 = pw[sc], wxm1 = (pw + sc)[xm], wxp1 = (pw + sc)[xp], wym1 = (pw + sc)[ym * Pc], wyp1 = (pw + sc)[yp * Pc];
-    const T ujm = mean(pu[ym * Pu], pu[ym * Pu + 1]), ujp = mean(pu[yp * Pu], pu[yp * Pu + 1]);
-    const T vim = mean(pv[xm], pv[xm + Pc]), vip = mean(pv[xp], pv[xp + Pc]);
-    T kxm = ki[c + xm], kxp = ki[c + xp], kym = ki[c + (ptrdiff_t)ym * Pc], kyp = ki[c + (ptrdiff_t)yp * Pc];
-    T oxm = oi[c + xm], oxp = oi[c + xp], oym = oi[c + (ptrdiff_t)ym * Pc], oyp = oi[c + (ptrdiff_t)yp * Pc];
+    const T w1 = W(pw + sc), wxm1 = W(pw + sc + xm), wxp1 = W(pw + sc + xp), wym1 = W(pw + sc + ym * Pc), wyp1 = W(pw + sc + yp * Pc);
+    const T ujm = mean(U(pu + ym * Pu), U(pu + (ym * Pu + 1))), ujp = mean(U(pu + yp * Pu), U(pu + (yp * Pu + 1)));
+    const T vim = mean(V(pv + xm), V(pv + (xm + Pc))), vip = mean(V(pv + xp), V(pv + (xp + Pc)));
+    T kxm = *C(ki, c + xm), kxp = *C(ki, c + xp), kym = *C(ki, c + (ptrdiff_t)ym * Pc), kyp = *C(ki, c + (ptrdiff_t)yp * Pc);
+    T oxm = *C(oi, c + xm), oxp = *C(oi, c + xp), oym = *C(oi, c + (ptrdiff_t)ym * Pc), oyp = *C(oi, c + (ptrdiff_t)yp * Pc);
     T un0 = u0, un1 = u1, vn0 = v0, vn1 = v1, kn = kc, on = oc;   // one plane above
     if (!top) {
-      un0 = pu[su];
-      un1 = (pu + su)[1];
-      vn0 = pv[sv];
-      vn1 = (pv + sv)[Pc];
-      kn = ki[c + sc];
-      on = oi[c + sc];
+      un0 = U(pu + su);
+      un1 = U(pu + su + 1);
+      vn0 = V(pv + sv);
+      vn1 = V(pv + sv + Pc);
+      kn = *C(ki, c + sc);
+      on = *C(oi, c + sc);
     }
     if (in_xm) { kxm = p.k_in; oxm = p.om_in; }
     if (in_xp) { kxp = p.k_in; oxp = p.om_in; }
@@ -801,8 +814,8 @@ __device__ __forceinline__ void turbulence_body(const StepParams<T>& p, const T*
     const T Pk = T(2) * nut * S2;
     const T rk = -adv_k + Pk - p.C_mu * kc * oc + (p.nu + p.sigma_star * nut) * lap_k * ih2;
     const T ro = -adv_o + T(2) * p.alpha * S2 - p.beta * oc * oc + (p.nu + p.sigma * nut) * lap_o * ih2;
-    ko[c] = fmax(kc + dt * rk, p.k_min);
-    oo[c] = fmax(oc + dt * ro, p.om_min);
+    *C(ko, c) = fmax(kc + dt * rk, p.k_min);
+    *C(oo, c) = fmax(oc + dt * ro, p.om_min);
     uz = uc; vz = vc; kz = kc; oz = oc;
     u0 = un0; u1 = un1; v0 = vn0; v1 = vn1; kc = kn; oc = on;
     w0 = w1; wxm0 = wxm1; wxp0 = wxp1; wym0 = wym1; wyp0 = wyp1;

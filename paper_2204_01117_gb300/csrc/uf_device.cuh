@@ -56,14 +56,17 @@ __device__ __forceinline__ double fma_rn(double a, double b, double c) { return 
 
 // ------------------------------------------------------- bounds checks --
 // Debug build (compiled with -DUF_BOUNDS_CHECK): every global index the
-// index helpers form (idx_u, idx_v, idx_c here, lidx for the multigrid
-// levels) is checked against its array: x within the row pitch, y and z
+// index helpers form (idx_u, idx_v, idx_c here, lidx for the grids of the
+// solvers) is checked against its array: x within the row pitch, y and z
 // within the stored rows and planes.  The first violation is recorded in
 // uf_bounds_hit (array, i, j, k) and the access is redirected to element 0,
 // so the kernel completes; the host reads the record after the call and
 // returns UF_ERR_BOUNDS.  Each translation unit has its own record, read by
 // its own host code.  The ordinary build compiles none of this.
-enum BoundsArray { BA_U = 0, BA_V = 1, BA_CW = 2, BA_LEVEL = 3 };
+// UF_PTR does the same for a pointer that a kernel moves along itself: `width`
+// values from p on must lie in the array of `planes` planes of `rows` rows of
+// P values at base; else it is recorded and base is used.
+enum BoundsArray { BA_U = 0, BA_V = 1, BA_CW = 2, BA_LEVEL = 3, BA_LATTICE = 4, BA_MATRIX = 5 };
 struct BoundsHit {
   int hit, array, i, j, k;
 };
@@ -79,6 +82,14 @@ __device__ __forceinline__ void bounds_check(bool ok, int array, int& i, int& j,
   }
   i = j = k = 0;
 }
+template <typename E>
+__device__ __forceinline__ E* bounds_ptr(E* p, const void* base, int P, int rows, long long planes, int width, int array) {
+  const long long o = p - (E*)base;
+  int i = (int)(o % P), j = (int)(o / P % rows), k = (int)(o / P / rows);
+  const bool ok = o >= 0 && o + width <= (long long)P * rows * planes;
+  bounds_check(ok, array, i, j, k);
+  return ok ? p : (E*)base;
+}
 // Reads (and clears) this translation unit's record after the work queued
 // on stream s; true if an index was out of bounds.
 static inline bool bounds_hit_take(cudaStream_t s, BoundsHit* out) {
@@ -92,8 +103,10 @@ static inline bool bounds_hit_take(cudaStream_t s, BoundsHit* out) {
   return true;
 }
 #define UF_BOUNDS(ok, array, i, j, k) ::uf::bounds_check((ok), (array), i, j, k)
+#define UF_PTR(p, base, P, rows, planes, width, array) ::uf::bounds_ptr((p), (base), (P), (rows), (planes), (width), (array))
 #else
 #define UF_BOUNDS(ok, array, i, j, k) ((void)0)
+#define UF_PTR(p, base, P, rows, planes, width, array) (p)
 #endif
 
 // ------------------------------------------------------------- indexing --
