@@ -514,7 +514,7 @@ __device__ __forceinline__ Vec16<T> sep_apply(const Level<T>& L, const SepCols<T
   constexpr int N = Vec16<T>::N;
   struct alignas(16) Row { E e[N]; };
   const int i0 = L.nx - C.left_x, j = (int)(C.c / L.P);
-  const E* __restrict__ f0 = f;
+  [[maybe_unused]] const E* __restrict__ f0 = f;   // (SEP_PTR)
   f += (size_t)k * C.PS + C.c;
   auto row = [&](const E* at) { return *reinterpret_cast<const Row*>(SEP_PTR(at, f0, L, N)); };
   const bool y0 = j > 0, y1 = j < L.ny - 1, z0 = k > 0, z1 = k < L.nz - 1;
