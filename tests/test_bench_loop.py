@@ -30,3 +30,13 @@ def test_v_cycle_labels_keep_the_count():
     # seven iterations: once per iteration, and once more at the set-up
     assert bench.loop_launches("mg_up_L0", 8, 7) == 1 and bench.loop_launches("b_mg_tail", 8, 7) == 1
     assert bench.loop_launches("mg_up_L0", 0, 0) == 0
+
+
+def test_the_solver_table_runs_what_its_rows_say():
+    """The V-cycle of the default settings has to be asked for, or the separable inverse runs under its name."""
+    rows = {name: (params, tuning) for name, params, tuning in bench.PRECONDITIONERS}
+    assert len(rows) == len(bench.PRECONDITIONERS)
+    default = [n for n, (p, _) in rows.items() if p.get("precond") == "mg" and p.get("mg_smoother", "cheby") == "cheby"
+               and p.get("mg_transfer", "linear") == "linear"]
+    assert sorted(default) == ["mg", "separable"]
+    assert rows["mg"][1].get("coarse_start") == -1 and rows["separable"][1].get("coarse_start", 0) == 0
