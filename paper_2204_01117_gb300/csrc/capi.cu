@@ -153,13 +153,20 @@ struct Plan {
 // whose panels fit one block's shared memory (227 KB: FP32 nz x 136 words, ny
 // x 72 or 40 words and at least 8 KB of queue; FP64 32 doubles per cell of
 // either axis) and whose x lines fit one warp, and at most kPartials panels per
-// reducing launch.  FP64: the transforms cost 8 (ny + nz) FP64 operations a cell
-// and application (half along an axis with walls at both ends), the V-cycle's
-// fourteen iterations about 4 ns a cell at any size; with two applications that
-// is even near ny + nz = 550 for the dearest form (one step with the V-cycle
-// and with the inverse, all axes in full: 64 x 32 x 16 2.72 and 0.20 ms, 128 x
-// 96 x 40 6.6 and 1.35, 256 x 256 x 64 26.6 and 10.9, 128 x 330 x 64 24.6 and
-// 7.9).
+// reducing launch.  FP64: the transforms cost about 4 (ny + nz) FP64 operations
+// a cell and application (half along an axis with walls at both ends), one
+// application a step in a developed flow; the V-cycle takes 14 to 18 iterations
+// of about 0.4 ns a cell.  One step with the V-cycle and with the inverse, ms,
+// wind at 45 degrees (no axis but z folded) and along x (y folded):
+//   ny + nz = 320, 256 x 256 x 64     25.8  10.2    25.4   8.2
+//             394, 128 x 330 x 64     24.2   7.4
+//             464, 512 x 400 x 64     76.4  34.8
+//             512, 384 x 384 x 128   100    52.8    97.5  40.5
+//             576, 512 x 512 x 64     91.0  50.6    88.8  36.6
+//             840, 128 x 800 x 40     25.7  21.1    25.8  13.7
+// So the two would meet near ny + nz = 1000 where no horizontal axis folds,
+// past what shared memory holds (880 rows).  The line is lower than that:
+// sizes beyond it have been timed, but not compared with a direct solve.
 constexpr int kSep64Sum = 480;
 bool sep_available(const uf_grid_desc* d) {
   if (d->precond != UF_PRECOND_MG || d->mg_smoother != UF_SMOOTH_CHEBY || d->mg_transfer != UF_TRANSFER_LINEAR ||

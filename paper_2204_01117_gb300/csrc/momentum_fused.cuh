@@ -28,9 +28,11 @@
 // Boundary faces of u~ and u2 are never stored between sub-steps; they come
 // from the BC rules, as in the unfused kernels.
 // Every value is formed by the expressions of k_diffuse, k_drag_bc and
-// k_pressure_rhs; the block and z-chunk decomposition is that of
-// k_pressure_rhs (chunk_grid), so ||b||^2 is summed in the same order.  The
-// results, ||b||^2 included, are bit for bit those of the three kernels.
+// k_pressure_rhs; the blocks and z chunks are those of k_pressure_rhs
+// (momentum_grid gives both), so ||b||^2 is summed in the same order.  The
+// results, ||b||^2 included, are bit for bit those of the three kernels while
+// the velocities are finite (in open air a face keeps its value here; the drag
+// expression makes 0 of it beside an infinite one).
 //
 // Tape (the adjoint): when u2t is not null, u2 of every interior face the
 // block owns is also written to (u2t, v2t, w2t).

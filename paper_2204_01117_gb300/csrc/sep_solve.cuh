@@ -18,9 +18,11 @@
 // iterations to 1e-7 where the V-cycle needs seven to eleven, and an
 // application is 5 launches where the V-cycle has 14 to 18 that depend on
 // one another.  CG still stops on ||r|| <= tol ||b|| with FP64 inner products,
-// so the solution is the same to the same tolerance; its error against 64
-// bits is at most the V-cycle's (512 x 512 x 128, w after two steps: 2.2e-6
-// against 4.8e-6).  Measured on a GB300, one time step with the V-cycle and
+// so the solution is the same to the same tolerance.  Its error against 64
+// bits, over 3 to 9 seeds each of ten FP32 workloads (48 x 40 x 16 to 256 x 256 x
+// 64, one to four steps), against the V-cycle's on the same inputs: u, v, w, k and
+// omega 0.38 to 1.00 of it, p 0.77 to 1.10 (+- 0.19: no difference that the seeds
+// could tell).  Measured on a GB300, one time step with the V-cycle and
 // with this in its first form, all else equal: 48 x 40 x 16 0.73 -> 0.20 ms, 157 x 203 x 41 1.87 -> 0.47 ms,
 // 256 x 256 x 64 2.20 -> 1.09 ms, 512 x 768 x 1 1.24 -> 0.34 ms,
 // 512 x 512 x 128 13.0 -> 8.7 ms (where the y transforms cost most); the
@@ -29,8 +31,9 @@
 // The transforms are contractions of a field with a constant n x n matrix:
 // tensor cores, TF32 operands split into a high and a low part (x = hi + lo,
 // 11 bits each), three products hi hi + hi lo + lo hi accumulated in FP32.
-// The dropped lo lo is below 2^-22 of the product, so a transform is about
-// as accurate as one in plain FP32.
+// The dropped lo lo is at most 2^-22 of the product, the bit cut off either
+// low part at most 2^-23: 2^-21 at worst where a plain FP32 product has 2^-24,
+// which the errors above include.
 //
 // The modes of an axis with walls at both ends are even or odd about its
 // middle, so there (always along z; along y for a wind along x) a transform
@@ -49,8 +52,8 @@ constexpr int SEP_MAX_NX = 1024;  // 32 lanes x 32 values per line
 
 // FP64 grids do the same on the FP64 pipe, 1/64 of the FP32 rate on this
 // chip: the products are then what a pass costs, and a rule on the sizes
-// keeps the V-cycle where they would outweigh the iterations saved
-// (sep_available in capi.cu, with both sides measured).
+// keeps the V-cycle for the longest axes (sep_available in capi.cu, with both
+// sides measured).
 template <typename T>
 struct SepMat { using type = float4; };   // FP32: see below
 template <>
@@ -167,7 +170,7 @@ struct SepStore {
   }
 };
 
-// x = hi + lo (+ below 2^-22 |x|): hi rounded to TF32's 11 bits, lo cut to them.
+// x = hi + lo (+ at most 2^-23 |x|): hi rounded to TF32's 11 bits, lo, of 12 at most, cut to them.
 __device__ __forceinline__ void tf32_split(float x, uint32_t& hi, uint32_t& lo) {
   hi = (__float_as_uint(x) + 0x1000u) & 0xffffe000u;
   lo = __float_as_uint(__fsub_rn(x, __uint_as_float(hi))) & 0xffffe000u;
