@@ -734,7 +734,7 @@ __device__ __forceinline__ double logistic(double t) { return 1.0 / (1.0 + exp(-
 // widths away.  (FP64 exp and division were what bounded both kernels; the
 // reverse one also added 3 terms per cell and box to shared memory with
 // FP64 atomics.)  Measured at 128 x 128 x 48 with 12 boxes, the map and its
-// transpose together: 11.8 -> 0.58 ms.
+// transpose together: 11.8 -> 0.50 ms.
 constexpr int DZ = 8;
 struct DesignTile {
   double xa[MAX_BOXES][BX], xb[MAX_BOXES][BX], ya[MAX_BOXES][BY], yb[MAX_BOXES][BY], z[MAX_BOXES][DZ];
@@ -817,30 +817,53 @@ __global__ void __launch_bounds__(NT) k_design_phi(int nx, int ny, int nz, int P
 // before and after b; dchi/dtheta = chi (dlog s/dtheta).  A thread sums its DZ
 // cells, a warp its threads.  A box that does not reach the tile has factors of
 // exactly 1 there, but its own chi is small, not zero: it drops out of the
-// products and keeps its term (where the tile has a sensitivity that is not
-// finite, also at chi = 0).
+// products and keeps its term (where a sensitivity of the tile or a product is
+// not finite, also at chi = 0).  What the sums need of a box is formed once per
+// tile: the ramps' products and derivative factors over x and over y in place
+// of the ramps, and z (1 - z) beside z.
+struct DesignVjpTile {
+  DesignTile t;
+  double zz[MAX_BOXES][DZ];
+};
 template <typename T>
 __global__ void __launch_bounds__(NT) k_design_phi_vjp(int nx, int ny, int nz, int P, double h,
                                                        const __grid_constant__ DesignBoxes boxes, int nbox, double wdt,
                                                        const T* __restrict__ lphi, double* g) {
-  __shared__ DesignTile t;
+  extern __shared__ __align__(16) unsigned char design_raw[];   // (past the 48 KB of a static array)
+  DesignVjpTile& V = *reinterpret_cast<DesignVjpTile*>(design_raw);
+  DesignTile& t = V.t;
   const int i0 = blockIdx.x * BX, j0 = blockIdx.y * BY, k0 = blockIdx.z * DZ;
   design_tile(t, boxes, nbox, h, wdt, i0, j0, k0);
+  constexpr int PER = BX + BY + DZ;
+  for (int e = threadIdx.x + BX * threadIdx.y; e < nbox * PER; e += NT) {
+    const int b = e / PER, o = e - b * PER;
+    if (o < BX + BY) {
+      double& lo = o < BX ? t.xa[b][o] : t.ya[b][o - BX];
+      double& hi = o < BX ? t.xb[b][o] : t.yb[b][o - BX];
+      const double u = lo, v = hi;
+      lo = u * v;
+      hi = -(1.0 - u) + (1.0 - v);
+    } else {
+      const int q = o - BX - BY;
+      V.zz[b][q] = t.z[b][q] * (1.0 - t.z[b][q]);
+    }
+  }
+  __syncthreads();
   const int i = i0 + threadIdx.x, j = j0 + threadIdx.y, n = t.n;
   double lam[DZ], pre[DZ];
-  bool wild = false;   // a sensitivity that is not finite
+  bool any = false;   // a sensitivity that is not zero
 #pragma unroll
   for (int q = 0; q < DZ; ++q) {
     lam[q] = i < nx && j < ny && k0 + q < nz ? (double)lphi[(size_t)i + (size_t)P * ((size_t)j + (size_t)ny * (k0 + q))] : 0.0;
-    wild |= !isfinite(lam[q]);
+    any |= lam[q] != 0.0;
     pre[q] = 1.0;   // product over the boxes before r
   }
   // Adds box b's terms: s1 the thread's sum of (dphi/dchi lam) z over its cells, s2 that of (dphi/dchi lam) z (1 - z).
   // The warp reduces the three together, halving what a lane holds, and divides once.
   auto add = [&](int b, double s1, double s2) {
-    const double sxa = t.xa[b][threadIdx.x], sxb = t.xb[b][threadIdx.x], sya = t.ya[b][threadIdx.y], syb = t.yb[b][threadIdx.y];
-    const double a = sxa * sxb * sya * syb, sum = a * s1;
-    const double v0 = a * s2, v1 = sum * (-(1.0 - sxa) + (1.0 - sxb)), v2 = sum * (-(1.0 - sya) + (1.0 - syb));
+    const double a = t.xa[b][threadIdx.x] * t.ya[b][threadIdx.y], sum = a * s1;
+    // (nothing from cells without sensitivities, also where a ramp is not a number)
+    const double v0 = any ? a * s2 : 0.0, v1 = any ? sum * t.xb[b][threadIdx.x] : 0.0, v2 = any ? sum * t.yb[b][threadIdx.y] : 0.0;
     const int lane = threadIdx.x;
     const bool h = lane & 16, l = lane & 8;
     const double p = (h ? v2 : v0) + __shfl_xor_sync(0xffffffffu, h ? v0 : v2, 16);
@@ -852,39 +875,43 @@ __global__ void __launch_bounds__(NT) k_design_phi_vjp(int nx, int ny, int nz, i
   };
   for (int r = 0; r < n; ++r) {
     const int b = t.list[r];
-    const double a = t.xa[b][threadIdx.x] * t.xb[b][threadIdx.x] * t.ya[b][threadIdx.y] * t.yb[b][threadIdx.y];
+    const double a = t.xa[b][threadIdx.x] * t.ya[b][threadIdx.y];
     double post[DZ];
 #pragma unroll
     for (int q = 0; q < DZ; ++q) post[q] = 1.0;
     for (int c = r + 1; c < n; ++c) {
       const int bc = t.list[c];
-      const double ac = t.xa[bc][threadIdx.x] * t.xb[bc][threadIdx.x] * t.ya[bc][threadIdx.y] * t.yb[bc][threadIdx.y];
+      const double ac = t.xa[bc][threadIdx.x] * t.ya[bc][threadIdx.y];
 #pragma unroll
       for (int q = 0; q < DZ; ++q) post[q] *= 1.0 - ac * t.z[bc][q];
     }
     double s1 = 0.0, s2 = 0.0;
 #pragma unroll
     for (int q = 0; q < DZ; ++q) {
-      const double sz = t.z[b][q];
-      const double base = lam[q] != 0.0 ? -(pre[q] * post[q]) * lam[q] * sz : 0.0;
-      s1 += base;
-      s2 += base * (1.0 - sz);
-      pre[q] *= 1.0 - a * sz;
+      const double base = -(pre[q] * post[q]) * lam[q];
+      if (lam[q] != 0.0) {
+        s1 += base * t.z[b][q];
+        s2 += base * V.zz[b][q];
+      }
+      pre[q] *= 1.0 - a * t.z[b][q];
     }
     add(b, s1, s2);
   }
-  const bool all = __syncthreads_or(wild);
+  bool wild = false;   // dphi/dchi lam of a cell is not finite
 #pragma unroll
-  for (int q = 0; q < DZ; ++q) lam[q] = lam[q] != 0.0 ? -pre[q] * lam[q] : 0.0;
+  for (int q = 0; q < DZ; ++q) {
+    lam[q] = lam[q] != 0.0 ? -pre[q] * lam[q] : 0.0;
+    wild |= !isfinite(lam[q]);
+  }
+  const bool all = __syncthreads_or(wild);
   for (int b = 0; b < nbox; ++b) {
     const unsigned int bit = 1u << (b & 31);
     if (!((t.far_mask[b >> 5] & bit) || (all && !(t.mask[b >> 5] & bit)))) continue;
     double s1 = 0.0, s2 = 0.0;
 #pragma unroll
     for (int q = 0; q < DZ; ++q) {
-      const double sz = t.z[b][q], base = lam[q] * sz;
-      s1 += base;
-      s2 += base * (1.0 - sz);
+      s1 += lam[q] * t.z[b][q];
+      s2 += lam[q] * V.zz[b][q];
     }
     add(b, s1, s2);
   }

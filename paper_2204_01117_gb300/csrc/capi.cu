@@ -619,6 +619,7 @@ class GridImpl final : public uf_grid {
     lim((const void*)uf::k_advect_fused<T, false>);
     lim((const void*)uf::k_advect_fused<T, true>);
     lim((const void*)uf::k_momentum_fused<T>);
+    lim((const void*)uf::k_design_phi_vjp<T>);
     lim((const void*)uf::k_mg_coarse<T, uf::SM_JACOBI>);
     lim((const void*)uf::k_mg_coarse<T, uf::SM_RBGS>);
     if (P.sep) {
@@ -1514,8 +1515,8 @@ class GridImpl final : public uf_grid {
     if (s != UF_OK) return s;
     double* g = at<double>(P.grad);
     UF_CUDA(cudaMemsetAsync(g, 0, sizeof(double) * 3 * nbox, stream));
-    uf::k_design_phi_vjp<T><<<design_grid(d.nx, d.ny, d.nz), dim3(uf::BX, uf::BY), 0, stream>>>(d.nx, d.ny, d.nz, P.Pc, d.h, hb, nbox,
-                                                                                                width, q, g);
+    uf::k_design_phi_vjp<T><<<design_grid(d.nx, d.ny, d.nz), dim3(uf::BX, uf::BY), sizeof(uf::DesignVjpTile), stream>>>(
+        d.nx, d.ny, d.nz, P.Pc, d.h, hb, nbox, width, q, g);
     UF_CUDA(cudaGetLastError());
     UF_CUDA(cudaMemcpyAsync(g_out, g, sizeof(double) * 3 * nbox, cudaMemcpyDeviceToHost, stream));
     UF_CUDA(cudaStreamSynchronize(stream));

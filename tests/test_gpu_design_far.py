@@ -51,3 +51,15 @@ def test_a_nan_reaches_every_box(precision):
     lam = np.zeros(g.shapes["phi"], dtype=g.np_dtype)
     lam[3, 40, 63] = np.nan
     assert np.isnan(g.design_vjp(BOXES, THETA, WIDTH, lam)).all()
+
+
+@pytest.mark.parametrize("precision", ["f32", "f64"])
+def test_a_nan_parameter_stays_with_the_sensitivities(precision):
+    """A box whose height is not a number: every gradient is, where there are sensitivities, and 0 where there are none."""
+    g = uf.Grid(*DIMS, h=H, precision=precision)
+    theta = THETA.copy()
+    theta[6] = np.nan
+    lam = np.zeros(g.shapes["phi"], dtype=g.np_dtype)
+    np.testing.assert_array_equal(g.design_vjp(BOXES, theta, WIDTH, lam), 0.0)
+    lam[3, 40, 60] = 1.0
+    assert np.isnan(g.design_vjp(BOXES, theta, WIDTH, lam)).all()
