@@ -26,9 +26,9 @@
 // functions below, each a call, which costs registers and moves even where
 // it is never made: a kernel of its own (FAR = true).  Measured, FP32 and
 // CFL time step, against general samples for all points, spread over the
-// threads by component: 256 x 256 x 64 375 -> 172 us (310 M -> 135 M warp
-// instructions, 1030 a cell), 512 x 512 x 128 2734 -> 1069 us; issue slots
-// 72 % busy at 3 blocks per SM.
+// threads by component: 256 x 256 x 64 375 -> 164 us (310 M -> 139 M warp
+// instructions, 1060 a cell), 512 x 512 x 128 2734 -> 1069 us; issue slots
+// 77 % busy at 3 blocks per SM.
 //
 // Every value is formed by the same expressions as the two-kernel form
 // (k_advect_forward, k_advect_backward) from the same inputs; only the

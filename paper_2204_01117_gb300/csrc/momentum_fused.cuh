@@ -21,8 +21,9 @@
 // the drag reads faces alike everywhere;
 // where the drag coefficient is zero (open air, most of a city) the face
 // keeps its value, which is what the drag expression gives.  Measured at
-// 256 x 256 x 64, FP32, against loops over the general expressions: 235 -> 141
-// us (197 M -> 118 M warp instructions), 512 x 512 x 128 1493 -> 777 us; the
+// 256 x 256 x 64, FP32, against loops over the general expressions: 235 -> 137
+// us (197 M -> 111 M warp instructions, issue slots 79 % busy), 512 x 512 x 128
+// 1493 -> 737 us; the
 // code of one variant more in the loop body cost 30 us in instruction fetch.
 //
 // Boundary faces of u~ and u2 are never stored between sub-steps; they come

@@ -21,8 +21,8 @@
 // so the solution is the same to the same tolerance.  Its error against 64
 // bits, over 3 to 9 seeds each of ten FP32 workloads (48 x 40 x 16 to 256 x 256 x
 // 64, one to four steps), against the V-cycle's on the same inputs: u, v, w, k and
-// omega 0.38 to 1.00 of it, p 0.77 to 1.10 (+- 0.19: no difference that the seeds
-// could tell).  Measured on a GB300, one time step with the V-cycle and
+// omega 0.38 to 1.00 of it, p 0.77 to 1.10 (standard errors to 0.3: no difference
+// that the seeds could tell).  Measured on a GB300, one time step with the V-cycle and
 // with this in its first form, all else equal: 48 x 40 x 16 0.73 -> 0.20 ms, 157 x 203 x 41 1.87 -> 0.47 ms,
 // 256 x 256 x 64 2.20 -> 1.09 ms, 512 x 768 x 1 1.24 -> 0.34 ms,
 // 512 x 512 x 128 13.0 -> 8.7 ms (where the y transforms cost most); the
