@@ -2158,11 +2158,10 @@ class GridImpl final : public uf_grid {
       e = cudaGetLastError();
     }
     if (e == cudaSuccess) {
-      const unsigned nb = uf::mesh_blocks(d.nx, d.ny, d.nz);
-      if (tables)
-        uf::k_mesh_phi<T, true><<<nb, 32 * uf::MESH_WARPS, 0, stream>>>(d.nx, d.ny, d.nz, P.Pc, d.h, sub, dtri, te, tf, dobj, nobj, dst);
-      else
-        uf::k_mesh_phi<T, false><<<nb, 32 * uf::MESH_WARPS, 0, stream>>>(d.nx, d.ny, d.nz, P.Pc, d.h, sub, dtri, te, tf, dobj, nobj, dst);
+      const uf::MeshBrick brick = uf::mesh_brick(d.nx, d.ny, d.nz);
+      auto k = tables ? uf::k_mesh_phi<T, true> : uf::k_mesh_phi<T, false>;
+      k<<<uf::mesh_blocks(d.nx, d.ny, d.nz, brick), 32 * uf::MESH_WARPS, 0, stream>>>(d.nx, d.ny, d.nz, P.Pc, d.h, sub, brick, dtri, te, tf,
+                                                                                     dobj, nobj, dst);
       e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);

@@ -125,92 +125,120 @@ __device__ __forceinline__ int ray_bound(float px, float py, float pz, float r, 
   return 0;
 }
 
-// A block takes a brick of 8 x 8 x 4 cells, a lane a cell: the brick's objects
+// A block takes a brick of cells, a warp one to 32 of them: the brick's objects
 // are listed once (a brick in the open, most of a city, is 1 at once), then
-// each warp works through those of its 32 cells that an object's cell range
-// holds.  For such a cell the lanes bound every triangle of the object over
-// the whole cell: a triangle that no ray from the cell can cross drops out,
-// one that every ray crosses only flips the parity, the few others are
+// each warp works through those of its cells that an object's cell range
+// holds.  For such a cell the lanes list its objects and bound every triangle of
+// each over the whole cell: a triangle that no ray from the cell can cross drops
+// out, one that every ray crosses only flips the parity, the few others are
 // listed.  The sub^3 sample points, 32 at a time, then test the listed ones,
 // in FP32 where its bound decides and with the test itself where it does not.
 // Every decision is the test's, so the field is the same bit for bit; what
 // bounded the kernel before were FP64 tests of every point against every
 // triangle (1/64 rate) and the serial object list of every cell.  Measured at
 // 256 x 256 x 64 with 100 objects (6500 triangles), the whole call: 23.4 ->
-// 1.15 ms.
+// 1.07 ms.
+// The brick: 8 x 8 x 4 cells, 32 to a warp, while the grid has cells for about
+// 32 warps on each SM, halved until it has, down to a cell to a warp: on a
+// coarse grid, whose cells hold many objects each, a warp would work through
+// its cells one after another while most of the chip had none (12 x 12 x 4 with
+// 300 objects 1.7 ms against 13.8, 50 x 50 x 8 with 4000 11 against
+// 114, also for the lists of 64 objects to a brick, past which every point met every
+// object).
 // TABLES = false: a mesh whose tables do not fit (an entry per object and
 // triangle, so objects that share long ranges need many) is tested triangle
 // by triangle.
-constexpr int MESH_LIST = 64;      // objects of a brick (more: every object is visited)
+constexpr int MESH_BRICK = 1024;   // objects of a brick (more: its cells look through all)
+constexpr int MESH_LIST = 64;      // objects of a cell (more: every point visits the brick's)
 constexpr int MESH_OPEN = 192;     // undecided triangles of a cell (more: every triangle is tested)
 constexpr int MESH_WARPS = 8;
-constexpr int MESH_BX = 8, MESH_BY = 8, MESH_BZ = 4;   // 32 MESH_WARPS cells
-
-inline unsigned mesh_blocks(int nx, int ny, int nz) {   // bricks, x fastest (in one dimension: any nz)
-  return (unsigned)((size_t)((nx + MESH_BX - 1) / MESH_BX) * ((ny + MESH_BY - 1) / MESH_BY) * ((nz + MESH_BZ - 1) / MESH_BZ));
+// Brick of 2^(x + y + z) cells, 2^(x + y + z - 3) to a warp.
+struct MeshBrick {
+  int x, y, z;
+};
+inline MeshBrick mesh_brick(int nx, int ny, int nz) {
+  const MeshBrick bricks[] = {{3, 3, 2}, {3, 2, 2}, {2, 2, 2}, {2, 2, 1}, {2, 1, 1}};
+  for (const MeshBrick& b : bricks)
+    if (((size_t)nx * ny * nz >> (b.x + b.y + b.z - 3)) >= 152 * 32) return b;
+  return {1, 1, 1};
+}
+inline unsigned mesh_blocks(int nx, int ny, int nz, MeshBrick b) {   // bricks, x fastest (in one dimension: any nz)
+  return (unsigned)((size_t)((nx + (1 << b.x) - 1) >> b.x) * ((ny + (1 << b.y) - 1) >> b.y) * ((nz + (1 << b.z) - 1) >> b.z));
 }
 template <typename T, bool TABLES>
-__global__ void __launch_bounds__(32 * MESH_WARPS) k_mesh_phi(int nx, int ny, int nz, int P, double h, int sub,
+__global__ void __launch_bounds__(32 * MESH_WARPS) k_mesh_phi(int nx, int ny, int nz, int P, double h, int sub, MeshBrick brick,
                                                               const double* __restrict__ tri, const MeshTri* __restrict__ te,
                                                               const MeshTriF* __restrict__ tf, const MeshObject* __restrict__ obj,
                                                               int nobj, T* __restrict__ phi) {
-  __shared__ int s_obj[MESH_LIST], s_nobj;
-  __shared__ int s_open[MESH_WARPS][MESH_OPEN];          // undecided triangles of the warp's cell, object by object
+  __shared__ int s_obj[MESH_BRICK], s_nobj;
+  __shared__ int s_cell[MESH_WARPS][MESH_LIST];          // objects of the warp's cell
+  __shared__ int s_open[MESH_WARPS][MESH_OPEN];          // its undecided triangles, object by object
   __shared__ int s_end[MESH_WARPS][MESH_LIST];           // where each object's end
-  __shared__ unsigned char s_odd[MESH_WARPS][MESH_LIST]; // parity of the crossings common to the whole cell; 2: not in the cell
+  __shared__ unsigned char s_odd[MESH_WARPS][MESH_LIST]; // parity of the crossings common to the whole cell
   __shared__ double s_val[MESH_WARPS][32];
   __shared__ double s_off[16];          // sample offsets (a + 1/2) / sub within a cell
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  const unsigned int nbx = (nx + MESH_BX - 1) / MESH_BX, nby = (ny + MESH_BY - 1) / MESH_BY, row = blockIdx.x / nbx;
-  const int bi = (int)(blockIdx.x % nbx) * MESH_BX, bj = (int)(row % nby) * MESH_BY, bk = (int)(row / nby) * MESH_BZ;
+  const unsigned int nbx = (nx + (1 << brick.x) - 1) >> brick.x, nby = (ny + (1 << brick.y) - 1) >> brick.y, row = blockIdx.x / nbx;
+  const int bi = (int)(blockIdx.x % nbx) << brick.x, bj = (int)(row % nby) << brick.y, bk = (int)(row / nby) << brick.z;
   if (t == 0) s_nobj = 0;
   if (t < sub) s_off[t] = __ddiv_rn(__dadd_rn((double)t, 0.5), (double)sub);
   __syncthreads();
   for (int o = t; o < nobj; o += 32 * MESH_WARPS) {
     const MeshObject& m = obj[o];
-    if (bi + MESH_BX - 1 < m.clo[0] || bi > m.chi[0] || bj + MESH_BY - 1 < m.clo[1] || bj > m.chi[1] || bk + MESH_BZ - 1 < m.clo[2] ||
-        bk > m.chi[2])
+    if (bi + (1 << brick.x) - 1 < m.clo[0] || bi > m.chi[0] || bj + (1 << brick.y) - 1 < m.clo[1] || bj > m.chi[1] ||
+        bk + (1 << brick.z) - 1 < m.clo[2] || bk > m.chi[2])
       continue;
     const int at = atomicAdd(&s_nobj, 1);
-    if (at < MESH_LIST) s_obj[at] = o;
+    if (at < MESH_BRICK) s_obj[at] = o;
   }
   __syncthreads();
-  const bool all = s_nobj > MESH_LIST;               // too many: visit every object
+  const bool all = s_nobj > MESH_BRICK;              // too many: look through every object
   const int n_obj = all ? nobj : s_nobj;
-  const int i = bi + t % MESH_BX, j = bj + t / MESH_BX % MESH_BY, k = bk + t / (MESH_BX * MESH_BY);
-  const bool in = i < nx && j < ny && k < nz;
+  const int per_warp = 1 << (brick.x + brick.y + brick.z - 3), cell = warp * per_warp + lane;
+  const int i = bi + (cell & ((1 << brick.x) - 1)), j = bj + (cell >> brick.x & ((1 << brick.y) - 1)), k = bk + (cell >> (brick.x + brick.y));
+  const bool in = lane < per_warp && i < nx && j < ny && k < nz;
   auto holds = [&](const MeshObject& m, int a, int b, int c) {
     return a >= m.clo[0] && a <= m.chi[0] && b >= m.clo[1] && b <= m.chi[1] && c >= m.clo[2] && c <= m.chi[2];
   };
-  bool hit = false;
-  for (int q = 0; q < n_obj && !hit; ++q) hit = holds(obj[all ? q : s_obj[q]], i, j, k);
+  bool hit = n_obj > MESH_LIST;                      // (then the cells' lists tell)
+  for (int q = 0; q < n_obj && !hit; ++q) hit = holds(obj[s_obj[q]], i, j, k);
   T out = T(1);                                      // the open: every point is 1, and so is their mean
   const int npts = sub * sub * sub;
   const double hh = 0.5 * h;
   for (unsigned int todo = __ballot_sync(0xffffffffu, in && hit); todo; todo &= todo - 1) {
     const int src = __ffs(todo) - 1;
     const int ci = __shfl_sync(0xffffffffu, i, src), cj = __shfl_sync(0xffffffffu, j, src), ck = __shfl_sync(0xffffffffu, k, src);
+    // list the cell's objects
+    int nl = 0;
+    for (int q = 0; q < n_obj; q += 32) {
+      const int o = q + lane < n_obj ? (all ? q + lane : s_obj[q + lane]) : -1;
+      const bool has = o >= 0 && holds(obj[o], ci, cj, ck);
+      const unsigned int m = __ballot_sync(0xffffffffu, has);
+      const int at = nl + __popc(m & ((1u << lane) - 1u));
+      if (has && at < MESH_LIST) s_cell[warp][at] = o;
+      nl += __popc(m);
+    }
+    if (nl == 0) continue;
+    const bool over = nl > MESH_LIST;                // too many: every point visits the brick's
+    __syncwarp();
     // bound the triangles over the cell
-    bool exact = !TABLES || all;                     // too much to list: test every triangle
+    bool exact = !TABLES || over;                    // too much to list: test every triangle
     int n = 0;
-    for (int q = 0; q < n_obj && !exact; ++q) {
-      const MeshObject& m = obj[s_obj[q]];
-      unsigned int odd = 2;
-      if (holds(m, ci, cj, ck)) {
-        odd = 0;
-        const float px = (float)(((ci + 0.5) * h - m.lo[0]) * m.scale), py = (float)(((cj + 0.5) * h - m.lo[1]) * m.scale),
-                    pz = (float)(((ck + 0.5) * h - m.lo[2]) * m.scale), r = (float)(hh * m.scale) * 1.0001f;
-        for (int e = 0; e < m.count; e += 32) {
-          int b = -1;
-          if (e + lane < m.count) b = ray_bound(px, py, pz, r, tf[m.entry + e + lane]);
-          odd ^= __popc(__ballot_sync(0xffffffffu, b == 1)) & 1u;
-          const unsigned int open = __ballot_sync(0xffffffffu, b == 0);
-          const int at = n + __popc(open & ((1u << lane) - 1u));
-          if (b == 0 && at < MESH_OPEN) s_open[warp][at] = m.entry + e + lane;
-          n += __popc(open);
-        }
-        if (n > MESH_OPEN) exact = true;
+    for (int q = 0; q < nl && !exact; ++q) {
+      const MeshObject& m = obj[s_cell[warp][q]];
+      unsigned int odd = 0;
+      const float px = (float)(((ci + 0.5) * h - m.lo[0]) * m.scale), py = (float)(((cj + 0.5) * h - m.lo[1]) * m.scale),
+                  pz = (float)(((ck + 0.5) * h - m.lo[2]) * m.scale), r = (float)(hh * m.scale) * 1.0001f;
+      for (int e = 0; e < m.count; e += 32) {
+        int b = -1;
+        if (e + lane < m.count) b = ray_bound(px, py, pz, r, tf[m.entry + e + lane]);
+        odd ^= __popc(__ballot_sync(0xffffffffu, b == 1)) & 1u;
+        const unsigned int open = __ballot_sync(0xffffffffu, b == 0);
+        const int at = n + __popc(open & ((1u << lane) - 1u));
+        if (b == 0 && at < MESH_OPEN) s_open[warp][at] = m.entry + e + lane;
+        n += __popc(open);
       }
+      if (n > MESH_OPEN) exact = true;
       if (lane == 0) {
         s_end[warp][q] = n;
         s_odd[warp][q] = (unsigned char)odd;
@@ -227,8 +255,8 @@ __global__ void __launch_bounds__(32 * MESH_WARPS) k_mesh_phi(int nx, int ny, in
       const double px = __dmul_rn(__dadd_rn((double)ci, s_off[pt ? a : 0]), h);
       const double py = __dmul_rn(__dadd_rn((double)cj, s_off[pt ? b : 0]), h);
       const double pz = __dmul_rn(__dadd_rn((double)ck, s_off[pt ? c : 0]), h);
-      for (int q = 0, at = 0; q < n_obj; ++q) {
-        const MeshObject& m = obj[exact && all ? q : s_obj[q]];
+      for (int q = 0, at = 0; q < (over ? n_obj : nl); ++q) {
+        const MeshObject& m = obj[over ? (all ? q : s_obj[q]) : s_cell[warp][q]];
         const bool box = pt && !(px < m.lo[0] || px > m.hi[0] || py < m.lo[1] || py > m.hi[1] || pz < m.lo[2] || pz > m.hi[2]);
         int cross = 0;
         if (exact) {
@@ -244,9 +272,7 @@ __global__ void __launch_bounds__(32 * MESH_WARPS) k_mesh_phi(int nx, int ny, in
             }
         } else {
           const int end = s_end[warp][q];
-          const unsigned int odd = s_odd[warp][q];
-          if (odd == 2) continue;
-          cross = (int)odd;
+          cross = (int)s_odd[warp][q];
           const float lx = (float)((px - m.lo[0]) * m.scale), ly = (float)((py - m.lo[1]) * m.scale), lz = (float)((pz - m.lo[2]) * m.scale);
           for (; at < end; ++at) {
             const int f = s_open[warp][at];
